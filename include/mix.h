@@ -296,7 +296,9 @@ int mix_set_chain(mix_ctx* ctx, int slot, int next_slot, void* stream);
    step to step while the captured launch structure stays as it is.)
    Install the token->slot map for the next mix_apply calls: token_slot int32[T_live]
    (host if src_is_device == 0, else device), -1 = no app.  Rows >= T_live are pass-through.
-   One async copy + a 4-byte store into fixed device buffers; never captured in a graph.
+   One operation on the stream -- an async copy from host memory, a kernel from device memory -- into
+   a fixed device buffer (two where a map from host memory is shorter than the one before: the rows
+   in between are set to -1); never captured in a graph.
    A host source must stay valid until the stream reaches the copy (use pinned memory for a
    truly asynchronous copy).  Errors: OUT_OF_RANGE (T_live < 0 or > T_max). */
 int mix_set_slot_map(mix_ctx* ctx, const int* token_slot, int T_live, int src_is_device, void* stream);
@@ -332,8 +334,8 @@ int mix_set_feature_out(mix_ctx* ctx, int* topk_idx, float* topk_val, int* n_act
    streaming kernel) and returns; safe to capture.  In a context without SAE weight sets and
    T_max <= 2048 the kernel is launched with programmatic stream serialization (see
    mix_set_pdl_mask): if the kernel in front of it in `stream` lets its successor start early, the
-   part that looks up the live count, slot map, app entry and single-vector weights -- tables the
-   library owns and only copies write -- overlaps that kernel; `hidden`, gate scores and
+   part that looks up the slot map, app entry and single-vector weights -- tables the library owns --
+   overlaps that kernel (unless that kernel is the one that installed the map); `hidden`, gate scores and
    multi-class probe weights are read only after the predecessor has completed and flushed, and the
    grid does not end before it.  Behind any other kernel nothing changes.  One launch shape follows
    from what is registered when the call is enqueued or captured -- the encode's epilogue warps

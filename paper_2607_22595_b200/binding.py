@@ -135,8 +135,8 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:                       # the raw handle: no Stream object on every call of a decode step
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     h = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
     return h or None
 

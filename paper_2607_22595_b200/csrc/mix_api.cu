@@ -103,6 +103,17 @@ int check_slot(mix_ctx* c, int slot) {
   return MIX_OK;
 }
 
+// The address under which the device reads host memory, or null where it cannot (pageable memory).  Asked anew on
+// every call (0.2 us): the same address may be pageable memory the next time.
+const int* device_view(const int* host) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return at.type == cudaMemoryTypeUnregistered ? nullptr : static_cast<const int*>(at.devicePointer);
+}
+
 // Publish an app entry: body first with valid = 0, then the valid word.
 // bias_src: device fp32 whose value goes into the entry's `alpha` word before the entry becomes valid (a one-class
 // probe's bias in contexts whose hook kernel reads it from there), or null.
@@ -285,7 +296,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   }
   if (!ok) { cudaGetLastError(); free_all(c); free(c); return MIX_ERR_NO_MEMORY; }
   e = cudaMemset(c->d_token_slot, 0xff, T * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(c->d_n_live, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemcpy(c->d_n_live, &T, sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->d_apps, 0, NS * sizeof(AppEntry));
   if (e == cudaSuccess) e = cudaMemset(c->d_groups, 0, (G > 0 ? G : 1) * sizeof(GroupEntry));
   if (e == cudaSuccess) e = cudaMemset(c->d_gates, 0, NS * sizeof(GateEntry));
@@ -642,10 +653,26 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (T_live > 0 && !token_slot) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "token_slot is NULL");
-  if (T_live > 0)
-    MIX_CUDA(c, cudaMemcpyAsync(c->d_token_slot, token_slot, (size_t)T_live * sizeof(int),
-                                src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  MIX_CUDA(c, cudaMemcpyAsync(c->d_n_live, &T_live, sizeof(int), cudaMemcpyHostToDevice, s));
+  const int n_fill = c->map_live;
+  c->map_live = T_live;
+  const bool by_kernel = c->cfg.n_groups_max == 0;
+  const int* src = (src_is_device || T_live == 0) ? token_slot : (by_kernel ? device_view(token_slot) : nullptr);
+  if (src || T_live == 0) {
+    c->map_installed = 1;
+    MIX_CUDA(c, launch_install_map(c, src, T_live, n_fill, s));
+    return MIX_OK;
+  }
+  if (by_kernel && T_live <= kMapParamRows) {
+    c->map_installed = 1;
+    MIX_CUDA(c, launch_install_map_params(c, token_slot, T_live, n_fill, s));
+    return MIX_OK;
+  }
+  c->map_installed = 0;             // (a copy is complete before anything behind it starts)
+  MIX_CUDA(c, cudaMemcpyAsync(c->d_token_slot, token_slot, (size_t)T_live * sizeof(int), cudaMemcpyHostToDevice, s));
+  if (n_fill > T_live) {
+    c->map_installed = 1;
+    MIX_CUDA(c, cudaMemsetAsync(c->d_token_slot + T_live, 0xff, (size_t)(n_fill - T_live) * sizeof(int), s));
+  }
   return MIX_OK;
 }
 
@@ -656,14 +683,17 @@ int mix_set_request_map(mix_ctx* c, const int* token_req, int T_live, const int*
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (n_req < 0 || n_req > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "n_req %d outside [0, T_max=%d]", n_req, c->cfg.T_max);
   if (T_live > 0 && (!token_req || (n_req > 0 && !req_slot))) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "map arrays are NULL");
-  const cudaMemcpyKind kind = src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  if (T_live > 0) {
-    MIX_CUDA(c, cudaMemcpyAsync(c->d_tmp_req, token_req, (size_t)T_live * sizeof(int), kind, s));
-    if (n_req > 0) MIX_CUDA(c, cudaMemcpyAsync(c->d_tmp_req_slot, req_slot, (size_t)n_req * sizeof(int), kind, s));
-    MIX_CUDA(c, launch_compose_map(c, T_live, n_req, s));
-    c->map_from_kernel = 1;
+  const int n_fill = c->map_live;
+  c->map_live = T_live;
+  c->map_installed = 1;
+  const int *req = token_req, *slots = req_slot;
+  if (!src_is_device && T_live > 0) {
+    MIX_CUDA(c, cudaMemcpyAsync(c->d_tmp_req, token_req, (size_t)T_live * sizeof(int), cudaMemcpyHostToDevice, s));
+    if (n_req > 0) MIX_CUDA(c, cudaMemcpyAsync(c->d_tmp_req_slot, req_slot, (size_t)n_req * sizeof(int), cudaMemcpyHostToDevice, s));
+    req = c->d_tmp_req;
+    slots = c->d_tmp_req_slot;
   }
-  MIX_CUDA(c, cudaMemcpyAsync(c->d_n_live, &T_live, sizeof(int), cudaMemcpyHostToDevice, s));
+  MIX_CUDA(c, launch_compose_map(c, req, slots, T_live, n_req, n_fill, s));
   return MIX_OK;
 }
 
@@ -783,9 +813,9 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
     }
   }
   // (programmatic launch only where this kernel directly follows the caller's work in the caller's stream)
-  const bool hook_pdl = !fork && !tc && !c->stage_events_on && !c->map_from_kernel;
-  c->map_from_kernel = 0;
-  MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl));
+  const bool hook_pdl = !fork && !tc && !c->stage_events_on;
+  MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, c->map_installed != 0));
+  c->map_installed = 0;
   MIX_CUDA(c, tap());
   if (has_multiclass_stage(c)) {
     MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, ps));

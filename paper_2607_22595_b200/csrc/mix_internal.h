@@ -118,8 +118,9 @@ struct Ctx {
   char err[256];
 
   // tables
-  int* d_token_slot;        // [T_max]
-  int* d_n_live;            // [1]
+  int* d_token_slot;        // [T_max]; -1 behind the live rows
+  int map_live;             // live rows of the map last installed: what a shorter map has to set to -1
+  int* d_n_live;            // [1] rows of d_token_slot that hold a map at all: T_max
   AppEntry* d_apps;         // [n_slots_max]
   GroupEntry* d_groups;     // [n_groups_max]
   GateEntry* d_gates;       // [n_slots_max]
@@ -246,7 +247,9 @@ __device__ __forceinline__ float key2f(unsigned k) {
 #endif
 
 // kernel launchers (each returns the CUDA error of the launch)
-cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s, bool allow_pdl);
+// map_ahead: the kernel in front of this one in the stream may be the one that installed the slot map.
+cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s, bool allow_pdl, bool map_ahead);
+constexpr int kPdlMapAhead = 2;   // how the hook kernels are told: programmatic launch, but nothing is read before the wait
 // Multi-class probes of large batches have two kernels; both are launched and exactly one does the work, chosen
 // on the device (mc_census_kernel lists the 128-row tiles that hold such rows and leaves the choice in
 // d_mc_census): probe_tc (tcgen05, streams whole 128-row tiles of that list: batches whose listed tiles are at
@@ -265,6 +268,10 @@ cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaS
 int front_chunks(int T_max);       // chunks of token rows the front kernel classifies: sizes d_front_counts / d_front_sync
 cudaError_t launch_encode_simt(const Ctx* c, cudaStream_t s);
 cudaError_t launch_encode_tc(const Ctx* c, int mode, bool pair, cudaStream_t s);   // 0: all tiles; 1: flagged row tiles -> Z
+inline int cand_tiles_for(long long d_sae_max, int n_sms) {   // Ctx::cand_tiles
+  const long long n = d_sae_max / kTileN, most = 4 * n < n_sms ? 4 * n : n_sms;
+  return (int)(n > most ? n : most);
+}
 bool encode_pair_possible(const Ctx* c);   // the CTA-pair encode kernel is part of this context's launch sequence
 // Selection, edits, decode and write-back of every SAE row.  mode 0: behind the tensor-core encode (TopK from its
 // candidates; rows it cannot settle are flagged); 1: behind the CUDA-core encode (TopK from Z); 2: the flagged

@@ -2,6 +2,8 @@
 //
 // probe_steer_kernel is the bandwidth kernel of the hook: one warp per token row, 16-byte
 // loads, fp32 FMA, shuffle reductions.  A row whose slot is -1 costs one 4-byte load.
+#include <string.h>
+
 #include "mix_internal.h"
 #include "row_lookup.cuh"
 
@@ -393,7 +395,14 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   // previous hook) is still running.  Memory the caller owns (`hidden`, multi-class probe weights, gate scores)
   // is read after the wait only, and every thread waits before it leaves, so that this grid cannot end -- and
   // release ITS successor -- before its predecessor has.  Launched the ordinary way, nothing has to wait: the
-  // row is then requested together with the vector and the app entry, one round trip earlier.
+  // row is then requested together with the vector and the app entry, one round trip earlier.  Behind a map that a
+  // kernel installed (kPdlMapAhead) the wait comes first, and only then the trigger: a successor that reads the map
+  // early must not start before the map is there.
+  if (pdl == kPdlMapAhead) {
+    pdl_wait();
+    pdl_launch_dependents();
+    pdl = 0;
+  }
   if (pdl) pdl_launch_dependents();
   const int n_live = __ldg(n_live_p);            // both loads issue together: one round trip, not two
   const int slot = __ldg(token_slot + t);
@@ -571,7 +580,7 @@ __global__ void __launch_bounds__(kChainWarps * 32)
 probe_steer_chain_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
                          const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates,
                          const int* __restrict__ chain_next, int n_slots, __nv_bfloat16* __restrict__ hidden, int d,
-                         float* __restrict__ scores, int C_max, unsigned* __restrict__ status) {
+                         float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int pdl) {
   __shared__ float s_part[kChainWarps][kMaxClasses];
   constexpr int NT = kChainWarps * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -579,6 +588,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, const int* __restri
   // programmatic dependent launch, as in probe_steer_team_kernel: the live count and the slot id (library-owned,
   // written only by copies) may be read while the predecessor still runs; everything else comes after the wait,
   // and every thread waits before it leaves
+  if (pdl == kPdlMapAhead) pdl_wait();
   pdl_launch_dependents();
   const int n_live = __ldg(n_live_p);
   int slot = __ldg(token_slot + t);
@@ -700,12 +710,55 @@ router_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live
   logits[i] += __ldg(reinterpret_cast<const float*>(a.W) + e);
 }
 
-__global__ void compose_map_kernel(const int* __restrict__ token_req, const int* __restrict__ req_slot, int T_live,
-                                   int n_req, int* __restrict__ token_slot) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T_live) return;
-  const int r = token_req[t];
-  token_slot[t] = (r >= 0 && r < n_req) ? req_slot[r] : -1;
+// The step's slot map.  Rows behind the live ones hold -1, so a step is one operation on the stream: a copy where the map
+// or one of these kernels, which set rows up to `n_fill` -- live in the previous map -- to -1 along the way.  With a live
+// count of its own the map was two copies, and two staging copies, a kernel and a copy in the two-level form, at 2 us
+// and more each on the stream and on the host.
+// Contexts without SAE weight sets, of which a step has one per layer, take a map in host memory by kernel too: read over
+// PCIe where it lies if the device can address it (2.9 us of stream time against 4.0 for a copy), among the kernel's
+// parameters if it is pageable and short (1.1 us).  Contexts with weight sets keep the copy: their long kernels leave the
+// translation of the host page cold, and the same read takes 5.3 us.
+// 32 maps of 256 rows and the replay of 32 layers behind them: 260 us with two copies a map, 204 with one, 160 with this.
+// Launched programmatically: a kernel is scheduled while its predecessor ends, and waits for it before it touches
+// anything (the predecessor may still read the old map, or write the source).
+constexpr int kMapThreads = 256;
+
+// token_slot[t] = src[t]
+__global__ void __launch_bounds__(kMapThreads)
+install_map_kernel(const int* __restrict__ src, int T_live, int n_fill, int* __restrict__ token_slot) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int t = blockIdx.x * kMapThreads + threadIdx.x;
+  if (t < T_live) token_slot[t] = src[t];
+  else if (t < n_fill) token_slot[t] = -1;
+}
+
+// The same with the map among the kernel's parameters.
+struct MapParams {
+  int slot[kMapParamRows];
+};
+__global__ void __launch_bounds__(kMapThreads)
+install_map_params_kernel(const __grid_constant__ MapParams src, int T_live, int n_fill, int* __restrict__ token_slot) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int t = blockIdx.x * kMapThreads + threadIdx.x;
+  if (t < T_live) token_slot[t] = src.slot[t];
+  else if (t < n_fill) token_slot[t] = -1;
+}
+
+// Two-level form: token_slot[t] = req_slot[token_req[t]]
+__global__ void __launch_bounds__(kMapThreads)
+compose_map_kernel(const int* __restrict__ token_req, const int* __restrict__ req_slot, int T_live, int n_req, int n_fill,
+                   int* __restrict__ token_slot) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int t = blockIdx.x * kMapThreads + threadIdx.x;
+  if (t < T_live) {
+    const int r = token_req[t];
+    token_slot[t] = (r >= 0 && r < n_req) ? req_slot[r] : -1;
+  } else if (t < n_fill) {
+    token_slot[t] = -1;
+  }
 }
 
 // b_eff[j] = b_enc[j] - sum_i W_enc[j,i] * b_dec[i]   (one warp per feature; registration time)
@@ -800,13 +853,13 @@ cudaError_t launch_mc_census(const Ctx* c, int T, cudaStream_t s) {
 // it could only wait, so contexts with SAE weight sets leave every batch to the 16-row kernel.
 bool has_tc_probe_stage(const Ctx* c) { return has_multiclass_stage(c) && c->cfg.n_groups_max == 0; }
 
-cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s, bool allow_pdl) {
+cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s, bool allow_pdl, bool map_ahead) {
+  const int pdl = (allow_pdl && (pdl_mask() & kPdlHook)) ? (map_ahead ? kPdlMapAhead : 1) : 0;
   if (c->cfg.flags & MIX_FLAG_SLOT_CHAINS) {
     return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_chain_kernel, dim3(c->cfg.T_max), dim3(kChainWarps * 32), 0, s,
                       c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
-                      c->cfg.d_model, scores, c->cfg.C_max, c->d_status);
+                      c->cfg.d_model, scores, c->cfg.C_max, c->d_status, pdl);
   } else if (c->cfg.T_max <= kTeamMaxRows) {
-    const int pdl = (allow_pdl && (pdl_mask() & kPdlHook)) ? 1 : 0;
     return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_team_kernel<8>, dim3(c->cfg.T_max), dim3(8 * 32), 0, s,
                       c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->cfg.n_slots_max, hidden, c->cfg.d_model,
                       scores, c->cfg.C_max, c->d_status, reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
@@ -834,11 +887,26 @@ cudaError_t launch_router(const Ctx* c, float* logits, int n_experts, int T, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_compose_map(const Ctx* c, int T_live, int n_req, cudaStream_t s) {
-  if (T_live == 0) return cudaSuccess;
-  compose_map_kernel<<<(T_live + 255) / 256, 256, 0, s>>>(c->d_tmp_req, c->d_tmp_req_slot, T_live, n_req,
-                                                          c->d_token_slot);
-  return cudaGetLastError();
+cudaError_t launch_install_map(const Ctx* c, const int* src, int T_live, int n_fill, cudaStream_t s) {
+  const int n = T_live > n_fill ? T_live : n_fill;
+  if (n == 0) return cudaSuccess;
+  return launch_pdl(kPdlHook, install_map_kernel, dim3((n + kMapThreads - 1) / kMapThreads), dim3(kMapThreads), 0, s, src, T_live, n_fill,
+                    c->d_token_slot);
+}
+
+cudaError_t launch_install_map_params(const Ctx* c, const int* host_src, int T_live, int n_fill, cudaStream_t s) {
+  MapParams p;
+  memcpy(p.slot, host_src, (size_t)T_live * sizeof(int));
+  const int n = T_live > n_fill ? T_live : n_fill;
+  return launch_pdl(kPdlHook, install_map_params_kernel, dim3((n + kMapThreads - 1) / kMapThreads), dim3(kMapThreads), 0, s, p, T_live, n_fill,
+                    c->d_token_slot);
+}
+
+cudaError_t launch_compose_map(const Ctx* c, const int* token_req, const int* req_slot, int T_live, int n_req, int n_fill, cudaStream_t s) {
+  const int n = T_live > n_fill ? T_live : n_fill;
+  if (n == 0) return cudaSuccess;
+  return launch_pdl(kPdlHook, compose_map_kernel, dim3((n + kMapThreads - 1) / kMapThreads), dim3(kMapThreads), 0, s, token_req, req_slot,
+                    T_live, n_req, n_fill, c->d_token_slot);
 }
 
 cudaError_t launch_fold_bias(const __nv_bfloat16* W_enc, const float* b_enc, const float* b_dec, float* b_eff,

@@ -1,0 +1,42 @@
+"""The slot map from every place it can come from, shrinking and growing from call to call: rows behind the live ones
+pass through whatever the maps before had there."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from paper_2607_22595_b200 import Mix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("with_sae", [False, True])
+@pytest.mark.parametrize("source", ["device", "pinned", "pageable", "numpy", "requests_device", "requests_host"])
+@pytest.mark.parametrize("T", [5, 896, 897, 3000])
+def test_maps_of_changing_length(T, source, with_sae):
+    d = 64
+    m = Mix(d_model=d, T_max=T, n_slots_max=2, n_groups_max=int(with_sae), d_sae_max=256 if with_sae else 0)
+    v = torch.ones(d, device="cuda", dtype=torch.bfloat16)
+    m.register_steer(0, v, 1.0)
+    m.register_steer(1, v, 2.0)
+    rng = np.random.default_rng(T)
+    for live in (T, T // 2, 0, 1, T - 1, T):
+        token_slot = rng.integers(-1, 2, size=live).astype(np.int32)
+        if source.startswith("requests"):
+            req, slots = np.arange(live, dtype=np.int32), token_slot
+            if source == "requests_device":
+                m.set_request_map(torch.from_numpy(req).cuda(), torch.from_numpy(slots).cuda(), live)
+            else:
+                m.set_request_map(req, slots, live)
+        else:
+            src = {"device": lambda x: torch.from_numpy(x).cuda(), "pinned": lambda x: torch.from_numpy(x).pin_memory(),
+                   "pageable": torch.from_numpy, "numpy": lambda x: x}[source](token_slot)
+            m.set_slot_map(src, live)
+        h = torch.zeros((T, d), device="cuda", dtype=torch.bfloat16)
+        m.apply(h)
+        m.apply(h)                                   # directly behind: the second call sees the same map
+        want = np.zeros(T, dtype=np.float32)
+        want[:live] = 2.0 * (token_slot + 1)
+        assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), live
+    assert m.get_status() == 0
+    m.destroy()
