@@ -177,8 +177,8 @@ struct Ctx {
   cudaEvent_t ev_fork, ev_join;
 
   // profiling taps
-  int map_from_kernel;      // the slot map was last written by compose_map_kernel, not by a copy: the next hook kernel
-                            // must not read it ahead of its predecessor
+  int map_installed;        // a map was installed (by a kernel) since the last call: the next hook kernel must not read it
+                            // ahead of its predecessor
   int stage_events_on;
   cudaEvent_t stage_events[16];
 
@@ -280,7 +280,11 @@ cudaError_t launch_tail(const Ctx* c, __nv_bfloat16* hidden, int mode, cudaStrea
 cudaError_t launch_edit_only(const Ctx* c, __nv_bfloat16* hidden, int T, cudaStream_t s);
 cudaError_t launch_edit_only_delta(const Ctx* c, __nv_bfloat16* hidden, cudaStream_t s);   // decode_delta_kernel on the shortcut's token-indexed records
 cudaError_t edit_only_prepare();   // opt in to the dynamic shared memory of the edit-only kernel
-cudaError_t launch_compose_map(const Ctx* c, int T_live, int n_req, cudaStream_t s);
+// The step's slot map, from memory the device can address or from the host; rows [T_live, n_fill) are set to -1.
+constexpr int kMapParamRows = 896;         // rows of a map that can travel as kernel parameters (3.5 of 4 KiB)
+cudaError_t launch_install_map(const Ctx* c, const int* src, int T_live, int n_fill, cudaStream_t s);
+cudaError_t launch_install_map_params(const Ctx* c, const int* host_src, int T_live, int n_fill, cudaStream_t s);   // 1 <= T_live <= kMapParamRows
+cudaError_t launch_compose_map(const Ctx* c, const int* token_req, const int* req_slot, int T_live, int n_req, int n_fill, cudaStream_t s);
 cudaError_t launch_fold_bias(const __nv_bfloat16* W_enc, const float* b_enc, const float* b_dec, float* b_eff,
                              long long d_sae, int d, cudaStream_t s);
 cudaError_t launch_retile(const __nv_bfloat16* W_enc, __nv_bfloat16* W_tiled, long long d_sae, int d, cudaStream_t s);
