@@ -72,6 +72,20 @@ int make_tmap(CUtensorMap* out, const void* base, unsigned long long rows, int d
   return r == CUDA_SUCCESS ? MIX_OK : MIX_ERR_CUDA;
 }
 
+// The packed panel as the encode reads it: all 128 rows of a tile at once, or 32 at a time.
+int make_panel_tmaps(Ctx* c) {
+  const int d = c->cfg.d_model;
+  const unsigned long long P = c->panel_rows_cap;
+  int rc = MIX_OK;
+  for (int i = 0; i < 2 && rc == MIX_OK; ++i) {
+    CUtensorMap* out = i == 0 ? &c->tmap_panel : &c->tmap_panel_32;
+    const int rows = i == 0 ? kTileM : 32;
+    rc = (c->cfg.flags & MIX_FLAG_FP8_W_ENC) ? make_tmap_e4m3(out, c->d_panel, 2 * P, d, rows)   // codes: P rows (8-bit input) or 2 P rows (hi, lo)
+                                             : make_tmap(out, c->d_panel, P, d, rows);
+  }
+  return rc;
+}
+
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t n) {
   *p = nullptr;
@@ -84,7 +98,7 @@ void free_all(mix_ctx* c) {
   cudaFree(c->d_edit_idx); cudaFree(c->d_edit_val); cudaFree(c->d_edit_mode); cudaFree(c->d_status);
   cudaFree(c->d_tmp_req); cudaFree(c->d_tmp_req_slot); cudaFree(c->d_panel); cudaFree(c->d_panel_row); cudaFree(c->d_act_scale); cudaFree(c->d_tau); cudaFree(c->d_tau_min); cudaFree(c->d_eo_row_delta); cudaFree(c->d_eo_coef);
   cudaFree(c->d_mtile_group); cudaFree(c->d_route); cudaFree(c->d_z);
-  cudaFree(c->d_tmap_w); cudaFree(c->d_tmap_w_half); cudaFree(c->d_phase_clk); cudaFree(c->d_tmap_probe); cudaFree(c->d_mc_census); cudaFree(c->d_mc_tiles); cudaFree(c->d_cand_val); cudaFree(c->d_cand_idx);
+  cudaFree(c->d_tmap_w); cudaFree(c->d_phase_clk); cudaFree(c->d_tmap_probe); cudaFree(c->d_mc_census); cudaFree(c->d_mc_tiles); cudaFree(c->d_cand_val); cudaFree(c->d_cand_idx);
   cudaFree(c->d_cand_ninth); cudaFree(c->d_row_flag); cudaFree(c->d_mtile_flag); cudaFree(c->d_n_flagged);
   if (c->owned_b_eff)
     for (int g = 0; g < c->cfg.n_groups_max; ++g) cudaFree(c->owned_b_eff[g]);
@@ -272,8 +286,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     ok = ok && dev_alloc(&c->d_front_sync, 2) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_route, 1) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_z, P * (size_t)cfg->d_sae_max) == cudaSuccess;
-    ok = ok && dev_alloc(&c->d_tmap_w, G) == cudaSuccess;
-    ok = ok && dev_alloc(&c->d_tmap_w_half, G) == cudaSuccess;
+    ok = ok && dev_alloc(&c->d_tmap_w, 3 * (size_t)G) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_row_rec, P) == cudaSuccess;
     if (getenv("MIX_PHASE_CLOCKS") && atoi(getenv("MIX_PHASE_CLOCKS")))
       ok = ok && dev_alloc(&c->d_phase_clk, 32) == cudaSuccess && cudaMemset(c->d_phase_clk, 0, 32 * sizeof(unsigned long long)) == cudaSuccess;
@@ -282,7 +295,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
       ok = ok && dev_alloc(&c->d_eo_coef, (size_t)T * (size_t)(cfg->r_max > 0 ? cfg->r_max : 1)) == cudaSuccess;
     }
     if (!(cfg->flags & MIX_FLAG_ENCODE_SIMT)) {
-      c->cand_tiles = (int)(cfg->d_sae_max / kTileN);
+      c->cand_tiles = cand_tiles_for(cfg->d_sae_max, c->n_sms);
       const size_t nc = P * (size_t)c->cand_tiles;
       ok = ok && dev_alloc(&c->d_cand_val, nc * kCandPerTile) == cudaSuccess;
       ok = ok && dev_alloc(&c->d_cand_idx, nc * kCandPerTile) == cudaSuccess;
@@ -312,9 +325,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     if (e == cudaSuccess && !(cfg->flags & MIX_FLAG_ENCODE_SIMT)) {
       if (load_encode_fn() != MIX_OK)
         e = cudaErrorUnknown;
-      else if ((cfg->flags & MIX_FLAG_FP8_W_ENC)    // codes: P rows (8-bit input) or 2 P rows (hi, lo) in the same buffer
-                   ? make_tmap_e4m3(&c->tmap_panel, c->d_panel, 2ull * c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK
-                   : make_tmap(&c->tmap_panel, c->d_panel, c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK)
+      else if (make_panel_tmaps(c) != MIX_OK)
         e = cudaErrorUnknown;
       if (e == cudaSuccess && c->d_act_scale) e = cudaMemset(c->d_act_scale, 0, c->panel_rows_cap * sizeof(float));
       if (e == cudaSuccess) e = encode_tc_prepare();
@@ -408,7 +419,8 @@ int mix_register_sae_weights(mix_ctx* c, int group, const mix_sae_weights* w, vo
     ge.b_eff = c->owned_b_eff[group];
   }
   if (!(c->cfg.flags & MIX_FLAG_ENCODE_SIMT)) {
-    CUtensorMap tm, tm_half;       // boxes of 256 features, and of 128 (one CTA's share when a CTA pair works on the tile)
+    CUtensorMap tm[3];             // boxes of 256 features, 128 (also one CTA's share when a CTA pair works on a tile) and 64
+    bool mapped = true;
     if (fp8) {
       // library-owned tile-ordered copy of the codes: [S/256][d/128][256][128] bytes, seen by TMA as a 128-byte-wide
       // matrix (128-byte swizzled boxes of 256 rows)
@@ -420,9 +432,8 @@ int mix_register_sae_weights(mix_ctx* c, int group, const mix_sae_weights* w, vo
       }
       unsigned char* tiled = reinterpret_cast<unsigned char*>(c->owned_w_tiled[group]);
       MIX_CUDA(c, launch_retile_fp8(static_cast<const unsigned char*>(w->W_enc), tiled, w->d_sae, c->cfg.d_model, 2 * kTileK, s));
-      if (make_tmap_e4m3(&tm, tiled, (unsigned long long)(n_el / (2 * kTileK)), 2 * kTileK, kTileN) != MIX_OK ||
-          make_tmap_e4m3(&tm_half, tiled, (unsigned long long)(n_el / (2 * kTileK)), 2 * kTileK, kTileN / 2) != MIX_OK)
-        MIX_FAIL(c, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the 8-bit W_enc");
+      for (int i = 0; i < 3; ++i)
+        mapped = mapped && make_tmap_e4m3(&tm[i], tiled, (unsigned long long)(n_el / (2 * kTileK)), 2 * kTileK, kTileN >> i) == MIX_OK;
     } else if (c->cfg.flags & MIX_FLAG_RETILE_W_ENC) {
       // library-owned tile-contiguous copy: [S/256][d/64][256][64], seen by TMA as a 64-column matrix
       if (c->owned_w_tiled[group]) { cudaStreamSynchronize(s); cudaFree(c->owned_w_tiled[group]); c->owned_w_tiled[group] = nullptr; }
@@ -432,15 +443,15 @@ int mix_register_sae_weights(mix_ctx* c, int group, const mix_sae_weights* w, vo
         MIX_FAIL(c, MIX_ERR_NO_MEMORY, "cannot allocate the re-tiled copy of W_enc");
       }
       MIX_CUDA(c, launch_retile(ge.W_enc, c->owned_w_tiled[group], w->d_sae, c->cfg.d_model, s));
-      if (make_tmap(&tm, c->owned_w_tiled[group], (unsigned long long)(n_el / kTileK), kTileK, kTileN) != MIX_OK ||
-          make_tmap(&tm_half, c->owned_w_tiled[group], (unsigned long long)(n_el / kTileK), kTileK, kTileN / 2) != MIX_OK)
-        MIX_FAIL(c, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the re-tiled W_enc");
-    } else if (make_tmap(&tm, w->W_enc, (unsigned long long)w->d_sae, c->cfg.d_model, kTileN) != MIX_OK ||
-               make_tmap(&tm_half, w->W_enc, (unsigned long long)w->d_sae, c->cfg.d_model, kTileN / 2) != MIX_OK) {
-      MIX_FAIL(c, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed for W_enc");
+      for (int i = 0; i < 3; ++i)
+        mapped = mapped && make_tmap(&tm[i], c->owned_w_tiled[group], (unsigned long long)(n_el / kTileK), kTileK, kTileN >> i) == MIX_OK;
+    } else {
+      for (int i = 0; i < 3; ++i)
+        mapped = mapped && make_tmap(&tm[i], w->W_enc, (unsigned long long)w->d_sae, c->cfg.d_model, kTileN >> i) == MIX_OK;
     }
-    MIX_CUDA(c, cudaMemcpyAsync(c->d_tmap_w + group, &tm, sizeof(tm), cudaMemcpyHostToDevice, s));
-    MIX_CUDA(c, cudaMemcpyAsync(c->d_tmap_w_half + group, &tm_half, sizeof(tm_half), cudaMemcpyHostToDevice, s));
+    if (!mapped) MIX_FAIL(c, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed for W_enc");
+    for (int i = 0; i < 3; ++i)
+      MIX_CUDA(c, cudaMemcpyAsync(c->d_tmap_w + (size_t)i * c->cfg.n_groups_max + group, &tm[i], sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
   }
   c->h_groups[group] = ge;
   GroupEntry tmp = ge;

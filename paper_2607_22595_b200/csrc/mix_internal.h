@@ -105,6 +105,7 @@ struct RouteState {
   int n_topk_rows;                  // SAE rows whose weight set is TopK
   int n_delta_rows;                 // ReLU / JumpReLU rows that keep the error term and have edits (the tail kernel's delta role)
   int use_pair;                     // some weight set of this call is encoded by CTA pairs (256-row tiles)
+  int tile_n;                       // features per tile of the single-CTA kernel this call: kTileN, kTileN / 2 or kTileN / 4
   int pair_mask;                    // bit g: weight set g is the pair kernel's this call, else the single-CTA kernel's
   int group_count[kMaxGroups];      // M_g
   int group_mtile0[kMaxGroups + 1]; // first m-tile of group g in the panel
@@ -154,22 +155,23 @@ struct Ctx {
   RouteState* d_route;
   float* d_z;               // [P, d_sae_max]
   float* d_cand_val;        // [P, cand_tiles, kCandPerTile] per-tile TopK candidates (fused epilogue)
-  int* d_cand_idx;          // same shape: feature ids
+  int* d_cand_idx;          // same shape: feature ids.  ReLU / JumpReLU rows that replace the residual: [d_sae / 32] words, a bit per active feature
   float* d_cand_ninth;      // [P, cand_tiles] the (kCandPerTile+1)-th largest value of each tile
   RowDelta* d_eo_row_delta; // [T_max] edit-only shortcut: per token row, what decode_delta_kernel adds (MIX_FLAG_SAE_EDIT_ONLY)
   float* d_eo_coef;         // [T_max, r_max]
   unsigned* d_tau_min;      // [P] the smallest of the row's first k slots, as last computed by a publisher
   unsigned* d_tau;          // [P, kTauSlots] order-preserving keys of pre-activations seen so far in this call (0 = empty)
-  int cand_tiles;           // d_sae_max / kTileN
+  int cand_tiles;           // tiles a row can have in a call: d_sae_max / kTileN, or as many narrower ones as there are SMs
   int* d_row_flag;          // [P] row needs the exact fallback selection
   int* d_mtile_flag;        // [P / kTileM] some row of the tile is flagged
   int* d_n_flagged;         // [1]
-  CUtensorMap* d_tmap_w;    // [n_groups_max] W_enc maps (box kTileK x kTileN, 128B swizzle)
-  CUtensorMap* d_tmap_w_half;   // [n_groups_max] the same with boxes of kTileN / 2 rows: what one CTA of a pair fetches
+  CUtensorMap* d_tmap_w;    // [3][n_groups_max] W_enc maps (128B swizzle): boxes of kTileN rows, of kTileN / 2 (half-width tiles; what
+                            // one CTA of a pair fetches) and of kTileN / 4
   CUtensorMap* d_tmap_probe;   // [n_slots_max] maps of multi-class probe matrices (box kTileK x 32), large-batch contexts only
   McCensus* d_mc_census;    // census of the 128-row tiles that hold multi-class probe rows, taken by mc_census_kernel every call
   int* d_mc_tiles;          // [ceil(T_max / 128)] those tiles, in no particular order
   CUtensorMap tmap_panel;   // panel map (box kTileK x kTileM, 128B swizzle)
+  CUtensorMap tmap_panel_32;   // the same with boxes of 32 rows: tiles with few valid rows
 
   // probe/steer kernels run beside the SAE chain on this stream (created with the context)
   cudaStream_t side_stream;

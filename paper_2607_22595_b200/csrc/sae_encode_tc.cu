@@ -37,7 +37,7 @@ namespace mix {
 
 namespace {
 
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 8;
 constexpr int kABytes = kTileM * kTileK * 2;   // 16 KiB: 128 rows of 128 bytes
 constexpr int kBBytes = kTileN * kTileK * 2;   // 32 KiB: 256 rows of 128 bytes
 constexpr int kXchgEntries = kCandPerTile + 2;  // a top-9 list and the bound it was collected under
@@ -49,7 +49,8 @@ template <int kEnc, int kEpi, bool kPair> struct TcCfg {
   static_assert(kEpi == 4 || kEpi == 8, "epilogue warps");
   static constexpr bool kSplit = kEnc == 1;            // two panel tiles (hi, lo) per stage
   static constexpr int kBBytesCta = kPair ? kBBytes / 2 : kBBytes;
-  static constexpr int kStageBytes = (kSplit ? 2 : 1) * kABytes + kBBytesCta;
+  static constexpr int kARingBytes = (kSplit ? 2 : 1) * kABytes;      // a stage's panel rows
+  static constexpr int kStageBytes = kARingBytes + kBBytesCta;        // (of a full-width tile; narrower tiles leave room for more stages)
   static constexpr int kStages = kPair ? (kSplit ? 4 : 6) : (kSplit ? 3 : 4);
   static constexpr int kRingBytes = kStages * kStageBytes;
   // epilogue warps: 4 (one per tensor-memory lane quarter, all 256 columns) or 8 (two per quarter, 128 columns
@@ -93,13 +94,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, TcShare
   return mbar_wait_bounded(bar, parity, &sh->abort_flag, &sh->wait_cycles, status);
 }
 
-constexpr unsigned kIdesc = idesc_f16(kTileM, kTileN);     // D fp32, A and B bf16, K-major, N = 256, M = 128
-constexpr unsigned kIdescE4 = idesc_e4m3(kTileM, kTileN);  // D fp32, A and B E4M3, K-major, N = 256, M = 128
 constexpr unsigned kIdescPair = idesc_f16(2 * kTileM, kTileN);     // the pair's instruction: M = 256
 constexpr unsigned kIdescE4Pair = idesc_e4m3(2 * kTileM, kTileN);
 
 struct Tile {
-  int group, n_tile, m_tile_global, rows_valid;
+  int group, n_tile, m_tile_global, rows_valid;      // n_tile: in tiles of this call's width
   int m_tile_peer;      // CTA pairs: the row tile the other CTA of the pair works on (the same one when the weight set has an odd tile left over)
 };
 
@@ -184,22 +183,20 @@ __device__ __forceinline__ void top9_insert(float (&tv)[kCandPerTile + 1], int (
 
 template <int kEnc, int kEpi, bool kPair>
 __global__ void __launch_bounds__(TcCfg<kEnc, kEpi, kPair>::kThreads, 1)
-encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorMap* __restrict__ tmap_w,
-                 const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
+encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_constant__ CUtensorMap tmap_panel_32,
+                 const CUtensorMap* __restrict__ tmap_w, const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
                  float* __restrict__ Z, long long ldz, int d, unsigned* __restrict__ status, int mode,
                  const int* __restrict__ mtile_flag, const int* __restrict__ n_flagged, float* __restrict__ cand_val,
                  int* __restrict__ cand_idx, float* __restrict__ cand_ninth, int cand_tiles, int w_tiled, int test_stall,
                  const float* __restrict__ act_scale, unsigned* __restrict__ tau_slots, unsigned* __restrict__ tau_min,
-                 int lo_row0, unsigned long long* __restrict__ clk) {
+                 int lo_row0, const RowRec* __restrict__ row_rec, unsigned long long* __restrict__ clk) {
   constexpr bool kE4 = kEnc != 0;                      // E4M3 x E4M3 contraction
   constexpr bool kSplit = kEnc == 1;                   // the panel row is hi + lo: two operand tiles per k-block
   constexpr int kBlockK = kE4 ? 2 * kTileK : kTileK;   // elements per 128-byte row of either operand
   using Cfg = TcCfg<kEnc, kEpi, kPair>;
-  constexpr int kStages = Cfg::kStages;
-  constexpr int kStageBytes = Cfg::kStageBytes;
   constexpr int kTcThreads = Cfg::kThreads;
   constexpr int kEpiWarps = Cfg::kEpiWarps;
-  constexpr int kEpiCols = kTileN / (kEpiWarps / 4);   // columns of a tile per epilogue warp
+  constexpr int kEpiColsMax = kTileN / (kEpiWarps / 4);
   pdl_wait();
   pdl_launch_dependents();
   const bool stamp = clk != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && mode == 0 && !kPair;
@@ -223,12 +220,19 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
   for (int i = threadIdx.x; i < (int)(sizeof(RouteState) / sizeof(int)); i += kTcThreads)
     reinterpret_cast<int*>(&sh->rs)[i] = reinterpret_cast<const int*>(rs_g)[i];
   __syncthreads();
+  // Feature width of this call's tiles: 256, or 128 / 64 where full-width tiles would leave half of the SMs or more without
+  // one (decided by the front kernel).  A narrower tile makes a shorter stage, so the ring holds more of them.
+  const int tile_n = kPair ? kTileN : sh->rs.tile_n;
+  const int n_sub = kTileN / tile_n;                   // tiles per 256 features
+  const int stage_bytes = Cfg::kARingBytes + (kPair ? Cfg::kBBytesCta : tile_n * (kTileK * 2));
+  const int n_stages = min(kMaxStages, Cfg::kRingBytes / stage_bytes);
+  const int epi_cols = tile_n / (kEpiWarps / 4);       // columns of a tile per epilogue warp
   if (threadIdx.x == 0) {
     {      // this kernel's weight sets: units (row tiles, or pairs of them) and tiles, numbered through
       int nu = 0, ut = 0;
       for (int g = 0; g < n_groups; ++g) {
         const int mt = sh->rs.group_mtile0[g + 1] - sh->rs.group_mtile0[g];
-        const int nt = mt > 0 ? (sh->rs.group_tile0[g + 1] - sh->rs.group_tile0[g]) / mt : 0;
+        const int nt = mt > 0 ? (sh->rs.group_tile0[g + 1] - sh->rs.group_tile0[g]) / mt * n_sub : 0;
         const bool mine = mode != 0 || (((sh->rs.pair_mask >> g) & 1) != 0) == kPair;
         const int units = !mine ? 0 : (kPair ? (mt + 1) / 2 : mt);
         sh->unit0[g] = (short)nu;
@@ -241,7 +245,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
         sh->utile0[g] = ut;
       }
     }
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < n_stages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
@@ -285,45 +289,57 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
       for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
         const Tile t = tile_of(tile);
         if (!tile_wanted(t, groups, mode, mtile_flag)) continue;
-        const CUtensorMap* tw = tmap_w + t.group;
+        // (boxes of as many W_enc rows as this kernel's tile has: a map array per width)
+        const CUtensorMap* tw = tmap_w + (kPair || n_sub == 2 ? n_groups : (n_sub == 4 ? 2 * n_groups : 0)) + t.group;
+        const int n256 = t.n_tile / n_sub, row_in_256 = kPair ? rank * (kTileN / 2) : (t.n_tile - n256 * n_sub) * tile_n;
+        // panel rows nobody's accumulator row needs are not fetched (32 at a time): a decode batch of 20 rows brings 4 KiB
+        // of panel per k-block into the SM instead of 16.  (What the unfetched shared memory rows hold reaches only
+        // accumulator rows that are never read.)
+        const int n32 = kPair ? 4 : (t.rows_valid + 31) >> 5;
+        const unsigned tx_bytes = stage_bytes - (kSplit ? 2 : 1) * (4 - n32) * (kABytes / 4);
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
           // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumer's
           // bounded wait runs out and the whole CTA leaves through the time-out path.
           if (test_stall) { ok = false; break; }
           const unsigned bar = smem_u32(&sh->full[stage]);
-          const unsigned sa = smem_u32(tiles + stage * kStageBytes);
-          const unsigned sw = sa + (kSplit ? 2 : 1) * kABytes;
+          const unsigned sa = smem_u32(tiles + stage * stage_bytes);
+          const unsigned sw = sa + Cfg::kARingBytes;
+          // W_enc tile: rows n_tile * tile_n .. of the row-major matrix, or -- when the weights were re-laid out at
+          // registration (always, for codes) -- rows of block (n256, kb) of the tile-contiguous copy
+          // [S/256][d/kBlockK][256][kBlockK]
+          const int wx = (kE4 || w_tiled) ? 0 : kb * kTileK;
+          const int wy = ((kE4 || w_tiled) ? n256 * num_kb + kb : n256) * kTileN + row_in_256;
           if (kPair) {
             // both CTAs' copies complete on the LEADER's barrier, which expects the bytes of both; this CTA
             // fetches its own 128 panel rows and its half (128 features) of the W_enc tile
-            if (leader) mbar_expect_tx(bar, 2 * kStageBytes);
+            if (leader) mbar_expect_tx(bar, 2 * stage_bytes);
             const unsigned bar_c = mapa_cluster(bar, 0);
             tma_load_2d_pair(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar_c);
             if (kSplit) tma_load_2d_pair(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar_c);
-            if (kE4 || w_tiled)
-              tma_load_2d_pair(sw, tw, 0, (t.n_tile * num_kb + kb) * kTileN + rank * (kTileN / 2), bar_c);
-            else
-              tma_load_2d_pair(sw, tw, kb * kTileK, t.n_tile * kTileN + rank * (kTileN / 2), bar_c);
+            tma_load_2d_pair(sw, tw, wx, wy, bar_c);
           } else {
-            mbar_expect_tx(bar, kStageBytes);
-            tma_load_2d(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar);
-            if (kSplit) tma_load_2d(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar);   // the lo codes
-            // W_enc tile: rows n_tile*256.. of the row-major matrix, or -- when the weights were re-laid
-            // out at registration (always, for codes) -- block (n_tile, kb) of the tile-contiguous copy
-            // [S/256][d/kBlockK][256][kBlockK]
-            if (kE4 || w_tiled)
-              tma_load_2d(sw, tw, 0, (t.n_tile * num_kb + kb) * kTileN, bar);
-            else
-              tma_load_2d(sw, tw, kb * kTileK, t.n_tile * kTileN, bar);
+            mbar_expect_tx(bar, tx_bytes);
+            if (n32 == 4) {
+              tma_load_2d(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar);
+              if (kSplit) tma_load_2d(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar);   // the lo codes
+            } else {
+              for (int i = 0; i < n32; ++i) {
+                tma_load_2d(sa + i * (kABytes / 4), &tmap_panel_32, kb * kBlockK, t.m_tile_global * kTileM + i * 32, bar);
+                if (kSplit)
+                  tma_load_2d(sa + kABytes + i * (kABytes / 4), &tmap_panel_32, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM + i * 32, bar);
+              }
+            }
+            tma_load_2d(sw, tw, wx, wy, bar);
           }
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
       }
       phase_stamp(clk, 28, stamp);          // the last copy of this CTA has been issued
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {
+      const unsigned idesc = kE4 ? idesc_e4m3(kTileM, tile_n) : idesc_f16(kTileM, tile_n);   // D fp32, operands K-major
       int stage = 0;
       unsigned phase = 0, acc = 0, acc_phase = 0;
       bool ok = true;
@@ -335,8 +351,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(smem_u32(&sh->full[stage]), phase, sh, status)) { ok = false; break; }
           tc_fence_after();
-          const unsigned sa = smem_u32(tiles + stage * kStageBytes);
-          const unsigned sb = sa + (kSplit ? 2 : 1) * kABytes;
+          const unsigned sa = smem_u32(tiles + stage * stage_bytes);
+          const unsigned sb = sa + Cfg::kARingBytes;
           const unsigned long long da = umma_desc(sa), db = umma_desc(sb);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {   // 16 bf16 or 32 codes = 32 bytes = 2 descriptor units per step
@@ -345,8 +361,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
               if (kE4) umma_e4m3_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescE4Pair, accum);
               else umma_f16_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescPair, accum);
             } else {
-              if (kE4) umma_e4m3(d_tmem, da + 2ull * k, db + 2ull * k, kIdescE4, accum);
-              else umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, kIdesc, accum);
+              if (kE4) umma_e4m3(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum);
+              else umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum);
             }
           }
           if (kSplit) {                   // + lo W into the same accumulator
@@ -354,13 +370,13 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               if (kPair) umma_e4m3_pair(d_tmem, dl + 2ull * k, db + 2ull * k, kIdescE4Pair, 1u);
-              else umma_e4m3(d_tmem, dl + 2ull * k, db + 2ull * k, kIdescE4, 1u);
+              else umma_e4m3(d_tmem, dl + 2ull * k, db + 2ull * k, idesc, 1u);
             }
           }
           // the stage is free again -- in both CTAs of a pair
           if (kPair) umma_commit_pair(smem_u32(&sh->empty[stage]));
           else umma_commit(smem_u32(&sh->empty[stage]));
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
         if (kPair) umma_commit_pair(smem_u32(&sh->tmem_full[acc]));
@@ -372,7 +388,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
   } else {
     const int q = warp & 3;                  // tensor-memory lane quarter this warp may read
     const int half = (warp - 2) >> 2;        // 8 epilogue warps: which 128 columns of the tile
-    const int c_lo = half * kEpiCols;
+    const int c_lo = half * epi_cols;
     unsigned acc = 0, acc_phase = 0;
     unsigned xchg_phase = 0;                 // bit a: phase of the next hand-over through xchg_full[a][q] (TopK tiles only)
     for (int tile = worker; tile < total_tiles; tile += n_workers) {
@@ -402,14 +418,14 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
       // against 210 us.  Asking one tile ahead, the vectors held in registers meanwhile, was slower still: 256 us.)
       constexpr bool kScaled = kEnc != 0;      // the accumulator is in units of the codes
       constexpr bool kStageVec = !(kEnc == 2 && kEpi == 8);
-      float* wb = epi_vec + (warp - 2) * kEpiCols;
-      float* ws = wb + kEpiWarps * kEpiCols;
-      const float* bias_t = groups[t.group].b_eff + (size_t)t.n_tile * kTileN + c_lo;
-      const float* wsc_t = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * kTileN + c_lo : nullptr;
+      float* wb = epi_vec + (warp - 2) * kEpiColsMax;
+      float* ws = wb + kEpiWarps * kEpiColsMax;
+      const float* bias_t = groups[t.group].b_eff + (size_t)t.n_tile * tile_n + c_lo;
+      const float* wsc_t = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * tile_n + c_lo : nullptr;
       if (kStageVec) {
-        const float* bias_g = groups[t.group].b_eff + (size_t)t.n_tile * kTileN + c_lo;
-        const float* wsc_g = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * kTileN + c_lo : nullptr;
-        for (int j = lane * 4; j < kEpiCols; j += 128) {
+        const float* bias_g = groups[t.group].b_eff + (size_t)t.n_tile * tile_n + c_lo;
+        const float* wsc_g = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * tile_n + c_lo : nullptr;
+        for (int j = lane * 4; j < epi_cols; j += 128) {
           *reinterpret_cast<float4*>(wb + j) = __ldg(reinterpret_cast<const float4*>(bias_g + j));
           if (kScaled) *reinterpret_cast<float4*>(ws + j) = __ldg(reinterpret_cast<const float4*>(wsc_g + j));
         }
@@ -432,7 +448,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
           ti[s] = 0;
         }
 #pragma unroll 1
-        for (int c = c_lo; c < c_lo + kEpiCols; c += 32) {
+        for (int c = c_lo; c < c_lo + epi_cols; c += 32) {
           float v[32];
           tmem_ld32(taddr + c, v);
 #pragma unroll
@@ -483,7 +499,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
           const size_t slot = p * (size_t)cand_tiles + (size_t)t.n_tile;
           float4* cv = reinterpret_cast<float4*>(cand_val + slot * kCandPerTile);
           int4* ci = reinterpret_cast<int4*>(cand_idx + slot * kCandPerTile);
-          const int j0 = t.n_tile * kTileN;
+          const int j0 = t.n_tile * tile_n;
           cv[0] = make_float4(tv[0], tv[1], tv[2], tv[3]);
           cv[1] = make_float4(tv[4], tv[5], tv[6], tv[7]);
           ci[0] = make_int4(j0 + ti[0], j0 + ti[1], j0 + ti[2], j0 + ti[3]);
@@ -520,9 +536,22 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
           }
         }
       } else {
-        float* out = Z + p * (size_t)ldz + (size_t)t.n_tile * kTileN;
+        float* out = Z + p * (size_t)ldz + (size_t)t.n_tile * tile_n;
+        // For rows that are rebuilt from their active features, which of the tile's are active goes beside Z, a bit each:
+        // the tail kernel then reads 3 KiB per row of 24576 features, and of Z what is active, instead of 100 KiB of Z and
+        // as much of theta.  (Lists of the active values instead of bits took this epilogue from 11 us a tile to 20.)
+        const bool want_bits = mode == 0 && valid && !(row_rec[p].group_flags & kRecAddError);
+        const bool any_bits = __any_sync(0xffffffffu, want_bits);
+        const bool jump = any_bits && groups[t.group].act == MIX_SAE_JUMPRELU;
+        const float* theta_t = jump ? groups[t.group].theta + (size_t)t.n_tile * tile_n + c_lo : nullptr;
+        float* wt = kScaled || !kStageVec ? nullptr : ws;       // (the scale's place is free where there is no scale)
+        if (jump && wt != nullptr) {
+          for (int j = lane * 4; j < epi_cols; j += 128) *reinterpret_cast<float4*>(wt + j) = __ldg(reinterpret_cast<const float4*>(theta_t + j));
+          __syncwarp();
+        }
+        unsigned* bits = reinterpret_cast<unsigned*>(cand_idx) + p * (size_t)cand_tiles * kCandPerTile + t.n_tile * (tile_n / 32);
 #pragma unroll 1
-        for (int c = c_lo; c < c_lo + kEpiCols; c += 32) {
+        for (int c = c_lo; c < c_lo + epi_cols; c += 32) {
           float v[32];
           tmem_ld32(taddr + c, v);
           if (valid) {
@@ -540,7 +569,22 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const CUtensorM
               o.z = kScaled ? fmaf(v[i + 2], s4.z, b4.z) : v[i + 2] + b4.z;
               o.w = kScaled ? fmaf(v[i + 3], s4.w, b4.w) : v[i + 3] + b4.w;
               *reinterpret_cast<float4*>(out + c + i) = o;
+              v[i] = o.x; v[i + 1] = o.y; v[i + 2] = o.z; v[i + 3] = o.w;
             }
+          }
+          if (any_bits) {
+            unsigned m = 0u;
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+              float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (jump) t4 = wt != nullptr ? *reinterpret_cast<const float4*>(wt + (c - c_lo) + i)
+                                           : __ldg(reinterpret_cast<const float4*>(theta_t + (c - c_lo) + i));
+              if (v[i] > t4.x && v[i] != 0.f) m |= 1u << i;
+              if (v[i + 1] > t4.y && v[i + 1] != 0.f) m |= 2u << i;
+              if (v[i + 2] > t4.z && v[i + 2] != 0.f) m |= 4u << i;
+              if (v[i + 3] > t4.w && v[i + 3] != 0.f) m |= 8u << i;
+            }
+            if (want_bits) bits[c >> 5] = m;
           }
         }
       }
@@ -681,14 +725,13 @@ static cudaError_t launch_encode_tc_as(const Ctx* c, int mode, cudaStream_t s) {
   }
   cfg.attrs = at;
   cfg.numAttrs = n_at;
-  const CUtensorMap* tmap_w = kPair ? c->d_tmap_w_half : c->d_tmap_w;
-  return cudaLaunchKernelEx(&cfg, encode_tc_kernel<kEnc, kEpi, kPair>, c->tmap_panel, tmap_w,
+  return cudaLaunchKernelEx(&cfg, encode_tc_kernel<kEnc, kEpi, kPair>, c->tmap_panel, c->tmap_panel_32, static_cast<const CUtensorMap*>(c->d_tmap_w),
                             static_cast<const RouteState*>(c->d_route), static_cast<const GroupEntry*>(c->d_groups),
                             c->cfg.n_groups_max, c->d_z, (long long)c->cfg.d_sae_max, c->cfg.d_model, c->d_status, mode,
                             static_cast<const int*>(c->d_mtile_flag), static_cast<const int*>(c->d_n_flagged), c->d_cand_val,
                             c->d_cand_idx, c->d_cand_ninth, c->cand_tiles, w_tiled, stall,
                             static_cast<const float*>(c->d_act_scale), c->d_tau, c->d_tau_min, c->panel_rows_cap,
-                            c->d_phase_clk);
+                            static_cast<const RowRec*>(c->d_row_rec), c->d_phase_clk);
 }
 
 // Eight epilogue warps pay off for the TopK epilogue (selection work per element); the plain store of the

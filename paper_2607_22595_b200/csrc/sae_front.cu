@@ -22,15 +22,13 @@ namespace {
 constexpr int kFrontThreads = 256;        // = token rows a CTA classifies
 constexpr int kFrontWarps = kFrontThreads / 32;   // = panel rows a CTA packs
 
-// bf16 row -> panel row (or zeros for the padding rows of a tile: they must be finite).
+// bf16 row -> panel row.  (The padding rows of a tile keep what they hold: an accumulator row depends on its own panel
+// row alone, and those of padding rows are never read.)
 __device__ __forceinline__ void pack_row_bf16(const __nv_bfloat16* __restrict__ hidden, int t, __nv_bfloat16* __restrict__ panel,
                                               size_t p, int d, int lane) {
   uint4* dst = reinterpret_cast<uint4*>(panel + p * d);
   const int nvec = d >> 3;
-  if (t < 0) {
-    for (int i = lane; i < nvec; i += 32) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
+  if (t < 0) return;
   const uint4* src = reinterpret_cast<const uint4*>(hidden + (size_t)t * d);
   for (int i = lane; i < nvec; i += 256) {               // eight loads in flight per lane, the ragged end included
     uint4 q[8];
@@ -59,14 +57,7 @@ __device__ __forceinline__ void pack_row_e4m3(const __nv_bfloat16* __restrict__ 
   uint2* dst = reinterpret_cast<uint2*>(panel + p * d);
   uint2* dst_lo = reinterpret_cast<uint2*>(panel + ((size_t)lo_row0 + p) * d);
   const int nvec = d >> 3;
-  if (t < 0) {   // padding rows of a tile
-    for (int i = lane; i < nvec; i += 32) {
-      dst[i] = make_uint2(0u, 0u);
-      if (kSplit) dst_lo[i] = make_uint2(0u, 0u);
-    }
-    if (lane == 0) act_scale[p] = 0.f;
-    return;
-  }
+  if (t < 0) return;
   const uint4* src = reinterpret_cast<const uint4*>(hidden + (size_t)t * d);
   unsigned m2 = 0u;                                     // two 15-bit magnitudes, compared as integers
   for (int i = lane; i < nvec; i += 32) {
@@ -138,6 +129,8 @@ struct FrontArgs {
   unsigned* tau_min;
   int lo_row0;
   unsigned long long* clk;   // profiling aid or null
+  int n_sms;
+  int cand_tiles;
   int pair_mode;             // 0: the encode runs on single CTAs, 1: on CTA pairs, 2: decided here from the routing result
 };
 
@@ -359,6 +352,19 @@ front_kernel(const FrontArgs a) {
           if (split_pays && split_total <= min(cost_single, cost_pair)) mask = split_mask;
           else mask = cost_pair < cost_single ? live_mask : 0;
         }
+        // A call with few tiles -- one dictionary of 16384 features is 64 -- leaves SMs without one, and the pass takes as
+        // long as one SM needs to stream a tile: tiles of 128 or 64 features then, as long as every SM gets at most one.
+        // (Pairs give way only where single CTAs can go down to 64: at 128 both forms bring the same bytes into an SM per
+        // k-block.)  91 rows, d = 4096, 16384 features: encode 50 us with 64 tiles, see encode_tc_kernel for what it is now.
+        int tile_n = kTileN;
+        if (a.pair_mode != 1 && 4 * tiles <= a.n_sms) mask = 0;
+        if (mask == 0) {
+          int nt_most = 1;
+          for (int q = 0; q < n_groups; ++q)
+            if (s_total[q] > 0) nt_most = max(nt_most, s_gtiles[q]);
+          for (int n = tiles; tile_n > kTileN / 4 && 2 * n <= a.n_sms && 2 * nt_most <= a.cand_tiles; n *= 2, nt_most *= 2) tile_n /= 2;
+        }
+        a.rs->tile_n = tile_n;
         a.rs->pair_mask = mask;
         a.rs->use_pair = mask != 0;
         if (a.n_flagged) *a.n_flagged = 0;       // fallback-selection flags of the fused TopK path start clear every call
@@ -411,7 +417,7 @@ front_kernel(const FrontArgs a) {
             }
           }
         }
-        if (a.tau_slots) {                               // the encode's TopK bound starts empty
+        if (a.tau_slots && t >= 0) {                     // the encode's TopK bound starts empty
           reinterpret_cast<uint4*>(a.tau_slots + (size_t)p * kTauSlots)[lane] = make_uint4(0u, 0u, 0u, 0u);
           if (lane == 0) a.tau_min[p] = 0u;
         }
@@ -490,6 +496,8 @@ cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaS
   a.tau_min = c->d_tau_min;
   a.lo_row0 = c->panel_rows_cap;
   a.clk = c->d_phase_clk;
+  a.n_sms = c->n_sms;
+  a.cand_tiles = c->cand_tiles;
   a.pair_mode = ((c->cfg.flags & MIX_FLAG_ENCODE_SIMT) || !encode_pair_possible(c)) ? 0 : encode_pair_mode(-1);
   const int chunks = front_chunks(T);
   const size_t smem = (size_t)front_chunks(c->cfg.T_max) * (c->cfg.n_groups_max + 1) * sizeof(int);

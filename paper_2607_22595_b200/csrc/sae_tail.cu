@@ -142,7 +142,7 @@ __device__ __forceinline__ void scan_keys(const Src& src, int n, int n_up, F&& f
 struct SelShared {
   __align__(16) int hist[kBins];            // radix histogram; afterwards the output of the counting sort (kBins / 2 composites)
   unsigned long long cand[kCand];
-  int n, res[2], count;
+  int n, res[2];
 };
 
 // Append `c` to sh.cand for every thread whose `take` is set: one shared-memory atomic per warp
@@ -429,16 +429,142 @@ struct TailArgs {
 struct RowShared {
   SelShared sel;
   __align__(16) unsigned keys[kCandMax];  // a TopK row's candidate keys (the radix passes run on shared memory)
+  int warp_n[kTailThreads / 32];          // entries of each warp's list
+  int count;
   GroupEntry grp[kMaxGroups];             // the weight-set table, fetched once per CTA
   float coef[kDecList];
   int feat[kDecList];
   int eidx[kMaxEdits];
   float ef[kMaxEdits];      // f_j of each edited feature before the edit
   float enew[kMaxEdits];    // f'_j
-  int n_list;
   int cum[kMaxGroups + 1];  // SAE rows in the weight sets before each one: work index -> packed row, padding rows skipped
   int row0[kMaxGroups];     // first packed row of each weight set
 };
+
+
+// Columns of one row from a list: h[v] = start + sum_e coef[e] W_dec[feat[e]], start = h itself (b_dec == nullptr and add) or
+// b_dec (or 0).  Passes of 256 vectors: first_pass, first_pass + pass_step, ...  A last pass of 128 vectors or fewer would
+// leave most of the CTA idle for as long as a full one takes (d = 2304 is 288 vectors: 31 rounds of loads instead of 16), so
+// there 2, 4 or 8 groups of threads take a part of the list each and the partial sums meet in shared memory (`part`).
+// Every thread of the CTA must call this.
+__device__ void gather_row(const float* coef, const int* feat, int n, const __nv_bfloat16* __restrict__ W_dec, int d, bool add,
+                           const float* __restrict__ b_dec, uint4* __restrict__ hrow, int first_pass, int pass_step, float* part) {
+  const int tid = threadIdx.x, nvec = d >> 3;
+  for (int v0 = first_pass * kTailThreads; v0 < nvec; v0 += pass_step * kTailThreads) {
+    const int rem = nvec - v0;
+    const bool split = rem <= kTailThreads / 2 && n > kGatherBatch;
+    const int cols = split ? (rem <= 32 ? 32 : (rem <= 64 ? 64 : 128)) : kTailThreads;
+    const int n_grp = kTailThreads / cols, grp = tid / cols, vl = tid - grp * cols, v = v0 + vl;
+    const bool in = vl < rem;
+    float acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    if (in && grp == 0) {
+      if (add) {
+        load8(acc, hrow[v]);
+      } else if (b_dec) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i] = b_dec[v * 8 + i];
+      }
+    }
+    const int e0 = n * grp / n_grp, e1 = n * (grp + 1) / n_grp;
+    gather_list(acc, coef + e0, feat + e0, e1 - e0, W_dec, d, v, in);
+    if (split) {
+      float4* p4 = reinterpret_cast<float4*>(part);
+      __syncthreads();
+      if (grp > 0) {
+        p4[((grp - 1) * cols + vl) * 2] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        p4[((grp - 1) * cols + vl) * 2 + 1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+      }
+      __syncthreads();
+      if (grp == 0) {
+        for (int g = 0; g < n_grp - 1; ++g) {
+          const float4 x = p4[(g * cols + vl) * 2], y = p4[(g * cols + vl) * 2 + 1];
+          acc[0] += x.x; acc[1] += x.y; acc[2] += x.z; acc[3] += x.w;
+          acc[4] += y.x; acc[5] += y.y; acc[6] += y.z; acc[7] += y.w;
+        }
+      }
+    }
+    if (in && grp == 0) hrow[v] = pack8(acc);
+  }
+}
+
+// A ReLU / JumpReLU row that is rebuilt from its features: h' = b_dec + edited entries (already in coef / feat) + active,
+// unedited features.  The encode left a bit per feature; the threads share the row's words, number their set bits through
+// (ids ascending), fetch those pre-activations, and the list is gathered.  A row with more active features than the list
+// holds is done 1024 features at a time, adding to what is in registers.  (Behind the CUDA-core encode the words are made
+// here, from Z.)
+// Bound by the gather: a row with 110 active features reads 110 decoder rows, out of L2 where W_dec fits.  1000 rows of
+// d = 2304, 24576 features, 0.4 % active: 480 us in the first form (a scan of Z and theta for every 2048 columns, in chunks
+// of 1024 with three barriers and a gather each), 245 us scanning once, 205 us from the bits, 118 us with the last pass split.
+__device__ void rebuild_row(const TailArgs& a, RowShared& sh, int p, const float* z, const float* theta, const float* b_dec,
+                            const __nv_bfloat16* W_dec, uint4* hrow, int S, int act, int n_edit, float* coef, int* feat) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int d = a.d, nvec = d >> 3, n_words = S / 32;
+  const unsigned* bits = reinterpret_cast<const unsigned*>(a.cand_idx) + (size_t)p * a.cand_tiles * kCandPerTile;
+  const bool from_bits = a.mode == kTailCand;
+  auto word = [&](int w) -> unsigned {
+    if (from_bits) return bits[w];
+    unsigned m = 0u;
+    for (int i = 0; i < 32; ++i) {
+      const float x = z[w * 32 + i];
+      if (x > (act == MIX_SAE_JUMPRELU ? theta[w * 32 + i] : 0.f) && x != 0.f) m |= 1u << i;
+    }
+    return m;
+  };
+  // entries for the set bits of words [w0, w1), behind the n_edit entries of the edits; their number (nothing is written
+  // if it exceeds the list)
+  auto list_words = [&](int w0, int w1) -> int {
+    int cnt = 0;
+    for (int w = w0 + tid; w < w1; w += kTailThreads) cnt += __popc(word(w));
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    __syncthreads();
+    if (lane == 31) sh.warp_n[warp] = incl;
+    __syncthreads();
+    int pos = n_edit + incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < kTailThreads / 32; ++w) {
+      const int c = sh.warp_n[w];
+      pos += w < warp ? c : 0;
+      total += c;
+    }
+    if (total > kDecList - kMaxEdits) return total;
+    for (int w = w0 + tid; w < w1; w += kTailThreads)
+      for (unsigned m = cnt > 0 ? word(w) : 0u; m != 0u; m &= m - 1u) {
+        const int f = w * 32 + __ffs(m) - 1;
+        float x = z[f];
+        for (int k = 0; k < n_edit; ++k) x = sh.eidx[k] == f ? 0.f : x;         // edited features have entries of their own
+        coef[pos] = x;
+        feat[pos] = f;
+        ++pos;
+      }
+    __syncthreads();
+    return total;
+  };
+  const int total = list_words(0, n_words);
+  if (total <= kDecList - kMaxEdits) {
+    gather_row(coef, feat, n_edit + total, W_dec, d, false, b_dec, hrow, 0, 1, reinterpret_cast<float*>(sh.keys));
+    return;
+  }
+  for (int v0 = 0; v0 < nvec; v0 += kTailThreads) {
+    const int v = v0 + tid;
+    const bool in = v < nvec;
+    float acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = (b_dec && in) ? b_dec[v * 8 + i] : 0.f;
+    gather_list(acc, coef, feat, n_edit, W_dec, d, v, in);
+    for (int w0 = 0; w0 < n_words; w0 += 32) {                // 1024 features always fit
+      const int n = list_words(w0, min(w0 + 32, n_words));
+      gather_list(acc, coef + n_edit, feat + n_edit, n, W_dec, d, v, in);
+    }
+    if (in) hrow[v] = pack8(acc);
+  }
+}
 
 
 // Row role.  Per row, the dependent round trips are: the row's record; then -- requested together -- the edit
@@ -505,10 +631,10 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
     }
     const int S = (int)gp->d_sae, k = gp->k;
     const float* z = a.Z + (size_t)p * a.ldz;
-    const int n_tiles = S / kTileN, n_cand = n_tiles * kCandPerTile;
+    const int n_tiles = S / a.rs->tile_n, n_cand = n_tiles * kCandPerTile;
     unsigned ninth_max = 0u;                           // largest key among this thread's share of the tiles' 9th values
     unsigned kmin = 0xffffffffu, kmax = 0u;            // range of this thread's share of the candidate keys
-    if (from_cand && n_cand >= k) {
+    if (from_cand && n_cand >= k && n_cand <= kCandMax) {
       // (16-byte pieces, four in flight per thread: 4096 candidates are one round trip)
       const float4* cv = reinterpret_cast<const float4*>(a.cand_val + (size_t)p * a.cand_tiles * kCandPerTile);
       const int n_vec = n_cand >> 2;
@@ -544,7 +670,7 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
         // candidates are the row's TopK unless some tile's 9th value reaches the k-th candidate, i.e. that tile
         // may hide a winner (or an exact tie whose order matters): such rows are flagged, their row tiles are
         // re-encoded to Z and the fallback launch selects exactly.
-        bool flag = n_cand < k;                        // uniform
+        bool flag = n_cand < k || n_cand > kCandMax;   // uniform
         if (!flag) {
           CandRow src{sh.keys, n_cand};
           flag = radix_collect<false, 8>(src, k, sh.sel, true, kmin, kmax, a.clk, stamp) == 0;
@@ -582,7 +708,7 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
       }
       __syncthreads();
       phase_stamp(a.clk, 12, stamp);
-      if (part == 0) emit_topk(win_id, win_val, k, a.k_max, t, a.out_idx, a.out_val, a.out_n_active, &sh.sel.count);
+      if (part == 0) emit_topk(win_id, win_val, k, a.k_max, t, a.out_idx, a.out_val, a.out_n_active, &sh.count);
     } else {
       if (a.out_n_active != nullptr) {
         int cnt = 0;
@@ -591,12 +717,12 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
           const float v = z[j];
           cnt += act == MIX_SAE_RELU ? v > 0.f : (v > theta[j] && v > 0.f);
         }
-        if (tid == 0) sh.sel.count = 0;
+        if (tid == 0) sh.count = 0;
         __syncthreads();
         cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if ((tid & 31) == 0) atomicAdd(&sh.sel.count, cnt);
+        if ((tid & 31) == 0) atomicAdd(&sh.count, cnt);
         __syncthreads();
-        if (tid == 0) a.out_n_active[t] = sh.sel.count;
+        if (tid == 0) a.out_n_active[t] = sh.count;
       }
       if (add_error) {                                 // the delta role's row
         __syncthreads();
@@ -623,12 +749,7 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
       }
       phase_stamp(a.clk, 13, stamp);
       if (__syncthreads_or(delta != 0.f)) {            // no effective edit: the row stays as it is, bit for bit
-        for (int v = part * kTailThreads + tid; v < nvec; v += n_split * kTailThreads) {
-          float acc[8];
-          load8(acc, hrow[v]);
-          gather_list(acc, sh.coef, sh.feat, n_edit, W_dec, d, v, true);
-          hrow[v] = pack8(acc);
-        }
+        gather_row(sh.coef, sh.feat, n_edit, W_dec, d, true, nullptr, hrow, part, n_split, reinterpret_cast<float*>(sh.keys));
       }
       __syncthreads();
       phase_stamp(a.clk, 14, stamp);
@@ -651,48 +772,9 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
         win_id[i] = in_range ? j : 0;
       }
       __syncthreads();
-      for (int v = part * kTailThreads + tid; v < nvec; v += n_split * kTailThreads) {
-        float acc[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = b_dec ? b_dec[v * 8 + i] : 0.f;
-        gather_list(acc, sh.coef, sh.feat, n_edit + k, W_dec, d, v, true);
-        hrow[v] = pack8(acc);
-      }
+      gather_row(sh.coef, sh.feat, n_edit + k, W_dec, d, false, b_dec, hrow, part, n_split, reinterpret_cast<float*>(sh.keys));
     } else {
-      // ReLU / JumpReLU: per pass of 2048 columns, the edited features first, then a dense scan of the
-      // activations in chunks of 1024 -- active, unedited features are compacted into shared memory and
-      // applied chunk by chunk.  (Every thread walks every pass: the scan needs the whole CTA.)
-      const float* theta = gp->theta;
-      for (int v0 = 0; v0 < nvec; v0 += kTailThreads) {
-        const int v = v0 + tid;
-        const bool in_cols = v < nvec;
-        float acc[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = (b_dec && in_cols) ? b_dec[v * 8 + i] : 0.f;
-        __syncthreads();
-        gather_list(acc, sh.coef, sh.feat, n_edit, W_dec, d, v, in_cols);
-        for (int c0 = 0; c0 < S; c0 += 1024) {
-          if (tid == 0) sh.n_list = 0;
-          __syncthreads();
-          for (int j = c0 + tid; j < min(S, c0 + 1024); j += kTailThreads) {
-            const float zj = z[j];
-            const float f = act == MIX_SAE_RELU ? fmaxf(zj, 0.f) : (zj > theta[j] ? zj : 0.f);
-            if (f != 0.f) {
-              bool edited = false;
-              for (int e = 0; e < n_edit; ++e) edited = edited || (sh.eidx[e] == j);
-              if (!edited) {
-                const int pos = atomicAdd(&sh.n_list, 1);
-                sh.coef[kMaxEdits + pos] = f;
-                sh.feat[kMaxEdits + pos] = j;
-              }
-            }
-          }
-          __syncthreads();
-          gather_list(acc, sh.coef + kMaxEdits, sh.feat + kMaxEdits, sh.n_list, W_dec, d, v, in_cols);
-          __syncthreads();
-        }
-        if (in_cols) hrow[v] = pack8(acc);
-      }
+      rebuild_row(a, sh, p, z, gp->theta, b_dec, W_dec, hrow, S, act, n_edit, sh.coef, sh.feat);
     }
     __syncthreads();                                   // the shared lists are reused by the next row
   }

@@ -1,0 +1,63 @@
+"""Encode tiles narrower than 256 features, panel tiles with few rows, and rows rebuilt from their active features, at the
+sizes where the splits change."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+from parity import check_parity, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(d, S, T, act, add_error, k=24, fp8=None, n_sets=1, b_enc_mean=-0.1, seed=0, extra_topk=False):
+    g = torch.Generator(device="cuda"); g.manual_seed(seed + S + T)
+    rng = np.random.default_rng(seed)
+    hidden = torch.randn((T, d), generator=g, device="cuda").to(torch.bfloat16)
+    groups = {i: W.make_sae_weights(g, "cuda", d, S, act, k=k if act == W.SAE_TOPK else 0, theta_range=(0.05, 0.3), b_enc_mean=b_enc_mean,
+                                    fp8=fp8 is not None) for i in range(n_sets)}
+    if extra_topk:                                            # registered, no rows: the encode runs with eight epilogue warps
+        groups[n_sets] = W.make_sae_weights(g, "cuda", d, 256, W.SAE_TOPK, k=4, fp8=fp8 is not None)
+    apps = {i: W.SaeApp(i, rng.choice(S, 3, replace=False).astype(np.int32), np.array([4.0, 0.0, 2.0], np.float32),
+                        np.array([0, 1, 0], np.uint8), add_error) for i in range(n_sets)}
+    token_slot = (np.arange(T) * n_sets // T).astype(np.int32)
+    return W.Workload("tiles", d, T, T, hidden, token_slot, apps, groups, n_slots_max=n_sets, n_groups_max=len(groups), C_max=1,
+                      k_max=k, r_max=3, d_sae_max=S, fp8_act=fp8 == "input")
+
+
+# features -> tiles of 256: 4 (width 64), 37 (64: 148 tiles), 38 (128), 74 (128), 75 (256); two sets halve the room
+@pytest.mark.parametrize("S,n_sets", [(1024, 1), (37 * 256, 1), (38 * 256, 1), (74 * 256, 1), (75 * 256, 1), (18 * 256, 2), (19 * 256, 2)])
+@pytest.mark.parametrize("act", [W.SAE_TOPK, W.SAE_JUMPRELU])
+def test_tile_widths(S, n_sets, act):
+    w = _workload(128, S, 50, act, True, n_sets=n_sets)
+    check_parity(W.host(w), run_gpu(w))
+
+
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 64, 96, 97, 127, 128, 129, 193, 256, 300])
+@pytest.mark.parametrize("fp8", [None, "weights", "input"])
+def test_rows_of_a_tile(T, fp8):
+    w = _workload(256, 2048, T, W.SAE_TOPK, False, fp8=fp8)
+    flags = {None: 0, "weights": 32, "input": 96}[fp8]
+    check_parity(W.host(w), run_gpu(w, flags=flags, graph=True, replays=2))
+
+
+# widths: one vector pass, and a last pass of 32, 64, 96, 128 and 160 vectors
+@pytest.mark.parametrize("d", [64, 2048, 2304, 2560, 2816, 3072, 3328])
+@pytest.mark.parametrize("act", [W.SAE_RELU, W.SAE_JUMPRELU])
+@pytest.mark.parametrize("extra_topk", [False, True])
+def test_rebuilt_rows(d, act, extra_topk):
+    w = _workload(d, 2048, 20, act, False, b_enc_mean=-1.8, extra_topk=extra_topk)
+    check_parity(W.host(w), run_gpu(w))
+
+
+def test_rebuilt_rows_with_more_active_features_than_a_list_holds():
+    w = _workload(320, 4096, 9, W.SAE_RELU, False, b_enc_mean=0.1)
+    out = run_gpu(w)
+    assert out["n_active"].min() > 1100
+    check_parity(W.host(w), out)
+
+
+def test_rebuilt_rows_on_cta_pairs():
+    w = _workload(320, 10240, 256, W.SAE_JUMPRELU, False, b_enc_mean=-2.0)
+    check_parity(W.host(w), run_gpu(w))
