@@ -61,31 +61,6 @@ int make_tmap_e4m3(CUtensorMap* out, const void* base, unsigned long long rows, 
   return r == CUDA_SUCCESS ? MIX_OK : MIX_ERR_CUDA;
 }
 
-int make_tmap(CUtensorMap* out, const void* base, unsigned long long rows, int d, int box_rows) {
-  cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MIX_OK : MIX_ERR_CUDA;
-}
-
-// The packed panel as the encode reads it: all 128 rows of a tile at once, or 32 at a time.
-int make_panel_tmaps(Ctx* c) {
-  const int d = c->cfg.d_model;
-  const unsigned long long P = c->panel_rows_cap;
-  int rc = MIX_OK;
-  for (int i = 0; i < 2 && rc == MIX_OK; ++i) {
-    CUtensorMap* out = i == 0 ? &c->tmap_panel : &c->tmap_panel_32;
-    const int rows = i == 0 ? kTileM : 32;
-    rc = (c->cfg.flags & MIX_FLAG_FP8_W_ENC) ? make_tmap_e4m3(out, c->d_panel, 2 * P, d, rows)   // codes: P rows (8-bit input) or 2 P rows (hi, lo)
-                                             : make_tmap(out, c->d_panel, P, d, rows);
-  }
-  return rc;
-}
-
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t n) {
   *p = nullptr;
@@ -209,6 +184,18 @@ int upload_chain(mix_ctx* c, int slot, cudaStream_t s) {
 }  // namespace
 
 namespace mix {
+int make_tmap(CUtensorMap* out, const void* base, unsigned long long rows, int d, int box_rows) {
+  if (load_encode_fn() != MIX_OK) return MIX_ERR_CUDA;
+  cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)d * 2};
+  cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MIX_OK : MIX_ERR_CUDA;
+}
+
 static int g_pdl_mask = -1;        // -1: not yet read from the environment
 int pdl_mask() {
   // default: not the full encode pass -- measured, its early-resident CTAs cost config 3 about 7 us
@@ -325,7 +312,9 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     if (e == cudaSuccess && !(cfg->flags & MIX_FLAG_ENCODE_SIMT)) {
       if (load_encode_fn() != MIX_OK)
         e = cudaErrorUnknown;
-      else if (make_panel_tmaps(c) != MIX_OK)
+      else if ((cfg->flags & MIX_FLAG_FP8_W_ENC)    // codes: P rows (8-bit input) or 2 P rows (hi, lo) in the same buffer
+                   ? make_tmap_e4m3(&c->tmap_panel, c->d_panel, 2ull * c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK
+                   : make_tmap(&c->tmap_panel, c->d_panel, c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK)
         e = cudaErrorUnknown;
       if (e == cudaSuccess && c->d_act_scale) e = cudaMemset(c->d_act_scale, 0, c->panel_rows_cap * sizeof(float));
       if (e == cudaSuccess) e = encode_tc_prepare();

@@ -170,8 +170,8 @@ struct Ctx {
   CUtensorMap* d_tmap_probe;   // [n_slots_max] maps of multi-class probe matrices (box kTileK x 32), large-batch contexts only
   McCensus* d_mc_census;    // census of the 128-row tiles that hold multi-class probe rows, taken by mc_census_kernel every call
   int* d_mc_tiles;          // [ceil(T_max / 128)] those tiles, in no particular order
+  CUtensorMap tmap_w_one;   // where d_tmap_w is null (the allocation-free call): the one weight set's map, at this call's tile width
   CUtensorMap tmap_panel;   // panel map (box kTileK x kTileM, 128B swizzle)
-  CUtensorMap tmap_panel_32;   // the same with boxes of 32 rows: tiles with few valid rows
 
   // probe/steer kernels run beside the SAE chain on this stream (created with the context)
   cudaStream_t side_stream;
@@ -268,11 +268,22 @@ cudaError_t launch_router(const Ctx* c, float* logits, int n_experts, int T, cud
 cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, unsigned long long cond = 0,
                          int use_cond = 0);
 int front_chunks(int T_max);       // chunks of token rows the front kernel classifies: sizes d_front_counts / d_front_sync
+// bf16 [rows, d] row-major, boxes of 64 columns x box_rows rows, 128-byte swizzle; host work only
+int make_tmap(CUtensorMap* out, const void* base, unsigned long long rows, int d, int box_rows);
 cudaError_t launch_encode_simt(const Ctx* c, cudaStream_t s);
 cudaError_t launch_encode_tc(const Ctx* c, int mode, bool pair, cudaStream_t s);   // 0: all tiles; 1: flagged row tiles -> Z
 inline int cand_tiles_for(long long d_sae_max, int n_sms) {   // Ctx::cand_tiles
   const long long n = d_sae_max / kTileN, most = 4 * n < n_sms ? 4 * n : n_sms;
   return (int)(n > most ? n : most);
+}
+// Features per tile of the single-CTA encode for a call of `tiles` full-width tiles, at most nt_most of them in one row.
+// A call with few tiles -- one dictionary of 16384 features is 64 -- leaves SMs without one, and the pass takes as long as
+// one SM needs to stream a tile: tiles of 128 or 64 features then, as long as every SM gets at most one.  91 rows, d = 4096,
+// 16384 features: the encode 50 us with 64 tiles, 43 with 128.
+__host__ __device__ inline int tile_width(int tiles, int nt_most, int n_sms, int cand_tiles) {
+  int tile_n = kTileN;
+  for (; tile_n > kTileN / 4 && 2 * tiles <= n_sms && 2 * nt_most <= cand_tiles; tiles *= 2, nt_most *= 2) tile_n /= 2;
+  return tile_n;
 }
 bool encode_pair_possible(const Ctx* c);   // the CTA-pair encode kernel is part of this context's launch sequence
 // Selection, edits, decode and write-back of every SAE row.  mode 0: behind the tensor-core encode (TopK from its

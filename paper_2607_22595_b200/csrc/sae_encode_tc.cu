@@ -62,7 +62,10 @@ template <int kEnc, int kEpi, bool kPair> struct TcCfg {
   // each epilogue warp keeps the bias (and, for codes, the feature scale) of its columns of the current tile in
   // shared memory, fetched while the tile's main loop still runs
   static constexpr int kEpiVecBytes = 2 * 4 * kTileN * 4;   // [bias, scale][warp][its columns] floats: 8 KiB with 4 or 8 warps
-  static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + 1024 /* TcShared */ + kXchgBytes + kEpiVecBytes;
+  // survivors of the top-8 search, 8 values and columns per row, of the four lower-half warps (the upper-half warps use
+  // their hand-over place)
+  static constexpr int kPickBytes = kEpiWarps == 8 ? 4 * 32 * kCandPerTile * 5 : 0;
+  static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + 1024 /* TcShared */ + kXchgBytes + kEpiVecBytes + kPickBytes;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
 constexpr int kTmemCols = 512;                 // two 128 x 256 fp32 accumulators
@@ -181,10 +184,65 @@ __device__ __forceinline__ void top9_insert(float (&tv)[kCandPerTile + 1], int (
   }
 }
 
+// Compare-exchange, larger value first; an 8-element sort (19 of them), and the merge of a bitonic sequence of 8 (12).
+__device__ __forceinline__ void cmpx(float& a, float& b) {
+  const float hi = fmaxf(a, b);
+  b = fminf(a, b);
+  a = hi;
+}
+__device__ __forceinline__ void sort8_desc(float (&b)[8]) {
+  cmpx(b[0], b[1]); cmpx(b[2], b[3]); cmpx(b[4], b[5]); cmpx(b[6], b[7]);
+  cmpx(b[0], b[2]); cmpx(b[1], b[3]); cmpx(b[4], b[6]); cmpx(b[5], b[7]);
+  cmpx(b[1], b[2]); cmpx(b[5], b[6]);
+  cmpx(b[0], b[4]); cmpx(b[1], b[5]); cmpx(b[2], b[6]); cmpx(b[3], b[7]);
+  cmpx(b[2], b[4]); cmpx(b[3], b[5]);
+  cmpx(b[1], b[2]); cmpx(b[3], b[4]); cmpx(b[5], b[6]);
+}
+__device__ __forceinline__ void merge8_desc(float (&b)[8]) {
+  cmpx(b[0], b[4]); cmpx(b[1], b[5]); cmpx(b[2], b[6]); cmpx(b[3], b[7]);
+  cmpx(b[0], b[2]); cmpx(b[1], b[3]); cmpx(b[4], b[6]); cmpx(b[5], b[7]);
+  cmpx(b[0], b[1]); cmpx(b[2], b[3]); cmpx(b[4], b[5]); cmpx(b[6], b[7]);
+}
+
+// The same on (value, column) pairs: the larger value first, of equal ones the lower column.
+__device__ __forceinline__ void cmpx(float& a, int& ca, float& b, int& cb) {
+  const bool swap = b > a || (b == a && cb < ca);
+  const float x = swap ? b : a, y = swap ? a : b;
+  const int cx = swap ? cb : ca, cy = swap ? ca : cb;
+  a = x; b = y; ca = cx; cb = cy;
+}
+#define MIX_CX(i, j) cmpx(v[i], c[i], v[j], c[j])
+__device__ __forceinline__ void sort8_pairs(float (&v)[kCandPerTile + 1], int (&c)[kCandPerTile + 1]) {
+  MIX_CX(0, 1); MIX_CX(2, 3); MIX_CX(4, 5); MIX_CX(6, 7);
+  MIX_CX(0, 2); MIX_CX(1, 3); MIX_CX(4, 6); MIX_CX(5, 7);
+  MIX_CX(1, 2); MIX_CX(5, 6);
+  MIX_CX(0, 4); MIX_CX(1, 5); MIX_CX(2, 6); MIX_CX(3, 7);
+  MIX_CX(2, 4); MIX_CX(3, 5);
+  MIX_CX(1, 2); MIX_CX(3, 4); MIX_CX(5, 6);
+}
+// Merges a second sorted list of 9 (columns all higher) into the first: the 8 largest of both, sorted, and the 9th value.
+template <class Get>
+__device__ __forceinline__ void merge_lists(float (&v)[kCandPerTile + 1], int (&c)[kCandPerTile + 1], float ninth2, Get&& second) {
+  float ninth = fmaxf(v[kCandPerTile], ninth2);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float x;
+    int cx;
+    second(7 - i, x, cx);
+    ninth = fmaxf(ninth, fminf(v[i], x));
+    c[i] = x > v[i] ? cx : c[i];
+    v[i] = fmaxf(v[i], x);
+  }
+  MIX_CX(0, 4); MIX_CX(1, 5); MIX_CX(2, 6); MIX_CX(3, 7);
+  MIX_CX(0, 2); MIX_CX(1, 3); MIX_CX(4, 6); MIX_CX(5, 7);
+  MIX_CX(0, 1); MIX_CX(2, 3); MIX_CX(4, 5); MIX_CX(6, 7);
+  v[kCandPerTile] = ninth;
+}
+#undef MIX_CX
+
 template <int kEnc, int kEpi, bool kPair>
 __global__ void __launch_bounds__(TcCfg<kEnc, kEpi, kPair>::kThreads, 1)
-encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_constant__ CUtensorMap tmap_panel_32,
-                 const CUtensorMap* __restrict__ tmap_w, const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
+encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_constant__ CUtensorMap tmap_w_one, const CUtensorMap* __restrict__ tmap_w, const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
                  float* __restrict__ Z, long long ldz, int d, unsigned* __restrict__ status, int mode,
                  const int* __restrict__ mtile_flag, const int* __restrict__ n_flagged, float* __restrict__ cand_val,
                  int* __restrict__ cand_idx, float* __restrict__ cand_ninth, int cand_tiles, int w_tiled, int test_stall,
@@ -209,6 +267,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   float* xchg_val = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sh) + 1024);
   int* xchg_idx = reinterpret_cast<int*>(xchg_val + 2 * 4 * kXchgEntries * 32);
   float* epi_vec = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sh) + 1024 + Cfg::kXchgBytes);
+  float* pick = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(epi_vec) + Cfg::kEpiVecBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // CTA pairs: rank 0 leads (it issues the pair's tensor-core instructions and owns the barriers both CTAs' copies
   // complete on); `worker` numbers the units that walk the tile list -- pairs, or single CTAs
@@ -286,17 +345,19 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
       int stage = 0;
       unsigned phase = 0;
       bool ok = true;
+      const unsigned long long stream = l2_evict_first();
       for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
         const Tile t = tile_of(tile);
         if (!tile_wanted(t, groups, mode, mtile_flag)) continue;
         // (boxes of as many W_enc rows as this kernel's tile has: a map array per width)
-        const CUtensorMap* tw = tmap_w + (kPair || n_sub == 2 ? n_groups : (n_sub == 4 ? 2 * n_groups : 0)) + t.group;
+        // (no array: a single weight set whose map came with the launch, at the width the front kernel arrives at too)
+        const CUtensorMap* tw = tmap_w == nullptr ? &tmap_w_one : tmap_w + (kPair || n_sub == 2 ? n_groups : (n_sub == 4 ? 2 * n_groups : 0)) + t.group;
         const int n256 = t.n_tile / n_sub, row_in_256 = kPair ? rank * (kTileN / 2) : (t.n_tile - n256 * n_sub) * tile_n;
-        // panel rows nobody's accumulator row needs are not fetched (32 at a time): a decode batch of 20 rows brings 4 KiB
-        // of panel per k-block into the SM instead of 16.  (What the unfetched shared memory rows hold reaches only
-        // accumulator rows that are never read.)
-        const int n32 = kPair ? 4 : (t.rows_valid + 31) >> 5;
-        const unsigned tx_bytes = stage_bytes - (kSplit ? 2 : 1) * (4 - n32) * (kABytes / 4);
+        // A W_enc tile that one worker alone reads goes through L2 as the first to be evicted: otherwise the stream leaves
+        // nothing of what the short kernels around it live on -- their code, the tables, the rows -- and each of them starts
+        // with a chain of DRAM round trips (91 rows, d = 4096, 16384 features: front 12.3 -> 8.5 us, tail 19.4 -> 15.6).
+        // Tiles that several row tiles share must stay (the mixed batch's encode 441 -> 480 us with the hint).
+        const bool once = sh->unit0[t.group + 1] - sh->unit0[t.group] == 1;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
           // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumer's
@@ -317,20 +378,14 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
             const unsigned bar_c = mapa_cluster(bar, 0);
             tma_load_2d_pair(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar_c);
             if (kSplit) tma_load_2d_pair(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar_c);
-            tma_load_2d_pair(sw, tw, wx, wy, bar_c);
+            if (once) tma_load_2d_pair_hint(sw, tw, wx, wy, bar_c, stream);
+            else tma_load_2d_pair(sw, tw, wx, wy, bar_c);
           } else {
-            mbar_expect_tx(bar, tx_bytes);
-            if (n32 == 4) {
-              tma_load_2d(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar);
-              if (kSplit) tma_load_2d(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar);   // the lo codes
-            } else {
-              for (int i = 0; i < n32; ++i) {
-                tma_load_2d(sa + i * (kABytes / 4), &tmap_panel_32, kb * kBlockK, t.m_tile_global * kTileM + i * 32, bar);
-                if (kSplit)
-                  tma_load_2d(sa + kABytes + i * (kABytes / 4), &tmap_panel_32, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM + i * 32, bar);
-              }
-            }
-            tma_load_2d(sw, tw, wx, wy, bar);
+            mbar_expect_tx(bar, stage_bytes);
+            tma_load_2d(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar);
+            if (kSplit) tma_load_2d(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar);   // the lo codes
+            if (once) tma_load_2d_hint(sw, tw, wx, wy, bar, stream);
+            else tma_load_2d(sw, tw, wx, wy, bar);
           }
           if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
@@ -447,12 +502,13 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
           tv[s] = below_tau;
           ti[s] = 0;
         }
-#pragma unroll 1
-        for (int c = c_lo; c < c_lo + epi_cols; c += 32) {
-          float v[32];
-          tmem_ld32(taddr + c, v);
+        // Eight columns of the accumulator as pre-activations.  (Eight, in loops that stay loops: this code runs once or a few
+        // times per call, and 32 unrolled columns of it are 30 KiB of instructions to fetch before the first has an effect --
+        // more than the selection itself takes.)
+        auto load_z = [&](int c, float (&v)[8]) {
+          tmem_ld8(taddr + c, v);
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
+          for (int i = 0; i < 8; i += 4) {
             const float4 b4 = kStageVec ? *reinterpret_cast<const float4*>(wb + (c - c_lo) + i)
                                         : __ldg(reinterpret_cast<const float4*>(bias_t + (c - c_lo) + i));
             float4 s4 = make_float4(1.f, 1.f, 1.f, 1.f);
@@ -464,9 +520,73 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
             v[i + 2] = kScaled ? fmaf(v[i + 2], s4.z, b4.z) : v[i + 2] + b4.z;
             v[i + 3] = kScaled ? fmaf(v[i + 3], s4.w, b4.w) : v[i + 3] + b4.w;
           }
-          // (the list's 9th value is at least below_tau, so the test inside top9_insert covers the bound too)
+        };
+        // Two ways to the list.  With a bound in force nearly every column fails one comparison, and the few that do not are
+        // inserted.  Without one (a call's first wave of tiles; every tile of a call that has one wave) some lane of the
+        // warp would insert at nearly every column, 60 instructions each for one lane's sake: there the 8 largest VALUES and
+        // the 9th are found first, by min / max networks in which all lanes take part (11 instructions a column), and a
+        // second look at the accumulator picks up the columns of those 8, which the lanes then sort together.
+        bool listed = false;
+        if (kEpiWarps == 8 && __any_sync(0xffffffffu, valid && tau_key <= 1u)) {
+          float top[8], ninth = -INFINITY;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) top9_insert(tv, ti, v[i], c + i);
+          for (int s = 0; s < 8; ++s) top[s] = -INFINITY;
+#pragma unroll 1
+          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
+            float b[8];
+            load_z(c, b);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) b[s] = fmaxf(b[s], -INFINITY);          // (a NaN is never selected)
+            sort8_desc(b);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {                                       // the 8 largest of both, and the largest of the rest
+              const float lo = fminf(top[s], b[7 - s]);
+              top[s] = fmaxf(top[s], b[7 - s]);
+              ninth = fmaxf(ninth, lo);
+            }
+            merge8_desc(top);
+          }
+          float* pick_v = half == 1 ? xchg_val + (size_t)((acc * 4 + q) * kXchgEntries) * 32 : pick + q * (32 * kCandPerTile);
+          unsigned char* pick_c = half == 1 ? reinterpret_cast<unsigned char*>(xchg_idx + (size_t)((acc * 4 + q) * kXchgEntries) * 32)
+                                            : reinterpret_cast<unsigned char*>(pick + 4 * 32 * kCandPerTile) + q * (32 * kCandPerTile);
+          const float eighth = valid ? top[7] : INFINITY;
+          int n = 0;
+#pragma unroll 1
+          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
+            float v[8];
+            load_z(c, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int at = min(n, kCandPerTile - 1) * 32 + lane;      // (a ninth survivor: see below)
+              if (v[i] >= eighth) {
+                pick_v[at] = v[i];
+                pick_c[at] = (unsigned char)(c - c_lo + i);
+                ++n;
+              }
+            }
+          }
+          if (__all_sync(0xffffffffu, n <= kCandPerTile)) {      // (more only where values are exactly equal: the insertion below)
+            listed = true;
+#pragma unroll
+            for (int s = 0; s < kCandPerTile; ++s) {
+              const bool in = s < n;
+              tv[s] = in ? pick_v[s * 32 + lane] : -INFINITY;
+              ti[s] = c_lo + (in ? (int)pick_c[s * 32 + lane] : 0);
+            }
+            sort8_pairs(tv, ti);
+            tv[kCandPerTile] = ninth;
+            __syncwarp();
+          }
+        }
+        if (!listed && __any_sync(0xffffffffu, valid)) {
+#pragma unroll 1
+          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
+            float v[8];
+            load_z(c, v);
+            // (the list's 9th value is at least below_tau, so the test inside top9_insert covers the bound too)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) top9_insert(tv, ti, v[i], c + i);
+          }
         }
         bool writer = true;
         unsigned tau_pub = tau_key;
@@ -487,8 +607,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
             writer = false;
           } else {
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->xchg_full[acc][q]), (xchg_phase >> acc) & 1u, sh, status))) break;
-#pragma unroll
-            for (int s = 0; s <= kCandPerTile; ++s) top9_insert(tv, ti, xv[s * 32], xi[s * 32]);
+            merge_lists(tv, ti, xv[kCandPerTile * 32], [&](int s, float& x, int& cx) { x = xv[s * 32]; cx = xi[s * 32]; });
             // the two warps may have read the bound at different times: what is at or above the larger one is a
             // real element of the row (each warp's fillers lie below its own bound)
             tau_pub = max(tau_key, (unsigned)xi[(kCandPerTile + 1) * 32]);
@@ -546,7 +665,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         const float* theta_t = jump ? groups[t.group].theta + (size_t)t.n_tile * tile_n + c_lo : nullptr;
         float* wt = kScaled || !kStageVec ? nullptr : ws;       // (the scale's place is free where there is no scale)
         if (jump && wt != nullptr) {
-          for (int j = lane * 4; j < epi_cols; j += 128) *reinterpret_cast<float4*>(wt + j) = __ldg(reinterpret_cast<const float4*>(theta_t + j));
+          for (int j = lane; j < epi_cols; j += 32) wt[j] = __ldg(theta_t + j);      // (theta need not be aligned)
           __syncwarp();
         }
         unsigned* bits = reinterpret_cast<unsigned*>(cand_idx) + p * (size_t)cand_tiles * kCandPerTile + t.n_tile * (tile_n / 32);
@@ -577,8 +696,11 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
               float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (jump) t4 = wt != nullptr ? *reinterpret_cast<const float4*>(wt + (c - c_lo) + i)
-                                           : __ldg(reinterpret_cast<const float4*>(theta_t + (c - c_lo) + i));
+              if (jump) {
+                const float* th = theta_t + (c - c_lo) + i;
+                t4 = wt != nullptr ? *reinterpret_cast<const float4*>(wt + (c - c_lo) + i)
+                                   : make_float4(__ldg(th), __ldg(th + 1), __ldg(th + 2), __ldg(th + 3));
+              }
               if (v[i] > t4.x && v[i] != 0.f) m |= 1u << i;
               if (v[i + 1] > t4.y && v[i + 1] != 0.f) m |= 2u << i;
               if (v[i + 2] > t4.z && v[i + 2] != 0.f) m |= 4u << i;
@@ -725,7 +847,8 @@ static cudaError_t launch_encode_tc_as(const Ctx* c, int mode, cudaStream_t s) {
   }
   cfg.attrs = at;
   cfg.numAttrs = n_at;
-  return cudaLaunchKernelEx(&cfg, encode_tc_kernel<kEnc, kEpi, kPair>, c->tmap_panel, c->tmap_panel_32, static_cast<const CUtensorMap*>(c->d_tmap_w),
+  return cudaLaunchKernelEx(&cfg, encode_tc_kernel<kEnc, kEpi, kPair>, c->tmap_panel, c->tmap_w_one,
+                            static_cast<const CUtensorMap*>(c->d_tmap_w),
                             static_cast<const RouteState*>(c->d_route), static_cast<const GroupEntry*>(c->d_groups),
                             c->cfg.n_groups_max, c->d_z, (long long)c->cfg.d_sae_max, c->cfg.d_model, c->d_status, mode,
                             static_cast<const int*>(c->d_mtile_flag), static_cast<const int*>(c->d_n_flagged), c->d_cand_val,

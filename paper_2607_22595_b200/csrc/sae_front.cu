@@ -352,17 +352,15 @@ front_kernel(const FrontArgs a) {
           if (split_pays && split_total <= min(cost_single, cost_pair)) mask = split_mask;
           else mask = cost_pair < cost_single ? live_mask : 0;
         }
-        // A call with few tiles -- one dictionary of 16384 features is 64 -- leaves SMs without one, and the pass takes as
-        // long as one SM needs to stream a tile: tiles of 128 or 64 features then, as long as every SM gets at most one.
-        // (Pairs give way only where single CTAs can go down to 64: at 128 both forms bring the same bytes into an SM per
-        // k-block.)  91 rows, d = 4096, 16384 features: encode 50 us with 64 tiles, see encode_tc_kernel for what it is now.
+        // (Pairs give way to narrow tiles only where single CTAs can go down to 64 features: at 128 both forms bring the same
+        // bytes into an SM per k-block.)
         int tile_n = kTileN;
         if (a.pair_mode != 1 && 4 * tiles <= a.n_sms) mask = 0;
         if (mask == 0) {
           int nt_most = 1;
           for (int q = 0; q < n_groups; ++q)
             if (s_total[q] > 0) nt_most = max(nt_most, s_gtiles[q]);
-          for (int n = tiles; tile_n > kTileN / 4 && 2 * n <= a.n_sms && 2 * nt_most <= a.cand_tiles; n *= 2, nt_most *= 2) tile_n /= 2;
+          tile_n = tile_width(tiles, nt_most, a.n_sms, a.cand_tiles);
         }
         a.rs->tile_n = tile_n;
         a.rs->pair_mask = mask;

@@ -64,6 +64,20 @@ __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map
       : "memory");
 }
 
+// The same for data that is read once (or by its readers at the same time) and larger than L2 -- a stream of weights: its
+// lines are the first to be evicted, so that what the kernels around it share (their code among it) stays in L2.
+__device__ __forceinline__ unsigned long long l2_evict_first() {
+  unsigned long long p;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ void tma_load_2d_hint(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar, unsigned long long policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+      : "memory");
+}
+
 // K-major operand tile, 128-byte swizzle: rows of 64 bf16 (128 B), 8-row groups 1024 B apart.
 __device__ __forceinline__ unsigned long long umma_desc(unsigned smem_addr) {
   unsigned long long d = 0;
@@ -124,6 +138,17 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
+  unsigned r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // ---- CTA pairs (a cluster of two CTAs working on one 256-row tile with tcgen05 cta_group::2) ----
 // Rank of this CTA in its cluster; the shared::cluster address of the same variable in CTA `rank` of the cluster;
 // a cluster-wide barrier; an arrival on an mbarrier that may live in the peer CTA.
@@ -150,6 +175,13 @@ __device__ __forceinline__ void tma_load_2d_pair(unsigned dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair_hint(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar_cluster,
+                                                      unsigned long long policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster), "l"(policy)
       : "memory");
 }
 // One instruction of the pair: M = 256 (rows 0..127 from the A tile in the leader's shared memory, 128..255 from
