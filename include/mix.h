@@ -446,7 +446,7 @@ int mix_debug_phase_clocks(mix_ctx* ctx, unsigned long long* out32);
  * untouched.  Such callers cannot use mix_create(), which allocates the hook's tables and
  * workspace.  This single call needs no context: all of its scratch (tables, routing state,
  * the packed bf16 row panel, the fp32 pre-activations, TopK lists) sits in one fixed array
- * inside the library image, about 5.2 MiB, which every GPU that loads the library keeps
+ * inside the library image, about 5.8 MiB, which every GPU that loads the library keeps
  * until the process exits.  The call allocates nothing and frees nothing.
  *
  * What it computes: the MIX_SAE function of mix_apply() for ONE app on EVERY one of the
@@ -455,7 +455,8 @@ int mix_debug_phase_clocks(mix_ctx* ctx, unsigned long long* out32);
  * `w` and `app` are host structs as for registration (w's pointers device, app's edit
  * arrays host, app->group ignored).  topk_idx int32 / topk_val fp32 [n_rows, w->k]: optional
  * device outputs for TopK SAEs (NULL = off), as in mix_set_feature_out with k_max = w->k.
- * The encode runs on the CUDA-core kernel (the one MIX_FLAG_ENCODE_SIMT selects).
+ * The encode runs on the tensor cores, as in mix_apply() (on the CUDA cores if b_enc is not 16-byte
+ * aligned).
  *
  * Limits (the array has a fixed size): n_rows <= MIX_STATIC_MAX_ROWS, d_model <=
  * MIX_STATIC_MAX_D_MODEL (multiple of 64), w->d_sae <= MIX_STATIC_MAX_D_SAE (multiple of 256),

@@ -4,8 +4,8 @@
 // tables, edit lists, routing state, the packed bf16 panel and the fp32 pre-activation
 // scratch) lives here in ONE file-scope device array of fixed size.  The array is
 // part of the library image: every GPU that loads libmix.so holds it until the process exits.
-// The call then runs the same routing / pack, encode (CUDA-core kernel) and selection / decode
-// kernels as mix_apply(), pointed at that array.
+// The call then runs the same routing / pack, encode and selection / decode kernels as mix_apply(),
+// pointed at that array.
 #include <stdio.h>
 #include <string.h>
 
@@ -41,10 +41,19 @@ constexpr size_t kOffFrontCounts = kOffRowMeta + align256(kStaticRows * sizeof(i
 constexpr size_t kOffFrontSync = kOffFrontCounts + 256;      // one chunk: a count per weight set + one, then epoch words
 constexpr size_t kOffChainNext = kOffFrontSync + 256;
 constexpr size_t kOffRowRec = kOffChainNext + 256;
-constexpr size_t kOffPanel = kOffRowRec + align256(kStaticRows * sizeof(RowRec));
+constexpr size_t kOffFlags = kOffRowRec + align256(kStaticRows * sizeof(RowRec));        // row flags, tile flag, flagged rows
+constexpr size_t kOffMtileFlag = kOffFlags + align256(kStaticRows * sizeof(int)), kOffNFlagged = kOffMtileFlag + 256;
+constexpr int kStaticTiles = (int)(kStaticDsae / (kTileN / 4));                         // the narrowest tiles of the widest SAE
+constexpr size_t kOffCandIdx = kOffNFlagged + 256;
+constexpr size_t kOffPanel = kOffCandIdx + align256((size_t)kStaticRows * kStaticTiles * kCandPerTile * sizeof(int));
 constexpr size_t kOffZ = kOffPanel + align256((size_t)kStaticRows * kStaticD * sizeof(__nv_bfloat16));
 constexpr size_t kScratchBytes = kOffZ + align256((size_t)kStaticRows * kStaticDsae * sizeof(float));
 static_assert(kScratchBytes < (6u << 20), "the header promises less than 6 MiB");
+// TopK candidates and pre-activations share their place: a row's Z is written (by the fallback pass) only when the
+// candidates have been read.
+constexpr size_t kOffCandVal = kOffZ;
+constexpr size_t kOffCandNinth = kOffCandVal + align256((size_t)kStaticRows * kStaticTiles * kCandPerTile * sizeof(float));
+static_assert(kOffCandNinth + (size_t)kStaticRows * kStaticTiles * sizeof(float) <= kScratchBytes, "the candidates fit in Z's place");
 
 // The scratch itself.  In host code this name is only a handle for cudaGetSymbolAddress();
 // it is NOT a device address and must never be handed to a kernel.
@@ -52,6 +61,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 unsigned char* g_scratch_addr[kMaxDevices];     // device address of the array, per device, once resolved
+int g_n_sms[kMaxDevices];
 
 // Everything the call's tables need, passed to the set-up kernel BY VALUE (well under the 4 KiB of kernel
 // parameters): no host pointer is handed to the stream, so nothing the stream does later depends on the
@@ -137,6 +147,9 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
     void* p = nullptr;
     const cudaError_t e = cudaGetSymbolAddress(&p, g_static_scratch);
     if (e != cudaSuccess || !p) return fail(errbuf, errbuf_len, MIX_ERR_CUDA, "cudaGetSymbolAddress failed (%lld)", (long long)e);
+    cudaError_t e2 = cudaDeviceGetAttribute(&g_n_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+    if (e2 == cudaSuccess) e2 = encode_tc_prepare();
+    if (e2 != cudaSuccess) return fail(errbuf, errbuf_len, MIX_ERR_CUDA, "cannot prepare the encode kernels (%lld)", (long long)e2);
     g_scratch_addr[dev] = static_cast<unsigned char*>(p);
   }
   unsigned char* base = g_scratch_addr[dev];
@@ -153,8 +166,11 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   c.cfg.k_max = w->act == MIX_SAE_TOPK ? w->k : 1;
   c.cfg.r_max = kMaxEdits;
   c.cfg.d_sae_max = w->d_sae;
-  c.cfg.flags = MIX_FLAG_ENCODE_SIMT;
+  // (the tensor-core encode reads the bias 16 bytes at a time; a bias that lies unaligned takes the CUDA-core kernel)
+  const bool simt = (reinterpret_cast<uintptr_t>(w->b_enc) & 15u) != 0;
+  c.cfg.flags = simt ? MIX_FLAG_ENCODE_SIMT : 0;
   c.device = dev;
+  c.n_sms = g_n_sms[dev];
   c.d_token_slot = reinterpret_cast<int*>(base + kOffTokenSlot);
   c.d_n_live = reinterpret_cast<int*>(base + kOffNLive);
   c.d_status = reinterpret_cast<unsigned*>(base + kOffStatus);
@@ -175,6 +191,14 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   c.d_row_rec = reinterpret_cast<RowRec*>(base + kOffRowRec);
   c.d_panel = reinterpret_cast<__nv_bfloat16*>(base + kOffPanel);
   c.d_z = reinterpret_cast<float*>(base + kOffZ);
+  c.d_cand_val = reinterpret_cast<float*>(base + kOffCandVal);
+  c.d_cand_idx = reinterpret_cast<int*>(base + kOffCandIdx);
+  c.d_cand_ninth = reinterpret_cast<float*>(base + kOffCandNinth);
+  c.cand_tiles = cand_tiles_for(w->d_sae, c.n_sms);
+  if (c.cand_tiles > kStaticTiles) c.cand_tiles = kStaticTiles;
+  c.d_row_flag = reinterpret_cast<int*>(base + kOffFlags);
+  c.d_mtile_flag = reinterpret_cast<int*>(base + kOffMtileFlag);
+  c.d_n_flagged = reinterpret_cast<int*>(base + kOffNFlagged);
   c.panel_rows_cap = kStaticRows;
   c.out_topk_idx = topk_idx;
   c.out_topk_val = topk_val;
@@ -198,6 +222,13 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   ge.W_dec = static_cast<const __nv_bfloat16*>(w->W_dec);
   ge.b_dec = w->b_dec;
 
+  c.h_groups = &ge;
+  // The tensor maps travel with the launches (they name addresses of this call only).
+  const int n_tiles = (int)(w->d_sae / kTileN);
+  if (make_tmap(&c.tmap_panel, c.d_panel, kStaticRows, d_model, kTileM) != MIX_OK ||
+      make_tmap(&c.tmap_w_one, w->W_enc, (unsigned long long)w->d_sae, d_model, tile_width(n_tiles, n_tiles, c.n_sms, c.cand_tiles)) != MIX_OK)
+    return fail(errbuf, errbuf_len, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed");
+
   // The array keeps whatever the previous call left: one small kernel rewrites every table this call reads,
   // from values it received as kernel parameters.  (Routing rewrites the row lists and counters itself; the
   // panel, Z and TopK lists are fully rewritten for the rows in use before they are read.)
@@ -217,8 +248,12 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   cudaError_t e = cudaGetLastError();
   __nv_bfloat16* h = static_cast<__nv_bfloat16*>(hidden);
   if (e == cudaSuccess) e = launch_front(&c, h, n_rows, s);       // routing + row pack
-  if (e == cudaSuccess) e = launch_encode_simt(&c, s);
-  if (e == cudaSuccess) e = launch_tail(&c, h, 1, s);             // selection, edits, decode, write-back
+  if (e == cudaSuccess) e = simt ? launch_encode_simt(&c, s) : launch_encode_tc(&c, 0, false, s);
+  if (e == cudaSuccess) e = launch_tail(&c, h, simt ? 1 : 0, s);  // selection, edits, decode, write-back
+  if (w->act == MIX_SAE_TOPK && !simt) {                                   // rows whose candidates cannot prove the TopK
+    if (e == cudaSuccess) e = launch_encode_tc(&c, 1, false, s);
+    if (e == cudaSuccess) e = launch_tail(&c, h, 2, s);
+  }
   if (e != cudaSuccess) return fail(errbuf, errbuf_len, MIX_ERR_CUDA, "CUDA error %lld while enqueuing the static SAE call", (long long)e);
   return MIX_OK;
 }

@@ -61,3 +61,39 @@ def test_rebuilt_rows_with_more_active_features_than_a_list_holds():
 def test_rebuilt_rows_on_cta_pairs():
     w = _workload(320, 10240, 256, W.SAE_JUMPRELU, False, b_enc_mean=-2.0)
     check_parity(W.host(w), run_gpu(w))
+
+
+@pytest.mark.parametrize("rows,d,S,act,k,add_error", [
+    (1, 64, 256, W.SAE_TOPK, 1, True), (33, 320, 2304, W.SAE_TOPK, 24, False), (128, 4096, 8192, W.SAE_TOPK, 64, True),
+    (7, 128, 8192, W.SAE_TOPK, 128, False), (128, 192, 4096, W.SAE_RELU, 0, True), (50, 2304, 1024, W.SAE_JUMPRELU, 0, False)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_allocation_free_call(rows, d, S, act, k, add_error, aligned):
+    import paper_2607_22595_b200 as mixlib
+    w = _workload(d, S, rows, act, add_error, k=max(k, 1), b_enc_mean=-0.1 if add_error or act == W.SAE_TOPK else -2.0)
+    if act == W.SAE_TOPK and k > 64:                          # duplicated encoder rows: ties at the k-th value, the exact fallback
+        w.groups[0].W_enc[1::2] = w.groups[0].W_enc[0::2]
+        w.groups[0].b_enc[1::2] = w.groups[0].b_enc[0::2]
+    if not aligned:
+        b = torch.empty(S + 1, device="cuda")
+        b[1:] = w.groups[0].b_enc
+        w.groups[0].b_enc = b[1:]
+    sw, app, h = w.groups[0], w.apps[0], w.hidden.clone()
+    idx = torch.full((rows, max(k, 1)), -559038737, dtype=torch.int32, device="cuda")
+    val = torch.from_numpy(np.full((rows, max(k, 1)), 0x7FC0DEAD, dtype=np.uint32).view(np.float32)).cuda()
+    for _ in range(2):                                        # the second call finds the first one's scratch
+        h.copy_(w.hidden)
+        mixlib.sae_apply_static(h, S, act, k, sw.W_enc, sw.b_enc, sw.W_dec, app.edit_idx, app.edit_val, app.edit_mode, add_error,
+                                theta=sw.theta, topk_idx=idx if k else None, topk_val=val if k else None)
+    from oracle import mi_hook as O
+    wh = W.host(w)
+    ref = O.apply_hook(wh, list(range(rows)), keep_z=True)
+    if k and k <= 64:
+        for t in range(rows):
+            z = ref.z[t]
+            picked = idx[t].cpu().numpy()
+            assert len(set(picked.tolist())) == k and z[picked].min() >= np.sort(z)[-k] - 1e-3
+            assert np.abs(val[t].cpu().numpy() - z[picked]).max() <= 1e-3
+    elif k:
+        assert (idx.cpu().numpy()[:, 0] % 2 == 0).all()       # of two equal ones the lower id comes first
+    hid, hmax = O.bf16_to_f64(W.bits(h)), np.abs(O.bf16_to_f64(wh.hidden)).max()
+    assert max(np.abs(hid[t] - ref.y[t]).max() for t in range(rows)) <= 1e-2 * hmax
