@@ -142,34 +142,181 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 
 constexpr long long kFrontWaitCycles = 2000000000ll;   // ~1 s: cap of the wait for the other CTAs' chunks
 
-// One launch, three steps, no CTA doing another's work:
-//   1. CTA c < chunks classifies token rows [256 c, 256 c + 256) -- slot -> app entry -> SAE row of which weight set --
-//      and PUBLISHES the chunk: per-row records, per-set counts, then one more on the call's counter of published chunks.
-//   2. Every CTA waits (one thread polls, bounded) until the counter says all chunks are there, reads the small count table and scans it: totals
-//      per weight set, the sets' first panel rows, and for every chunk the rank of its first row within each set.
-//      The publishing CTAs never wait before they publish, and CTAs are dispatched in index order, so whoever waits,
-//      waits for work that is already running.
-//   3. CTA b packs panel rows [8 b, 8 b + 8), one per warp: the row's set and rank follow from its position, the
-//      chunk that holds that rank from the scan, the token from that chunk's published records.
-// CTA 0 alone writes what exists once (the routing result the encode reads, the tile -> weight-set map, the
-// conditional handle).  The last CTA of the launch to leave puts the two counters back to zero for the next call.
+constexpr int kFrontLocal = 4;            // chunks (of 256 token rows) up to which every CTA routes the whole call for itself
+
+// What the slot map says about one token row.
+struct RowClass {
+  int meta;        // (weight set + 1) | edit count << 8 | error-term flag << 16; 0: not an SAE row
+  int slot;
+  bool delta;      // a row of the tail kernel's delta role
+};
+
+// Slot and the part of the app entry that routing needs, requested together.
+struct RowEntry {
+  int slot;
+  int2 q0;         // valid, kind
+  int g, n_edit, add_error;
+};
+__device__ __forceinline__ RowEntry load_entry(const FrontArgs& a, int slot) {
+  RowEntry r;
+  r.slot = slot;
+  r.q0 = make_int2(0, 0);
+  r.g = -1;
+  r.n_edit = r.add_error = 0;
+  if (slot >= 0) {
+    const AppEntry* e = a.apps + slot;
+    r.q0 = __ldg(reinterpret_cast<const int2*>(e));
+    r.g = __ldg(&e->group);
+    const int2 ne = __ldg(reinterpret_cast<const int2*>(&e->n_edit));
+    r.n_edit = ne.x;
+    r.add_error = ne.y != 0;
+  }
+  return r;
+}
+
+__device__ __forceinline__ RowClass classify(const FrontArgs& a, RowEntry r, int t, const int* s_gact, const int* s_gtiles) {
+  // a row whose slot starts a chain is an SAE row if the chain ends in an SAE app: follow the links
+  if (r.q0.x && (r.q0.y & kKindChained) && (r.q0.y & kKindMask) != MIX_SAE) {
+    int s2 = r.slot;
+    int2 h2 = r.q0;
+    for (int depth = 1; depth < kMaxChain && s2 >= 0; ++depth) {
+      s2 = (h2.y & kKindChained) ? __ldg(a.chain_next + s2) : -1;
+      if (s2 < 0 || s2 >= a.n_slots) { s2 = -1; break; }
+      h2 = __ldg(reinterpret_cast<const int2*>(a.apps + s2));
+      if (!h2.x) { s2 = -1; break; }
+      if ((h2.y & kKindMask) == MIX_SAE) break;
+    }
+    if (s2 >= 0 && (h2.y & kKindMask) != MIX_SAE) s2 = -1;
+    r = load_entry(a, s2);
+  }
+  RowClass c;
+  c.meta = 0;
+  c.slot = r.slot;
+  c.delta = false;
+  if (r.q0.x && (r.q0.y & kKindMask) == MIX_SAE) {
+    if (r.g < 0 || r.g >= a.n_groups || s_gtiles[r.g] == 0) {
+      atomicOr(a.status, MIX_STATUS_BAD_GROUP);
+    } else if (a.edit_only && r.add_error && s_gact[r.g] != MIX_SAE_TOPK) {
+      // handled by sae_edit_only_kernel: with the error term on, a ReLU / JumpReLU row needs
+      // only the pre-activations of its edited features, not the whole encode
+    } else if (!(r.q0.y & kKindGated) || gate_open(a.gates, r.slot, t)) {
+      c.meta = (r.g + 1) | (r.n_edit << 8) | (r.add_error << 16);
+      c.delta = r.add_error && r.n_edit > 0 && s_gact[r.g] != MIX_SAE_TOPK;
+    }
+  }
+  return c;
+}
+
+__device__ __forceinline__ int warp_scan(int v, int lane) {      // inclusive
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+__device__ __forceinline__ long long warp_sum64(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// What exists once per call, written by one warp (lane q: weight set q): the routing result the encode and the tail read,
+// and which encode kernel takes which weight set.
+__device__ __forceinline__ void write_route(const FrontArgs& a, int total, int nt, bool topk, int mt0, int mt, int n_delta, int lane) {
+  const bool live = total > 0;
+  const int m_tiles = (total + kTileM - 1) / kTileM;
+  const int my_tiles = live ? m_tiles * nt : 0;
+  const int tiles_incl = warp_scan(my_tiles, lane);
+  const int tiles = __shfl_sync(0xffffffffu, tiles_incl, 31);
+  a.rs->group_count[lane] = total;                  // (lanes of sets that do not exist: no rows)
+  a.rs->group_mtile0[lane] = mt0;
+  a.rs->group_tile0[lane] = tiles_incl - my_tiles;
+  const int rows = __reduce_add_sync(0xffffffffu, total);
+  const int topk_rows = __reduce_add_sync(0xffffffffu, topk ? total : 0);
+  const int nt_most = max(1, __reduce_max_sync(0xffffffffu, live ? nt : 0));
+  // per feature tile, in units of 1/40 of the time the W_enc tile takes to stream from HBM (measured on one
+  // weight set with 64 ... 1024 rows): single CTAs stream at the full rate for one row tile, and from two row
+  // tiles on every further tile costs 25 -- each of them fetches the W_enc tile again, from L2; a pair costs 46
+  // per 256-row tile whether its second half has rows or not, streaming at a slightly lower rate
+  const long long cs = live ? (long long)(m_tiles == 1 ? 40 : 25 * m_tiles) * nt : 0;
+  const long long cp = live ? (long long)(46 * ((m_tiles + 1) / 2)) * nt : 0;
+  const long long cost_single = warp_sum64(cs), cost_pair = warp_sum64(cp), cost_split = warp_sum64(min(cs, cp));
+  const int live_mask = (int)__ballot_sync(0xffffffffu, live);
+  const int split_mask = (int)__ballot_sync(0xffffffffu, live && cp < cs);
+  const bool odd3 = __ballot_sync(0xffffffffu, live && cp >= cs && m_tiles >= 3) != 0u;
+  // Pairs win where a weight set has an even number of row tiles (two tiles share one fetch of W_enc, and the
+  // pair's instruction fills less shared memory per flop) and lose where half of a pair would repeat the other
+  // half's work: one row tile, or three.  Each weight set may go to the form that is cheaper for it -- the two
+  // encode kernels then both work, one after the other, which costs a second ramp-up and drain (about 25 us:
+  // in the units above 25 x 40 / (time to stream one tile of 512 d bytes at 6.3 TB/s) = 1.23e7 / d).
+  // Measured on config 4's replays, the split pays when two or more sets go to the pairs, or when a set of
+  // three or more row tiles stays with the single CTAs; ONE two-tile set among one-tile sets does not: inside
+  // the single-CTA kernel its second fetch of each W_enc tile and its tensor time hide behind the other sets'
+  // streams (1.67 ms all single against 1.71-1.74 ms split for sets of 1, 1, 1, 1, 2 tiles), so such a call
+  // stays with one form.
+  int mask = a.pair_mode == 1 ? live_mask : 0;
+  if (a.pair_mode == 2) {
+    const bool both = split_mask != 0 && split_mask != live_mask;
+    const long long split_total = cost_split + (both ? 12300000ll / max(a.d, 1) : 0ll);
+    const bool split_pays = !both || __popc(split_mask) >= 2 || odd3;
+    if (split_pays && split_total <= min(cost_single, cost_pair)) mask = split_mask;
+    else mask = cost_pair < cost_single ? live_mask : 0;
+  }
+  // (Pairs give way to narrow tiles only where single CTAs can go down to 64 features: at 128 both forms bring the same
+  // bytes into an SM per k-block.)
+  if (a.pair_mode != 1 && 4 * tiles <= a.n_sms) mask = 0;
+  if (lane == 0) {
+    a.rs->group_mtile0[kMaxGroups] = mt;
+    a.rs->group_tile0[kMaxGroups] = tiles;
+    a.rs->n_panel_rows = mt * kTileM;
+    a.rs->n_mtiles = mt;
+    a.rs->n_sae_rows = rows;
+    a.rs->total_tiles = tiles;
+    a.rs->n_topk_rows = topk_rows;
+    a.rs->n_delta_rows = n_delta;
+    a.rs->tile_n = mask == 0 ? tile_width(tiles, nt_most, a.n_sms, a.cand_tiles) : kTileN;
+    a.rs->pair_mask = mask;
+    a.rs->use_pair = mask != 0;
+    if (a.n_flagged) *a.n_flagged = 0;       // fallback-selection flags of the fused TopK path start clear every call
+    // graph-conditional form: the rest of the SAE chain sits in the body of an IF node that runs only when a row needs it
+    if (a.use_cond) cudaGraphSetConditional(a.cond, rows > 0 ? 1u : 0u);
+  }
+}
+
+// Routing and row pack in one launch.
+//   Calls of up to 1024 rows: every CTA classifies ALL token rows -- slot -> app entry -> SAE row of which weight set, four
+//      rows a thread, their loads in flight together -- and so knows every row's place in the panel; the eight rows that
+//      fall to the CTA are noted along the way.  No CTA waits for another.  (91 rows behind a 16384-feature encode: 8.2 us
+//      with the exchange below, 4.7 without.)
+//   Longer calls, where that would cost T rows times a CTA for every eight: CTA c < chunks classifies token rows
+//      [256 c, 256 c + 256) and PUBLISHES the chunk -- per-row records, per-set counts, then one more on the call's counter
+//      of published chunks.  Every CTA waits (one thread polls, bounded) until the counter says all chunks are there, reads
+//      the small count table and scans it.  The publishing CTAs never wait before they publish, and CTAs are dispatched in
+//      index order, so whoever waits, waits for work that is already running.  The rows of a CTA are found through the
+//      scan and the published records.
+// Then CTA b packs panel rows [8 b, 8 b + 8), one per warp.  The last CTA -- whose panel rows a call seldom needs -- writes
+// what exists once (routing result, tile -> weight-set map, conditional handle), beside the others' packing.  The last CTA
+// of the launch to leave puts the two counters back to zero for the next call.
 // kPack: 0 the bf16 row, 1 E4M3 hi + lo (exact split), 2 E4M3 quantised.
 template <int kPack>
 __global__ void __launch_bounds__(kFrontThreads)
 front_kernel(const FrontArgs a) {
   extern __shared__ int s_tab[];                      // [chunks][n_groups + 1]: counts, then exclusive prefixes over the chunks
-  __shared__ int s_total[kMaxGroups + 1], s_base[kMaxGroups + 1];
+  __shared__ int s_total[kMaxGroups + 1];
   __shared__ int s_gact[kMaxGroups], s_gtiles[kMaxGroups];   // per weight set: activation, feature tiles (0: not registered)
   __shared__ const __nv_bfloat16* s_gwdec[kMaxGroups];
   __shared__ const float* s_gtheta[kMaxGroups];
-  __shared__ int s_wcnt[kFrontWarps][kMaxGroups + 1];
-  __shared__ int s_n_panel_rows;
+  __shared__ int s_wcnt[kFrontLocal * kFrontWarps][kMaxGroups + 1];   // rows per (chunk, warp) and weight set; then what comes before them
+  __shared__ int s_row[kFrontWarps][3];                // this CTA's panel rows: token row, record, slot
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x;
-  const bool first_cta = cta == 0;
+  const bool first_cta = cta == 0, route_cta = cta == (int)gridDim.x - 1;
   const int n_groups = a.n_groups, n_slots = a.n_slots, ncol = n_groups + 1;
   const int n_chunks = (a.T + kFrontThreads - 1) / kFrontThreads;     // the same in every CTA: who publishes is fixed by the launch
+  const bool local = n_chunks <= kFrontLocal;
   phase_stamp(a.clk, 0, first_cta && tid == 0);
+  const int n_live = min(a.T, __ldg(a.n_live_p));      // (all of these loads issue together)
   if (tid < n_groups) {                                // requested now, needed after the first barrier
     const bool valid = __ldg(&a.groups[tid].valid) != 0;
     s_gact[tid] = __ldg(&a.groups[tid].act);
@@ -177,244 +324,192 @@ front_kernel(const FrontArgs a) {
     s_gwdec[tid] = a.groups[tid].W_dec;
     s_gtheta[tid] = a.groups[tid].theta;
   }
-  // ---- step 1: classify and publish one chunk
-  if (cta < n_chunks) {
-    const int t = cta * kFrontThreads + tid;
-    const int n_live = min(a.T, __ldg(a.n_live_p));   // both loads issue together
-    int slot = t < a.T ? __ldg(a.token_slot + t) : -1;
-    if (t >= n_live || slot >= n_slots) slot = -1;
-    int2 q0 = make_int2(0, 0);                         // valid, kind
-    int g = -1, n_edit = 0, add_error = 0;
-    if (slot >= 0) {
-      const AppEntry* e = a.apps + slot;
-      q0 = __ldg(reinterpret_cast<const int2*>(e));
-      g = __ldg(&e->group);
-      const int2 ne = __ldg(reinterpret_cast<const int2*>(&e->n_edit));
-      n_edit = ne.x;
-      add_error = ne.y != 0;
-    }
-    // a row whose slot starts a chain is an SAE row if the chain ends in an SAE app: follow the links
-    if (q0.x && (q0.y & kKindChained) && (q0.y & kKindMask) != MIX_SAE) {
-      int s2 = slot;
-      int2 h2 = q0;
-      for (int depth = 1; depth < kMaxChain && s2 >= 0; ++depth) {
-        s2 = (h2.y & kKindChained) ? __ldg(a.chain_next + s2) : -1;
-        if (s2 < 0 || s2 >= n_slots) { s2 = -1; break; }
-        h2 = __ldg(reinterpret_cast<const int2*>(a.apps + s2));
-        if (!h2.x) { s2 = -1; break; }
-        if ((h2.y & kKindMask) == MIX_SAE) break;
-      }
-      if (s2 >= 0 && (h2.y & kKindMask) != MIX_SAE) s2 = -1;
-      slot = s2;
-      q0 = s2 >= 0 ? h2 : make_int2(0, 0);
-      if (s2 >= 0) {
-        g = __ldg(&a.apps[s2].group);
-        n_edit = __ldg(&a.apps[s2].n_edit);
-        add_error = __ldg(&a.apps[s2].add_error) != 0;
-      }
-    }
-    __syncthreads();                                   // the weight-set table is in shared memory
-    int meta = 0, is_delta = 0;
-    if (q0.x && (q0.y & kKindMask) == MIX_SAE) {
-      if (g < 0 || g >= n_groups || s_gtiles[g] == 0) {
-        atomicOr(a.status, MIX_STATUS_BAD_GROUP);
-      } else if (a.edit_only && add_error && s_gact[g] != MIX_SAE_TOPK) {
-        // handled by sae_edit_only_kernel: with the error term on, a ReLU / JumpReLU row needs
-        // only the pre-activations of its edited features, not the whole encode
-      } else if (!(q0.y & kKindGated) || gate_open(a.gates, slot, t)) {
-        meta = (g + 1) | (n_edit << 8) | (add_error << 16);
-        is_delta = add_error && n_edit > 0 && s_gact[g] != MIX_SAE_TOPK;
-      }
-    }
-    if (t < a.T) a.row_meta[t] = make_int2(meta, slot);
-    const int grp = (meta & 0xff) - 1;
-    for (int q = 0; q < n_groups; ++q) {
-      const unsigned m = __ballot_sync(0xffffffffu, grp == q);
-      if (lane == 0) s_wcnt[warp][q] = __popc(m);
-    }
-    {
-      const unsigned m = __ballot_sync(0xffffffffu, is_delta != 0);
-      if (lane == 0) s_wcnt[warp][n_groups] = __popc(m);
-    }
-    __syncthreads();
-    if (tid < ncol) {
-      int sum = 0;
-#pragma unroll
-      for (int w = 0; w < kFrontWarps; ++w) sum += s_wcnt[w][tid];
-      a.counts[cta * ncol + tid] = sum;
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) atomicAdd(a.sync, 1);                // (fence above + this: the chunk is published)
-  } else {
-    __syncthreads();                                   // (the weight-set table)
-  }
-  phase_stamp(a.clk, 1, first_cta && tid == 0);
-  // ---- step 2: wait for every chunk, scan the counts
+  auto slot_of = [&](int t) {
+    const int slot = t < a.T ? __ldg(a.token_slot + t) : -1;
+    return t < n_live && slot < n_slots ? slot : -1;
+  };
+  int rank[kFrontLocal], grp[kFrontLocal];             // local: this thread's rows -- weight set or -1, place among the warp's rows of the set
+  RowClass row[kFrontLocal];
   bool ok = true;
-  if (tid == 0 && ld_acquire(a.sync) < n_chunks) {     // one polling thread per CTA, backing off: a thousand CTAs ask about one word
-    const long long t0 = clock64();
-    unsigned ns = 32;
-    while (ld_acquire(a.sync) < n_chunks) {
-      if (clock64() - t0 > kFrontWaitCycles) { ok = false; break; }
-      __nanosleep(ns);
-      if (ns < 256) ns *= 2;
+  if (local) {
+    RowEntry e[kFrontLocal];
+#pragma unroll
+    for (int u = 0; u < kFrontLocal; ++u) e[u].slot = u < n_chunks ? slot_of(u * kFrontThreads + tid) : -1;
+#pragma unroll
+    for (int u = 0; u < kFrontLocal; ++u) e[u] = load_entry(a, e[u].slot);
+    for (int i = tid; i < n_chunks * kFrontWarps * ncol; i += kFrontThreads) s_wcnt[i / ncol][i % ncol] = 0;
+    if (tid < kFrontWarps) s_row[tid][0] = -1;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kFrontLocal; ++u) {
+      grp[u] = -1;
+      rank[u] = 0;
+      if (u < n_chunks) {
+        row[u] = classify(a, e[u], u * kFrontThreads + tid, s_gact, s_gtiles);
+        grp[u] = (row[u].meta & 0xff) - 1;
+        const unsigned same = __match_any_sync(0xffffffffu, grp[u]);
+        rank[u] = __popc(same & ((1u << lane) - 1u));
+        if (grp[u] >= 0 && rank[u] == 0) s_wcnt[u * kFrontWarps + warp][grp[u]] = __popc(same);
+        const unsigned dm = __ballot_sync(0xffffffffu, row[u].delta);
+        if (lane == 0) s_wcnt[u * kFrontWarps + warp][n_groups] = __popc(dm);
+      }
+    }
+    phase_stamp(a.clk, 1, first_cta && tid == 0);
+    __syncthreads();
+    for (int q = warp; q < ncol; q += kFrontWarps) {   // exclusive scan over (chunk, warp), one column per warp
+      const int v = lane < n_chunks * kFrontWarps ? s_wcnt[lane][q] : 0;
+      const int incl = warp_scan(v, lane);
+      if (lane < n_chunks * kFrontWarps) s_wcnt[lane][q] = incl - v;
+      if (lane == 31) s_total[q] = incl;
+    }
+  } else {
+    if (cta < n_chunks) {                              // classify and publish one chunk
+      const int t = cta * kFrontThreads + tid;
+      const RowEntry e = load_entry(a, slot_of(t));
+      __syncthreads();                                 // the weight-set table is in shared memory
+      const RowClass c = classify(a, e, t, s_gact, s_gtiles);
+      if (t < a.T) a.row_meta[t] = make_int2(c.meta, c.slot);
+      const int g = (c.meta & 0xff) - 1;
+      for (int q = 0; q < n_groups; ++q) {
+        const unsigned m = __ballot_sync(0xffffffffu, g == q);
+        if (lane == 0) s_wcnt[warp][q] = __popc(m);
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, c.delta);
+      if (lane == 0) s_wcnt[warp][n_groups] = __popc(m);
+      __syncthreads();
+      if (tid < ncol) {
+        int sum = 0;
+#pragma unroll
+        for (int w = 0; w < kFrontWarps; ++w) sum += s_wcnt[w][tid];
+        a.counts[cta * ncol + tid] = sum;
+      }
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) atomicAdd(a.sync, 1);              // (fence above + this: the chunk is published)
+    } else {
+      __syncthreads();                                 // (the weight-set table)
+    }
+    phase_stamp(a.clk, 1, first_cta && tid == 0);
+    // wait for every chunk, scan the counts
+    if (tid == 0 && ld_acquire(a.sync) < n_chunks) {   // one polling thread per CTA, backing off: a thousand CTAs ask about one word
+      const long long t0 = clock64();
+      unsigned ns = 32;
+      while (ld_acquire(a.sync) < n_chunks) {
+        if (clock64() - t0 > kFrontWaitCycles) { ok = false; break; }
+        __nanosleep(ns);
+        if (ns < 256) ns *= 2;
+      }
+    }
+    ok = __syncthreads_and(ok) != 0;
+    if (ok) {
+      for (int i = tid; i < n_chunks * ncol; i += kFrontThreads) s_tab[i] = __ldcg(a.counts + i);   // (never through L1: written by other SMs)
+      __syncthreads();
+      for (int q = warp; q < ncol; q += kFrontWarps) { // exclusive scan over the chunks, one column per warp
+        int carry = 0;
+        for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+          const int c = c0 + lane;
+          const int v = c < n_chunks ? s_tab[c * ncol + q] : 0;
+          const int incl = warp_scan(v, lane);
+          if (c < n_chunks) s_tab[c * ncol + q] = carry + incl - v;
+          carry += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) s_total[q] = carry;
+      }
     }
   }
-  ok = __syncthreads_and(ok) != 0;
   if (ok) {
-    for (int i = tid; i < n_chunks * ncol; i += kFrontThreads) s_tab[i] = __ldcg(a.counts + i);   // (never through L1: written by other SMs)
-    __syncthreads();
-    for (int q = warp; q < ncol; q += kFrontWarps) {   // exclusive scan over the chunks, one column per warp
-      int carry = 0;
-      for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-        const int c = c0 + lane;
-        const int v = c < n_chunks ? s_tab[c * ncol + q] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        if (c < n_chunks) s_tab[c * ncol + q] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-      }
-      if (lane == 0) s_total[q] = carry;
-    }
     __syncthreads();
     phase_stamp(a.clk, 2, first_cta && tid == 0);
-    if (tid == 0) {
-      int mt = 0, tiles = 0, rows = 0, topk_rows = 0;
-      long long cost_single = 0, cost_pair = 0, cost_split = 0;
-      int live_mask = 0, split_mask = 0, n_even = 0, n_odd3 = 0;
-      for (int q = 0; q < n_groups; ++q) {
-        s_base[q] = mt * kTileM;
-        const int m_tiles = (s_total[q] + kTileM - 1) / kTileM;
-        if (first_cta) {
-          a.rs->group_count[q] = s_total[q];
-          a.rs->group_mtile0[q] = mt;
-          a.rs->group_tile0[q] = tiles;
-          for (int m = 0; m < m_tiles; ++m) a.mtile_group[mt + m] = q;
-        }
-        mt += m_tiles;
-        rows += s_total[q];
-        if (s_total[q] > 0 && s_gact[q] == MIX_SAE_TOPK) topk_rows += s_total[q];
-        tiles += s_total[q] > 0 ? m_tiles * s_gtiles[q] : 0;
-        if (s_total[q] > 0) {
-          // per feature tile, in units of 1/40 of the time the W_enc tile takes to stream from HBM (measured on one
-          // weight set with 64 ... 1024 rows): single CTAs stream at the full rate for one row tile, and from two row
-          // tiles on every further tile costs 25 -- each of them fetches the W_enc tile again, from L2; a pair costs 46
-          // per 256-row tile whether its second half has rows or not, streaming at a slightly lower rate
-          const long long cs = (long long)(m_tiles == 1 ? 40 : 25 * m_tiles) * s_gtiles[q];
-          const long long cp = (long long)(46 * ((m_tiles + 1) / 2)) * s_gtiles[q];
-          cost_single += cs;
-          cost_pair += cp;
-          cost_split += min(cs, cp);
-          live_mask |= 1 << q;
-          if (cp < cs) {
-            split_mask |= 1 << q;
-            ++n_even;
-          } else if (m_tiles >= 3) {
-            ++n_odd3;
-          }
-        }
-      }
-      s_base[n_groups] = mt * kTileM;
-      s_n_panel_rows = mt * kTileM;
-      if (first_cta) {
-        for (int q = n_groups; q <= kMaxGroups; ++q) {
-          a.rs->group_mtile0[q] = mt;
-          a.rs->group_tile0[q] = tiles;
-          if (q < kMaxGroups) a.rs->group_count[q] = 0;
-        }
-        for (int m = mt; m < a.panel_cap / kTileM; ++m) a.mtile_group[m] = -1;
-        a.rs->n_panel_rows = mt * kTileM;
-        a.rs->n_mtiles = mt;
-        a.rs->n_sae_rows = rows;
-        a.rs->total_tiles = tiles;
-        a.rs->n_topk_rows = topk_rows;
-        a.rs->n_delta_rows = s_total[n_groups];
-        // Pairs win where a weight set has an even number of row tiles (two tiles share one fetch of W_enc, and the
-        // pair's instruction fills less shared memory per flop) and lose where half of a pair would repeat the other
-        // half's work: one row tile, or three.  Each weight set may go to the form that is cheaper for it -- the two
-        // encode kernels then both work, one after the other, which costs a second ramp-up and drain (about 25 us:
-        // in the units above 25 x 40 / (time to stream one tile of 512 d bytes at 6.3 TB/s) = 1.23e7 / d).
-        // Measured on config 4's replays, the split pays when two or more sets go to the pairs, or when a set of
-        // three or more row tiles stays with the single CTAs; ONE two-tile set among one-tile sets does not: inside
-        // the single-CTA kernel its second fetch of each W_enc tile and its tensor time hide behind the other sets'
-        // streams (1.67 ms all single against 1.71-1.74 ms split for sets of 1, 1, 1, 1, 2 tiles), so such a call
-        // stays with one form.
-        int mask = a.pair_mode == 1 ? live_mask : 0;
-        if (a.pair_mode == 2) {
-          const bool both = split_mask != 0 && split_mask != live_mask;
-          const long long split_total = cost_split + (both ? 12300000ll / max(a.d, 1) : 0ll);
-          const bool split_pays = !both || n_even >= 2 || n_odd3 >= 1;
-          if (split_pays && split_total <= min(cost_single, cost_pair)) mask = split_mask;
-          else mask = cost_pair < cost_single ? live_mask : 0;
-        }
-        // (Pairs give way to narrow tiles only where single CTAs can go down to 64 features: at 128 both forms bring the same
-        // bytes into an SM per k-block.)
-        int tile_n = kTileN;
-        if (a.pair_mode != 1 && 4 * tiles <= a.n_sms) mask = 0;
-        if (mask == 0) {
-          int nt_most = 1;
-          for (int q = 0; q < n_groups; ++q)
-            if (s_total[q] > 0) nt_most = max(nt_most, s_gtiles[q]);
-          tile_n = tile_width(tiles, nt_most, a.n_sms, a.cand_tiles);
-        }
-        a.rs->tile_n = tile_n;
-        a.rs->pair_mask = mask;
-        a.rs->use_pair = mask != 0;
-        if (a.n_flagged) *a.n_flagged = 0;       // fallback-selection flags of the fused TopK path start clear every call
-        // graph-conditional form: the rest of the SAE chain sits in the body of an IF node that runs only when a row needs it
-        if (a.use_cond) cudaGraphSetConditional(a.cond, rows > 0 ? 1u : 0u);
-      }
-    }
-    if (first_cta && a.mtile_flag)
-      for (int m = tid; m < a.panel_cap / kTileM; m += kFrontThreads) a.mtile_flag[m] = 0;
-    __syncthreads();
-    phase_stamp(a.clk, 3, first_cta && tid == 0);
-    // ---- step 3: this CTA's panel rows, one per warp
+    // every warp works out where the weight sets' rows start (lane q: set q)
+    const int my_total = lane < n_groups ? s_total[lane] : 0;
+    const int my_mt = (my_total + kTileM - 1) / kTileM;
+    const int mt_incl = warp_scan(my_mt, lane);
+    const int n_mtiles = __shfl_sync(0xffffffffu, mt_incl, 31), n_panel_rows = n_mtiles * kTileM;
+    const int my_base = (mt_incl - my_mt) * kTileM;
+    int t = -1, meta = 0, slot = -1;
     const int p = cta * kFrontWarps + warp;
-    if (p < a.panel_cap) {
-      int t = -1, meta = 0, slot = -1;
-      if (p < s_n_panel_rows) {
-        int g = 0;
-        while (g + 1 < n_groups && p >= s_base[g + 1]) ++g;
-        const int r = p - s_base[g];                   // rank of the row within its weight set
-        if (r < s_total[g]) {
-          // the chunk that holds rank r: the last one whose first rank is <= r
-          int c_hit = 0;
-          for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-            const int c = c0 + lane;
-            const unsigned m = __ballot_sync(0xffffffffu, c < n_chunks && s_tab[c * ncol + g] <= r);
-            if (m) c_hit = c0 + 31 - __clz(m);
-          }
-          int left = r - s_tab[c_hit * ncol + g];      // rank inside the chunk
-          int2 mm[kFrontThreads / 32];
+    if (local) {
 #pragma unroll
-          for (int i = 0; i < kFrontThreads / 32; ++i) {
-            const int tt = c_hit * kFrontThreads + i * 32 + lane;
-            mm[i] = tt < a.T ? __ldcg(a.row_meta + tt) : make_int2(0, -1);
+      for (int u = 0; u < kFrontLocal; ++u) {
+        if (u >= n_chunks) break;
+        const int base = __shfl_sync(0xffffffffu, my_base, grp[u] & 31);
+        if (grp[u] >= 0) {
+          const int pp = base + s_wcnt[u * kFrontWarps + warp][grp[u]] + rank[u];
+          if (pp / kFrontWarps == cta) {
+            int* r = s_row[pp % kFrontWarps];
+            r[0] = u * kFrontThreads + tid;
+            r[1] = row[u].meta;
+            r[2] = row[u].slot;
           }
-          bool found = false;
+        }
+      }
+      __syncthreads();
+      t = s_row[warp][0];
+      if (t >= 0) {
+        meta = s_row[warp][1];
+        slot = s_row[warp][2];
+      }
+    } else if (p < n_panel_rows) {
+      // the set is the last one that starts at or before p; the row's rank within it follows
+      const int g = 31 - __clz(__ballot_sync(0xffffffffu, lane < n_groups && my_mt > 0 && my_base <= p));
+      const int r = p - __shfl_sync(0xffffffffu, my_base, g);
+      if (r < __shfl_sync(0xffffffffu, my_total, g)) {
+        // the chunk that holds rank r: the last one whose first rank is <= r
+        int c_hit = 0;
+        for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+          const int c = c0 + lane;
+          const unsigned m = __ballot_sync(0xffffffffu, c < n_chunks && s_tab[c * ncol + g] <= r);
+          if (m) c_hit = c0 + 31 - __clz(m);
+        }
+        int left = r - s_tab[c_hit * ncol + g];        // rank inside the chunk
+        int2 mm[kFrontThreads / 32];
 #pragma unroll
-          for (int i = 0; i < kFrontThreads / 32; ++i) {
-            const unsigned m = __ballot_sync(0xffffffffu, (mm[i].x & 0xff) - 1 == g);
-            const int cnt = __popc(m);
-            if (!found) {
-              if (left < cnt) {
-                const int src = __fns(m, 0, left + 1);
-                t = c_hit * kFrontThreads + i * 32 + src;
-                meta = __shfl_sync(0xffffffffu, mm[i].x, src);
-                slot = __shfl_sync(0xffffffffu, mm[i].y, src);
-                found = true;
-              } else {
-                left -= cnt;
-              }
+        for (int i = 0; i < kFrontThreads / 32; ++i) {
+          const int tt = c_hit * kFrontThreads + i * 32 + lane;
+          mm[i] = tt < a.T ? __ldcg(a.row_meta + tt) : make_int2(0, -1);
+        }
+        bool found = false;
+#pragma unroll
+        for (int i = 0; i < kFrontThreads / 32; ++i) {
+          const unsigned m = __ballot_sync(0xffffffffu, (mm[i].x & 0xff) - 1 == g);
+          const int cnt = __popc(m);
+          if (!found) {
+            if (left < cnt) {
+              const int src = __fns(m, 0, left + 1);
+              t = c_hit * kFrontThreads + i * 32 + src;
+              meta = __shfl_sync(0xffffffffu, mm[i].x, src);
+              slot = __shfl_sync(0xffffffffu, mm[i].y, src);
+              found = true;
+            } else {
+              left -= cnt;
             }
           }
         }
+      }
+    }
+    phase_stamp(a.clk, 3, first_cta && tid == 0);
+    if (route_cta) {
+      if (warp == 0) {
+        const bool topk = lane < n_groups && s_gact[lane] == MIX_SAE_TOPK;
+        write_route(a, my_total, lane < n_groups ? s_gtiles[lane] : 0, topk, mt_incl - my_mt, n_mtiles, s_total[n_groups], lane);
+      } else {
+        for (int m0 = (warp - 1) * 32; m0 < a.panel_cap / kTileM; m0 += (kFrontWarps - 1) * 32) {
+          const int m = m0 + lane;
+          int g = -1;
+          for (int q = 0; q < n_groups; ++q) {         // (whole warps: the shuffles)
+            const int first = __shfl_sync(0xffffffffu, mt_incl - my_mt, q), n = __shfl_sync(0xffffffffu, my_mt, q);
+            if (m >= first && m < first + n) g = q;
+          }
+          if (m < a.panel_cap / kTileM) {
+            a.mtile_group[m] = g;
+            if (a.mtile_flag) a.mtile_flag[m] = 0;
+          }
+        }
+      }
+    }
+    // this CTA's panel rows, one per warp
+    if (p < a.panel_cap) {
+      if (p < n_panel_rows) {
         if (a.tau_slots && t >= 0) {                     // the encode's TopK bound starts empty
           reinterpret_cast<uint4*>(a.tau_slots + (size_t)p * kTauSlots)[lane] = make_uint4(0u, 0u, 0u, 0u);
           if (lane == 0) a.tau_min[p] = 0u;
@@ -446,12 +541,14 @@ front_kernel(const FrontArgs a) {
   // registers and shared memory, and resident any earlier they would crowd out the CTAs that still have rows to pack.
   pdl_launch_dependents();
   // the last CTA to leave closes the call: both counters are zero again when the next launch starts
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    if (atomicAdd(a.sync + 1, 1) == (int)gridDim.x - 1) {
-      a.sync[0] = 0;
-      a.sync[1] = 0;
+  if (!local) {
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(a.sync + 1, 1) == (int)gridDim.x - 1) {
+        a.sync[0] = 0;
+        a.sync[1] = 0;
+      }
     }
   }
 }
