@@ -327,8 +327,8 @@ int mix_set_feature_out(mix_ctx* ctx, int* topk_idx, float* topk_val, int* n_act
    hidden: device bf16 [T_max, d], modified in place.  T: number of rows of
    `hidden` that may be live (<= T_max; rows >= min(T, T_live) are pass-through).  scores_out:
    device fp32 [T_max, C_max] or NULL; only the first n_classes entries of probe rows are
-   written.  Enqueues kernels on `stream` (when the context has SAE weight sets, the probe /
-   steering kernels run on a context-owned side stream forked from and joined back into `stream`
+   written.  Enqueues kernels on `stream` (when the context has SAE weight sets, more than 2048 rows
+   and no slot chains, the probe / steering kernels run on a context-owned side stream forked from and joined back into `stream`
    by events, so they overlap the SAE chain; in a context for more than 2048 rows with multi-class
    probes and no SAE weight sets, the tensor-core probe kernel runs on that side stream beside the
    streaming kernel) and returns; safe to capture.  In a context without SAE weight sets and
@@ -409,9 +409,9 @@ int mix_bench_param_update(mix_ctx* ctx, int iters, float* us_table, float* us_n
 /* Which launches of the library use programmatic dependent launch (a kernel's CTAs may become resident,
    and run the part of the kernel that reads only library-owned tables, while the kernel in front of
    it in the stream is still running; everything the predecessor may have written is read after an
-   in-kernel wait).  Bits: 1 unused (the row pack is part of the first kernel of the SAE chain),
+   in-kernel wait).  Bits: 1 the first kernel of the SAE chain behind the hook kernel of a context of up to 2048 rows,
    2 the full SAE encode pass (the kernel in front of it lets it start only when its own rows are packed),
-   4 the kernels after it, 8 the one-CTA-per-row probe / steering kernel of a context that has no SAE weight sets
+   4 the kernels after it, 8 the one-CTA-per-row probe / steering kernel and the kernels that install a slot map
    (T_max <= 2048).  Default 1 | 2 | 4 | 8, or the value of MIX_PDL_MASK in the environment when the
    library first launches.  Process-wide; affects launches (and captures) made afterwards; meant
    for A/B measurement.  Returns the previous mask.  mask < 0 only queries. */

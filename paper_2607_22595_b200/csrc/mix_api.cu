@@ -785,7 +785,11 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // joined back into the caller's stream with events, which stream capture turns into graph
   // edges), the SAE chain on the caller's stream.  With the timing taps on, everything runs in
   // order on the caller's stream so that the per-stage times mean something.
-  const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on;
+  // In contexts of up to 2048 rows the hook kernel is a few microseconds, less than fork and join cost on the host and on
+  // the stream: there both run in the caller's stream, the front kernel launched programmatically, so that its look-ups
+  // overlap the hook kernel (tiny configuration, eagerly: 41 -> 38 us; 555 rows with 8-bit input: 213 -> 203).
+  const bool small = c->cfg.T_max <= kTeamMaxRows || (c->cfg.flags & MIX_FLAG_SLOT_CHAINS);
+  const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on && !small;
   cudaStream_t ps = fork ? c->side_stream : s;
   if (fork) {
     MIX_CUDA(c, cudaEventRecord(c->ev_fork, s));
@@ -828,10 +832,8 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   if (tc_fork) MIX_CUDA(c, cudaStreamWaitEvent(ps, c->ev_join, 0));
   if (fork) MIX_CUDA(c, cudaEventRecord(c->ev_join, ps));
   if (c->cfg.n_groups_max > 0) {
-    // with slot chains a steering app may precede an SAE app on the same row: the SAE chain reads
-    // the hidden state (first in the front kernel's row pack) only after the probe / steering kernel is done
-    if (fork && (c->cfg.flags & MIX_FLAG_SLOT_CHAINS)) MIX_CUDA(c, cudaStreamWaitEvent(s, c->ev_join, 0));
-    MIX_CUDA(c, launch_front(c, h, T, s, handle, conditional ? 1 : 0));   // routing + row pack
+    // (with slot chains a steering app may precede an SAE app on the same row: the hook kernel is in front of this one)
+    MIX_CUDA(c, launch_front(c, h, T, s, small && !c->stage_events_on, handle, conditional ? 1 : 0));   // routing + row pack
     MIX_CUDA(c, tap());
     const int rc = conditional ? sae_chain_conditional(c, h, s, graph, handle) : sae_chain(c, h, s, tap);
     if (rc != MIX_OK) return rc;

@@ -202,7 +202,7 @@ struct Ctx {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Which launches use programmatic dependent launch: bit 0 unused (the pack step is part of the front kernel now), bit 1
+// Which launches use programmatic dependent launch: bit 0 the front kernel behind a small context's hook kernel, bit 1
 // the full encode pass, bit 2 everything after it (tail, flagged-tile encode, flagged tail, edit-only kernels), bit 3
 // the one-CTA-per-row probe / steering kernel of a context without weight sets.
 // MIX_PDL_MASK in the environment overrides the default (A/B timing); read once.
@@ -265,7 +265,8 @@ bool has_tc_probe_stage(const Ctx* c);     // ... and, in contexts without SAE w
 cudaError_t launch_router(const Ctx* c, float* logits, int n_experts, int T, cudaStream_t s);
 // Routing + row pack in one launch.  cond/use_cond: graph-conditional handle the kernel sets to (SAE rows
 // routed > 0); plain calls pass 0, 0
-cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, unsigned long long cond = 0,
+// pdl: the kernel in front of it in the stream is the hook kernel
+cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, bool pdl = false, unsigned long long cond = 0,
                          int use_cond = 0);
 int front_chunks(int T_max);       // chunks of token rows the front kernel classifies: sizes d_front_counts / d_front_sync
 // bf16 [rows, d] row-major, boxes of 64 columns x box_rows rows, 128-byte swizzle; host work only

@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(NW * 32)
 probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
-                        unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl) {
+                        unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl, int late) {
   __shared__ float s_part[NW][kMaxClasses];
   constexpr int NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -416,15 +416,17 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   // into row `slot` of the context's vector arena, so their address follows from the slot id
   // alone: the row AND its vector are requested together, before the app entry is known.
   uint4 hq[kTeamVec], vq[kTeamVec];
+  // (`late`, contexts with SAE weight sets: most rows may be another kernel's; nothing is requested before the entry says
+  // that the row is this one's.  1000 SAE rows of d = 2304: 6.2 -> 4.5 us)
   const bool slot_ok = slot >= 0 && slot < n_slots;
-  if (slot_ok) {
+  if (slot_ok && !late) {
 #pragma unroll
     for (int u = 0; u < kTeamVec; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
     }
   }
-  if (!pdl && slot_ok) {
+  if (!pdl && slot_ok && !late) {
 #pragma unroll
     for (int u = 0; u < kTeamVec; ++u) {
       const int v = threadIdx.x + u * NT;
@@ -432,8 +434,18 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
     }
   }
   RowApp a = lookup(slot, t, apps, gates, n_slots, status, threadIdx.x == 0, /*eval_gate=*/false);
-  if (pdl) {
-    pdl_wait();
+  if (pdl) pdl_wait();
+  if (late) {
+    if (a.kind == 0 || a.kind == MIX_SAE || a.kind == MIX_ROUTER) return;
+#pragma unroll
+    for (int u = 0; u < kTeamVec; ++u) {
+      const int v = threadIdx.x + u * NT;
+      if (v < nvec) {
+        vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
+        hq[u] = __ldcs(hrow + v);
+      }
+    }
+  } else if (pdl) {
     if (slot_ok) {
 #pragma unroll
       for (int u = 0; u < kTeamVec; ++u) {
@@ -862,7 +874,8 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
   } else if (c->cfg.T_max <= kTeamMaxRows) {
     return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_team_kernel<8>, dim3(c->cfg.T_max), dim3(8 * 32), 0, s,
                       c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->cfg.n_slots_max, hidden, c->cfg.d_model,
-                      scores, c->cfg.C_max, c->d_status, reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
+                      scores, c->cfg.C_max, c->d_status, reinterpret_cast<const uint4*>(c->d_vec_arena), pdl,
+                      c->cfg.n_groups_max > 0 ? 1 : 0);
   } else {
     const int blocks = (c->cfg.T_max + kWarpsPerBlock - 1) / kWarpsPerBlock;
     probe_steer_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,

@@ -295,6 +295,8 @@ __device__ __forceinline__ void write_route(const FrontArgs& a, int total, int n
 //      the small count table and scans it.  The publishing CTAs never wait before they publish, and CTAs are dispatched in
 //      index order, so whoever waits, waits for work that is already running.  The rows of a CTA are found through the
 //      scan and the published records.
+// Launched programmatically behind the hook kernel of a small context: what is read before the wait is the slot map and the
+// tables, as in that kernel; gates, `hidden` and everything that is written come after it.
 // Then CTA b packs panel rows [8 b, 8 b + 8), one per warp.  The last CTA -- whose panel rows a call seldom needs -- writes
 // what exists once (routing result, tile -> weight-set map, conditional handle), beside the others' packing.  The last CTA
 // of the launch to leave puts the two counters back to zero for the next call.
@@ -337,6 +339,7 @@ front_kernel(const FrontArgs a) {
     for (int u = 0; u < kFrontLocal; ++u) e[u].slot = u < n_chunks ? slot_of(u * kFrontThreads + tid) : -1;
 #pragma unroll
     for (int u = 0; u < kFrontLocal; ++u) e[u] = load_entry(a, e[u].slot);
+    pdl_wait();
     for (int i = tid; i < n_chunks * kFrontWarps * ncol; i += kFrontThreads) s_wcnt[i / ncol][i % ncol] = 0;
     if (tid < kFrontWarps) s_row[tid][0] = -1;
     __syncthreads();
@@ -366,6 +369,7 @@ front_kernel(const FrontArgs a) {
     if (cta < n_chunks) {                              // classify and publish one chunk
       const int t = cta * kFrontThreads + tid;
       const RowEntry e = load_entry(a, slot_of(t));
+      pdl_wait();
       __syncthreads();                                 // the weight-set table is in shared memory
       const RowClass c = classify(a, e, t, s_gact, s_gtiles);
       if (t < a.T) a.row_meta[t] = make_int2(c.meta, c.slot);
@@ -387,6 +391,7 @@ front_kernel(const FrontArgs a) {
       __syncthreads();
       if (tid == 0) atomicAdd(a.sync, 1);              // (fence above + this: the chunk is published)
     } else {
+      pdl_wait();
       __syncthreads();                                 // (the weight-set table)
     }
     phase_stamp(a.clk, 1, first_cta && tid == 0);
@@ -557,7 +562,7 @@ front_kernel(const FrontArgs a) {
 
 int front_chunks(int T_max) { return (T_max + kFrontThreads - 1) / kFrontThreads; }
 
-cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, unsigned long long cond, int use_cond) {
+cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, bool pdl, unsigned long long cond, int use_cond) {
   FrontArgs a;
   a.token_slot = c->d_token_slot;
   a.n_live_p = c->d_n_live;
@@ -598,13 +603,11 @@ cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaS
   const size_t smem = (size_t)front_chunks(c->cfg.T_max) * (c->cfg.n_groups_max + 1) * sizeof(int);
   const int pack_ctas = (c->panel_rows_cap + kFrontWarps - 1) / kFrontWarps;
   const dim3 grid(chunks > pack_ctas ? chunks : pack_ctas);
-  if (c->cfg.flags & MIX_FLAG_FP8_ACT)
-    front_kernel<2><<<grid, kFrontThreads, smem, s>>>(a);
-  else if (c->cfg.flags & MIX_FLAG_FP8_W_ENC)      // hi codes in rows [0, P), lo codes in rows [P, 2P) of the same buffer
-    front_kernel<1><<<grid, kFrontThreads, smem, s>>>(a);
-  else
-    front_kernel<0><<<grid, kFrontThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  const int which = pdl ? kPdlPack : 0;
+  if (c->cfg.flags & MIX_FLAG_FP8_ACT) return launch_pdl(which, front_kernel<2>, grid, dim3(kFrontThreads), smem, s, a);
+  // (MIX_FLAG_FP8_W_ENC alone: hi codes in rows [0, P), lo codes in rows [P, 2P) of the same buffer)
+  if (c->cfg.flags & MIX_FLAG_FP8_W_ENC) return launch_pdl(which, front_kernel<1>, grid, dim3(kFrontThreads), smem, s, a);
+  return launch_pdl(which, front_kernel<0>, grid, dim3(kFrontThreads), smem, s, a);
 }
 
 }  // namespace mix
