@@ -4,11 +4,13 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libmix.so")
+FAST_PATH = os.path.join(PKG_DIR, "_fastcall.so")      # CPython module of the binding's per-step calls, linked to libmix.so
 
 SOURCES = ["mix_api.cu", "route_probe_steer.cu", "probe_tc.cu", "sae_front.cu", "sae_simt_edit_only.cu", "sae_encode_tc.cu", "sae_tail.cu",
            "sae_static.cu"]
@@ -22,9 +24,9 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not (os.path.exists(LIB_PATH) and os.path.exists(FAST_PATH)):
         return True
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(FAST_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "mix.h")]
     return any(os.path.getmtime(p) > t for p in deps)
 
@@ -46,4 +48,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
     if verbose:
         print(res.stderr)
+    cmd = [shutil.which("gcc") or "gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+           "-o", FAST_PATH, os.path.join(CSRC, "fastcall.c"), "-L", PKG_DIR, "-l:libmix.so", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("gcc failed:\n" + res.stdout + res.stderr)
     return LIB_PATH

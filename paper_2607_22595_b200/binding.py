@@ -74,11 +74,12 @@ class MixError(RuntimeError):
 
 
 _lib = None
+_fast = None          # the CPython module of the calls a step makes (csrc/fastcall.c), loaded with the library
 
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
     """Load libmix.so (built in-tree).  Raises if it is absent: there is no other path."""
-    global _lib
+    global _lib, _fast
     if _lib is not None and path is None:
         return _lib
     path = path or _build.LIB_PATH
@@ -117,7 +118,8 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
         if name != "mix_last_error":
             getattr(lib, name).restype = ci
     if path == _build.LIB_PATH:
-        _lib = lib
+        from . import _fastcall
+        _lib, _fast = lib, _fastcall
     return lib
 
 
@@ -154,6 +156,7 @@ class Mix:
         rc = self.lib.mix_create(C.byref(self.ctx), C.byref(self.cfg))
         if rc != 0:
             raise MixError(rc, "mix_create failed")
+        self._addr = self.ctx.value
         self._keep = {}          # borrowed weights must outlive their registration
 
     def _check(self, rc):
@@ -164,6 +167,7 @@ class Mix:
         if self.ctx:
             self.lib.mix_destroy(self.ctx)
             self.ctx = C.c_void_p()
+            self._addr = 0
             self._keep.clear()
 
     def __del__(self):
@@ -256,10 +260,9 @@ class Mix:
             n = len(token_slot) if T_live is None else T_live
             self._check(self.lib.mix_set_slot_map(self.ctx, token_slot.ctypes.data, n, 0, _stream(stream)))
             return
-        assert token_slot.dtype == torch.int32 and token_slot.is_contiguous()
-        n = token_slot.numel() if T_live is None else T_live
-        self._check(self.lib.mix_set_slot_map(self.ctx, token_slot.data_ptr(), n, int(token_slot.is_cuda),
-                                              _stream(stream)))
+        rc = _fast.set_slot_map(self._addr, token_slot, T_live, stream)
+        if rc != 0:
+            self._check(rc)
 
     def set_request_map(self, token_req, req_slot, T_live=None, stream=None):
         if isinstance(token_req, np.ndarray):
@@ -269,18 +272,18 @@ class Mix:
             self._check(self.lib.mix_set_request_map(self.ctx, token_req.ctypes.data, n, req_slot.ctypes.data,
                                                      len(req_slot), 0, _stream(stream)))
             return
-        n = token_req.numel() if T_live is None else T_live
-        self._check(self.lib.mix_set_request_map(self.ctx, token_req.data_ptr(), n, req_slot.data_ptr(),
-                                                 req_slot.numel(), int(token_req.is_cuda), _stream(stream)))
+        rc = _fast.set_request_map(self._addr, token_req, req_slot, T_live, stream)
+        if rc != 0:
+            self._check(rc)
 
     def set_feature_out(self, topk_idx=None, topk_val=None, n_active=None):
         self._check(self.lib.mix_set_feature_out(self.ctx, _ptr(topk_idx), _ptr(topk_val), _ptr(n_active)))
         self._keep["fo"] = (topk_idx, topk_val, n_active)
 
     def apply(self, hidden, scores_out=None, T=None, stream=None):
-        assert hidden.dtype == torch.bfloat16 and hidden.is_cuda and hidden.is_contiguous()
-        T = hidden.shape[0] if T is None else T
-        self._check(self.lib.mix_apply(self.ctx, hidden.data_ptr(), int(T), _ptr(scores_out), _stream(stream)))
+        rc = _fast.apply(self._addr, hidden, scores_out, T, stream)
+        if rc != 0:
+            self._check(rc)
 
     def apply_conditional(self, hidden, scores_out=None, T=None, stream=None):
         """As apply(), inside a stream capture only: the SAE chain becomes the body of a graph IF node."""
