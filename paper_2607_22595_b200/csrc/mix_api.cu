@@ -73,7 +73,7 @@ void free_all(mix_ctx* c) {
   cudaFree(c->d_edit_idx); cudaFree(c->d_edit_val); cudaFree(c->d_edit_mode); cudaFree(c->d_status);
   cudaFree(c->d_tmp_req); cudaFree(c->d_tmp_req_slot); cudaFree(c->d_panel); cudaFree(c->d_panel_row); cudaFree(c->d_act_scale); cudaFree(c->d_tau); cudaFree(c->d_tau_min); cudaFree(c->d_eo_row_delta); cudaFree(c->d_eo_coef);
   cudaFree(c->d_mtile_group); cudaFree(c->d_route); cudaFree(c->d_z);
-  cudaFree(c->d_tmap_w); cudaFree(c->d_phase_clk); cudaFree(c->d_tmap_probe); cudaFree(c->d_mc_census); cudaFree(c->d_mc_tiles); cudaFree(c->d_cand_val); cudaFree(c->d_cand_idx);
+  cudaFree(c->d_tmap_w); cudaFree(c->d_phase_clk); cudaFree(c->d_tmap_probe); cudaFree(c->d_mc_census); cudaFree(c->d_mc_tiles); cudaFree(c->d_part_logits); cudaFree(c->d_part_done); cudaFree(c->d_cand_val); cudaFree(c->d_cand_idx);
   cudaFree(c->d_cand_ninth); cudaFree(c->d_row_flag); cudaFree(c->d_mtile_flag); cudaFree(c->d_n_flagged);
   if (c->owned_b_eff)
     for (int g = 0; g < c->cfg.n_groups_max; ++g) cudaFree(c->owned_b_eff[g]);
@@ -326,7 +326,8 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   if (e == cudaSuccess && has_tc_probe_stage(c)) {
     // large batches with multi-class probes: the tensor-core probe kernel needs a map per probe matrix
     if (dev_alloc(&c->d_tmap_probe, NS) != cudaSuccess || dev_alloc(&c->d_mc_census, 1) != cudaSuccess ||
-        dev_alloc(&c->d_mc_tiles, (size_t)(T + kTileM - 1) / kTileM) != cudaSuccess) {
+        dev_alloc(&c->d_mc_tiles, (size_t)(T + kTileM - 1) / kTileM) != cudaSuccess ||
+        dev_alloc(&c->d_part_logits, (size_t)kPPartItems * kTileM * 32) != cudaSuccess || dev_alloc(&c->d_part_done, kPPartItems * 4) != cudaSuccess) {
       cudaGetLastError(); free_all(c); free(c); return MIX_ERR_NO_MEMORY;
     }
     e = cudaMemset(c->d_mc_census, 0, sizeof(McCensus));
@@ -798,9 +799,9 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   MIX_CUDA(c, tap());
   // Multi-class probes of a large batch have two kernels of which exactly one does the work: the 16-row
   // kernel takes batches sparse in such rows (and every batch of a context with SAE weight sets), the
-  // tensor-core kernel dense ones.  Where both exist, a one-CTA kernel makes the choice first and the
-  // tensor-core kernel -- whose rows no other kernel of this call touches -- runs on the context's side
-  // stream, beside the streaming kernel's pass over the batch.
+  // tensor-core kernel dense ones.  Where both exist, a census makes the choice first and both -- their rows
+  // no other kernel of this call touches -- run on the context's side stream, beside the streaming kernel's
+  // pass over the batch.
   const bool tc = has_tc_probe_stage(c);
   const bool tc_fork = tc && !c->stage_events_on;
   CUtensorMap tm_hidden;                         // host-side encoding only: no device work, fine under capture
@@ -813,6 +814,7 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
       MIX_CUDA(c, cudaEventRecord(c->ev_fork, ps));
       MIX_CUDA(c, cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
       MIX_CUDA(c, launch_probe_tc(c, tm_hidden, T, scores_out, c->side_stream));
+      MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, c->side_stream));
       MIX_CUDA(c, cudaEventRecord(c->ev_join, c->side_stream));
     }
   }
@@ -821,7 +823,7 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, c->map_installed != 0));
   c->map_installed = 0;
   MIX_CUDA(c, tap());
-  if (has_multiclass_stage(c)) {
+  if (has_multiclass_stage(c) && !tc_fork) {
     MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, ps));
     MIX_CUDA(c, tap());
   }

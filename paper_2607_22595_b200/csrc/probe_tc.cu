@@ -6,14 +6,16 @@
 // nothing, the job is to stream `hidden` from HBM once, at HBM speed.  That is what the TMA ->
 // tcgen05 pipeline of the SAE encode is good at, so the same machinery is used: one persistent CTA
 // per SM; warp 0 = TMA producer (a 128 x 64 tile of `hidden`, straight from the caller's tensor, and
-// a 32 x 64 tile of each probe matrix that occurs in the tile, per k-block, into a 5-stage ring:
-// ~80 KiB of `hidden` in flight per SM without holding a single register), warp 1 = MMA issuer
-// (M = 128, N = 32 per distinct probe of the tile, up to 4 probes side by side, fp32 accumulators
+// a 32 x 64 tile of each probe matrix that occurs in the tile, per k-block, into a 4-stage ring:
+// 64 KiB of `hidden` in flight per SM without holding a single register), warp 1 = MMA issuer
+// (M = 128, N = 32 per distinct probe of the tile, up to 8 probes side by side, fp32 accumulators
 // in tensor memory, double buffered), warps 2..5 = epilogue (one lane per row: its probe's 32
 // columns, + bias, softmax / sigmoid / identity, scores out), warp 6 = scout (reads the tile's slot
 // ids and app entries, evaluates gates, groups the rows by probe and hands the other roles one
 // descriptor per pass through a small ring).  Rows of other kinds inside a tile are streamed but
-// ignored.  The CTAs share out the tiles that a census kernel listed as holding such rows (mc_census_kernel), and the
+// ignored.  A work item is a tile, or -- where the listed tiles are few -- a part of its columns (see column_parts): the
+// items' partial logits meet in a scratch, and the last one to finish a quarter of the tile's rows adds them up, in order.
+// The CTAs share out the tiles that a census kernel listed as holding such rows (mc_census_kernel), and the
 // kernel takes the call when those tiles are at least half full of such rows; thinly scattered rows go to the 16-row mma.sync kernel.  No TMA multicast, no clusters; every wait is
 // bounded (on expiry: MIX_STATUS_WAIT_TIMEOUT, copies are given time to land, tensor memory freed).
 #include "mix_internal.h"
@@ -26,21 +28,27 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPStages = 9;
+constexpr int kPStages = 4;
 constexpr int kPABytes = kTileM * kTileK * 2;          // 16 KiB: 128 rows x 64 columns of hidden
 constexpr int kPBlockCols = 32;                        // accumulator columns per probe (= most classes taken)
-constexpr int kPBlocks = 2;                            // probes side by side in one pass
+// Probes side by side in one pass over the tile.  Batches of short requests have many probes in a tile, and every further
+// pass streams it again; eight leave room for four stages, which stream as fast as nine did with two (32768 rows of
+// d = 4096: 67 us either way; 11111 rows of 8 probes in requests of 16 tokens: 147 -> 68 us).
+constexpr int kPBlocks = 8;
 constexpr int kPBlockBytes = kPBlockCols * kTileK * 2; // 4 KiB: 32 classes x 64 columns
-constexpr int kPBBytes = kPBlocks * kPBlockBytes;      // 8 KiB
+constexpr int kPBBytes = kPBlocks * kPBlockBytes;      // 32 KiB
 constexpr int kPStageBytes = kPABytes + kPBBytes;
 constexpr int kPThreads = 7 * 32;
-constexpr int kPTmemCols = 2 * kPBlocks * kPBlockCols; // 128: two accumulators of 64 columns
+constexpr int kPTmemCols = 2 * kPBlocks * kPBlockCols; // 512: two accumulators of 256 columns
 constexpr long long kPWaitCycles = 4000000000ll;       // ~2 s at 2 GHz
 constexpr long long kPWaitCyclesTest = 2000000ll;      // ~1 ms: the cap under MIX_FLAG_TEST_STALL_ENCODE
 
 struct PDesc {
   int t0;                       // first row of the tile
-  int n_blocks;                 // probes in this pass (1..4); 0 = no more work for this CTA
+  int kb0, kb1;                 // this item's k-blocks
+  int list_tile, part;          // the tile's place in the census's list; which part of its columns
+  int last_pass;                // the item's last pass: the rows' partial logits are complete after it
+  int n_blocks;                 // probes in this pass (1..8); 0 = no more work for this CTA
   int slot[kPBlocks];
   signed char row_block[kTileM];   // block of each row in this pass, or -1
 };
@@ -61,16 +69,36 @@ constexpr int kPSmemBytes = kPStages * kPStageBytes + 1024 /* alignment slack */
 static_assert(kPSmemBytes <= 227 * 1024, "shared memory per CTA");
 static_assert(sizeof(PShared) <= 1024, "PShared must fit the space reserved for it");
 
+// Into how many parts of d the listed tiles are cut.  A tile is num_kb k-blocks of 16 KiB that one SM streams at 0.44 us each
+// (d = 5120: 80 of them, 35 us), so 30 tiles took as long as 148; the parts are chosen so that the longest CTA has the fewest
+// k-blocks, a part counting two more for its descriptor and epilogue.
+// 4000 rows of 16-class probes, d = 5120: 45 -> 26 us; 15873 rows with every kind of app, 2778 of them such probes: the call
+// 75 -> 58 us.
+constexpr int kPMostParts = 8;
+__device__ __forceinline__ int column_parts(int n_tiles, int num_kb, int n_ctas) {
+  int best = 1, best_cost = 1 << 30;
+  for (int parts = 1; parts <= kPMostParts && parts <= num_kb; ++parts) {
+    if (parts > 1 && n_tiles * parts > kPPartItems) break;
+    const int cost = (n_tiles * parts + n_ctas - 1) / n_ctas * ((num_kb + parts - 1) / parts + 2);
+    if (cost < best_cost) {
+      best = parts;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 __device__ __forceinline__ bool pwait(unsigned bar, unsigned parity, PShared* sh, unsigned* status) {
   return mbar_wait_bounded(bar, parity, &sh->abort_flag, &sh->wait_cycles, status);
 }
 
-__global__ void __launch_bounds__(kPThreads, 1)
+// (96 registers a thread, hence the bound of three CTAs: with the streaming kernel beside it, whose 20 Ki registers per CTA then fit twice into what is left)
+__global__ void __launch_bounds__(kPThreads, 3)
 probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorMap* __restrict__ tmap_probe,
                 const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
                 const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots, int d,
                 float* __restrict__ scores, int C_max, unsigned* __restrict__ status, const McCensus* __restrict__ census,
-                const int* __restrict__ census_tiles, int test_stall) {
+                const int* __restrict__ census_tiles, float* __restrict__ part_logits, int* __restrict__ part_done, int test_stall) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   PShared* sh = reinterpret_cast<PShared*>(tiles + kPStages * kPStageBytes);
@@ -80,7 +108,9 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
   // CTAs share THEM out, so a batch whose hooked requests are clustered still spreads evenly over the SMs
   if (!census->use_tc) return;                         // rows scattered thinly: probe_multiclass_kernel's call
   const int n_tiles = census->n_tiles;
-  if ((int)blockIdx.x >= n_tiles) return;              // CTA-uniform: this CTA owns no tile
+  const int num_kb = d / kTileK;
+  const int n_parts = column_parts(n_tiles, num_kb, gridDim.x), n_items = n_tiles * n_parts;
+  if ((int)blockIdx.x >= n_items) return;              // CTA-uniform: this CTA has no work
   if (threadIdx.x == 0) {
     for (int s = 0; s < kPStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
@@ -103,14 +133,14 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
   __syncthreads();
   tc_fence_after();
   const unsigned tmem_base = sh->tmem_base;
-  const int num_kb = d / kTileK;
 
   if (warp == 6) {
-    // ---- scout: one descriptor per (tile, pass of up to 4 probes), then a terminator
+    // ---- scout: one descriptor per (tile, pass of up to 8 probes), then a terminator
     int di = 0;
     unsigned dphase = 0;
     bool ok = true;
-    for (int ti = blockIdx.x; ti < n_tiles && ok; ti += gridDim.x) {
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      const int ti = item / n_parts, part = item - ti * n_parts;
       const int tile = __ldg(census_tiles + ti);
       int s[4], blk[4];
 #pragma unroll
@@ -153,6 +183,11 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
         PDesc* ds = &sh->desc[di];
         if (lane == 0) {
           ds->t0 = tile * kTileM;
+          ds->kb0 = num_kb * part / n_parts;
+          ds->kb1 = num_kb * (part + 1) / n_parts;
+          ds->list_tile = ti;
+          ds->part = part;
+          ds->last_pass = p == n_pass - 1;
           ds->n_blocks = min(kPBlocks, nd - p * kPBlocks);
         }
 #pragma unroll
@@ -182,7 +217,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
       for (;;) {
         if (!pwait(smem_u32(&sh->desc_full[di]), dphase, sh, status)) break;
         const PDesc* ds = &sh->desc[di];
-        const int nb = ds->n_blocks, t0 = ds->t0;
+        const int nb = ds->n_blocks, t0 = ds->t0, kb0 = ds->kb0, kb1 = ds->kb1;
         int slot[kPBlocks];
 #pragma unroll
         for (int b = 0; b < kPBlocks; ++b) slot[b] = ds->slot[b];
@@ -191,7 +226,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
         if (di == 0) dphase ^= 1u;
         if (nb == 0) break;
         bool ok = true;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!pwait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
           // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumers' bounded
           // waits run out and the whole CTA leaves through the time-out path.
@@ -214,7 +249,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
       unsigned dphase = 0, phase = 0, acc = 0, acc_phase = 0;
       for (;;) {
         if (!pwait(smem_u32(&sh->desc_full[di]), dphase, sh, status)) break;
-        const int nb = sh->desc[di].n_blocks;
+        const int nb = sh->desc[di].n_blocks, kb0 = sh->desc[di].kb0, kb1 = sh->desc[di].kb1;
         mbar_arrive(smem_u32(&sh->desc_empty[di]));
         di ^= 1;
         if (di == 0) dphase ^= 1u;
@@ -224,13 +259,13 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
         const unsigned d_tmem = tmem_base + acc * (kPBlocks * kPBlockCols);
         const unsigned idesc = idesc_f16(kTileM, nb * kPBlockCols);
         bool ok = true;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!pwait(smem_u32(&sh->full[stage]), phase, sh, status)) { ok = false; break; }
           tc_fence_after();
           const unsigned sa = smem_u32(tiles + stage * kPStageBytes);
           const unsigned long long da = umma_desc(sa), db = umma_desc(sa + kPABytes);
 #pragma unroll
-          for (int k = 0; k < kTileK / 16; ++k) umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, (unsigned)((kb | k) != 0));
+          for (int k = 0; k < kTileK / 16; ++k) umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, (unsigned)(kb != kb0 || k != 0));
           umma_commit(smem_u32(&sh->empty[stage]));
           if (++stage == kPStages) { stage = 0; phase ^= 1u; }
         }
@@ -245,6 +280,39 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
     const int q = warp & 3;                            // tensor-memory lane quarter this warp may read
     int di = 0;
     unsigned dphase = 0, acc = 0, acc_phase = 0;
+    int my_slot = -1;                                  // the probe of this lane's row in the present item
+    // logits of one row (bias not yet in them) -> scores
+    auto finish = [&](float (&v)[32], int slot, int t) {
+      const AppEntry* e = apps + slot;
+      const int C = __ldg(&e->n_classes), act = __ldg(&e->act);
+      const float* bias = reinterpret_cast<const float*>(__ldg(reinterpret_cast<const unsigned long long*>(&e->b)));
+      float mx = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        if (c < C) {
+          v[c] += bias ? __ldg(bias + c) : 0.f;
+          mx = fmaxf(mx, v[c]);
+        }
+      }
+      float* out = scores + (size_t)t * C_max;
+      if (act == MIX_ACT_SOFTMAX) {
+        float sum = 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          if (c < C) {
+            v[c] = expf(v[c] - mx);
+            sum += v[c];
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+          if (c < C) out[c] = v[c] / sum;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+          if (c < C) out[c] = act == MIX_ACT_SIGMOID ? 1.f / (1.f + expf(-v[c])) : v[c];
+      }
+    };
     for (;;) {
       if (!__all_sync(0xffffffffu, pwait(smem_u32(&sh->desc_full[di]), dphase, sh, status))) break;
       const PDesc* ds = &sh->desc[di];
@@ -260,39 +328,50 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
       if (!__all_sync(0xffffffffu, pwait(smem_u32(&sh->tmem_full[acc]), acc_phase, sh, status))) break;
       tc_fence_after();
       const unsigned taddr = tmem_base + ((unsigned)(q * 32) << 16) + acc * (kPBlocks * kPBlockCols);
-      for (int b = 0; b < nb; ++b) {
-        float v[32];
-        tmem_ld32(taddr + b * kPBlockCols, v);
-        if (my_block != b) continue;                   // the load above is warp-wide; the rest is per row
-        const AppEntry* e = apps + ds->slot[b];
-        const int C = __ldg(&e->n_classes), act = __ldg(&e->act);
-        const float* bias = reinterpret_cast<const float*>(__ldg(reinterpret_cast<const unsigned long long*>(&e->b)));
-        float mx = -INFINITY;
+      float mine[32];                                  // the row's logits
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          if (c < C) {
-            v[c] += bias ? __ldg(bias + c) : 0.f;
-            mx = fmaxf(mx, v[c]);
-          }
+      for (int c = 0; c < 32; c += 8) {                // (eight columns at a time: a block's worth of registers, not two)
+        for (int b = 0; b < nb; ++b) {
+          float v[8];
+          tmem_ld8(taddr + b * kPBlockCols + c, v);    // (warp-wide)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mine[c + i] = b == 0 || my_block == b ? v[i] : mine[c + i];
         }
-        float* out = scores + (size_t)t * C_max;
-        if (act == MIX_ACT_SOFTMAX) {
-          float sum = 0.f;
+      }
+      if (my_block >= 0) my_slot = ds->slot[my_block];
+      bool complete = my_block >= 0 && n_parts == 1;
+      if (n_parts > 1) {
+        if (my_block >= 0) {
+          float4* p = reinterpret_cast<float4*>(part_logits + ((size_t)(ds->list_tile * n_parts + ds->part) * kTileM + row) * 32);
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            if (c < C) {
-              v[c] = expf(v[c] - mx);
-              sum += v[c];
+          for (int c = 0; c < 8; ++c) __stcg(p + c, make_float4(mine[4 * c], mine[4 * c + 1], mine[4 * c + 2], mine[4 * c + 3]));
+        }
+        if (ds->last_pass) {
+          // these 32 rows' part is in the scratch; whoever is the last of the parts finds all of them there
+          __threadfence();
+          __syncwarp();
+          int done = 0;
+          if (lane == 0) done = atomicAdd(part_done + ds->list_tile * 4 + q, 1);
+          done = __shfl_sync(0xffffffffu, done, 0);
+          complete = done == n_parts - 1 && my_slot >= 0;
+          if (complete) {
+            __threadfence();
+#pragma unroll
+            for (int c = 0; c < 32; ++c) mine[c] = 0.f;
+            for (int k = 0; k < n_parts; ++k) {
+              const float4* p = reinterpret_cast<const float4*>(part_logits + ((size_t)(ds->list_tile * n_parts + k) * kTileM + row) * 32);
+#pragma unroll
+              for (int c = 0; c < 8; ++c) {
+                const float4 x = __ldcg(p + c);
+                mine[4 * c] += x.x; mine[4 * c + 1] += x.y; mine[4 * c + 2] += x.z; mine[4 * c + 3] += x.w;
+              }
             }
           }
-#pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c < C) out[c] = v[c] / sum;
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c < C) out[c] = act == MIX_ACT_SIGMOID ? 1.f / (1.f + expf(-v[c])) : v[c];
         }
+      }
+      if (complete) finish(mine, my_slot, t);
+      if (ds->last_pass) {
+        my_slot = -1;
       }
       tc_fence_before();
       __syncwarp();
@@ -330,7 +409,7 @@ cudaError_t launch_probe_tc(const Ctx* c, const CUtensorMap& tmap_hidden, int T,
   if (scores == nullptr) return cudaSuccess;
   probe_tc_kernel<<<c->n_sms, kPThreads, kPSmemBytes, s>>>(tmap_hidden, c->d_tmap_probe, c->d_token_slot, c->d_n_live, T,
                                                            c->d_apps, c->d_gates, c->cfg.n_slots_max, c->cfg.d_model, scores,
-                                                           c->cfg.C_max, c->d_status, c->d_mc_census, c->d_mc_tiles,
+                                                           c->cfg.C_max, c->d_status, c->d_mc_census, c->d_mc_tiles, c->d_part_logits, c->d_part_done,
                                                            (c->cfg.flags & MIX_FLAG_TEST_STALL_ENCODE) ? 1 : 0);
   return cudaGetLastError();
 }

@@ -157,7 +157,6 @@ __device__ __forceinline__ void finish_probe(const float* logit, int C, int act,
   if (lane + 32 < C) out[lane + 32] = z1;
 }
 
-constexpr int kWarpsPerBlock = 8;      // = rows per CTA of the large-batch kernel
 constexpr int kCoopMaxClasses = 32;    // widest probe the cooperative tensor-core pass takes
 
 // One row, one warp: steer, single-class probe, or multi-class probe.
@@ -203,17 +202,21 @@ __device__ __forceinline__ void warp_row(const RowApp& a, __nv_bfloat16* __restr
   finish_probe(s_logit, a.C, a.act, out, lane);
 }
 
-// Large batches: a CTA owns 8 consecutive rows, one warp per row: streaming work (steering,
+// Large batches: a CTA owns kWarps consecutive rows, one warp per row: streaming work (steering,
 // single-class probes).  Multi-class probes up to kCoopMaxClasses classes are left to
 // probe_tc_kernel (probe_tc.cu) when `multiclass_elsewhere` is set.
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, 3)
+// Bound by the bytes in flight.  Small CTAs, as many warps as 56 registers let an SM hold (11111 rows of d = 5120, steering,
+// one-class probes and projections: 37.2 us with eight-warp CTAs at 66 registers, 35.3 so) -- except beside the
+// tensor-core kernel, which leaves room for eight warps at a time.
+template <int kWarps, int kMinCtas>
+__global__ void __launch_bounds__(kWarps * 32, kMinCtas)
 probe_steer_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
                    const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                    __nv_bfloat16* __restrict__ hidden, int d,
                    float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int multiclass_elsewhere) {
-  __shared__ float s_logit[kWarpsPerBlock][kMaxClasses];
+  __shared__ float s_logit[kWarps][kMaxClasses];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kWarpsPerBlock + warp;
+  const int t = blockIdx.x * kWarps + warp;
   const int n_live = __ldg(n_live_p);            // issued together with the slot id: one round trip, not two
   const int slot = t < T ? __ldg(token_slot + t) : -1;
   if (t >= min(T, n_live)) return;
@@ -795,7 +798,10 @@ __global__ void fold_bias_kernel(const __nv_bfloat16* __restrict__ W_enc, const 
 constexpr int kCensusWarps = 8;
 __global__ void __launch_bounds__(kCensusWarps * 32)
 mc_census_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
-                 const AppEntry* __restrict__ apps, int n_slots, McCensus* __restrict__ census, int* __restrict__ tiles) {
+                 const AppEntry* __restrict__ apps, int n_slots, McCensus* __restrict__ census, int* __restrict__ tiles,
+                 int* __restrict__ part_done) {
+  if (blockIdx.x == 0)                                   // the tensor-core kernel's counters of finished column parts
+    for (int i = threadIdx.x; i < kPPartItems * 4; i += kCensusWarps * 32) part_done[i] = 0;
   __shared__ int s_cnt[kCensusWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int live = min(T, __ldg(n_live_p));
@@ -857,7 +863,7 @@ bool has_multiclass_stage(const Ctx* c) {
 cudaError_t launch_mc_census(const Ctx* c, int T, cudaStream_t s) {
   const int rows_per_cta = kCensusWarps * kTileM;
   mc_census_kernel<<<(c->cfg.T_max + rows_per_cta - 1) / rows_per_cta, kCensusWarps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps,
-                                                                           c->cfg.n_slots_max, c->d_mc_census, c->d_mc_tiles);
+                                                                           c->cfg.n_slots_max, c->d_mc_census, c->d_mc_tiles, c->d_part_done);
   return cudaGetLastError();
 }
 
@@ -877,10 +883,13 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
                       scores, c->cfg.C_max, c->d_status, reinterpret_cast<const uint4*>(c->d_vec_arena), pdl,
                       c->cfg.n_groups_max > 0 ? 1 : 0);
   } else {
-    const int blocks = (c->cfg.T_max + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    probe_steer_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
-                                                              c->cfg.n_slots_max, hidden, c->cfg.d_model, scores,
-                                                              c->cfg.C_max, c->d_status, has_multiclass_stage(c) ? 1 : 0);
+    auto run = [&](auto kernel, int warps) {
+      kernel<<<(c->cfg.T_max + warps - 1) / warps, warps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+                                                                      c->cfg.n_slots_max, hidden, c->cfg.d_model, scores,
+                                                                      c->cfg.C_max, c->d_status, has_multiclass_stage(c) ? 1 : 0);
+    };
+    if (has_tc_probe_stage(c)) run(probe_steer_kernel<8, 3>, 8);
+    else run(probe_steer_kernel<4, 8>, 4);
   }
   return cudaGetLastError();
 }

@@ -139,3 +139,32 @@ def test_time_out_path_of_the_tensor_core_probe_kernel():
     good = run_gpu(w)
     assert good["status"] == 0
     check_parity(W.host(w), good)
+
+
+@pytest.mark.parametrize("d", [64, 448, 2048])
+@pytest.mark.parametrize("T,rows", [(2049, 64), (2049, 2049), (6000, 128 * 40), (40000, 128 * 150), (60000, 128 * 400)])
+def test_columns_cut_into_parts(d, T, rows):
+    """Batches of 1 ... 400 listed tiles: the kernel cuts a tile's columns into one to eight parts; twice, on the same scratch."""
+    g = torch.Generator(device="cuda"); g.manual_seed(d + T)
+    mixlib = _mixlib()
+    m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=3, C_max=17)
+    C = [17, 2, 5]
+    Wp = [(torch.randn((c, d), generator=g, device="cuda") * d ** -0.5).to(torch.bfloat16) for c in C]
+    b = [torch.randn(c, generator=g, device="cuda") for c in C]
+    for i in range(3):
+        m.register_probe(i, Wp[i], b[i], mixlib.MIX_ACT_SOFTMAX)
+    slot = torch.full((T,), -1, dtype=torch.int32, device="cuda")
+    slot[:rows] = (torch.arange(rows, device="cuda") // 70 % 3).int()
+    m.set_slot_map(slot)
+    for _ in range(2):
+        hidden = torch.randn((T, d), generator=g, device="cuda").to(torch.bfloat16)
+        scores = torch.full((T, 17), -1.0, device="cuda")
+        m.apply(hidden, scores)
+        for i in range(3):
+            pick = slot == i
+            want = torch.softmax(hidden[pick].double() @ Wp[i].double().T + b[i].double(), dim=1)
+            assert ((scores[pick, :C[i]].double() - want).abs() <= 1e-3 * want).all()
+            assert (scores[pick, C[i]:] == -1.0).all()
+        assert (scores[slot < 0] == -1.0).all()
+    assert m.get_status() == 0
+    m.destroy()
