@@ -255,11 +255,6 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   constexpr int kTcThreads = Cfg::kThreads;
   constexpr int kEpiWarps = Cfg::kEpiWarps;
   constexpr int kEpiColsMax = kTileN / (kEpiWarps / 4);
-  pdl_wait();
-  pdl_launch_dependents();
-  const bool stamp = clk != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && mode == 0 && !kPair;
-  phase_stamp(clk, 26, stamp);
-  if (mode == 1 && *n_flagged == 0) return;
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: required by the 128-byte swizzle atoms
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -276,35 +271,9 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   const int worker = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int n_workers = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 
-  for (int i = threadIdx.x; i < (int)(sizeof(RouteState) / sizeof(int)); i += kTcThreads)
-    reinterpret_cast<int*>(&sh->rs)[i] = reinterpret_cast<const int*>(rs_g)[i];
-  __syncthreads();
-  // Feature width of this call's tiles: 256, or 128 / 64 where full-width tiles would leave half of the SMs or more without
-  // one (decided by the front kernel).  A narrower tile makes a shorter stage, so the ring holds more of them.
-  const int tile_n = kPair ? kTileN : sh->rs.tile_n;
-  const int n_sub = kTileN / tile_n;                   // tiles per 256 features
-  const int stage_bytes = Cfg::kARingBytes + (kPair ? Cfg::kBBytesCta : tile_n * (kTileK * 2));
-  const int n_stages = min(kMaxStages, Cfg::kRingBytes / stage_bytes);
-  const int epi_cols = tile_n / (kEpiWarps / 4);       // columns of a tile per epilogue warp
+  // what does not depend on the routing is done before the wait
   if (threadIdx.x == 0) {
-    {      // this kernel's weight sets: units (row tiles, or pairs of them) and tiles, numbered through
-      int nu = 0, ut = 0;
-      for (int g = 0; g < n_groups; ++g) {
-        const int mt = sh->rs.group_mtile0[g + 1] - sh->rs.group_mtile0[g];
-        const int nt = mt > 0 ? (sh->rs.group_tile0[g + 1] - sh->rs.group_tile0[g]) / mt * n_sub : 0;
-        const bool mine = mode != 0 || (((sh->rs.pair_mask >> g) & 1) != 0) == kPair;
-        const int units = !mine ? 0 : (kPair ? (mt + 1) / 2 : mt);
-        sh->unit0[g] = (short)nu;
-        sh->utile0[g] = ut;
-        nu += units;
-        ut += units * nt;
-      }
-      for (int g = n_groups; g <= kMaxGroups; ++g) {
-        sh->unit0[g] = (short)nu;
-        sh->utile0[g] = ut;
-      }
-    }
-    for (int s = 0; s < n_stages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
@@ -318,20 +287,55 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();
+  pdl_launch_dependents();
+  const bool stamp = clk != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && mode == 0 && !kPair;
+  phase_stamp(clk, 26, stamp);
+  if (mode == 1 && *n_flagged == 0) return;
+  for (int i = threadIdx.x; i < (int)(sizeof(RouteState) / sizeof(int)); i += kTcThreads)
+    reinterpret_cast<int*>(&sh->rs)[i] = reinterpret_cast<const int*>(rs_g)[i];
   __syncthreads();
-  // the full pass has two kernels, single CTAs and CTA pairs, and the front kernel dealt this call's weight sets
-  // between them: nothing routed to any SAE, or no set for this kernel -- no tensor memory is taken (both CTAs
-  // of a pair see the same)
-  const int total_tiles = sh->utile0[n_groups];
-  if (total_tiles == 0) return;
-
-  if (warp == 1) {
-    if (kPair) tmem_alloc_pair(smem_u32(&sh->tmem_base), kTmemCols);
-    else tmem_alloc(smem_u32(&sh->tmem_base), kTmemCols);
+  // Feature width of this call's tiles: 256, or 128 / 64 where full-width tiles would leave half of the SMs or more without
+  // one (decided by the front kernel).  A narrower tile makes a shorter stage, so the ring holds more of them.
+  const int tile_n = kPair ? kTileN : sh->rs.tile_n;
+  const int n_sub = kTileN / tile_n;                   // tiles per 256 features
+  const int stage_bytes = Cfg::kARingBytes + (kPair ? Cfg::kBBytesCta : tile_n * (kTileK * 2));
+  const int n_stages = min(kMaxStages, Cfg::kRingBytes / stage_bytes);
+  const int epi_cols = tile_n / (kEpiWarps / 4);       // columns of a tile per epilogue warp
+  if (warp < 2) {
+    // this kernel's weight sets (lane g: set g): units (row tiles, or pairs of them) and tiles, numbered through.  The full
+    // pass has two kernels, single CTAs and CTA pairs, and the front kernel dealt this call's weight sets between them.
+    static_assert(kMaxGroups == 32, "a lane per weight set");
+    const int mt = lane < n_groups ? sh->rs.group_mtile0[lane + 1] - sh->rs.group_mtile0[lane] : 0;
+    const int nt = mt > 0 ? (sh->rs.group_tile0[lane + 1] - sh->rs.group_tile0[lane]) / mt * n_sub : 0;
+    const bool mine = mode != 0 || (((sh->rs.pair_mask >> lane) & 1) != 0) == kPair;
+    const int units = !mine ? 0 : (kPair ? (mt + 1) / 2 : mt);
+    if (warp == 0) {
+      int nu = units, ut = units * nt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, nu, o), z = __shfl_up_sync(0xffffffffu, ut, o);
+        if (lane >= o) {
+          nu += y;
+          ut += z;
+        }
+      }
+      sh->unit0[lane + 1] = (short)nu;
+      sh->utile0[lane + 1] = ut;
+      if (lane == 0) {
+        sh->unit0[0] = 0;
+        sh->utile0[0] = 0;
+      }
+    } else if (__any_sync(0xffffffffu, units * nt != 0)) {     // (nothing for this kernel: no tensor memory is taken)
+      if (kPair) tmem_alloc_pair(smem_u32(&sh->tmem_base), kTmemCols);
+      else tmem_alloc(smem_u32(&sh->tmem_base), kTmemCols);
+    }
   }
   tc_fence_before();
+  __syncthreads();
+  const int total_tiles = sh->utile0[n_groups];
+  if (total_tiles == 0) return;            // (both CTAs of a pair see the same)
   if (kPair) cluster_sync_all();           // the peer's barriers are initialised before anything is sent to them
-  else __syncthreads();
   tc_fence_after();
   const unsigned tmem_base = sh->tmem_base;
   phase_stamp(clk, 27, stamp);

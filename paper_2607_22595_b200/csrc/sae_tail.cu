@@ -424,6 +424,7 @@ struct TailArgs {
   int n_col_slices;         // delta role: ceil(d / 2048)
   unsigned long long* clk;  // profiling aid or null
   int n_groups;
+  int panel_cap;
 };
 
 struct RowShared {
@@ -573,21 +574,21 @@ __device__ void rebuild_row(const TailArgs& a, RowShared& sh, int p, const float
 // L2 while the selection runs was tried twice: line by line, one 128-byte line per lane, the 1024 prefetches of a
 // row cost more issue time -- 3 us -- than the latency they hid; one bulk prefetch per decoder row made the
 // staging step 1.5 us slower and the gather no faster.)
-__device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
+__device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups, const RouteState& rs, const RowRec* guess) {
   const int tid = threadIdx.x;
   const int d = a.d, nvec = d >> 3;
   // the call's SAE rows, numbered through the weight sets without the padding rows of their last tiles
-  constexpr int kGrpVecs = (int)(sizeof(GroupEntry) / sizeof(uint4));
-  if (tid >= 32 && tid < 32 + n_groups * kGrpVecs)
-    reinterpret_cast<uint4*>(sh.grp)[tid - 32] = reinterpret_cast<const uint4*>(a.groups)[tid - 32];
-  if (tid == 0) {
-    int cum = 0;
-    for (int g = 0; g < n_groups; ++g) {
-      sh.cum[g] = cum;
-      sh.row0[g] = a.rs->group_mtile0[g] * kTileM;
-      cum += a.rs->group_count[g];
+  if (tid < 32) {
+    const int n = tid < n_groups ? rs.group_count[tid] : 0;
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (tid >= o) incl += y;
     }
-    sh.cum[n_groups] = cum;
+    sh.cum[tid + 1] = incl;
+    if (tid == 0) sh.cum[0] = 0;
+    sh.row0[tid] = rs.group_mtile0[tid] * kTileM;
   }
   __syncthreads();
   const int n_work = sh.cum[n_groups];
@@ -607,7 +608,8 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
     const int p = sh.row0[g_w] + (w - sh.cum[g_w]);
     const bool stamp = item == 0 && tid == 0 && a.mode != kTailFallback;
     phase_stamp(a.clk, 9, stamp);
-    const RowRec rec = a.row_rec[p];
+    const int shift = n_split == 4 ? 2 : n_split - 1;
+    const RowRec rec = item == (int)blockIdx.x && p == item >> shift ? guess[shift] : a.row_rec[p];   // (requested with the routing result)
     const int t = rec.t;
     if (t < 0) continue;                               // padding row of a tile (uniform across the CTA, like every branch below)
     // (the weight-set entry field by field, not as a struct held in registers across the whole row)
@@ -631,7 +633,7 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups) {
     }
     const int S = (int)gp->d_sae, k = gp->k;
     const float* z = a.Z + (size_t)p * a.ldz;
-    const int n_tiles = S / a.rs->tile_n, n_cand = n_tiles * kCandPerTile;
+    const int n_tiles = S / rs.tile_n, n_cand = n_tiles * kCandPerTile;
     unsigned ninth_max = 0u;                           // largest key among this thread's share of the tiles' 9th values
     unsigned kmin = 0xffffffffu, kmax = 0u;            // range of this thread's share of the candidate keys
     if (from_cand && n_cand >= k && n_cand <= kCandMax) {
@@ -954,8 +956,26 @@ tail_kernel(const TailArgs a) {
     stamp_launch_end(a.clk, a.mode);
     return;
   }
-  const int n_rows = a.rs->n_panel_rows, n_delta = a.rs->n_delta_rows, n_sae = a.rs->n_sae_rows;
-  if (a.mode == kTailFallback || n_sae > n_delta || (a.out_n_active != nullptr && n_sae > 0)) tail_rows(a, s_row, a.n_groups);
+  // One round trip for all that the first row needs to know: the routing result, the weight-set table, and the record of the
+  // row this CTA will have if the call's rows all belong to the first weight set that has any (the usual short call), for
+  // each way of sharing rows between CTAs.
+  __shared__ RouteState s_rs;
+  __shared__ RowRec s_guess[3];
+  {
+    constexpr int kRsWords = (int)(sizeof(RouteState) / sizeof(int)), kGrpVecs = (int)(sizeof(GroupEntry) / sizeof(uint4));
+    static_assert(kRsWords <= kTailThreads - 6, "a thread per word of the routing result");
+    const int tid = threadIdx.x;
+    if (tid < kRsWords) reinterpret_cast<int*>(&s_rs)[tid] = reinterpret_cast<const int*>(a.rs)[tid];
+    if (tid >= kTailThreads - 6) {
+      const int i = (tid - (kTailThreads - 6)) >> 1, half = tid & 1, p = min((int)blockIdx.x >> i, a.panel_cap - 1);
+      reinterpret_cast<uint4*>(s_guess + i)[half] = reinterpret_cast<const uint4*>(a.row_rec + p)[half];
+    }
+    for (int i = tid; i < a.n_groups * kGrpVecs; i += kTailThreads)
+      reinterpret_cast<uint4*>(s_row.grp)[i] = reinterpret_cast<const uint4*>(a.groups)[i];
+    __syncthreads();
+  }
+  const int n_rows = s_rs.n_panel_rows, n_delta = s_rs.n_delta_rows, n_sae = s_rs.n_sae_rows;
+  if (a.mode == kTailFallback || n_sae > n_delta || (a.out_n_active != nullptr && n_sae > 0)) tail_rows(a, s_row, a.n_groups, s_rs, s_guess);
   if (a.mode != kTailFallback && n_delta > 0) {
     const int n_rg = n_rows / kDlRows;
     const int n_cg = min(a.n_col_slices, max(1, (int)gridDim.x / n_rg));
@@ -998,6 +1018,7 @@ cudaError_t launch_tail(const Ctx* c, __nv_bfloat16* hidden, int mode, cudaStrea
   a.mode = mode;
   a.clk = c->d_phase_clk;
   a.n_groups = c->cfg.n_groups_max;
+  a.panel_cap = c->panel_rows_cap;
   const int n_sms = c->n_sms > 0 ? c->n_sms : 148;
   a.n_col_slices = (c->cfg.d_model / 8 + kTailThreads - 1) / kTailThreads;
   const int work_cap = c->panel_rows_cap > (c->panel_rows_cap / kDlRows) * a.n_col_slices ? c->panel_rows_cap
