@@ -103,6 +103,12 @@ const int* device_view(const int* host) {
   return at.type == cudaMemoryTypeUnregistered ? nullptr : static_cast<const int*>(at.devicePointer);
 }
 
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();   // (what is enqueued next reports it)
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Publish an app entry: body first with valid = 0, then the valid word.
 // bias_src: device fp32 whose value goes into the entry's `alpha` word before the entry becomes valid (a one-class
 // probe's bias in contexts whose hook kernel reads it from there), or null.
@@ -712,6 +718,10 @@ namespace {
 // The SAE chain behind the front kernel: encode ... write-back.  `tap` records a stage event after each launch.
 template <class Tap>
 int sae_chain(mix_ctx* c, __nv_bfloat16* h, cudaStream_t s, Tap&& tap) {
+  // The two fallback launches serve rows of TopK sets.  A call that is not being captured knows whether there are any; a
+  // captured one may be replayed with sets registered later.  (reconstruct() on a JumpReLU set: 247 -> 243 us.)
+  bool topk = is_capturing(s);
+  for (int g = 0; g < c->cfg.n_groups_max; ++g) topk = topk || (c->h_groups[g].valid && c->h_groups[g].act == MIX_SAE_TOPK);
   if (c->cfg.flags & MIX_FLAG_ENCODE_SIMT) {
     MIX_CUDA(c, launch_encode_simt(c, s));
     MIX_CUDA(c, tap());
@@ -726,9 +736,9 @@ int sae_chain(mix_ctx* c, __nv_bfloat16* h, cudaStream_t s, Tap&& tap) {
     MIX_CUDA(c, tap());
     MIX_CUDA(c, launch_tail(c, h, 0, s));        // exact TopK from candidates (or a flag), edits, decode
     MIX_CUDA(c, tap());
-    MIX_CUDA(c, launch_encode_tc(c, 1, false, s));   // flagged row tiles -> Z (returns at once if none)
+    if (topk) MIX_CUDA(c, launch_encode_tc(c, 1, false, s));   // flagged row tiles -> Z (returns at once if none)
     MIX_CUDA(c, tap());
-    MIX_CUDA(c, launch_tail(c, h, 2, s));        // the flagged rows (returns at once if none)
+    if (topk) MIX_CUDA(c, launch_tail(c, h, 2, s));        // the flagged rows (returns at once if none)
     MIX_CUDA(c, tap());
   }
   return MIX_OK;
