@@ -40,3 +40,44 @@ def test_maps_of_changing_length(T, source, with_sae):
         assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), live
     assert m.get_status() == 0
     m.destroy()
+
+
+@pytest.mark.parametrize("live", [1, 256, 257, 896, 897])
+@pytest.mark.parametrize("before", [0, 1000])
+def test_pinned_maps_in_a_graph_and_in_eager_calls(live, before):
+    d, T = 64, 1000
+    ms, pins, hs = [], [], []
+    for _ in range(2):
+        m = Mix(d_model=d, T_max=T, n_slots_max=2)
+        for slot in range(2):
+            m.register_steer(slot, torch.ones(d, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+        m.set_slot_map(torch.zeros(before, dtype=torch.int32, device="cuda"), before)
+        ms.append(m)
+        pins.append(torch.full((live,), -1, dtype=torch.int32).pin_memory())
+        hs.append(torch.zeros((T, d), device="cuda", dtype=torch.bfloat16))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for m, pin, h in zip(ms, pins, hs):
+            m.set_slot_map(pin, live)
+            m.apply(h)
+    for replay in range(3):
+        for i, (pin, h) in enumerate(zip(pins, hs)):
+            pin.copy_(torch.from_numpy(np.random.default_rng(2 * replay + i).integers(-1, 2, size=live).astype(np.int32)))
+            h.zero_()
+        torch.cuda.synchronize()
+        if replay < 2:
+            graph.replay()
+        else:
+            for m, pin, h in zip(ms, pins, hs):
+                m.set_slot_map(pin, live)
+                m.apply(h)
+        torch.cuda.synchronize()
+        for pin, h in zip(pins, hs):
+            want = np.zeros(T, dtype=np.float32)
+            want[:live] = pin.numpy() + 1.0
+            assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), replay
+    assert all(m.get_status() == 0 for m in ms)
+    del graph
+    for m in ms:
+        m.destroy()

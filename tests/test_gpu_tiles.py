@@ -97,3 +97,12 @@ def test_allocation_free_call(rows, d, S, act, k, add_error, aligned):
         assert (idx.cpu().numpy()[:, 0] % 2 == 0).all()       # of two equal ones the lower id comes first
     hid, hmax = O.bf16_to_f64(W.bits(h)), np.abs(O.bf16_to_f64(wh.hidden)).max()
     assert max(np.abs(hid[t] - ref.y[t]).max() for t in range(rows)) <= 1e-2 * hmax
+
+
+# rows of one CTA of the front kernel: 256; from 1025 rows on its CTAs exchange their counts
+@pytest.mark.parametrize("T", [255, 257, 1023, 1024, 1025])
+def test_rows_scattered_over_sets(T):
+    w = _workload(64, 256, T, W.SAE_TOPK, True, k=4, n_sets=3)
+    w.token_slot[:] = np.random.default_rng(T).integers(-1, 3, size=T)
+    w.token_slot[: T // 2] = np.minimum(w.token_slot[: T // 2], 0)
+    check_parity(W.host(w), run_gpu(w))
