@@ -662,7 +662,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         float* out = Z + p * (size_t)ldz + (size_t)t.n_tile * tile_n;
         // For rows that are rebuilt from their active features, which of the tile's are active goes beside Z, a bit each:
         // the tail kernel then reads 3 KiB per row of 24576 features, and of Z what is active, instead of 100 KiB of Z and
-        // as much of theta.  (Lists of the active values instead of bits took this epilogue from 11 us a tile to 20.)
+        // as much of theta; and of Z only the groups of four with an active feature are written -- all of it (98 MB for 1000
+        // rows) pushed W_dec out of L2 ahead of the gather.  1000 rows of d = 2304: the call 244 -> 219 us.  (Lists of the active values instead of bits took this epilogue from 11 us a tile to 20.)
         const bool want_bits = mode == 0 && valid && !(row_rec[p].group_flags & kRecAddError);
         const bool any_bits = __any_sync(0xffffffffu, want_bits);
         const bool jump = any_bits && groups[t.group].act == MIX_SAE_JUMPRELU;
@@ -691,7 +692,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
               o.y = kScaled ? fmaf(v[i + 1], s4.y, b4.y) : v[i + 1] + b4.y;
               o.z = kScaled ? fmaf(v[i + 2], s4.z, b4.z) : v[i + 2] + b4.z;
               o.w = kScaled ? fmaf(v[i + 3], s4.w, b4.w) : v[i + 3] + b4.w;
-              *reinterpret_cast<float4*>(out + c + i) = o;
+              if (!want_bits) *reinterpret_cast<float4*>(out + c + i) = o;
               v[i] = o.x; v[i + 1] = o.y; v[i + 2] = o.z; v[i + 3] = o.w;
             }
           }
@@ -710,7 +711,12 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
               if (v[i + 2] > t4.z && v[i + 2] != 0.f) m |= 4u << i;
               if (v[i + 3] > t4.w && v[i + 3] != 0.f) m |= 8u << i;
             }
-            if (want_bits) bits[c >> 5] = m;
+            if (want_bits) {
+              bits[c >> 5] = m;
+#pragma unroll
+              for (int i = 0; i < 32; i += 4)
+                if ((m >> i) & 15u) *reinterpret_cast<float4*>(out + c + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            }
           }
         }
       }

@@ -715,9 +715,15 @@ __device__ void tail_rows(const TailArgs& a, RowShared& sh, int n_groups, const 
       if (a.out_n_active != nullptr) {
         int cnt = 0;
         const float* theta = gp->theta;
-        for (int j = tid; j < S; j += kTailThreads) {
-          const float v = z[j];
-          cnt += act == MIX_SAE_RELU ? v > 0.f : (v > theta[j] && v > 0.f);
+        if (a.mode == kTailCand && !add_error) {       // of a row that is rebuilt, Z holds the active features only
+          const unsigned* bits = reinterpret_cast<const unsigned*>(a.cand_idx) + (size_t)p * a.cand_tiles * kCandPerTile;
+          for (int w = tid; w < S / 32; w += kTailThreads)
+            for (unsigned m = bits[w]; m != 0u; m &= m - 1u) cnt += z[w * 32 + __ffs(m) - 1] > 0.f;
+        } else {
+          for (int j = tid; j < S; j += kTailThreads) {
+            const float v = z[j];
+            cnt += act == MIX_SAE_RELU ? v > 0.f : (v > theta[j] && v > 0.f);
+          }
         }
         if (tid == 0) sh.count = 0;
         __syncthreads();
