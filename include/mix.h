@@ -421,8 +421,9 @@ int mix_set_pdl_mask(int mask);
 /* Test / profiling taps into the SAE workspace after a mix_apply (device pointers owned by
    the context; valid until mix_destroy):  panel_rows int32 [n_panel_rows] gives the token
    index of each packed panel row (-1 = padding), z the fp32 pre-activations
-   [n_panel_rows, ld_z] of ReLU / JumpReLU rows (of rows whose app replaces the residual, the tensor-core
-   encode stores the active features, in aligned groups of four, only).  Any out pointer may be NULL. */
+   [n_panel_rows, ld_z] of ReLU / JumpReLU rows.  The tensor-core encode stores, in aligned groups of four,
+   what the call needs: of rows whose app replaces the residual the active features, of the others the edited ones
+   (all of them while mix_set_feature_out() asks for active counts).  Any out pointer may be NULL. */
 int mix_debug_workspace(mix_ctx* ctx, const int** panel_rows, const float** z, long long* ld_z,
                         int* n_panel_rows);
 

@@ -247,7 +247,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
                  const int* __restrict__ mtile_flag, const int* __restrict__ n_flagged, float* __restrict__ cand_val,
                  int* __restrict__ cand_idx, float* __restrict__ cand_ninth, int cand_tiles, int w_tiled, int test_stall,
                  const float* __restrict__ act_scale, unsigned* __restrict__ tau_slots, unsigned* __restrict__ tau_min,
-                 int lo_row0, const RowRec* __restrict__ row_rec, unsigned long long* __restrict__ clk) {
+                 int lo_row0, const RowRec* __restrict__ row_rec, const int* __restrict__ edit_idx, int r_max, int all_z,
+                 unsigned long long* __restrict__ clk) {
   constexpr bool kE4 = kEnc != 0;                      // E4M3 x E4M3 contraction
   constexpr bool kSplit = kEnc == 1;                   // the panel row is hi + lo: two operand tiles per k-block
   constexpr int kBlockK = kE4 ? 2 * kTileK : kTileK;   // elements per 128-byte row of either operand
@@ -490,6 +491,53 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         }
         __syncwarp();
       }
+      const float* theta_t = nullptr;
+      float* wt = kScaled || !kStageVec ? nullptr : ws;         // (the scale's place is free where there is no scale)
+      bool want_bits = false, any_bits = false, jump = false, only_edits = false, any_full = false;
+      unsigned edited = 0u;
+      if (!topk_tile) {
+        // For rows that are rebuilt from their active features, which of the tile's are active goes beside Z, a bit each:
+        // the tail kernel then reads 3 KiB per row of 24576 features, and of Z what is active, instead of 100 KiB of Z and
+        // as much of theta; and of Z only the groups of four with an active feature are written -- all of it (98 MB for 1000
+        // rows) pushed W_dec out of L2 ahead of the gather.  1000 rows of d = 2304: the call 244 -> 219 us.  (Lists of the active
+        // values instead of bits took this epilogue from 11 us a tile to 20.)
+        const bool add_error = valid && (row_rec[p].group_flags & kRecAddError);
+        want_bits = mode == 0 && valid && !add_error;
+        any_bits = __any_sync(0xffffffffu, want_bits);
+        // Of a row that keeps the error term only the edited features are needed (unless its active count is read out): the
+        // groups of four that hold one, for any row of the warp, are written, and where that was, in the place of the bits --
+        // the tail does not take Z's word for an edit that arrived on another stream after this kernel had looked.
+        // 8192 rows, d = 5120, 23 % of them edited in two sets of 32768: the call 670 -> 630 us; d = 2304, 16384: 212 -> 186.  (Looked
+        // up here, before the wait: behind it, the look-up showed in calls of one wave, 42 -> 44 us for 64 rows.)
+        only_edits = mode == 0 && add_error && all_z == 0;
+        any_full = __any_sync(0xffffffffu, valid && !want_bits && !only_edits);
+        // (`edited`: lane w: the edited features among columns [32 w, 32 w + 32).)
+        if (__any_sync(0xffffffffu, only_edits)) {
+          const int n_edit = only_edits ? min(row_rec[p].n_edit, r_max) : 0;
+          const int* list = edit_idx + (only_edits ? (size_t)row_rec[p].slot * r_max : 0);
+          const int n_most = __reduce_max_sync(0xffffffffu, n_edit);
+          for (int e0 = 0; e0 < n_most; e0 += 8) {
+            int rel[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) rel[u] = e0 + u < n_edit ? list[e0 + u] - t.n_tile * tile_n : -1;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const bool in = (unsigned)rel[u] < (unsigned)tile_n;
+              for (unsigned b = __ballot_sync(0xffffffffu, in); b != 0u;) {
+                const int x = __shfl_sync(0xffffffffu, rel[u], __ffs(b) - 1);
+                if (lane == (x >> 5)) edited |= 1u << (x & 31);
+                b &= ~__ballot_sync(0xffffffffu, in && rel[u] == x);
+              }
+            }
+          }
+        }
+        jump = any_bits && groups[t.group].act == MIX_SAE_JUMPRELU;
+        if (jump) theta_t = groups[t.group].theta + (size_t)t.n_tile * tile_n + c_lo;
+        if (jump && wt != nullptr) {
+          for (int j = lane; j < epi_cols; j += 32) wt[j] = __ldg(theta_t + j);      // (theta need not be aligned)
+          __syncwarp();
+        }
+      }
       // warp-uniform decision: tcgen05.ld below needs the whole warp
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->tmem_full[acc]), acc_phase, sh, status))) break;
       tc_fence_after();
@@ -660,22 +708,12 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         }
       } else {
         float* out = Z + p * (size_t)ldz + (size_t)t.n_tile * tile_n;
-        // For rows that are rebuilt from their active features, which of the tile's are active goes beside Z, a bit each:
-        // the tail kernel then reads 3 KiB per row of 24576 features, and of Z what is active, instead of 100 KiB of Z and
-        // as much of theta; and of Z only the groups of four with an active feature are written -- all of it (98 MB for 1000
-        // rows) pushed W_dec out of L2 ahead of the gather.  1000 rows of d = 2304: the call 244 -> 219 us.  (Lists of the active values instead of bits took this epilogue from 11 us a tile to 20.)
-        const bool want_bits = mode == 0 && valid && !(row_rec[p].group_flags & kRecAddError);
-        const bool any_bits = __any_sync(0xffffffffu, want_bits);
-        const bool jump = any_bits && groups[t.group].act == MIX_SAE_JUMPRELU;
-        const float* theta_t = jump ? groups[t.group].theta + (size_t)t.n_tile * tile_n + c_lo : nullptr;
-        float* wt = kScaled || !kStageVec ? nullptr : ws;       // (the scale's place is free where there is no scale)
-        if (jump && wt != nullptr) {
-          for (int j = lane; j < epi_cols; j += 32) wt[j] = __ldg(theta_t + j);      // (theta need not be aligned)
-          __syncwarp();
-        }
         unsigned* bits = reinterpret_cast<unsigned*>(cand_idx) + p * (size_t)cand_tiles * kCandPerTile + t.n_tile * (tile_n / 32);
 #pragma unroll 1
         for (int c = c_lo; c < c_lo + epi_cols; c += 32) {
+          const unsigned here = __shfl_sync(0xffffffffu, edited, c >> 5);
+          if (only_edits) bits[c >> 5] = here;
+          if (!any_full && !any_bits && here == 0u) continue;
           float v[32];
           tmem_ld32(taddr + c, v);
           if (valid) {
@@ -692,7 +730,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
               o.y = kScaled ? fmaf(v[i + 1], s4.y, b4.y) : v[i + 1] + b4.y;
               o.z = kScaled ? fmaf(v[i + 2], s4.z, b4.z) : v[i + 2] + b4.z;
               o.w = kScaled ? fmaf(v[i + 3], s4.w, b4.w) : v[i + 3] + b4.w;
-              if (!want_bits) *reinterpret_cast<float4*>(out + c + i) = o;
+              if (!want_bits && (!only_edits || ((here >> i) & 15u))) *reinterpret_cast<float4*>(out + c + i) = o;
               v[i] = o.x; v[i + 1] = o.y; v[i + 2] = o.z; v[i + 3] = o.w;
             }
           }
@@ -864,7 +902,8 @@ static cudaError_t launch_encode_tc_as(const Ctx* c, int mode, cudaStream_t s) {
                             static_cast<const int*>(c->d_mtile_flag), static_cast<const int*>(c->d_n_flagged), c->d_cand_val,
                             c->d_cand_idx, c->d_cand_ninth, c->cand_tiles, w_tiled, stall,
                             static_cast<const float*>(c->d_act_scale), c->d_tau, c->d_tau_min, c->panel_rows_cap,
-                            static_cast<const RowRec*>(c->d_row_rec), c->d_phase_clk);
+                            static_cast<const RowRec*>(c->d_row_rec), static_cast<const int*>(c->d_edit_idx), c->cfg.r_max,
+                            c->out_n_active != nullptr ? 1 : 0, c->d_phase_clk);
 }
 
 // Eight epilogue warps pay off for the TopK epilogue (selection work per element); the plain store of the

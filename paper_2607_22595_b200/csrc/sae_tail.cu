@@ -877,6 +877,10 @@ __device__ void tail_delta(const TailArgs& a, DeltaShared& sh, int item, int n_r
 #pragma unroll
       for (int r2 = 0; r2 < kDlRows; ++r2) {
         if (sh.slot[r2] == slot && alive) {
+          if (a.mode == kTailCand && a.out_n_active == nullptr) {   // the encode wrote the edits that it found: not this one?
+            const unsigned* stored = reinterpret_cast<const unsigned*>(a.cand_idx) + (size_t)(p0 + r2) * a.cand_tiles * kCandPerTile;
+            if (((stored[j >> 5] >> (j & 28)) & 15u) == 0u) continue;
+          }
           const float zj = a.Z[(size_t)(p0 + r2) * a.ldz + j];
           const float f = act == MIX_SAE_RELU ? fmaxf(zj, 0.f) : (zj > theta ? zj : 0.f);
           c[r2] = fnew - f;

@@ -106,3 +106,26 @@ def test_rows_scattered_over_sets(T):
     w.token_slot[:] = np.random.default_rng(T).integers(-1, 3, size=T)
     w.token_slot[: T // 2] = np.minimum(w.token_slot[: T // 2], 0)
     check_parity(W.host(w), run_gpu(w))
+
+
+# pre-activations stored for the edited features alone (no read-out) against all of them: the same rows, bit for bit
+@pytest.mark.parametrize("T", [1, 33, 130, 700])
+@pytest.mark.parametrize("n_edit", [1, 9, 64])
+@pytest.mark.parametrize("act", [W.SAE_RELU, W.SAE_JUMPRELU])
+@pytest.mark.parametrize("fp8", [None, "weights", "input"])
+def test_only_edited_features_stored(T, n_edit, act, fp8):
+    S = 2048
+    w = _workload(128, S, T, act, True, fp8=fp8, extra_topk=T == 33)
+    rng = np.random.default_rng(T + n_edit)
+    edges = np.array([0, 3, 4, 31, 32, 63, 64, 127, 128, 255, 256, S - 4, S - 1], np.int32)
+    for slot in range(5):                                     # the last one replaces the residual
+        idx = np.concatenate([rng.choice(edges, min(n_edit, 9)), rng.integers(0, S, max(n_edit - 9, 0))]).astype(np.int32)
+        w.apps[slot] = W.SaeApp(0, idx, rng.normal(size=n_edit).astype(np.float32), rng.integers(0, 2, n_edit).astype(np.uint8), slot < 4)
+    w.n_slots_max, w.r_max = 5, n_edit
+    w.token_slot[:] = rng.integers(-1, 5, size=T) if T > 1 else 0
+    flags = {None: 0, "weights": 32, "input": 96}[fp8]
+    full = run_gpu(w, flags=flags)
+    check_parity(W.host(w), full)
+    sparse = run_gpu(w, flags=flags, feature_out=False, replays=2, graph=True)
+    assert np.array_equal(full["hidden"], sparse["hidden"])
+    assert sparse["status"] == 0
