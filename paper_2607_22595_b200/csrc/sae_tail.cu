@@ -358,19 +358,49 @@ __device__ __forceinline__ void axpy8(float* acc, float c, const uint4& q) {
 // The gather of the decode.  A row is rebuilt in passes of 2048 columns: thread `tid` owns the 16-byte column
 // vector v = pass * 256 + tid, so one decoder row is read as 4 KiB of contiguous 16-byte loads per pass, and
 // acc (8 columns) += sum_e coef[e] * W_dec[feat[e], 8v .. 8v+7] with kGatherBatch decoder rows in flight per
-// thread -- the loop is bound by load latency, not arithmetic.  Entries with a zero coefficient are not fetched.
+// thread.  Entries with a zero coefficient are not fetched.
+// A whole batch without a zero is the usual one and has a path of its own: entries four at a time out of shared memory
+// (kAligned: both lists start on 16 bytes), no test and no zeroed register per entry
+// (the loop keeps the issue slots half busy: with every load an L1 hit it still takes 60 % of its time).  1000 rows with 110
+// active features each: the call 219 -> 216 us.  (Packed two-column multiply-adds on top: 217, and 244 bytes of spills.)
+template <bool kAligned>
 __device__ __forceinline__ void gather_list(float (&acc)[8], const float* coef, const int* feat, int n,
                                             const __nv_bfloat16* __restrict__ W_dec, int d, int v, bool in_cols) {
+  if (!in_cols) return;
+  const uint4* base = reinterpret_cast<const uint4*>(W_dec) + v;
+  const unsigned row_vecs = (unsigned)d >> 3;
 #pragma unroll 1
   for (int e0 = 0; e0 < n; e0 += kGatherBatch) {
     uint4 q[kGatherBatch];
     float c[kGatherBatch];
+    bool full = e0 + kGatherBatch <= n;
+    if (full) {
+      int f[kGatherBatch];
 #pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u) {
-      const int e = e0 + u;
-      c[u] = e < n ? coef[e] : 0.f;
-      q[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (c[u] != 0.f && in_cols) q[u] = __ldg(reinterpret_cast<const uint4*>(W_dec + (size_t)feat[e] * d) + v);
+      for (int u = 0; u < kGatherBatch; u += 4) {
+        if (kAligned) {
+          *reinterpret_cast<float4*>(c + u) = *reinterpret_cast<const float4*>(coef + e0 + u);
+          *reinterpret_cast<int4*>(f + u) = *reinterpret_cast<const int4*>(feat + e0 + u);
+        } else {
+#pragma unroll
+          for (int w = u; w < u + 4; ++w) { c[w] = coef[e0 + w]; f[w] = feat[e0 + w]; }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kGatherBatch; ++u) full = full && c[u] != 0.f;
+      if (full) {
+#pragma unroll
+        for (int u = 0; u < kGatherBatch; ++u) q[u] = __ldg(base + (unsigned long long)(unsigned)f[u] * row_vecs);
+      }
+    }
+    if (!full) {
+#pragma unroll
+      for (int u = 0; u < kGatherBatch; ++u) {
+        const int e = e0 + u;
+        c[u] = e < n ? coef[e] : 0.f;
+        q[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (c[u] != 0.f) q[u] = __ldg(base + (unsigned long long)(unsigned)feat[e] * row_vecs);
+      }
     }
 #pragma unroll
     for (int u = 0; u < kGatherBatch; ++u) axpy8(acc, c[u], q[u]);
@@ -433,8 +463,8 @@ struct RowShared {
   int warp_n[kTailThreads / 32];          // entries of each warp's list
   int count;
   GroupEntry grp[kMaxGroups];             // the weight-set table, fetched once per CTA
-  float coef[kDecList];
-  int feat[kDecList];
+  __align__(16) float coef[kDecList];
+  __align__(16) int feat[kDecList];
   int eidx[kMaxEdits];
   float ef[kMaxEdits];      // f_j of each edited feature before the edit
   float enew[kMaxEdits];    // f'_j
@@ -468,8 +498,8 @@ __device__ void gather_row(const float* coef, const int* feat, int n, const __nv
         for (int i = 0; i < 8; ++i) acc[i] = b_dec[v * 8 + i];
       }
     }
-    const int e0 = n * grp / n_grp, e1 = n * (grp + 1) / n_grp;
-    gather_list(acc, coef + e0, feat + e0, e1 - e0, W_dec, d, v, in);
+    const int e0 = (n * grp / n_grp) & ~3, e1 = grp + 1 == n_grp ? n : (n * (grp + 1) / n_grp) & ~3;
+    gather_list<true>(acc, coef + e0, feat + e0, e1 - e0, W_dec, d, v, in);
     if (split) {
       float4* p4 = reinterpret_cast<float4*>(part);
       __syncthreads();
@@ -558,10 +588,10 @@ __device__ void rebuild_row(const TailArgs& a, RowShared& sh, int p, const float
     float acc[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i] = (b_dec && in) ? b_dec[v * 8 + i] : 0.f;
-    gather_list(acc, coef, feat, n_edit, W_dec, d, v, in);
+    gather_list<true>(acc, coef, feat, n_edit, W_dec, d, v, in);
     for (int w0 = 0; w0 < n_words; w0 += 32) {                // 1024 features always fit
       const int n = list_words(w0, min(w0 + 32, n_words));
-      gather_list(acc, coef + n_edit, feat + n_edit, n, W_dec, d, v, in);
+      gather_list<false>(acc, coef + n_edit, feat + n_edit, n, W_dec, d, v, in);
     }
     if (in) hrow[v] = pack8(acc);
   }
