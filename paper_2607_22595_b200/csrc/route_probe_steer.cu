@@ -382,12 +382,14 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, const int* __restric
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
 constexpr int kTeamVec = 4;     // NW * 32 * kTeamVec * 8 >= d_model: 8192 columns at NW = 8
 
-template <int NW>
+enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
+
+template <int NW, TeamForm kForm>
 __global__ void __launch_bounds__(NW * 32)
 probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
-                        unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl, int late) {
+                        unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl) {
   __shared__ float s_part[NW][kMaxClasses];
   constexpr int NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -401,11 +403,12 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   // row is then requested together with the vector and the app entry, one round trip earlier.  Behind a map that a
   // kernel installed (kPdlMapAhead) the wait comes first, and only then the trigger: a successor that reads the map
   // early must not start before the map is there.
-  if (pdl == kPdlMapAhead) {
+  if (kForm == kTeamMapAhead || (kForm == kTeamLate && pdl == kPdlMapAhead)) {
     pdl_wait();
     pdl_launch_dependents();
     pdl = 0;
   }
+  constexpr bool kLate = kForm == kTeamLate;
   if (pdl) pdl_launch_dependents();
   const int n_live = __ldg(n_live_p);            // both loads issue together: one round trip, not two
   const int slot = __ldg(token_slot + t);
@@ -419,17 +422,17 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   // into row `slot` of the context's vector arena, so their address follows from the slot id
   // alone: the row AND its vector are requested together, before the app entry is known.
   uint4 hq[kTeamVec], vq[kTeamVec];
-  // (`late`, contexts with SAE weight sets: most rows may be another kernel's; nothing is requested before the entry says
-  // that the row is this one's.  1000 SAE rows of d = 2304: 6.2 -> 4.5 us)
+  // (kLate, contexts with SAE weight sets: most rows may be another kernel's; nothing is requested before the entry says
+  // that the row is this one's.  1000 SAE rows of d = 2304: 6.2 -> 4.5 us.)
   const bool slot_ok = slot >= 0 && slot < n_slots;
-  if (slot_ok && !late) {
+  if (!kLate && slot_ok) {
 #pragma unroll
     for (int u = 0; u < kTeamVec; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
     }
   }
-  if (!pdl && slot_ok && !late) {
+  if (!kLate && !pdl && slot_ok) {
 #pragma unroll
     for (int u = 0; u < kTeamVec; ++u) {
       const int v = threadIdx.x + u * NT;
@@ -438,7 +441,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   }
   RowApp a = lookup(slot, t, apps, gates, n_slots, status, threadIdx.x == 0, /*eval_gate=*/false);
   if (pdl) pdl_wait();
-  if (late) {
+  if (kLate) {
     if (a.kind == 0 || a.kind == MIX_SAE || a.kind == MIX_ROUTER) return;
 #pragma unroll
     for (int u = 0; u < kTeamVec; ++u) {
@@ -878,10 +881,12 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
                       c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
                       c->cfg.d_model, scores, c->cfg.C_max, c->d_status, pdl);
   } else if (c->cfg.T_max <= kTeamMaxRows) {
-    return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_team_kernel<8>, dim3(c->cfg.T_max), dim3(8 * 32), 0, s,
-                      c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->cfg.n_slots_max, hidden, c->cfg.d_model,
-                      scores, c->cfg.C_max, c->d_status, reinterpret_cast<const uint4*>(c->d_vec_arena), pdl,
-                      c->cfg.n_groups_max > 0 ? 1 : 0);
+    auto kernel = c->cfg.n_groups_max > 0 ? probe_steer_team_kernel<8, kTeamLate>
+                                          : (pdl == kPdlMapAhead ? probe_steer_team_kernel<8, kTeamMapAhead> : probe_steer_team_kernel<8, kTeamPlain>);
+    return launch_pdl(allow_pdl ? kPdlHook : 0, kernel,
+                      dim3(c->cfg.T_max), dim3(8 * 32), 0, s, c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+                      c->cfg.n_slots_max, hidden, c->cfg.d_model, scores, c->cfg.C_max, c->d_status,
+                      reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
   } else {
     auto run = [&](auto kernel, int warps) {
       kernel<<<(c->cfg.T_max + warps - 1) / warps, warps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
