@@ -3,7 +3,9 @@
  *
  * An eager decode step is two of these calls and two kernels, and the host sets its pace: of 4.2 us for an apply, 2.2 were
  * the launch, the rest attribute look-ups in Python and ctypes' conversions.  The checks are the binding's own, made here on
- * the same tensor attributes; a call that fails one raises what the Python code raised.
+ * the same tensor attributes; a call that fails one raises what the Python code raised.  The GIL is released round the call
+ * into the library, as ctypes releases it: a launch can wait for room in a full queue, and a copy from pageable memory for
+ * everything in front of it, which may be a host function that itself needs the GIL.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -88,7 +90,11 @@ static PyObject* fast_apply(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     if (data_ptr(a[2], &scores) < 0) return NULL;
   }
   if (stream_of(a[4], &stream) < 0) return NULL;
-  return PyLong_FromLong(mix_apply(c, h, (int)T, (float*)scores, stream));
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = mix_apply(c, h, (int)T, (float*)scores, stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 /* set_slot_map(ctx, token_slot int32 tensor, T_live | None, stream | None) -> status */
@@ -105,7 +111,11 @@ static PyObject* fast_set_slot_map(PyObject* self, PyObject* const* a, Py_ssize_
   if (cuda < 0 || data_ptr(a[1], &src) < 0) return NULL;
   if (number(a[2] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Long(a[2]), &T) < 0) return NULL;
   if (stream_of(a[3], &stream) < 0) return NULL;
-  return PyLong_FromLong(mix_set_slot_map(c, (const int*)src, (int)T, cuda, stream));
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = mix_set_slot_map(c, (const int*)src, (int)T, cuda, stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 /* set_request_map(ctx, token_req, req_slot, T_live | None, stream | None) -> status */
@@ -120,7 +130,11 @@ static PyObject* fast_set_request_map(PyObject* self, PyObject* const* a, Py_ssi
   if (number(a[3] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Long(a[3]), &T) < 0) return NULL;
   if (number(PyObject_CallMethodNoArgs(a[2], s_numel), &n_req) < 0) return NULL;
   if (stream_of(a[4], &stream) < 0) return NULL;
-  return PyLong_FromLong(mix_set_request_map(c, (const int*)req, (int)T, (const int*)slots, (int)n_req, cuda, stream));
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = mix_set_request_map(c, (const int*)req, (int)T, (const int*)slots, (int)n_req, cuda, stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 static PyMethodDef methods[] = {
