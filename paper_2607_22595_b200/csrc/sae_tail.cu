@@ -360,9 +360,14 @@ __device__ __forceinline__ void axpy8(float* acc, float c, const uint4& q) {
 // acc (8 columns) += sum_e coef[e] * W_dec[feat[e], 8v .. 8v+7] with kGatherBatch decoder rows in flight per
 // thread.  Entries with a zero coefficient are not fetched.
 // A whole batch without a zero is the usual one and has a path of its own: entries four at a time out of shared memory
-// (kAligned: both lists start on 16 bytes), no test and no zeroed register per entry
-// (the loop keeps the issue slots half busy: with every load an L1 hit it still takes 60 % of its time).  1000 rows with 110
-// active features each: the call 219 -> 216 us.  (Packed two-column multiply-adds on top: 217, and 244 bytes of spills.)
+// (kAligned: both lists start on 16 bytes), no test and no zeroed register per entry.  Its coefficients are read twice, for the
+// test and again when the rows are here: 8 registers less while 32 hold the rows.  Kept instead, the kernel spilled 292 bytes
+// (100 now, 92 without the path), and every role paid: 128 rows, 16384 features: the call 63.9 us kept, 62.5 read twice;
+// 1000 rows with 110 active features each, d = 2304: 215.5 and 210.3, without the path 4 more.
+template <bool kAligned, class V, class S>
+__device__ __forceinline__ V list4(const S* p) {
+  return kAligned ? *reinterpret_cast<const V*>(p) : V{p[0], p[1], p[2], p[3]};
+}
 template <bool kAligned>
 __device__ __forceinline__ void gather_list(float (&acc)[8], const float* coef, const int* feat, int n,
                                             const __nv_bfloat16* __restrict__ W_dec, int d, int v, bool in_cols) {
@@ -371,36 +376,36 @@ __device__ __forceinline__ void gather_list(float (&acc)[8], const float* coef, 
   const unsigned row_vecs = (unsigned)d >> 3;
 #pragma unroll 1
   for (int e0 = 0; e0 < n; e0 += kGatherBatch) {
-    uint4 q[kGatherBatch];
-    float c[kGatherBatch];
     bool full = e0 + kGatherBatch <= n;
     if (full) {
-      int f[kGatherBatch];
 #pragma unroll
       for (int u = 0; u < kGatherBatch; u += 4) {
-        if (kAligned) {
-          *reinterpret_cast<float4*>(c + u) = *reinterpret_cast<const float4*>(coef + e0 + u);
-          *reinterpret_cast<int4*>(f + u) = *reinterpret_cast<const int4*>(feat + e0 + u);
-        } else {
-#pragma unroll
-          for (int w = u; w < u + 4; ++w) { c[w] = coef[e0 + w]; f[w] = feat[e0 + w]; }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kGatherBatch; ++u) full = full && c[u] != 0.f;
-      if (full) {
-#pragma unroll
-        for (int u = 0; u < kGatherBatch; ++u) q[u] = __ldg(base + (unsigned long long)(unsigned)f[u] * row_vecs);
+        const float4 x = list4<kAligned, float4>(coef + e0 + u);
+        full = full && x.x != 0.f && x.y != 0.f && x.z != 0.f && x.w != 0.f;
       }
     }
-    if (!full) {
+    uint4 q[kGatherBatch];
+    if (full) {
 #pragma unroll
-      for (int u = 0; u < kGatherBatch; ++u) {
-        const int e = e0 + u;
-        c[u] = e < n ? coef[e] : 0.f;
-        q[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (c[u] != 0.f) q[u] = __ldg(base + (unsigned long long)(unsigned)feat[e] * row_vecs);
+      for (int u = 0; u < kGatherBatch; u += 4) {
+        const int4 f = list4<kAligned, int4>(feat + e0 + u);
+        q[u] = __ldg(base + (unsigned long long)(unsigned)f.x * row_vecs);
+        q[u + 1] = __ldg(base + (unsigned long long)(unsigned)f.y * row_vecs);
+        q[u + 2] = __ldg(base + (unsigned long long)(unsigned)f.z * row_vecs);
+        q[u + 3] = __ldg(base + (unsigned long long)(unsigned)f.w * row_vecs);
       }
+      asm volatile("" ::: "memory");             // (the coefficients are read again, not kept while the rows are in flight)
+#pragma unroll
+      for (int u = 0; u < kGatherBatch; ++u) axpy8(acc, coef[e0 + u], q[u]);
+      continue;
+    }
+    float c[kGatherBatch];
+#pragma unroll
+    for (int u = 0; u < kGatherBatch; ++u) {
+      const int e = e0 + u;
+      c[u] = e < n ? coef[e] : 0.f;
+      q[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (c[u] != 0.f) q[u] = __ldg(base + (unsigned long long)(unsigned)feat[e] * row_vecs);
     }
 #pragma unroll
     for (int u = 0; u < kGatherBatch; ++u) axpy8(acc, c[u], q[u]);
