@@ -12,6 +12,9 @@ LIMITS = [
     # four CTAs of 256 threads per SM leave 64 registers.  What lives across a row's steps does not fit, with or without the
     # gather (88 bytes of spill stores before it read its lists in whole batches, 292 after): outside the loops, some 100 bytes.
     ("sae_tail.cu", "tail_kernel", 64, 112),
+    # beside it two CTAs of the streaming kernel (72 registers a thread) are to fit into the SM's 64 Ki registers: at most 112,
+    # and at the launch bound of three CTAs 80
+    ("probe_tc.cu", "probe_tc_kernel", 80, 0),
 ]
 
 
