@@ -22,10 +22,15 @@ namespace {
     return (code);                                        \
   } while (0)
 
+// (The error that is returned is also taken out of the runtime's record: left there, the next check of that record, the
+// library's behind a launch or the caller's own, would report it as its own.)
 #define MIX_CUDA(ctx, expr)                                                                  \
   do {                                                                                       \
     cudaError_t e_ = (expr);                                                                 \
-    if (e_ != cudaSuccess) MIX_FAIL(ctx, MIX_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e_)); \
+    if (e_ != cudaSuccess) {                                                                 \
+      cudaGetLastError();                                                                    \
+      MIX_FAIL(ctx, MIX_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e_));                  \
+    }                                                                                        \
   } while (0)
 
 __global__ void bench_add_from_table(const float* __restrict__ table, float* __restrict__ acc) {

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import workloads as W
-from paper_2607_22595_b200 import Mix
+from paper_2607_22595_b200 import Mix, MixError
 
 pytestmark = pytest.mark.gpu
 
@@ -81,3 +81,29 @@ def test_pinned_maps_in_a_graph_and_in_eager_calls(live, before):
     del graph
     for m in ms:
         m.destroy()
+
+
+def _refused_install(m, src, n):
+    """An install on the legacy stream while a blocking stream is being captured: CUDA refuses it, nothing is enqueued."""
+    from cuda.bindings import runtime as rt
+
+    err, blocking = rt.cudaStreamCreate()
+    assert int(err) == 0
+    assert int(rt.cudaStreamBeginCapture(blocking, rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal)[0]) == 0
+    with pytest.raises(MixError):
+        m.set_slot_map(src, n, stream=0)
+    err, graph = rt.cudaStreamEndCapture(blocking)   # (the failed call has invalidated it)
+    if int(err) == 0:
+        rt.cudaGraphDestroy(graph)
+    rt.cudaStreamDestroy(blocking)
+    rt.cudaGetLastError()
+
+
+def test_an_error_that_a_call_returned_is_not_reported_again():
+    m = Mix(d_model=64, T_max=3000, n_slots_max=1)
+    src = torch.zeros(5, dtype=torch.int32, device="cuda")
+    h = torch.ones((3000, 64), device="cuda", dtype=torch.bfloat16)
+    _refused_install(m, src, 5)
+    m.apply(h)                                       # (checks the runtime's record behind its launch)
+    assert bool((h == 1).all())                      # (so does torch)
+    m.destroy()
