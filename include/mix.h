@@ -296,11 +296,15 @@ int mix_set_chain(mix_ctx* ctx, int slot, int next_slot, void* stream);
    step to step while the captured launch structure stays as it is.)
    Install the token->slot map for the next mix_apply calls: token_slot int32[T_live]
    (host if src_is_device == 0, else device), -1 = no app.  Rows >= T_live are pass-through.
-   One operation on the stream -- an async copy from host memory, a kernel from device memory -- into
-   a fixed device buffer (two where a map from host memory is shorter than the one before: the rows
-   in between are set to -1); never captured in a graph.
-   A host source must stay valid until the stream reaches the copy (use pinned memory for a
-   truly asynchronous copy).  Errors: OUT_OF_RANGE (T_live < 0 or > T_max). */
+   One operation on the stream into a fixed device buffer: from device memory a kernel; from host memory an async
+   copy or, in contexts without weight sets, mostly a kernel, which reads memory that the device can address where it
+   lies and takes up to 896 rows of any other among its parameters; two operations where a map that is copied is
+   shorter than the one before (the rows in between are set to -1).
+   Meant to be called between replays.  A captured call reads its source, which must then stay valid as long as the
+   graph, at every replay; from the capture on every install of the context sets all rows up to T_max, since a
+   replay may have put a longer map in front of it.
+   A host source must stay valid until the stream reaches the call (use pinned memory for a
+   truly asynchronous one).  Errors: OUT_OF_RANGE (T_live < 0 or > T_max). */
 int mix_set_slot_map(mix_ctx* ctx, const int* token_slot, int T_live, int src_is_device, void* stream);
 
 /* Two-level form of the same map (Section 4.2 "Toggling semantics": activation is per REQUEST; a

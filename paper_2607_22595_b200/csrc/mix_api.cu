@@ -112,8 +112,21 @@ const int* device_view(const int* host) {
 
 bool is_capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();   // (what is enqueued next reports it)
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();                                 // (what is enqueued next reports it)
+    return false;
+  }
   return st != cudaStreamCaptureStatusNone;
+}
+
+// Rows that an install of T_live has to cover: those behind it that the map in front of it left, as far as the host knows
+// which map that is.  A captured install runs when its graph is replayed, in front of or behind any other: a context that
+// had one captured sets all T_max rows in every install.
+int map_fill(mix_ctx* c, int T_live, bool capturing) {
+  if (capturing) c->map_captured = 1;
+  const int n_fill = c->map_captured ? c->cfg.T_max : c->map_live;
+  c->map_live = n_fill > T_live ? n_fill : T_live;      // until everything is enqueued: a call that fails on the way may have left either
+  return n_fill;
 }
 
 // Publish an app entry: body first with valid = 0, then the valid word.
@@ -671,8 +684,8 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (T_live > 0 && !token_slot) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "token_slot is NULL");
-  const int n_fill = c->map_live;
-  c->map_live = T_live;
+  const bool capturing = is_capturing(s);
+  const int n_fill = map_fill(c, T_live, capturing);
   const bool by_kernel = c->cfg.n_groups_max == 0;
   const int* src = (src_is_device || T_live == 0) ? token_slot : (by_kernel ? device_view(token_slot) : nullptr);
   // With few hooks in the program a short map goes by a copy, which does not hold up the launch of a graph behind it; a
@@ -681,15 +694,17 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   // one hook on 512 rows 11.9 and 10.3, on 2000 rows 22.9 and 16.4.
   // As a node of a graph the kernel is never slower (two hooks: 8.3 ... 10.3 us, copies 11.7).
   const bool by_copy = src && !src_is_device && T_live <= kMapCopyRows && n_fill <= T_live && g_hook_contexts <= kMapCopyHooks &&
-                       !is_capturing(s);
+                       !capturing;
   if ((src && !by_copy) || T_live == 0) {
     c->map_installed = 1;
     MIX_CUDA(c, launch_install_map(c, src, T_live, n_fill, s));
+    c->map_live = T_live;
     return MIX_OK;
   }
-  if (by_kernel && !by_copy && T_live <= kMapParamRows) {
+  if (by_kernel && !by_copy && !capturing && T_live <= kMapParamRows) {     // (a captured install reads its source when it is replayed)
     c->map_installed = 1;
     MIX_CUDA(c, launch_install_map_params(c, token_slot, T_live, n_fill, s));
+    c->map_live = T_live;
     return MIX_OK;
   }
   c->map_installed = 0;             // (a copy is complete before anything behind it starts)
@@ -698,6 +713,7 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
     c->map_installed = 1;
     MIX_CUDA(c, cudaMemsetAsync(c->d_token_slot + T_live, 0xff, (size_t)(n_fill - T_live) * sizeof(int), s));
   }
+  c->map_live = T_live;
   return MIX_OK;
 }
 
@@ -708,8 +724,7 @@ int mix_set_request_map(mix_ctx* c, const int* token_req, int T_live, const int*
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (n_req < 0 || n_req > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "n_req %d outside [0, T_max=%d]", n_req, c->cfg.T_max);
   if (T_live > 0 && (!token_req || (n_req > 0 && !req_slot))) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "map arrays are NULL");
-  const int n_fill = c->map_live;
-  c->map_live = T_live;
+  const int n_fill = map_fill(c, T_live, is_capturing(s));
   c->map_installed = 1;
   const int *req = token_req, *slots = req_slot;
   if (!src_is_device && T_live > 0) {
@@ -719,6 +734,7 @@ int mix_set_request_map(mix_ctx* c, const int* token_req, int T_live, const int*
     slots = c->d_tmp_req_slot;
   }
   MIX_CUDA(c, launch_compose_map(c, req, slots, T_live, n_req, n_fill, s));
+  c->map_live = T_live;
   return MIX_OK;
 }
 

@@ -121,6 +121,7 @@ struct Ctx {
   // tables
   int* d_token_slot;        // [T_max]; -1 behind the live rows
   int map_live;             // live rows of the map last installed: what a shorter map has to set to -1
+  int map_captured;         // an install was captured: which map is in force when another runs, the host cannot know
   int* d_n_live;            // [1] rows of d_token_slot that hold a map at all: T_max
   AppEntry* d_apps;         // [n_slots_max]
   GroupEntry* d_groups;     // [n_groups_max]

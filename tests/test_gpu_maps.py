@@ -107,3 +107,74 @@ def test_an_error_that_a_call_returned_is_not_reported_again():
     m.apply(h)                                       # (checks the runtime's record behind its launch)
     assert bool((h == 1).all())                      # (so does torch)
     m.destroy()
+
+
+@pytest.mark.parametrize("with_sae", [False, True])
+@pytest.mark.parametrize("source", ["device", "pinned", "pageable", "requests_device"])
+def test_a_captured_map_among_eager_ones(source, with_sae):
+    d, T = 64, 1000
+    m = Mix(d_model=d, T_max=T, n_slots_max=2, n_groups_max=int(with_sae), d_sae_max=256 if with_sae else 0)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(d, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+    h = torch.zeros((T, d), device="cuda", dtype=torch.bfloat16)
+
+    def make(slots):
+        x = torch.from_numpy(np.ascontiguousarray(slots, dtype=np.int32))
+        return {"device": lambda: x.cuda(), "pinned": x.pin_memory, "pageable": lambda: x, "requests_device": lambda: x.cuda()}[source]()
+
+    def install(src, n):
+        if source == "requests_device":
+            m.set_request_map(every, src, n)
+        else:
+            m.set_slot_map(src, n)
+
+    def check(slots, note):
+        want = np.zeros(T, dtype=np.float32)
+        want[:len(slots)] = np.asarray(slots) + 1.0
+        assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), note
+        h.zero_()
+
+    every = torch.arange(T, dtype=torch.int32, device="cuda")
+    rng = np.random.default_rng(5)
+    long, short, ten = rng.integers(-1, 2, T), rng.integers(-1, 2, 20), rng.integers(-1, 2, 10)
+    src_long, src_short, src_ten = make(long), make(short), make(ten)
+    install(src_long, T)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        install(src_ten, 10)
+        m.apply(h)
+    install(src_short, 20)                           # captured, not replayed: the long map is the one in front
+    m.apply(h)
+    check(short, "behind a capture")
+    install(src_long, T)
+    m.apply(h)
+    check(long, "long")
+    graph.replay()                                   # the captured map is shorter than the one installed meanwhile
+    check(ten, "replayed behind a longer map")
+    src_ten.copy_(torch.from_numpy(ten[::-1].copy().astype(np.int32)))
+    torch.cuda.synchronize()
+    graph.replay()
+    check(ten[::-1], "replayed with another map in its source")
+    install(src_long, T)
+    install(src_short, 20)
+    m.apply(h)
+    check(short, "eager behind eager")
+    assert m.get_status() == 0
+    del graph
+    m.destroy()
+
+
+def test_an_install_that_fails_leaves_the_rows_of_the_map_before_to_the_next_one():
+    d, T = 64, 500
+    m = Mix(d_model=d, T_max=T, n_slots_max=1)
+    m.register_steer(0, torch.ones(d, device="cuda", dtype=torch.bfloat16), 1.0)
+    src = torch.zeros(T, dtype=torch.int32, device="cuda")
+    m.set_slot_map(src, T)
+    torch.cuda.synchronize()
+    _refused_install(m, src, 5)
+    h = torch.zeros((T, d), device="cuda", dtype=torch.bfloat16)
+    m.set_slot_map(src, 20)
+    m.apply(h)
+    assert int((h[:, 0] != 0).sum()) == 20
+    m.destroy()
