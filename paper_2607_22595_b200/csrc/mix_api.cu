@@ -110,13 +110,47 @@ const int* device_view(const int* host) {
   return at.type == cudaMemoryTypeUnregistered ? nullptr : static_cast<const int*>(at.devicePointer);
 }
 
-bool is_capturing(cudaStream_t s) {
+// The capture that the stream takes part in; 0: none.
+unsigned long long capture_of(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo_v2(s, &st, &id, nullptr, nullptr, nullptr) != cudaSuccess) {
     cudaGetLastError();                                 // (what is enqueued next reports it)
-    return false;
+    return 0;
   }
-  return st != cudaStreamCaptureStatusNone;
+  return st == cudaStreamCaptureStatusNone ? 0 : id + 1;
+}
+
+// Installs by kernel that no hook kernel has waited for yet, by the stream (and capture) they are in: a hook kernel there
+// must not read the map ahead of its wait.  Behind one that waits before it lets its own successor start, the map is there;
+// but a call on another stream or in another capture stands behind nothing of this one.
+cudaStream_t map_stream(cudaStream_t s) { return s == cudaStreamLegacy ? nullptr : s; }      // (one handle where there are two)
+void map_by_kernel(mix_ctx* c, cudaStream_t s, unsigned long long capture) {
+  s = map_stream(s);
+  for (int i = 0; i < c->n_map_pending; ++i)
+    if (c->map_pending[i].stream == s && c->map_pending[i].capture == capture) return;
+  if (c->n_map_pending == kMapPending) {
+    c->map_pending_any = 1;                             // every hook kernel waits first from here on
+    return;
+  }
+  c->map_pending[c->n_map_pending].stream = s;
+  c->map_pending[c->n_map_pending++].capture = capture;
+}
+bool map_is_pending(const mix_ctx* c, cudaStream_t s, unsigned long long capture) {
+  s = map_stream(s);
+  for (int i = 0; i < c->n_map_pending; ++i)            // (any stream of the same capture: it may have been forked since)
+    if (c->map_pending[i].capture == capture && (capture != 0 || c->map_pending[i].stream == s)) return true;
+  // (a replayed install stands in no stream that this list knows)
+  return c->map_pending_any || (c->map_captured && capture == 0);
+}
+void map_arrived(mix_ctx* c, cudaStream_t s, unsigned long long capture) {
+  s = map_stream(s);
+  if (s == cudaStreamPerThread) return;                 // (another stream in every thread: none of them speaks for the others)
+  for (int i = 0; i < c->n_map_pending; ++i)
+    if (c->map_pending[i].stream == s && c->map_pending[i].capture == capture) {
+      c->map_pending[i] = c->map_pending[--c->n_map_pending];
+      return;
+    }
 }
 
 // Rows that an install of T_live has to cover: those behind it that the map in front of it left, as far as the host knows
@@ -684,7 +718,8 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (T_live > 0 && !token_slot) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "token_slot is NULL");
-  const bool capturing = is_capturing(s);
+  const unsigned long long capture = capture_of(s);
+  const bool capturing = capture != 0;
   const int n_fill = map_fill(c, T_live, capturing);
   const bool by_kernel = c->cfg.n_groups_max == 0;
   const int* src = (src_is_device || T_live == 0) ? token_slot : (by_kernel ? device_view(token_slot) : nullptr);
@@ -696,21 +731,21 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   const bool by_copy = src && !src_is_device && T_live <= kMapCopyRows && n_fill <= T_live && g_hook_contexts <= kMapCopyHooks &&
                        !capturing;
   if ((src && !by_copy) || T_live == 0) {
-    c->map_installed = 1;
+    map_by_kernel(c, s, capture);
     MIX_CUDA(c, launch_install_map(c, src, T_live, n_fill, s));
     c->map_live = T_live;
     return MIX_OK;
   }
   if (by_kernel && !by_copy && !capturing && T_live <= kMapParamRows) {     // (a captured install reads its source when it is replayed)
-    c->map_installed = 1;
+    map_by_kernel(c, s, capture);
     MIX_CUDA(c, launch_install_map_params(c, token_slot, T_live, n_fill, s));
     c->map_live = T_live;
     return MIX_OK;
   }
-  c->map_installed = 0;             // (a copy is complete before anything behind it starts)
   MIX_CUDA(c, cudaMemcpyAsync(c->d_token_slot, token_slot, (size_t)T_live * sizeof(int), cudaMemcpyHostToDevice, s));
+  map_arrived(c, s, capture);       // (a copy is complete before anything behind it starts)
   if (n_fill > T_live) {
-    c->map_installed = 1;
+    map_by_kernel(c, s, capture);
     MIX_CUDA(c, cudaMemsetAsync(c->d_token_slot + T_live, 0xff, (size_t)(n_fill - T_live) * sizeof(int), s));
   }
   c->map_live = T_live;
@@ -724,8 +759,9 @@ int mix_set_request_map(mix_ctx* c, const int* token_req, int T_live, const int*
   if (T_live < 0 || T_live > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "T_live %d outside [0, T_max=%d]", T_live, c->cfg.T_max);
   if (n_req < 0 || n_req > c->cfg.T_max) MIX_FAIL(c, MIX_ERR_OUT_OF_RANGE, "n_req %d outside [0, T_max=%d]", n_req, c->cfg.T_max);
   if (T_live > 0 && (!token_req || (n_req > 0 && !req_slot))) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "map arrays are NULL");
-  const int n_fill = map_fill(c, T_live, is_capturing(s));
-  c->map_installed = 1;
+  const unsigned long long capture = capture_of(s);
+  const int n_fill = map_fill(c, T_live, capture != 0);
+  map_by_kernel(c, s, capture);
   const int *req = token_req, *slots = req_slot;
   if (!src_is_device && T_live > 0) {
     MIX_CUDA(c, cudaMemcpyAsync(c->d_tmp_req, token_req, (size_t)T_live * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -754,7 +790,7 @@ template <class Tap>
 int sae_chain(mix_ctx* c, __nv_bfloat16* h, cudaStream_t s, Tap&& tap) {
   // The two fallback launches serve rows of TopK sets.  A call that is not being captured knows whether there are any; a
   // captured one may be replayed with sets registered later.  (reconstruct() on a JumpReLU set: 247 -> 243 us.)
-  bool topk = is_capturing(s);
+  bool topk = capture_of(s) != 0;
   for (int g = 0; g < c->cfg.n_groups_max; ++g) topk = topk || (c->h_groups[g].valid && c->h_groups[g].act == MIX_SAE_TOPK);
   if (c->cfg.flags & MIX_FLAG_ENCODE_SIMT) {
     MIX_CUDA(c, launch_encode_simt(c, s));
@@ -864,8 +900,9 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   }
   // (programmatic launch only where this kernel directly follows the caller's work in the caller's stream)
   const bool hook_pdl = !fork && !tc && !c->stage_events_on;
-  MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, c->map_installed != 0));
-  c->map_installed = 0;
+  const unsigned long long capture = c->n_map_pending || c->map_captured ? capture_of(s) : 0;
+  MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, map_is_pending(c, s, capture)));
+  map_arrived(c, s, capture);
   MIX_CUDA(c, tap());
   if (has_multiclass_stage(c) && !tc_fork) {
     MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, ps));

@@ -112,6 +112,13 @@ struct RouteState {
   int group_tile0[kMaxGroups + 1];  // first linear encode tile of group g
 };
 
+// Where an install of the slot map was enqueued.
+struct MapInstall {
+  cudaStream_t stream;
+  unsigned long long capture;       // 0: not captured
+};
+constexpr int kMapPending = 8;
+
 struct Ctx {
   mix_config cfg;
   int device;
@@ -122,6 +129,9 @@ struct Ctx {
   int* d_token_slot;        // [T_max]; -1 behind the live rows
   int map_live;             // live rows of the map last installed: what a shorter map has to set to -1
   int map_captured;         // an install was captured: which map is in force when another runs, the host cannot know
+  MapInstall map_pending[kMapPending];   // installs by kernel that no hook kernel of the same stream and capture has waited for
+  int n_map_pending;
+  int map_pending_any;      // there were too many to keep: every hook kernel waits
   int* d_n_live;            // [1] rows of d_token_slot that hold a map at all: T_max
   AppEntry* d_apps;         // [n_slots_max]
   GroupEntry* d_groups;     // [n_groups_max]
@@ -182,8 +192,6 @@ struct Ctx {
   cudaEvent_t ev_fork, ev_join;
 
   // profiling taps
-  int map_installed;        // a map was installed (by a kernel) since the last call: the next hook kernel must not read it
-                            // ahead of its predecessor
   int stage_events_on;
   cudaEvent_t stage_events[16];
 

@@ -124,6 +124,72 @@ def test_request_map_composed_by_a_kernel_is_seen_by_the_next_hook():
     m.destroy()
 
 
+@pytest.mark.parametrize("between", ["capture", "other stream", "other capture"])
+def test_a_hook_behind_a_map_that_a_call_elsewhere_has_used(between):
+    """A call in a capture, or on another stream, does not stand behind the kernel that installs the map on this one: the
+    next call here still does, and must not read the map ahead of it."""
+    mixlib = _mixlib()
+    T, d = 2048, 1024
+    m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=2)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(d, device=DEV, dtype=torch.bfloat16), 1.0 + slot)
+    maps = [torch.full((T,), slot, dtype=torch.int32, device=DEV) for slot in range(2)]
+    h, unused = torch.zeros((T, d), device=DEV, dtype=torch.bfloat16), torch.zeros((T, d), device=DEV, dtype=torch.bfloat16)
+    graphs = []
+    s, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for i in range(1, 7):
+        h.zero_()
+        torch.cuda.synchronize()
+        event = torch.cuda.Event()
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(20_000_000)            # everything below is enqueued before the first of it runs
+            m.apply(unused, stream=s)
+            m.set_slot_map(maps[i % 2], T, stream=s)
+            event.record(s)
+        if between == "other stream":
+            other.wait_event(event)
+            m.apply(unused, stream=other)
+        else:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.stream(other):
+                graph.capture_begin(capture_error_mode="thread_local")
+                if between == "other capture":
+                    m.set_slot_map(maps[0], T, stream=other)
+                m.apply(unused, stream=other)
+                graph.capture_end()
+            graphs.append(graph)
+        m.apply(h, stream=s)
+        torch.cuda.synchronize()
+        assert bool((h == 1.0 + i % 2).all()), i
+    assert m.get_status() == 0
+    graphs.clear()
+    m.destroy()
+
+
+def test_more_streams_with_a_pending_map_than_are_kept():
+    mixlib = _mixlib()
+    T, d = 64, 64
+    m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=2)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(d, device=DEV, dtype=torch.bfloat16), 1.0 + slot)
+    maps = [torch.full((T,), slot, dtype=torch.int32, device=DEV) for slot in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(12)]
+    for i, s in enumerate(streams):
+        m.set_slot_map(maps[i % 2], T, stream=s)     # ... and no call on most of them
+        torch.cuda.synchronize()
+    h = torch.zeros((T, d), device=DEV, dtype=torch.bfloat16)
+    for i, s in enumerate(streams):
+        h.zero_()
+        torch.cuda.synchronize()
+        m.set_slot_map(maps[i % 2], T, stream=s)
+        m.apply(h, stream=s)
+        m.apply(h, stream=s)
+        torch.cuda.synchronize()
+        assert bool((h == 2 * (1.0 + i % 2)).all())
+    m.destroy()
+
+
 def _run_sae_calls(w, n_calls, mask, flags=0):
     """One graph: n_calls x (copy a fresh batch into `h` -> mix_apply -> copy `h` out); returns the bits of every result."""
     mixlib = _mixlib()
