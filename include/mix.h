@@ -251,7 +251,12 @@ int mix_unregister_app(mix_ctx* ctx, int slot, void* stream);
 
 /* Cheap toggles that never touch launch structure (Section 4.2 "Toggling semantics").
    mix_update_steer_alpha also sets beta of a MIX_PROJECT app.  mix_update_sae_edits validates the
-   whole list first: a call that fails has changed nothing, on the host or on the device. */
+   whole list first: a call that fails has changed nothing, on the host or on the device.
+   Both are ordered by their stream, like registration.  An update on another stream than a mix_apply that is
+   running reaches it in part: the call takes the length of the edit list from its beginning, and on rows of a ReLU /
+   JumpReLU set that keep the error term it leaves out a feature that was not in the list when its encode looked
+   (only there are the pre-activations kept).  The next call applies the whole list; where one call must not mix two
+   lists, order the update in front of it or behind it with an event. */
 int mix_update_steer_alpha(mix_ctx* ctx, int slot, float alpha, void* stream);
 int mix_update_sae_edits(mix_ctx* ctx, int slot, int n_edit, const int* idx, const float* val,
                          const unsigned char* mode, void* stream);

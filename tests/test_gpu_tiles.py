@@ -129,3 +129,84 @@ def test_only_edited_features_stored(T, n_edit, act, fp8):
     sparse = run_gpu(w, flags=flags, feature_out=False, replays=2, graph=True)
     assert np.array_equal(full["hidden"], sparse["hidden"])
     assert sparse["status"] == 0
+
+
+def test_an_edit_list_that_another_stream_replaces_between_encode_and_decode():
+    """The call is captured, and a host function put between its encode and its tail: while that runs, another stream replaces
+    the edit list.  What the encode did not know to store is left out of this call; the next one applies the whole list."""
+    import ctypes
+    import threading
+
+    from cuda.bindings import runtime as rt
+
+    import paper_2607_22595_b200 as mixlib
+
+    def ok(result):
+        assert int(result[0]) == 0, result
+        return result[1:]
+
+    S, T = 2048, 40
+    w = _workload(128, S, T, W.SAE_RELU, True)
+    w.apps[0] = W.SaeApp(0, np.array([8, 20], np.int32), np.array([5.0, 2.0], np.float32), np.array([0, 0], np.uint8), True)
+    w.token_slot[:] = 0
+    replaced = np.array([9, 700], np.int32), np.array([3.0, -4.0], np.float32), np.array([0, 0], np.uint8)
+
+    def expected(idx, val, mode):
+        w.apps[0] = W.SaeApp(0, idx, val, mode, True)
+        return run_gpu(w, feature_out=False)["hidden"]
+
+    old_mask = mixlib.set_pdl_mask(0)                         # (plain edges: a programmatic one cannot be cut)
+    try:
+        m = W.make_context(mixlib.Mix, w)
+        h = w.hidden.clone()
+        m.apply(h)
+        h.copy_(w.hidden)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph):
+            m.apply(h)
+    finally:
+        mixlib.set_pdl_mask(old_mask)
+    raw = rt.cudaGraph_t(init_value=graph.raw_cuda_graph())
+    n = ok(rt.cudaGraphGetEdges(raw))[-1]
+    start, end = ok(rt.cudaGraphGetEdges(raw, n))[:2]
+    after = {int(a): b for a, b in zip(start[:n], end[:n])}
+    node = next(a for a in start[:n] if int(a) not in {int(b) for b in end[:n]})
+    chain = [node]
+    while int(chain[-1]) in after:
+        chain.append(after[int(chain[-1])])
+    assert len(chain) == 6                                    # hook, front, encode, tail and the two of the fallback
+    encode, tail = chain[2], chain[3]
+    reached, done = threading.Event(), threading.Event()
+
+    @ctypes.CFUNCTYPE(None, ctypes.c_void_p)
+    def pause(_):
+        reached.set()
+        done.wait(2.0)
+
+    params = rt.cudaHostNodeParams()
+    params.fn = rt.cudaHostFn_t(init_value=ctypes.cast(pause, ctypes.c_void_p).value)
+    between = ok(rt.cudaGraphAddHostNode(raw, [encode], 1, params))[0]
+    ok(rt.cudaGraphRemoveDependencies(raw, [encode], [tail], 1))
+    ok(rt.cudaGraphAddDependencies(raw, [between], [tail], 1))
+    graph.instantiate()
+
+    other = torch.cuda.Stream()
+    graph.replay()
+    assert reached.wait(10.0)
+    m.update_sae_edits(0, *replaced, stream=other)
+    other.synchronize()
+    assert not done.is_set()
+    done.set()
+    torch.cuda.synchronize()
+    # feature 9 shares a group of four with the edited feature 8, so its value was stored; feature 700's was not
+    during = W.bits(h)
+    assert np.array_equal(during, expected(*[x[:1] for x in replaced]))
+    assert not np.array_equal(during, expected(*replaced))
+    h.copy_(w.hidden)
+    m.apply(h)
+    assert np.array_equal(W.bits(h), expected(*replaced))
+    assert m.get_status() == 0
+    torch.cuda.synchronize()
+    del graph
+    m.destroy()
