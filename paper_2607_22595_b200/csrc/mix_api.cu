@@ -262,7 +262,9 @@ int pdl_mask() {
   if (g_pdl_mask < 0) g_pdl_mask = getenv("MIX_PDL_MASK") ? (atoi(getenv("MIX_PDL_MASK")) & 15) : (kPdlPack | kPdlEncode | kPdlTail | kPdlHook);
   return g_pdl_mask;
 }
-static std::atomic<int> g_hook_contexts{0};      // live contexts without weight sets: how many hooks the program has
+// Contexts without weight sets that the device has: how many hooks a step there is likely to have.
+static std::atomic<int> g_hook_contexts[64];
+std::atomic<int>& hook_contexts(int device) { return g_hook_contexts[device & 63]; }
 
 }  // namespace mix
 
@@ -405,14 +407,14 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { free_all(c); free(c); return MIX_ERR_CUDA; }
   c->err[0] = 0;
-  if (G == 0) ++mix::g_hook_contexts;
+  if (G == 0) ++mix::hook_contexts(c->device);
   *out = c;
   return MIX_OK;
 }
 
 int mix_destroy(mix_ctx* c) {
   if (!c) return MIX_OK;
-  if (c->cfg.n_groups_max == 0) --mix::g_hook_contexts;
+  if (c->cfg.n_groups_max == 0) --mix::hook_contexts(c->device);
   cudaDeviceSynchronize();
   free_all(c);
   free(c);
@@ -723,12 +725,15 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   const int n_fill = map_fill(c, T_live, capturing);
   const bool by_kernel = c->cfg.n_groups_max == 0;
   const int* src = (src_is_device || T_live == 0) ? token_slot : (by_kernel ? device_view(token_slot) : nullptr);
-  // With few hooks in the program a short map goes by a copy, which does not hold up the launch of a graph behind it; a
-  // row of hooks and longer maps go by the kernel, whose start and end cost less than a copy's.  Map and replay, 8 ... 256
-  // rows, copy against kernel: one hook 6.2 and 8.2 ... 9.1 us, two 12.3 and 13.0, four 24.6 and 23.3, sixteen 101 and 88;
-  // one hook on 512 rows 11.9 and 10.3, on 2000 rows 22.9 and 16.4.
+  // Where there are few hooks a short map goes by a copy, which does not hold up the launch of a graph behind it; a row of
+  // hooks and longer maps go by the kernel, whose start and end cost less than a copy's.  Maps and replay, 8 ... 256 rows, one
+  // after the other, copy against kernel: one hook 5.4 ... 6.2 and 8.2 us, two 11.2 ... 12.3 and 10.6 ... 12.3, three 16.4 ...
+  // 18.5 and 16.4, four 21.8 ... 22.6 and 20.5, sixteen 78 ... 88 and 68 ... 73; on an idle GPU 11.5 ... 13 and 15 ... 17, 16.5 and
+  // 19.7, 21 ... 22 and 24.5, 26 ... 27 and 28.5, 83 ... 93 and 78 ... 85.  One hook on 512 rows 11.9 and 10.3, on 2000 rows
+  // 22.9 and 16.4.  (The count is a guess at the length of the row, from the contexts that the device has; either way
+  // installs the same map.)
   // As a node of a graph the kernel is never slower (two hooks: 8.3 ... 10.3 us, copies 11.7).
-  const bool by_copy = src && !src_is_device && T_live <= kMapCopyRows && n_fill <= T_live && g_hook_contexts <= kMapCopyHooks &&
+  const bool by_copy = src && !src_is_device && T_live <= kMapCopyRows && n_fill <= T_live && hook_contexts(c->device) <= kMapCopyHooks &&
                        !capturing;
   if ((src && !by_copy) || T_live == 0) {
     map_by_kernel(c, s, capture);

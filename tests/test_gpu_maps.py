@@ -178,3 +178,31 @@ def test_an_install_that_fails_leaves_the_rows_of_the_map_before_to_the_next_one
     m.apply(h)
     assert int((h[:, 0] != 0).sum()) == 20
     m.destroy()
+
+
+# one and two hooks take a short pinned map by a copy, three by the kernel
+@pytest.mark.parametrize("hooks", [1, 2, 3])
+@pytest.mark.parametrize("live", [1, 255, 256, 257])
+def test_pinned_maps_of_a_row_of_hooks(hooks, live):
+    d, T = 64, 300
+    ms, hs = [], []
+    for _ in range(hooks):
+        m = Mix(d_model=d, T_max=T, n_slots_max=2)
+        for slot in range(2):
+            m.register_steer(slot, torch.ones(d, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+        ms.append(m)
+        hs.append(torch.zeros((T, d), device="cuda", dtype=torch.bfloat16))
+    rng = np.random.default_rng(live)
+    for n in (live, T, live, live // 2, live):               # longer, shorter, as long
+        slots = [rng.integers(-1, 2, size=n).astype(np.int32) for _ in ms]
+        pins = [torch.from_numpy(x).pin_memory() for x in slots]
+        for m, pin, h in zip(ms, pins, hs):
+            h.zero_()
+            m.set_slot_map(pin, n)
+            m.apply(h)
+        for x, h in zip(slots, hs):
+            want = np.zeros(T, dtype=np.float32)
+            want[:n] = x + 1.0
+            assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), n
+    for m in ms:
+        m.destroy()
