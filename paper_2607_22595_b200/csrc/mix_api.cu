@@ -391,7 +391,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     // large batches with multi-class probes: the tensor-core probe kernel needs a map per probe matrix
     if (dev_alloc(&c->d_tmap_probe, NS) != cudaSuccess || dev_alloc(&c->d_mc_census, 1) != cudaSuccess ||
         dev_alloc(&c->d_mc_tiles, (size_t)(T + kTileM - 1) / kTileM) != cudaSuccess ||
-        dev_alloc(&c->d_part_logits, (size_t)kPPartItems * kTileM * 32) != cudaSuccess || dev_alloc(&c->d_part_done, kPPartItems * 4) != cudaSuccess) {
+        dev_alloc(&c->d_part_logits, (size_t)part_items(T) * kTileM * 32) != cudaSuccess || dev_alloc(&c->d_part_done, kPPartItems * 4) != cudaSuccess) {
       cudaGetLastError(); free_all(c); free(c); return MIX_ERR_NO_MEMORY;
     }
     e = cudaMemset(c->d_mc_census, 0, sizeof(McCensus));

@@ -181,7 +181,7 @@ struct Ctx {
   CUtensorMap* d_tmap_probe;   // [n_slots_max] maps of multi-class probe matrices (box kTileK x 32), large-batch contexts only
   McCensus* d_mc_census;    // census of the 128-row tiles that hold multi-class probe rows, taken by mc_census_kernel every call
   int* d_mc_tiles;          // [ceil(T_max / 128)] those tiles, in no particular order
-  float* d_part_logits;     // [kPPartItems][128 rows][32] tensor-core probe kernel: partial logits of tiles whose columns are cut into parts
+  float* d_part_logits;     // [part_items(T_max)][128 rows][32] tensor-core probe kernel: partial logits of tiles whose columns are cut into parts
   int* d_part_done;         // [kPPartItems][4] finished parts of each quarter of a tile (zeroed by the census)
   CUtensorMap tmap_w_one;   // where d_tmap_w is null (the allocation-free call): the one weight set's map, at this call's tile width
   CUtensorMap tmap_panel;   // panel map (box kTileK x kTileM, 128B swizzle)
@@ -269,6 +269,11 @@ constexpr int kPdlMapAhead = 2;   // how the hook kernels are told: programmatic
 // least half full of such rows) or probe_multiclass (mma.sync, 16-row tiles: rows scattered thinly).
 cudaError_t launch_mc_census(const Ctx* c, int T, cudaStream_t s);
 constexpr int kPPartItems = 448;           // most (tile, part of the columns) items of a call that cuts its tiles: three per SM
+constexpr int kPMostParts = 8;             // most parts of a tile
+inline int part_items(int T_max) {         // most such items of a context: what Ctx::d_part_logits holds (16 KiB each)
+  const int most = (T_max + kTileM - 1) / kTileM * kPMostParts;
+  return most < kPPartItems ? most : kPPartItems;
+}
 cudaError_t launch_probe_tc(const Ctx* c, const CUtensorMap& tmap_hidden, int T, float* scores, cudaStream_t s);
 cudaError_t launch_probe_multiclass(const Ctx* c, const __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s);
 cudaError_t probe_tc_prepare();   // opt in to the large dynamic shared memory size

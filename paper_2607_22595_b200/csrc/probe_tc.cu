@@ -74,7 +74,6 @@ static_assert(sizeof(PShared) <= 1024, "PShared must fit the space reserved for 
 // k-blocks, a part counting two more for its descriptor and epilogue.
 // 4000 rows of 16-class probes, d = 5120: 45 -> 26 us; 15873 rows with every kind of app, 2778 of them such probes: the call
 // 75 -> 58 us.
-constexpr int kPMostParts = 8;
 __device__ __forceinline__ int column_parts(int n_tiles, int num_kb, int n_ctas) {
   int best = 1, best_cost = 1 << 30;
   for (int parts = 1; parts <= kPMostParts && parts <= num_kb; ++parts) {

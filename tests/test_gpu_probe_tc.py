@@ -168,3 +168,22 @@ def test_columns_cut_into_parts(d, T, rows):
         assert (scores[slot < 0] == -1.0).all()
     assert m.get_status() == 0
     m.destroy()
+
+
+def test_scratch_of_the_smallest_batches():
+    # every tile cut into as many parts as there are, which fills the scratch to its end; it costs no more memory than that
+    T, d = 17 * 128, 8192
+    mixlib = _mixlib()
+
+    def bytes_of(C_max):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=2, C_max=C_max)
+        used = free - torch.cuda.mem_get_info()[0]
+        m.destroy()
+        return used
+
+    bytes_of(16)                                         # (loads the kernels)
+    assert bytes_of(16) - bytes_of(1) <= 5 << 20         # 17 x 8 items of 16 KiB, in pages of 2 MiB
+    w = _probe_workload(T, T, d, np.arange(T) // 300 % 2, [16, 9], [W.ACT_SOFTMAX, W.ACT_NONE])
+    check_parity(W.host(w), run_gpu(w))
