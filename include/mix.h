@@ -384,7 +384,7 @@ int mix_get_status(mix_ctx* ctx, unsigned* bits, void* stream);
 /* Number of kernels one mix_apply() call launches on this context (fixed at mix_create):
    1 without SAE weight sets, else 7 (4 with MIX_FLAG_ENCODE_SIMT); one more when T_max > 2048
    and C_max > 1 (multi-class probes of large batches run in a kernel of their own), and two more
-   with MIX_FLAG_SAE_EDIT_ONLY.  An uncaptured call leaves two of the 7 out while no TopK set is
+   with MIX_FLAG_SAE_EDIT_ONLY.  An uncaptured call leaves two of the 7 out until a TopK set is
    registered: they serve its fallback. */
 int mix_launches_per_apply(const mix_ctx* ctx);
 

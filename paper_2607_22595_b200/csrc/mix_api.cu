@@ -509,6 +509,7 @@ int mix_register_sae_weights(mix_ctx* c, int group, const mix_sae_weights* w, vo
     for (int i = 0; i < 3; ++i)
       MIX_CUDA(c, cudaMemcpyAsync(c->d_tmap_w + (size_t)i * c->cfg.n_groups_max + group, &tm[i], sizeof(CUtensorMap), cudaMemcpyHostToDevice, s));
   }
+  if (w->act == MIX_SAE_TOPK) c->topk_seen = 1;
   c->h_groups[group] = ge;
   GroupEntry tmp = ge;
   tmp.valid = 0;
@@ -793,10 +794,10 @@ namespace {
 // The SAE chain behind the front kernel: encode ... write-back.  `tap` records a stage event after each launch.
 template <class Tap>
 int sae_chain(mix_ctx* c, __nv_bfloat16* h, cudaStream_t s, Tap&& tap) {
-  // The two fallback launches serve rows of TopK sets.  A call that is not being captured knows whether there are any; a
-  // captured one may be replayed with sets registered later.  (reconstruct() on a JumpReLU set: 247 -> 243 us.)
-  bool topk = capture_of(s) != 0;
-  for (int g = 0; g < c->cfg.n_groups_max; ++g) topk = topk || (c->h_groups[g].valid && c->h_groups[g].act == MIX_SAE_TOPK);
+  // The two fallback launches serve rows of TopK sets.  A call that is not being captured knows whether there ever were any (a
+  // set that another stream is about to replace may still be the one in the device's table); a captured one may be replayed
+  // with sets registered later.  (reconstruct() on a JumpReLU set: 247 -> 243 us.)
+  const bool topk = c->topk_seen || capture_of(s) != 0;
   if (c->cfg.flags & MIX_FLAG_ENCODE_SIMT) {
     MIX_CUDA(c, launch_encode_simt(c, s));
     MIX_CUDA(c, tap());

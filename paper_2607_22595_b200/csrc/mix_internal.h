@@ -150,6 +150,7 @@ struct Ctx {
   // host mirrors (validation only)
   AppEntry* h_apps;
   GroupEntry* h_groups;
+  int topk_seen;            // a TopK set has been registered
   float** owned_b_eff;      // per group: library-owned folded bias or null
   __nv_bfloat16** owned_w_tiled;   // per group: library-owned tile-contiguous copy of W_enc or null
 

@@ -210,3 +210,27 @@ def test_an_edit_list_that_another_stream_replaces_between_encode_and_decode():
     torch.cuda.synchronize()
     del graph
     m.destroy()
+
+
+def test_a_set_that_another_stream_is_about_to_remove():
+    """The host's table has lost the TopK set, the device's has not: rows that need the exact fallback still get it."""
+    import paper_2607_22595_b200 as mixlib
+    w = _workload(128, 2048, 30, W.SAE_TOPK, False)
+    w.groups[0].W_enc[256:512] = w.groups[0].W_enc[256].clone()          # 256 equal features: no tile's eight candidates can tell
+    w.groups[0].b_enc[256:512] = 3.0
+    want = run_gpu(w, feature_out=False)
+    check_parity(W.host(w), want, check_features=False)
+    assert not np.array_equal(want["hidden"], W.bits(w.hidden))
+    m = W.make_context(mixlib.Mix, w)
+    h = w.hidden.clone()
+    late, now = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(late):
+        torch.cuda._sleep(100_000_000)                        # 50 ms
+    m.unregister_sae_weights(0, stream=late)
+    m.apply(h, stream=now)
+    now.synchronize()
+    assert not late.query()                                   # the set is still there
+    assert np.array_equal(W.bits(h), want["hidden"])
+    torch.cuda.synchronize()
+    m.destroy()
