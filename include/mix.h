@@ -371,7 +371,7 @@ int mix_apply_conditional(mix_ctx* ctx, void* hidden, int T, float* scores_out, 
 /* The hook on a different target tensor: router logits (device fp32 [T_max, n_experts], modified in
    place).  Rows whose slot holds a MIX_ROUTER app with the same n_experts (and an open gate, if it
    has one) get logits[t, :] += delta; every other row is neither read nor written.  Uses the same
-   slot map, live count and gates as mix_apply(); one kernel, capturable.
+   slot map and gates as mix_apply(); one kernel, capturable.
    Errors: INVALID_ARG (NULL logits, n_experts < 1), OUT_OF_RANGE (T). */
 int mix_apply_router(mix_ctx* ctx, float* logits, int n_experts, int T, void* stream);
 

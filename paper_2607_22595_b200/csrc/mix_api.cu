@@ -76,7 +76,7 @@ cudaError_t dev_alloc(T** p, size_t n) {
 }
 
 void free_all(mix_ctx* c) {
-  cudaFree(c->d_token_slot); cudaFree(c->d_n_live); cudaFree(c->d_apps); cudaFree(c->d_groups); cudaFree(c->d_gates); cudaFree(c->d_vec_arena); cudaFree(c->d_chain_next); cudaFree(c->d_row_meta); cudaFree(c->d_front_counts); cudaFree(c->d_front_sync); cudaFree(c->d_row_rec);
+  cudaFree(c->d_token_slot); cudaFree(c->d_apps); cudaFree(c->d_groups); cudaFree(c->d_gates); cudaFree(c->d_vec_arena); cudaFree(c->d_chain_next); cudaFree(c->d_row_meta); cudaFree(c->d_front_counts); cudaFree(c->d_front_sync); cudaFree(c->d_row_rec);
   cudaFree(c->d_edit_idx); cudaFree(c->d_edit_val); cudaFree(c->d_edit_mode); cudaFree(c->d_status);
   cudaFree(c->d_tmp_req); cudaFree(c->d_tmp_req_slot); cudaFree(c->d_panel); cudaFree(c->d_panel_row); cudaFree(c->d_act_scale); cudaFree(c->d_tau); cudaFree(c->d_tau_min); cudaFree(c->d_eo_row_delta); cudaFree(c->d_eo_coef);
   cudaFree(c->d_mtile_group); cudaFree(c->d_route); cudaFree(c->d_z);
@@ -313,7 +313,6 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   if (!c->h_apps || !c->h_groups || !c->h_chain_next || !c->h_edit_idx || !c->owned_b_eff || !c->owned_w_tiled) { free_all(c); free(c); return MIX_ERR_NO_MEMORY; }
   bool ok = true;
   ok = ok && dev_alloc(&c->d_token_slot, T) == cudaSuccess;
-  ok = ok && dev_alloc(&c->d_n_live, 1) == cudaSuccess;
   ok = ok && dev_alloc(&c->d_apps, NS) == cudaSuccess;
   ok = ok && dev_alloc(&c->d_groups, G > 0 ? G : 1) == cudaSuccess;
   ok = ok && dev_alloc(&c->d_gates, NS) == cudaSuccess;
@@ -360,7 +359,6 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   }
   if (!ok) { cudaGetLastError(); free_all(c); free(c); return MIX_ERR_NO_MEMORY; }
   e = cudaMemset(c->d_token_slot, 0xff, T * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpy(c->d_n_live, &T, sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->d_apps, 0, NS * sizeof(AppEntry));
   if (e == cudaSuccess) e = cudaMemset(c->d_groups, 0, (G > 0 ? G : 1) * sizeof(GroupEntry));
   if (e == cudaSuccess) e = cudaMemset(c->d_gates, 0, NS * sizeof(GateEntry));

@@ -1,6 +1,6 @@
 // Internal declarations shared by the translation units of libmix.so.
 // Device tables live at fixed addresses owned by the context; kernels read every piece of
-// dynamic state (slot map, live count, app table, edit lists, route results) from them, so
+// dynamic state (slot map, app table, edit lists, route results) from them, so
 // a captured graph never needs its kernel parameters changed.
 #pragma once
 
@@ -132,7 +132,6 @@ struct Ctx {
   MapInstall map_pending[kMapPending];   // installs by kernel that no hook kernel of the same stream and capture has waited for
   int n_map_pending;
   int map_pending_any;      // there were too many to keep: every hook kernel waits
-  int* d_n_live;            // [1] rows of d_token_slot that hold a map at all: T_max
   AppEntry* d_apps;         // [n_slots_max]
   GroupEntry* d_groups;     // [n_groups_max]
   GateEntry* d_gates;       // [n_slots_max]

@@ -97,7 +97,7 @@ __device__ __forceinline__ bool pwait(unsigned bar, unsigned parity, PShared* sh
 // with every kind of app: the call 58.0 -> 57.0 us.)
 __global__ void __launch_bounds__(kPThreads, 3)
 probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorMap* __restrict__ tmap_probe,
-                const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+                const int* __restrict__ token_slot, int T,
                 const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots, int d,
                 float* __restrict__ scores, int C_max, unsigned* __restrict__ status, const McCensus* __restrict__ census,
                 const int* __restrict__ census_tiles, float* __restrict__ part_logits, int* __restrict__ part_done, int test_stall) {
@@ -105,7 +105,6 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   PShared* sh = reinterpret_cast<PShared*>(tiles + kPStages * kPStageBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_live = min(T, __ldg(n_live_p));
   // the tiles of this call that hold multi-class probe rows, as the census listed them (in no particular order):
   // CTAs share THEM out, so a batch whose hooked requests are clustered still spreads evenly over the SMs
   if (!census->use_tc) return;                         // rows scattered thinly: probe_multiclass_kernel's call
@@ -150,7 +149,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
         s[i] = -1;
         blk[i] = -1;
         const int t = tile * kTileM + i * 32 + lane;
-        if (t < n_live) {
+        if (t < T) {
           const int sl = __ldg(token_slot + t);
           const RowApp a = lookup(sl, t, apps, gates, n_slots, nullptr, false);   // bad slots: flagged by probe_steer_kernel
           if (a.kind == MIX_PROBE && a.C > 1 && a.C <= kPBlockCols) s[i] = sl;
@@ -413,7 +412,7 @@ cudaError_t probe_tc_prepare() {
 
 cudaError_t launch_probe_tc(const Ctx* c, const CUtensorMap& tmap_hidden, int T, float* scores, cudaStream_t s) {
   if (scores == nullptr) return cudaSuccess;
-  probe_tc_kernel<<<c->n_sms, kPThreads, kPSmemBytes, s>>>(tmap_hidden, c->d_tmap_probe, c->d_token_slot, c->d_n_live, T,
+  probe_tc_kernel<<<c->n_sms, kPThreads, kPSmemBytes, s>>>(tmap_hidden, c->d_tmap_probe, c->d_token_slot, T,
                                                            c->d_apps, c->d_gates, c->cfg.n_slots_max, c->cfg.d_model, scores,
                                                            c->cfg.C_max, c->d_status, c->d_mc_census, c->d_mc_tiles, c->d_part_logits, c->d_part_done,
                                                            (c->cfg.flags & MIX_FLAG_TEST_STALL_ENCODE) ? 1 : 0);

@@ -210,16 +210,15 @@ __device__ __forceinline__ void warp_row(const RowApp& a, __nv_bfloat16* __restr
 // tensor-core kernel, which leaves room for eight warps at a time.
 template <int kWarps, int kMinCtas>
 __global__ void __launch_bounds__(kWarps * 32, kMinCtas)
-probe_steer_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+probe_steer_kernel(const int* __restrict__ token_slot, int T,
                    const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                    __nv_bfloat16* __restrict__ hidden, int d,
                    float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int multiclass_elsewhere) {
   __shared__ float s_logit[kWarps][kMaxClasses];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * kWarps + warp;
-  const int n_live = __ldg(n_live_p);            // issued together with the slot id: one round trip, not two
-  const int slot = t < T ? __ldg(token_slot + t) : -1;
-  if (t >= min(T, n_live)) return;
+  if (t >= T) return;
+  const int slot = __ldg(token_slot + t);
   const RowApp a = lookup(slot, t, apps, gates, n_slots, status, lane == 0);
   if (a.kind == 0) return;
   if (multiclass_elsewhere && a.kind == MIX_PROBE && a.C > 1 && a.C <= kCoopMaxClasses) return;
@@ -309,7 +308,7 @@ struct McRow {
 // 16 rows against that probe's matrix, which is therefore streamed from L2 once per 16 rows;
 // only the rows that belong to the probe keep their result.
 __global__ void __launch_bounds__(kMcWarps * 32, 2)
-probe_multiclass_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         const __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
                         const McCensus* __restrict__ census) {
@@ -319,8 +318,7 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, const int* __restric
   __shared__ int s_any;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t0 = blockIdx.x * kMcRows;
-  const int n_live = min(T, __ldg(n_live_p));
-  if (t0 >= n_live || scores == nullptr) return;
+  if (t0 >= T || scores == nullptr) return;
   if (census != nullptr && census->use_tc) return;          // this call's batch is probe_tc_kernel's
   if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
@@ -328,7 +326,7 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, const int* __restric
     const int t = t0 + threadIdx.x;
     McRow r;
     r.slot = -1;
-    if (t < n_live) {
+    if (t < T) {
       const int s = __ldg(token_slot + t);
       const RowApp a = lookup(s, t, apps, gates, n_slots, nullptr, false);   // bad slots are flagged by probe_steer_kernel
       if (a.kind == MIX_PROBE && a.C > 1 && a.C <= kCoopMaxClasses) {
@@ -345,8 +343,8 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, const int* __restric
   __syncthreads();
   if (!s_any) return;                    // CTA-uniform
   const int g = lane >> 2;
-  const uint4* h_lo = reinterpret_cast<const uint4*>(hidden + (size_t)min(t0 + g, n_live - 1) * d);
-  const uint4* h_hi = reinterpret_cast<const uint4*>(hidden + (size_t)min(t0 + g + 8, n_live - 1) * d);
+  const uint4* h_lo = reinterpret_cast<const uint4*>(hidden + (size_t)min(t0 + g, T - 1) * d);
+  const uint4* h_hi = reinterpret_cast<const uint4*>(hidden + (size_t)min(t0 + g + 8, T - 1) * d);
   const int n_chunks = d >> 5, row_vecs = d >> 3;
   for (int r = 0; r < kMcRows; ++r) {
     const McRow ci = s_row[r];
@@ -386,7 +384,7 @@ enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own
 
 template <int NW, TeamForm kForm>
 __global__ void __launch_bounds__(NW * 32)
-probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
                         unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl) {
@@ -395,7 +393,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
   // Programmatic dependent launch (`pdl`: the launch asked for it): everything up to pdl_wait() reads only
-  // tables the LIBRARY owns and that only copies write -- live count, slot map, app entry, vector arena -- so it
+  // tables the LIBRARY owns and that only copies write -- slot map, app entry, vector arena -- so it
   // may run while the kernel in front of this one in the stream (the layer that produces `hidden`, or the
   // previous hook) is still running.  Memory the caller owns (`hidden`, multi-class probe weights, gate scores)
   // is read after the wait only, and every thread waits before it leaves, so that this grid cannot end -- and
@@ -410,9 +408,8 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
   }
   constexpr bool kLate = kForm == kTeamLate;
   if (pdl) pdl_launch_dependents();
-  const int n_live = __ldg(n_live_p);            // both loads issue together: one round trip, not two
   const int slot = __ldg(token_slot + t);
-  if (t >= min(T, n_live) || slot == -1) {
+  if (t >= T || slot == -1) {
     if (pdl) pdl_wait();
     return;
   }
@@ -595,7 +592,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, const int* __restric
 constexpr int kChainWarps = 8;
 
 __global__ void __launch_bounds__(kChainWarps * 32)
-probe_steer_chain_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
                          const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates,
                          const int* __restrict__ chain_next, int n_slots, __nv_bfloat16* __restrict__ hidden, int d,
                          float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int pdl) {
@@ -603,15 +600,14 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, const int* __restri
   constexpr int NT = kChainWarps * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
-  // programmatic dependent launch, as in probe_steer_team_kernel: the live count and the slot id (library-owned,
+  // programmatic dependent launch, as in probe_steer_team_kernel: the slot id (library-owned,
   // written only by copies) may be read while the predecessor still runs; everything else comes after the wait,
   // and every thread waits before it leaves
   if (pdl == kPdlMapAhead) pdl_wait();
   pdl_launch_dependents();
-  const int n_live = __ldg(n_live_p);
   int slot = __ldg(token_slot + t);
   pdl_wait();
-  if (t >= min(T, n_live) || slot == -1) return;
+  if (t >= T || slot == -1) return;
   const int nvec = d >> 3;
   uint4* hrow = reinterpret_cast<uint4*>(hidden + (size_t)t * d);
   uint4 hq[kTeamVec];
@@ -717,12 +713,12 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, const int* __restri
 
 // Router-logit steering: one thread per (row, expert).
 __global__ void __launch_bounds__(256)
-router_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+router_kernel(const int* __restrict__ token_slot, int T,
               const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
               float* __restrict__ logits, int n_experts) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(i / n_experts), e = (int)(i - (long long)t * n_experts);
-  if (t >= min(T, __ldg(n_live_p))) return;
+  if (t >= T) return;
   const RowApp a = lookup(__ldg(token_slot + t), t, apps, gates, n_slots, nullptr, false);
   if (a.kind != MIX_ROUTER || a.C != n_experts) return;
   logits[i] += __ldg(reinterpret_cast<const float*>(a.W) + e);
@@ -800,20 +796,19 @@ __global__ void fold_bias_kernel(const __nv_bfloat16* __restrict__ W_enc, const 
 // it takes the call when the listed tiles are, on average, at least half full of such rows.
 constexpr int kCensusWarps = 8;
 __global__ void __launch_bounds__(kCensusWarps * 32)
-mc_census_kernel(const int* __restrict__ token_slot, const int* __restrict__ n_live_p, int T,
+mc_census_kernel(const int* __restrict__ token_slot, int T,
                  const AppEntry* __restrict__ apps, int n_slots, McCensus* __restrict__ census, int* __restrict__ tiles,
                  int* __restrict__ part_done) {
   if (blockIdx.x == 0)                                   // the tensor-core kernel's counters of finished column parts
     for (int i = threadIdx.x; i < kPPartItems * 4; i += kCensusWarps * 32) part_done[i] = 0;
   __shared__ int s_cnt[kCensusWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int live = min(T, __ldg(n_live_p));
   const int tile = blockIdx.x * kCensusWarps + warp;
   int slot[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int t = tile * kTileM + i * 32 + lane;
-    slot[i] = t < live ? __ldg(token_slot + t) : -1;
+    slot[i] = t < T ? __ldg(token_slot + t) : -1;
   }
   int4 q[4];
 #pragma unroll
@@ -865,7 +860,7 @@ bool has_multiclass_stage(const Ctx* c) {
 
 cudaError_t launch_mc_census(const Ctx* c, int T, cudaStream_t s) {
   const int rows_per_cta = kCensusWarps * kTileM;
-  mc_census_kernel<<<(c->cfg.T_max + rows_per_cta - 1) / rows_per_cta, kCensusWarps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps,
+  mc_census_kernel<<<(c->cfg.T_max + rows_per_cta - 1) / rows_per_cta, kCensusWarps * 32, 0, s>>>(c->d_token_slot, T, c->d_apps,
                                                                            c->cfg.n_slots_max, c->d_mc_census, c->d_mc_tiles, c->d_part_done);
   return cudaGetLastError();
 }
@@ -878,18 +873,18 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
   const int pdl = (allow_pdl && (pdl_mask() & kPdlHook)) ? (map_ahead ? kPdlMapAhead : 1) : 0;
   if (c->cfg.flags & MIX_FLAG_SLOT_CHAINS) {
     return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_chain_kernel, dim3(c->cfg.T_max), dim3(kChainWarps * 32), 0, s,
-                      c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
+                      c->d_token_slot, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
                       c->cfg.d_model, scores, c->cfg.C_max, c->d_status, pdl);
   } else if (c->cfg.T_max <= kTeamMaxRows) {
     auto kernel = c->cfg.n_groups_max > 0 ? probe_steer_team_kernel<8, kTeamLate>
                                           : (pdl == kPdlMapAhead ? probe_steer_team_kernel<8, kTeamMapAhead> : probe_steer_team_kernel<8, kTeamPlain>);
     return launch_pdl(allow_pdl ? kPdlHook : 0, kernel,
-                      dim3(c->cfg.T_max), dim3(8 * 32), 0, s, c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+                      dim3(c->cfg.T_max), dim3(8 * 32), 0, s, c->d_token_slot, T, c->d_apps, c->d_gates,
                       c->cfg.n_slots_max, hidden, c->cfg.d_model, scores, c->cfg.C_max, c->d_status,
                       reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
   } else {
     auto run = [&](auto kernel, int warps) {
-      kernel<<<(c->cfg.T_max + warps - 1) / warps, warps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+      kernel<<<(c->cfg.T_max + warps - 1) / warps, warps * 32, 0, s>>>(c->d_token_slot, T, c->d_apps, c->d_gates,
                                                                       c->cfg.n_slots_max, hidden, c->cfg.d_model, scores,
                                                                       c->cfg.C_max, c->d_status, has_multiclass_stage(c) ? 1 : 0);
     };
@@ -901,7 +896,7 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
 
 cudaError_t launch_probe_multiclass(const Ctx* c, const __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s) {
   const int blocks = (c->cfg.T_max + kMcRows - 1) / kMcRows;
-  probe_multiclass_kernel<<<blocks, kMcWarps * 32, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+  probe_multiclass_kernel<<<blocks, kMcWarps * 32, 0, s>>>(c->d_token_slot, T, c->d_apps, c->d_gates,
                                                                  c->cfg.n_slots_max, hidden, c->cfg.d_model, scores,
                                                                  c->cfg.C_max, has_tc_probe_stage(c) ? c->d_mc_census : nullptr);
   return cudaGetLastError();
@@ -909,7 +904,7 @@ cudaError_t launch_probe_multiclass(const Ctx* c, const __nv_bfloat16* hidden, i
 
 cudaError_t launch_router(const Ctx* c, float* logits, int n_experts, int T, cudaStream_t s) {
   const long long n = (long long)c->cfg.T_max * n_experts;
-  router_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates,
+  router_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c->d_token_slot, T, c->d_apps, c->d_gates,
                                                             c->cfg.n_slots_max, logits, n_experts);
   return cudaGetLastError();
 }

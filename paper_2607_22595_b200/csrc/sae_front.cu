@@ -95,7 +95,6 @@ __device__ __forceinline__ void pack_row_e4m3(const __nv_bfloat16* __restrict__ 
 struct FrontArgs {
   // slot map and tables (read)
   const int* token_slot;
-  const int* n_live_p;
   int T;
   const AppEntry* apps;
   const GateEntry* gates;
@@ -318,7 +317,6 @@ front_kernel(const FrontArgs a) {
   const int n_chunks = (a.T + kFrontThreads - 1) / kFrontThreads;     // the same in every CTA: who publishes is fixed by the launch
   const bool local = n_chunks <= kFrontLocal;
   phase_stamp(a.clk, 0, first_cta && tid == 0);
-  const int n_live = min(a.T, __ldg(a.n_live_p));      // (all of these loads issue together)
   if (tid < n_groups) {                                // requested now, needed after the first barrier
     const bool valid = __ldg(&a.groups[tid].valid) != 0;
     s_gact[tid] = __ldg(&a.groups[tid].act);
@@ -328,7 +326,7 @@ front_kernel(const FrontArgs a) {
   }
   auto slot_of = [&](int t) {
     const int slot = t < a.T ? __ldg(a.token_slot + t) : -1;
-    return t < n_live && slot < n_slots ? slot : -1;
+    return slot < n_slots ? slot : -1;
   };
   int rank[kFrontLocal], grp[kFrontLocal];             // local: this thread's rows -- weight set or -1, place among the warp's rows of the set
   RowClass row[kFrontLocal];
@@ -565,7 +563,6 @@ int front_chunks(int T_max) { return (T_max + kFrontThreads - 1) / kFrontThreads
 cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, bool pdl, unsigned long long cond, int use_cond) {
   FrontArgs a;
   a.token_slot = c->d_token_slot;
-  a.n_live_p = c->d_n_live;
   a.T = T;
   a.apps = c->d_apps;
   a.gates = c->d_gates;

@@ -242,8 +242,8 @@ struct EoRow {
 };
 
 __global__ void __launch_bounds__(kEoThreads)
-sae_edit_only_kernel(__nv_bfloat16* __restrict__ hidden, int d, const int* __restrict__ token_slot,
-                     const int* __restrict__ n_live_p, int T, const AppEntry* __restrict__ apps,
+sae_edit_only_kernel(__nv_bfloat16* __restrict__ hidden, int d, const int* __restrict__ token_slot, int T,
+                     const AppEntry* __restrict__ apps,
                      const GateEntry* __restrict__ gates, int n_slots, const GroupEntry* __restrict__ groups,
                      int n_groups, const int* __restrict__ edit_idx, const float* __restrict__ edit_val,
                      const unsigned char* __restrict__ edit_mode, int r_max, RowDelta* __restrict__ row_delta,
@@ -265,7 +265,7 @@ sae_edit_only_kernel(__nv_bfloat16* __restrict__ hidden, int d, const int* __res
     r.slot = -1;
     r.n_edit = 0;
     const int t = t0 + tid;
-    if (t < min(T, *n_live_p)) {
+    if (t < T) {
       const int slot = token_slot[t];
       if (slot >= 0 && slot < n_slots) {
         const AppEntry app = apps[slot];
@@ -428,7 +428,7 @@ cudaError_t edit_only_prepare() {
 cudaError_t launch_edit_only(const Ctx* c, __nv_bfloat16* hidden, int T, cudaStream_t s) {
   const size_t smem = (size_t)kEoRows * c->cfg.d_model * sizeof(__nv_bfloat16);
   cudaError_t e = launch_pdl(kPdlTail, sae_edit_only_kernel, dim3((c->cfg.T_max + kEoRows - 1) / kEoRows), dim3(kEoThreads), smem, s,
-                             hidden, c->cfg.d_model, c->d_token_slot, c->d_n_live, T, c->d_apps, c->d_gates, c->cfg.n_slots_max,
+                             hidden, c->cfg.d_model, c->d_token_slot, T, c->d_apps, c->d_gates, c->cfg.n_slots_max,
                              c->d_groups, c->cfg.n_groups_max, c->d_edit_idx, c->d_edit_val, c->d_edit_mode, c->cfg.r_max,
                              c->d_eo_row_delta, c->d_eo_coef, c->cfg.T_max);
   return e;

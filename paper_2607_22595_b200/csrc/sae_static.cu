@@ -25,8 +25,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // byte offsets inside the scratch array (each 256-byte aligned)
 constexpr size_t kOffTokenSlot = 0;
-constexpr size_t kOffNLive = kOffTokenSlot + align256(kStaticRows * sizeof(int));
-constexpr size_t kOffStatus = kOffNLive + 256;
+constexpr size_t kOffStatus = kOffTokenSlot + align256(kStaticRows * sizeof(int));
 constexpr size_t kOffApp = kOffStatus + 256;
 constexpr size_t kOffGate = kOffApp + align256(sizeof(AppEntry));
 constexpr size_t kOffGroup = kOffGate + align256(sizeof(GateEntry));
@@ -78,9 +77,9 @@ struct StaticSetup {
 
 // Rewrites every table of the scratch array that this call's kernels read before writing.
 __global__ void __launch_bounds__(128)
-static_setup_kernel(const StaticSetup su, int* __restrict__ token_slot, int* __restrict__ n_live,
-                    unsigned* __restrict__ status, AppEntry* __restrict__ app, GroupEntry* __restrict__ group,
-                    int* __restrict__ edit_idx, float* __restrict__ edit_val, unsigned char* __restrict__ edit_mode) {
+static_setup_kernel(const StaticSetup su, int* __restrict__ token_slot, unsigned* __restrict__ status,
+                    AppEntry* __restrict__ app, GroupEntry* __restrict__ group, int* __restrict__ edit_idx,
+                    float* __restrict__ edit_val, unsigned char* __restrict__ edit_mode) {
   const int tid = threadIdx.x;
   if (tid < su.n_rows) token_slot[tid] = 0;             // every row -> slot 0 (n_rows <= 128 = blockDim.x)
   if (tid < su.n_edit) {
@@ -89,7 +88,6 @@ static_setup_kernel(const StaticSetup su, int* __restrict__ token_slot, int* __r
     edit_mode[tid] = su.edit_mode[tid];
   }
   if (tid == 0) {
-    *n_live = su.n_rows;
     *status = 0u;
     *app = su.app;
     *group = su.group;
@@ -172,7 +170,6 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   c.device = dev;
   c.n_sms = g_n_sms[dev];
   c.d_token_slot = reinterpret_cast<int*>(base + kOffTokenSlot);
-  c.d_n_live = reinterpret_cast<int*>(base + kOffNLive);
   c.d_status = reinterpret_cast<unsigned*>(base + kOffStatus);
   c.d_apps = reinterpret_cast<AppEntry*>(base + kOffApp);
   c.d_gates = reinterpret_cast<GateEntry*>(base + kOffGate);     // never read: the app entry carries no gate flag
@@ -243,7 +240,7 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
     su.edit_val[i] = app->val[i];
     su.edit_mode[i] = app->mode[i];
   }
-  static_setup_kernel<<<1, 128, 0, s>>>(su, c.d_token_slot, c.d_n_live, c.d_status, c.d_apps, c.d_groups, c.d_edit_idx,
+  static_setup_kernel<<<1, 128, 0, s>>>(su, c.d_token_slot, c.d_status, c.d_apps, c.d_groups, c.d_edit_idx,
                                         c.d_edit_val, c.d_edit_mode);
   cudaError_t e = cudaGetLastError();
   __nv_bfloat16* h = static_cast<__nv_bfloat16*>(hidden);
