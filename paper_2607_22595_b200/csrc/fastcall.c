@@ -109,7 +109,7 @@ static PyObject* fast_set_slot_map(PyObject* self, PyObject* const* a, Py_ssize_
   if (!ok2) return PyErr_Format(PyExc_AssertionError, "token_slot must be a contiguous int32 tensor");
   const int cuda = flag(a[1], s_is_cuda, 0);
   if (cuda < 0 || data_ptr(a[1], &src) < 0) return NULL;
-  if (number(a[2] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Long(a[2]), &T) < 0) return NULL;
+  if (number(a[2] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Index(a[2]), &T) < 0) return NULL;
   if (stream_of(a[3], &stream) < 0) return NULL;
   int rc;
   Py_BEGIN_ALLOW_THREADS
@@ -127,7 +127,7 @@ static PyObject* fast_set_request_map(PyObject* self, PyObject* const* a, Py_ssi
   if (context(a[0], &c) < 0) return NULL;
   const int cuda = flag(a[1], s_is_cuda, 0);
   if (cuda < 0 || data_ptr(a[1], &req) < 0 || data_ptr(a[2], &slots) < 0) return NULL;
-  if (number(a[3] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Long(a[3]), &T) < 0) return NULL;
+  if (number(a[3] == Py_None ? PyObject_CallMethodNoArgs(a[1], s_numel) : PyNumber_Index(a[3]), &T) < 0) return NULL;
   if (number(PyObject_CallMethodNoArgs(a[2], s_numel), &n_req) < 0) return NULL;
   if (stream_of(a[4], &stream) < 0) return NULL;
   int rc;

@@ -1,5 +1,6 @@
-"""The calls of a step let other Python threads run while they are in the library: a launch into a full queue, or a copy
-from pageable memory, may wait for as long as the stream does."""
+"""The CPython module of a step's calls, against a library that only waits.  The calls let other Python threads run while they
+are in the library (a launch into a full queue, or a copy from pageable memory, may wait for as long as the stream does), and
+refuse what ctypes refused."""
 import importlib.util
 import os
 import shutil
@@ -8,6 +9,7 @@ import sysconfig
 import threading
 import time
 
+import numpy as np
 import pytest
 
 from paper_2607_22595_b200 import _build
@@ -83,3 +85,13 @@ def test_other_threads_run_during_a_call(fastcall, name):
     assert end - start >= 0.3
     # 60 ticks fit into the call; without the GIL's release there is at most one, at either end
     assert sum(start + 0.01 < t < end - 0.01 for t in ticks) >= 5
+
+
+@pytest.mark.parametrize("T_live", [3.7, "3", [3]])
+def test_a_live_count_is_a_whole_number(fastcall, T_live):
+    import torch
+    with pytest.raises(TypeError):
+        fastcall.set_slot_map(1, Tensor(torch.int32, 7), T_live, 16)
+    with pytest.raises(TypeError):
+        fastcall.set_request_map(1, Tensor(torch.int32, 7), Tensor(torch.int32, 5), T_live, 16)
+    assert fastcall.set_slot_map(1, Tensor(torch.int32, 7), np.int32(3), 16) == 3
