@@ -99,15 +99,24 @@ int check_slot(mix_ctx* c, int slot) {
   return MIX_OK;
 }
 
-// The address under which the device reads host memory, or null where it cannot (pageable memory).  Asked anew on
-// every call (0.2 us): the same address may be pageable memory the next time.
-const int* device_view(const int* host) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return at.type == cudaMemoryTypeUnregistered ? nullptr : static_cast<const int*>(at.devicePointer);
+// The address under which the device reads `n` words of host memory, or null where it cannot (pageable memory).  Asked anew on
+// every call (0.2 us): the same address may be pageable memory the next time.  Of memory that is registered in part a kernel
+// would fault on the rest, so the last byte is asked about too if it lies on another page (pages are what is registered).
+const int* device_view(const int* host, int n) {
+  auto view = [](const char* p) -> const char* {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return at.type == cudaMemoryTypeUnregistered ? nullptr : static_cast<const char*>(at.devicePointer);
+  };
+  const char* first = reinterpret_cast<const char*>(host);
+  const size_t last = (size_t)n * sizeof(int) - 1;
+  const char* seen = view(first);
+  const bool one_page = (reinterpret_cast<uintptr_t>(first) ^ reinterpret_cast<uintptr_t>(first + last)) >> 12 == 0;
+  if (seen && !one_page && view(first + last) != seen + last) return nullptr;
+  return reinterpret_cast<const int*>(seen);
 }
 
 // The capture that the stream takes part in; 0: none.
@@ -723,7 +732,10 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   const bool capturing = capture != 0;
   const int n_fill = map_fill(c, T_live, capturing);
   const bool by_kernel = c->cfg.n_groups_max == 0;
-  const int* src = (src_is_device || T_live == 0) ? token_slot : (by_kernel ? device_view(token_slot) : nullptr);
+  // where a kernel can read the map (a copy takes words that do not lie on 4 bytes too)
+  const int* src = token_slot;
+  if (T_live > 0 && !src_is_device) src = by_kernel ? device_view(token_slot, T_live) : nullptr;
+  if (T_live > 0 && (reinterpret_cast<uintptr_t>(token_slot) & 3u)) src = nullptr;
   // Where there are few hooks a short map goes by a copy, which does not hold up the launch of a graph behind it; a row of
   // hooks and longer maps go by the kernel, whose start and end cost less than a copy's.  Maps and replay, 8 ... 256 rows, one
   // after the other, copy against kernel: one hook 5.4 ... 6.2 and 8.2 us, two 11.2 ... 12.3 and 10.6 ... 12.3, three 16.4 ...
@@ -740,16 +752,17 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
     c->map_live = T_live;
     return MIX_OK;
   }
-  if (by_kernel && !by_copy && !capturing && T_live <= kMapParamRows) {     // (a captured install reads its source when it is replayed)
+  if (by_kernel && !by_copy && !capturing && !src_is_device && T_live <= kMapParamRows) {     // (a captured install reads its source when it is replayed)
     map_by_kernel(c, s, capture);
     MIX_CUDA(c, launch_install_map_params(c, token_slot, T_live, n_fill, s));
     c->map_live = T_live;
     return MIX_OK;
   }
-  MIX_CUDA(c, cudaMemcpyAsync(c->d_token_slot, token_slot, (size_t)T_live * sizeof(int), cudaMemcpyHostToDevice, s));
-  map_arrived(c, s, capture);       // (a copy is complete before anything behind it starts)
+  MIX_CUDA(c, cudaMemcpyAsync(c->d_token_slot, token_slot, (size_t)T_live * sizeof(int),
+                              src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+  map_arrived(c, s, capture);       // (a copy from the host is complete before anything behind it starts)
+  if (n_fill > T_live || src_is_device) map_by_kernel(c, s, capture);   // (a memset, and a copy inside the device, may be kernels)
   if (n_fill > T_live) {
-    map_by_kernel(c, s, capture);
     MIX_CUDA(c, cudaMemsetAsync(c->d_token_slot + T_live, 0xff, (size_t)(n_fill - T_live) * sizeof(int), s));
   }
   c->map_live = T_live;

@@ -206,3 +206,51 @@ def test_pinned_maps_of_a_row_of_hooks(hooks, live):
             assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), n
     for m in ms:
         m.destroy()
+
+
+def _installs(m, T, live, ptr, src_is_device, slots):
+    stream = torch.cuda.current_stream().cuda_stream
+    assert m.lib.mix_set_slot_map(m.ctx, ptr, live, src_is_device, stream) == 0
+    h = torch.zeros((T, 64), device="cuda", dtype=torch.bfloat16)
+    m.apply(h)
+    want = np.zeros(T, dtype=np.float32)
+    want[:live] = slots + 1.0
+    assert np.array_equal(h[:, 0].float().cpu().numpy(), want)
+
+
+# sources that a copy takes and a kernel cannot read
+@pytest.mark.parametrize("with_sae", [False, True])
+@pytest.mark.parametrize("live", [3, 700, 1000])
+def test_maps_that_do_not_lie_on_four_bytes(live, with_sae):
+    T = 1000
+    m = Mix(d_model=64, T_max=T, n_slots_max=2, n_groups_max=int(with_sae), d_sae_max=256 if with_sae else 0)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(64, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+    slots = np.random.default_rng(live).integers(-1, 2, live).astype(np.int32)
+    raw = torch.zeros(4 * live + 4, dtype=torch.uint8)
+    raw[1:4 * live + 1] = torch.from_numpy(slots.view(np.uint8))
+    for where, src_is_device in ((raw.cuda(), 1), (raw.pin_memory(), 0), (raw, 0)):
+        m.set_slot_map(torch.zeros(T, dtype=torch.int32, device="cuda"), T)
+        _installs(m, T, live, where.data_ptr() + 1, src_is_device, slots)
+    assert m.get_status() == 0
+    m.destroy()
+
+
+def test_a_map_in_memory_that_is_registered_in_part():
+    T = live = 700
+    m = Mix(d_model=64, T_max=T, n_slots_max=2)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(64, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+    slots = np.random.default_rng(1).integers(-1, 2, live).astype(np.int32)
+    memory = np.zeros(4 * 4096, dtype=np.uint8)
+    page = -memory.ctypes.data % 4096                # the first page in it is registered, the second is not
+    start = page + 4096 - 4 * 100
+    memory[start:start + 4 * live] = slots.view(np.uint8)
+    cudart = torch.cuda.cudart()
+    assert int(cudart.cudaHostRegister(memory.ctypes.data + page, 4096, 0)) == 0
+    try:
+        _installs(m, T, live, memory.ctypes.data + start, 0, slots)
+        torch.cuda.synchronize()
+    finally:
+        cudart.cudaHostUnregister(memory.ctypes.data + page)
+    m.destroy()
