@@ -448,6 +448,7 @@ int mix_register_sae_weights(mix_ctx* c, int group, const mix_sae_weights* w, vo
   const bool fp8 = (c->cfg.flags & MIX_FLAG_FP8_W_ENC) != 0;
   if (fp8 && (!w->W_enc_scale || w->center_input))
     MIX_FAIL(c, MIX_ERR_INVALID_ARG, "an 8-bit encoder needs W_enc_scale and does not take center_input");
+  if (fp8 && !aligned16(w->W_enc_scale)) MIX_FAIL(c, MIX_ERR_INVALID_ARG, "weight pointers must be 16-byte aligned");   // (read four at a time)
   // Replacing a weight set: the edit lists of the apps attached to it were range-checked against the old
   // d_sae and index W_enc / W_dec rows on the device, so the new set must still cover every edited feature.
   for (int sl = 0; sl < c->cfg.n_slots_max; ++sl) {

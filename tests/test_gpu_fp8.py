@@ -114,6 +114,17 @@ def test_fp8_api_errors():
     m.destroy()
 
 
+def test_an_unaligned_scale_is_refused():
+    mixlib = _mixlib()
+    m = mixlib.Mix(d_model=128, T_max=8, n_slots_max=1, n_groups_max=1, k_max=4, r_max=1, d_sae_max=256, flags=mixlib.MIX_FLAG_FP8_W_ENC)
+    g = torch.Generator(device=DEV); g.manual_seed(0)
+    sae = W.make_sae_weights(g, DEV, 128, 256, W.SAE_TOPK, k=4, fp8=True)
+    with pytest.raises(mixlib.MixError) as e:
+        m.register_sae_weights(0, 256, sae.act, 4, sae.W_enc, sae.b_enc, sae.W_dec, w_scale=torch.ones(257, device=DEV)[1:])
+    assert e.value.code == -1
+    m.destroy()
+
+
 def test_fp8_sae_heavy_full_size_sampled_rows():
     w = W.make_sae_heavy(DEV, edit_hint=oracle_edit_hint, fp8=True)
     out = run_gpu(w, flags=_mixlib().MIX_FLAG_FP8_W_ENC, graph=True)
