@@ -1,4 +1,4 @@
-"""Thin ctypes binding of libmix.so: argument marshalling only.
+"""Thin binding of libmix.so: argument marshalling only, by ctypes for set-up and by a CPython module for the calls of a step.
 
 Every step of the hook runs in the CUDA kernels behind the C ABI (include/mix.h); this
 module turns torch tensors into device pointers and checks return codes.  There is no CPU

@@ -393,7 +393,8 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
   // Programmatic dependent launch (`pdl`: the launch asked for it): everything up to pdl_wait() reads only
-  // tables the LIBRARY owns and that only copies write -- slot map, app entry, vector arena -- so it
+  // tables the LIBRARY owns -- slot map, app entry, vector arena; copies write them, which are complete before a kernel
+  // behind them starts, and, the map alone, kernels (see below) -- so it
   // may run while the kernel in front of this one in the stream (the layer that produces `hidden`, or the
   // previous hook) is still running.  Memory the caller owns (`hidden`, multi-class probe weights, gate scores)
   // is read after the wait only, and every thread waits before it leaves, so that this grid cannot end -- and
@@ -600,9 +601,9 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
   constexpr int NT = kChainWarps * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
-  // programmatic dependent launch, as in probe_steer_team_kernel: the slot id (library-owned,
-  // written only by copies) may be read while the predecessor still runs; everything else comes after the wait,
-  // and every thread waits before it leaves
+  // programmatic dependent launch, as in probe_steer_team_kernel: the slot id (library-owned) may be read while the
+  // predecessor still runs, unless a kernel has just installed the map; everything else comes after the wait, and every
+  // thread waits before it leaves
   if (pdl == kPdlMapAhead) pdl_wait();
   pdl_launch_dependents();
   int slot = __ldg(token_slot + t);

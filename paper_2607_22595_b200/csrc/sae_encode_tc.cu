@@ -3,9 +3,9 @@
 //   Z[p, j] = sum_i panel[p, i] * W_enc[j, i] + b_eff[j]        bf16 x bf16 -> fp32
 //
 // One persistent CTA per SM walks a device-built tile schedule (group, feature tile, row tile).
-// Warp roles:  warp 0 = TMA producer (panel tile 128x64 and W_enc tile 256x64 per k-block into
-// a 4-stage ring of 128-byte-swizzled shared memory), warp 1 = MMA issuer (tcgen05.mma
-// 128x256x16, fp32 accumulators in tensor memory, double buffered so the epilogue of one tile
+// Warp roles:  warp 0 = TMA producer (panel tile 128x64 and W_enc tile 256x64 -- or 128x64, 64x64 where a call has few
+// tiles -- per k-block into a ring of 128-byte-swizzled shared memory: TcCfg::kStages of full-width tiles, up to kMaxStages
+// of narrower ones), warp 1 = MMA issuer (tcgen05.mma 128x256x16, fp32 accumulators in tensor memory, double buffered so the epilogue of one tile
 // overlaps the main loop of the next), warps 2..9 = epilogue, two per tensor-memory lane quarter
 // with 128 columns of the tile each (tcgen05.ld, + bias -- the warp's columns of it copied to shared
 // memory before the accumulator is waited for -- then either

@@ -2,10 +2,11 @@
 //
 // Routing is integer work on the slot map: which rows carry an SAE app, of which weight set, and where each of
 // them goes in the packed panel (weight set by weight set, ascending token order inside a set, every set
-// starting on a 128-row tile).  The kernel does it as a chunked scan inside one grid -- every CTA classifies 256
-// token rows and publishes their counts, every CTA then reads the small count table -- and packs the rows right
-// after, each CTA the eight panel rows it owns, found through the published per-row records.  The only waiting
-// between CTAs is a bounded wait for the published chunks; see front_kernel.
+// starting on a 128-row tile).  Calls of up to kFrontLocal chunks of 256 token rows route without an exchange: every CTA
+// classifies all rows for itself.  Longer ones do it as a chunked scan inside one grid -- every CTA classifies 256
+// token rows and publishes their counts, every CTA then reads the small count table.  Either way the rows are packed right
+// after, each CTA the eight panel rows it owns, found through its own classification or the published per-row records.
+// The only waiting between CTAs is a bounded wait for the published chunks; see front_kernel.
 //
 // Pack forms: the bf16 row as it is; with an 8-bit encoder the row as E4M3 codes with a power-of-two row
 // scale -- quantised (MIX_FLAG_FP8_ACT), or split exactly into two E4M3 operands hi + lo.

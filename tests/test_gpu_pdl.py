@@ -95,7 +95,7 @@ def test_back_to_back_hooks_accumulate_identically():
 
 def test_request_map_composed_by_a_kernel_is_seen_by_the_next_hook():
     """mix_set_request_map composes the slot map with a kernel; the hook enqueued right behind it must see the new
-    map (the library launches that one hook the ordinary way: the map is then not a table only copies write)."""
+    map (that hook is launched early too, but waits for the kernel in front before it reads anything)."""
     mixlib = _mixlib()
     w = W.make_decode(DEV)
     m = W.make_context(mixlib.Mix, w)
