@@ -28,16 +28,21 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPStages = 4;
 constexpr int kPABytes = kTileM * kTileK * 2;          // 16 KiB: 128 rows x 64 columns of hidden
 constexpr int kPBlockCols = 32;                        // accumulator columns per probe (= most classes taken)
 // Probes side by side in one pass over the tile.  Batches of short requests have many probes in a tile, and every further
-// pass streams it again; eight leave room for four stages, which stream as fast as nine did with two (32768 rows of
-// d = 4096: 67 us either way; 11111 rows of 8 probes in requests of 16 tokens: 147 -> 68 us).
+// pass streams it again (11111 rows of 8 probes in requests of 16 tokens: 147 us with two a pass, 68 with eight).
 constexpr int kPBlocks = 8;
 constexpr int kPBlockBytes = kPBlockCols * kTileK * 2; // 4 KiB: 32 classes x 64 columns
-constexpr int kPBBytes = kPBlocks * kPBlockBytes;      // 32 KiB
-constexpr int kPStageBytes = kPABytes + kPBBytes;
+// The ring is cut by the pass: nine stages for one or two probes -- what a tile of long requests has -- and four for more.
+// Bound by the bytes of `hidden` in flight.
+struct PRing {
+  int n_stages, stage_bytes;
+};
+constexpr PRing kPNarrow = {9, kPABytes + 2 * kPBlockBytes}, kPWide = {4, kPABytes + kPBlocks * kPBlockBytes};
+constexpr int kPNarrowBlocks = 2, kPMostStages = 9;
+constexpr int kPRingBytes = 216 * 1024;
+static_assert(kPNarrow.n_stages * kPNarrow.stage_bytes <= kPRingBytes && kPWide.n_stages * kPWide.stage_bytes <= kPRingBytes, "the ring");
 constexpr int kPThreads = 7 * 32;
 constexpr int kPTmemCols = 2 * kPBlocks * kPBlockCols; // 512: two accumulators of 256 columns
 constexpr long long kPWaitCycles = 4000000000ll;       // ~2 s at 2 GHz
@@ -54,8 +59,8 @@ struct PDesc {
 };
 
 struct __align__(8) PShared {
-  unsigned long long full[kPStages];
-  unsigned long long empty[kPStages];
+  unsigned long long full[kPMostStages];
+  unsigned long long empty[kPMostStages];
   unsigned long long tmem_full[2];
   unsigned long long tmem_empty[2];
   unsigned long long desc_full[2];
@@ -64,8 +69,9 @@ struct __align__(8) PShared {
   volatile int abort_flag;
   long long wait_cycles;        // cap of every bounded wait in this launch
   PDesc desc[2];
+  int pass_slot[kPBlocks];      // the producer's own copy of its pass's probes
 };
-constexpr int kPSmemBytes = kPStages * kPStageBytes + 1024 /* alignment slack */ + 1024 /* PShared */;
+constexpr int kPSmemBytes = kPRingBytes + 1024 /* alignment slack */ + 1024 /* PShared */;
 static_assert(kPSmemBytes <= 227 * 1024, "shared memory per CTA");
 static_assert(sizeof(PShared) <= 1024, "PShared must fit the space reserved for it");
 
@@ -103,7 +109,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
                 const int* __restrict__ census_tiles, float* __restrict__ part_logits, int* __restrict__ part_done, int test_stall) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  PShared* sh = reinterpret_cast<PShared*>(tiles + kPStages * kPStageBytes);
+  PShared* sh = reinterpret_cast<PShared*>(tiles + kPRingBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the tiles of this call that hold multi-class probe rows, as the census listed them (in no particular order):
   // CTAs share THEM out, so a batch whose hooked requests are clustered still spreads evenly over the SMs
@@ -113,7 +119,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
   const int n_parts = column_parts(n_tiles, num_kb, gridDim.x), n_items = n_tiles * n_parts;
   if ((int)blockIdx.x >= n_items) return;              // CTA-uniform: this CTA has no work
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kPStages; ++s) {
+    for (int s = 0; s < kPMostStages; ++s) {
       mbar_init(smem_u32(&sh->full[s]), 1);
       mbar_init(smem_u32(&sh->empty[s]), 1);
     }
@@ -214,32 +220,39 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
     // ---- producer
     if (lane == 0) {
       int di = 0, stage = 0;
-      unsigned dphase = 0, phase = 0;
+      unsigned dphase = 0, phases = 0;                 // bit s: parity of stage s's next use
+      PRing ring = kPNarrow;
       for (;;) {
         if (!pwait(smem_u32(&sh->desc_full[di]), dphase, sh, status)) break;
         const PDesc* ds = &sh->desc[di];
-        const int nb = ds->n_blocks, t0 = ds->t0, kb0 = ds->kb0, kb1 = ds->kb1;
-        int slot[kPBlocks];
-#pragma unroll
-        for (int b = 0; b < kPBlocks; ++b) slot[b] = ds->slot[b];
+        const int nb = ds->n_blocks, t0 = ds->t0, kb0 = ds->kb0, kb1 = ds->kb1, slot0 = ds->slot[0];
+        for (int b = 1; b < nb; ++b) sh->pass_slot[b] = ds->slot[b];
         mbar_arrive(smem_u32(&sh->desc_empty[di]));    // everything this role needs has been copied out
         di ^= 1;
         if (di == 0) dphase ^= 1u;
         if (nb == 0) break;
         bool ok = true;
+        const PRing cut = nb > kPNarrowBlocks ? kPWide : kPNarrow;
+        if (cut.n_stages != ring.n_stages) {           // cut anew: only when every stage of the old cut is free
+          for (int s = 0; s < ring.n_stages && ok; ++s) ok = pwait(smem_u32(&sh->empty[s]), ((phases >> s) & 1u) ^ 1u, sh, status);
+          if (!ok) break;
+          ring = cut;
+          stage = 0;
+        }
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!pwait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
+          if (!pwait(smem_u32(&sh->empty[stage]), ((phases >> stage) & 1u) ^ 1u, sh, status)) { ok = false; break; }
           // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumers' bounded
           // waits run out and the whole CTA leaves through the time-out path.
           if (test_stall) { ok = false; break; }
           const unsigned bar = smem_u32(&sh->full[stage]);
           mbar_expect_tx(bar, kPABytes + nb * kPBlockBytes);
-          const unsigned sa = smem_u32(tiles + stage * kPStageBytes);
+          const unsigned sa = smem_u32(tiles + stage * ring.stage_bytes);
           tma_load_2d(sa, &tmap_hidden, kb * kTileK, t0, bar);
-#pragma unroll
-          for (int b = 0; b < kPBlocks; ++b)
-            if (b < nb) tma_load_2d(sa + kPABytes + b * kPBlockBytes, tmap_probe + slot[b], kb * kTileK, 0, bar);
-          if (++stage == kPStages) { stage = 0; phase ^= 1u; }
+          tma_load_2d(sa + kPABytes, tmap_probe + slot0, kb * kTileK, 0, bar);
+          for (int b = 1; b < nb; ++b)
+            tma_load_2d(sa + kPABytes + b * kPBlockBytes, tmap_probe + sh->pass_slot[b], kb * kTileK, 0, bar);
+          phases ^= 1u << stage;
+          if (++stage == ring.n_stages) stage = 0;
         }
         if (!ok) break;
       }
@@ -248,7 +261,8 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
     // ---- MMA issuer
     if (lane == 0) {
       int di = 0, stage = 0;
-      unsigned dphase = 0, phase = 0, acc = 0, acc_phase = 0;
+      unsigned dphase = 0, phases = 0, acc = 0, acc_phase = 0;
+      PRing ring = kPNarrow;
       for (;;) {
         if (!pwait(smem_u32(&sh->desc_full[di]), dphase, sh, status)) break;
         const int nb = sh->desc[di].n_blocks, kb0 = sh->desc[di].kb0, kb1 = sh->desc[di].kb1;
@@ -258,18 +272,24 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const CUtensorM
         if (nb == 0) break;
         if (!pwait(smem_u32(&sh->tmem_empty[acc]), acc_phase ^ 1u, sh, status)) break;
         tc_fence_after();
+        const PRing cut = nb > kPNarrowBlocks ? kPWide : kPNarrow;
+        if (cut.n_stages != ring.n_stages) {
+          ring = cut;
+          stage = 0;
+        }
         const unsigned d_tmem = tmem_base + acc * (kPBlocks * kPBlockCols);
         const unsigned idesc = idesc_f16(kTileM, nb * kPBlockCols);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!pwait(smem_u32(&sh->full[stage]), phase, sh, status)) { ok = false; break; }
+          if (!pwait(smem_u32(&sh->full[stage]), (phases >> stage) & 1u, sh, status)) { ok = false; break; }
           tc_fence_after();
-          const unsigned sa = smem_u32(tiles + stage * kPStageBytes);
+          const unsigned sa = smem_u32(tiles + stage * ring.stage_bytes);
           const unsigned long long da = umma_desc(sa), db = umma_desc(sa + kPABytes);
 #pragma unroll
           for (int k = 0; k < kTileK / 16; ++k) umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, (unsigned)(kb != kb0 || k != 0));
           umma_commit(smem_u32(&sh->empty[stage]));
-          if (++stage == kPStages) { stage = 0; phase ^= 1u; }
+          phases ^= 1u << stage;
+          if (++stage == ring.n_stages) stage = 0;
         }
         if (!ok) break;
         umma_commit(smem_u32(&sh->tmem_full[acc]));

@@ -5,13 +5,12 @@
 // One persistent CTA per SM walks a device-built tile schedule (group, feature tile, row tile).
 // Warp roles:  warp 0 = TMA producer (panel tile 128x64 and W_enc tile 256x64 -- or 128x64, 64x64 where a call has few
 // tiles -- per k-block into a ring of 128-byte-swizzled shared memory: TcCfg::kStages of full-width tiles, up to kMaxStages
-// of narrower ones), warp 1 = MMA issuer (tcgen05.mma 128x256x16, fp32 accumulators in tensor memory, double buffered so the epilogue of one tile
-// overlaps the main loop of the next), warps 2..9 = epilogue, two per tensor-memory lane quarter
-// with 128 columns of the tile each (tcgen05.ld, + bias -- the warp's columns of it copied to shared
-// memory before the accumulator is waited for -- then either
-// the fp32 pre-activations to the Z scratch, or -- for TopK weight sets -- only the tile's 8
-// largest values per row plus its 9th, which the tail kernel turns into the exact TopK; the two
-// warps of a quarter merge their lists through shared memory).
+// of narrower ones), warp 1 = MMA issuer (tcgen05.mma 128x256x16, fp32 accumulators in tensor memory, double
+// buffered so the epilogue of one tile overlaps the main loop of the next), warps 2..9 = epilogue, two per
+// tensor-memory lane quarter with 128 columns of the tile each (tcgen05.ld, + bias -- the warp's columns of it
+// copied to shared memory before the accumulator is waited for -- then either the fp32 pre-activations to the Z
+// scratch, or -- for TopK weight sets -- only the tile's 8 largest values per row plus its 9th, which the tail
+// kernel turns into the exact TopK; the two warps of a quarter merge their lists through shared memory).
 // A second form (kPair) runs on clusters of two CTAs that share a 256-row tile through
 // tcgen05.mma.cta_group::2; which form works on a call is decided on the device (see TcCfg).
 // No TMA multicast in either form.  Every wait is bounded: on expiry the CTA raises

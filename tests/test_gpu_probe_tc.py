@@ -187,3 +187,34 @@ def test_scratch_of_the_smallest_batches():
     assert bytes_of(16) - bytes_of(1) <= 5 << 20         # 17 x 8 items of 16 KiB, in pages of 2 MiB
     w = _probe_workload(T, T, d, np.arange(T) // 300 % 2, [16, 9], [W.ACT_SOFTMAX, W.ACT_NONE])
     check_parity(W.host(w), run_gpu(w))
+
+
+@pytest.mark.parametrize("d", [64, 704])
+@pytest.mark.parametrize("T", [3000, 50000])
+def test_tiles_of_few_and_of_many_probes(d, T):
+    """The ring is cut for one or two probes in a pass or for more: tiles with 1 ... 12 probes in turn, so that a CTA's passes
+    go from one cut to the other and back."""
+    g = torch.Generator(device="cuda"); g.manual_seed(d + T)
+    mixlib = _mixlib()
+    rng = np.random.default_rng(T)
+    n, C = 12, 6
+    m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=n, C_max=C)
+    Wp = (torch.randn((n, C, d), generator=g, device="cuda") * d ** -0.5).to(torch.bfloat16)
+    b = torch.randn((n, C), generator=g, device="cuda")
+    for i in range(n):
+        m.register_probe(i, Wp[i], b[i], mixlib.MIX_ACT_SOFTMAX)
+    slot = np.empty(T, np.int32)
+    for t in range(0, T, 128):
+        some = rng.permutation(n)[:rng.choice([1, 1, 2, 3, 8, 9, 10, 12])]
+        slot[t:t + 128] = rng.choice(some, size=128)[:T - t]
+    slot = torch.from_numpy(slot).cuda()
+    m.set_slot_map(slot)
+    for _ in range(2):
+        hidden = torch.randn((T, d), generator=g, device="cuda").to(torch.bfloat16)
+        scores = torch.full((T, C), -1.0, device="cuda")
+        m.apply(hidden, scores)
+        logits = torch.einsum("td,scd->tsc", hidden.double(), Wp.double())[torch.arange(T, device="cuda"), slot.long()] + b.double()[slot.long()]
+        want = torch.softmax(logits, dim=1)
+        assert ((scores.double() - want).abs() <= 1e-3 * want).all()
+    assert m.get_status() == 0
+    m.destroy()
