@@ -6,8 +6,8 @@
 // nothing, the job is to stream `hidden` from HBM once, at HBM speed.  That is what the TMA ->
 // tcgen05 pipeline of the SAE encode is good at, so the same machinery is used: one persistent CTA
 // per SM; warp 0 = TMA producer (a 128 x 64 tile of `hidden`, straight from the caller's tensor, and
-// a 32 x 64 tile of each probe matrix that occurs in the tile, per k-block, into a 4-stage ring:
-// 64 KiB of `hidden` in flight per SM without holding a single register), warp 1 = MMA issuer
+// a 32 x 64 tile of each probe matrix that occurs in the tile, per k-block, into a ring of
+// eight stages, or four where many probes meet: 128 or 64 KiB of `hidden` in flight per SM without holding a register), warp 1 = MMA issuer
 // (M = 128, N = 32 per distinct probe of the tile, up to 8 probes side by side, fp32 accumulators
 // in tensor memory, double buffered), warps 2..5 = epilogue (one lane per row: its probe's 32
 // columns, + bias, softmax / sigmoid / identity, scores out), warp 6 = scout (reads the tile's slot
@@ -34,14 +34,16 @@ constexpr int kPBlockCols = 32;                        // accumulator columns pe
 // pass streams it again (11111 rows of 8 probes in requests of 16 tokens: 147 us with two a pass, 68 with eight).
 constexpr int kPBlocks = 8;
 constexpr int kPBlockBytes = kPBlockCols * kTileK * 2; // 4 KiB: 32 classes x 64 columns
-// The ring is cut by the pass: nine stages for one or two probes -- what a tile of long requests has -- and four for more.
-// Bound by the bytes of `hidden` in flight.
+// The ring is cut by the pass: eight stages for one or two probes -- what a tile of long requests has -- and four for more.
+// Bound by the bytes of `hidden` in flight: 65536 rows of d = 4096 in requests of 256, in the kernel, 102 us with 8 or 9 stages,
+// 115 with 4.  (192 KiB in all, not the 216 of nine stages: those leave the kernels beside this one the smallest L1, for the
+// sake of a launch that mostly returns at once -- 32768 rows, a quarter of them scattered multi-class probes: the call 110 and 140 us.)
 struct PRing {
   int n_stages, stage_bytes;
 };
-constexpr PRing kPNarrow = {9, kPABytes + 2 * kPBlockBytes}, kPWide = {4, kPABytes + kPBlocks * kPBlockBytes};
-constexpr int kPNarrowBlocks = 2, kPMostStages = 9;
-constexpr int kPRingBytes = 216 * 1024;
+constexpr PRing kPNarrow = {8, kPABytes + 2 * kPBlockBytes}, kPWide = {4, kPABytes + kPBlocks * kPBlockBytes};
+constexpr int kPNarrowBlocks = 2, kPMostStages = 8;
+constexpr int kPRingBytes = 192 * 1024;
 static_assert(kPNarrow.n_stages * kPNarrow.stage_bytes <= kPRingBytes && kPWide.n_stages * kPWide.stage_bytes <= kPRingBytes, "the ring");
 constexpr int kPThreads = 7 * 32;
 constexpr int kPTmemCols = 2 * kPBlocks * kPBlockCols; // 512: two accumulators of 256 columns
