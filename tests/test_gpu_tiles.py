@@ -234,3 +234,27 @@ def test_a_set_that_another_stream_is_about_to_remove():
     assert np.array_equal(W.bits(h), want["hidden"])
     torch.cuda.synchronize()
     m.destroy()
+
+
+def test_padding_rows_of_a_tile_are_zero():
+    """Rows of the panel behind a set's own are zeros, whatever a longer call before had there (seen through the CUDA-core
+    encode, which writes the pre-activations of whole tiles)."""
+    from cuda.bindings import runtime as rt
+
+    import paper_2607_22595_b200 as mixlib
+    S, T = 512, 200
+    w = _workload(128, S, T, W.SAE_RELU, True)
+    w.token_slot[:] = 0
+    m = W.make_context(mixlib.Mix, w, flags=mixlib.MIX_FLAG_ENCODE_SIMT)
+    h = w.hidden.clone()
+    m.apply(h)
+    m.set_slot_map(w.token_slot, 5)
+    m.apply(h)
+    torch.cuda.synchronize()
+    _, z_ptr, ld, _ = m.debug_workspace()
+    z = np.empty((128, ld), np.float32)
+    assert int(rt.cudaMemcpy(z.ctypes.data, z_ptr, z.nbytes, rt.cudaMemcpyKind.cudaMemcpyDeviceToHost)[0]) == 0
+    b = w.groups[0].b_enc.cpu().numpy()
+    assert np.array_equal(z[5:, :S], np.broadcast_to(b, (123, S)))
+    assert not np.array_equal(z[:5, :S], np.broadcast_to(b, (5, S)))
+    m.destroy()
