@@ -742,8 +742,9 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   // after the other, copy against kernel: one hook 5.4 ... 6.2 and 8.2 us, two 11.2 ... 12.3 and 10.6 ... 12.3, three 16.4 ...
   // 18.5 and 16.4, four 21.8 ... 22.6 and 20.5, sixteen 78 ... 88 and 68 ... 73; on an idle GPU 11.5 ... 13 and 15 ... 17, 16.5 and
   // 19.7, 21 ... 22 and 24.5, 26 ... 27 and 28.5, 83 ... 93 and 78 ... 85.  One hook on 512 rows 11.9 and 10.3, on 2000 rows
-  // 22.9 and 16.4.  (The count is a guess at the length of the row, from the contexts that the device has; either way
-  // installs the same map.)
+  // 22.9 and 16.4.  At three the one measure says about as much for the copy as the other against it.  (The count is a guess at
+  // the length of the row, from the contexts that the device has -- a program may have three and step through one --; either
+  // way installs the same map.)
   // As a node of a graph the kernel is never slower (two hooks: 8.3 ... 10.3 us, copies 11.7).
   const bool by_copy = src && !src_is_device && T_live <= kMapCopyRows && n_fill <= T_live && hook_contexts(c->device) <= kMapCopyHooks &&
                        !capturing;
