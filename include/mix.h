@@ -339,7 +339,7 @@ int mix_set_feature_out(mix_ctx* ctx, int* topk_idx, float* topk_val, int* n_act
    written.  Enqueues kernels on `stream` (when the context has SAE weight sets, more than 2048 rows
    and no slot chains, the probe / steering kernels run on a context-owned side stream forked from and joined back into `stream`
    by events, so they overlap the SAE chain; in a context for more than 2048 rows with multi-class
-   probes and no SAE weight sets, the tensor-core probe kernel runs on that side stream beside the
+   probes and no SAE weight sets, the two kernels for those run on two such streams beside the
    streaming kernel) and returns; safe to capture.  In a context without SAE weight sets and
    T_max <= 2048 the kernel is launched with programmatic stream serialization (see
    mix_set_pdl_mask): if the kernel in front of it in `stream` lets its successor start early, the

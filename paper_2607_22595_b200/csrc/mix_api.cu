@@ -90,6 +90,7 @@ void free_all(mix_ctx* c) {
   free(c->owned_b_eff); free(c->h_apps); free(c->h_groups); free(c->h_chain_next); free(c->h_edit_idx);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->ev_join2) cudaEventDestroy(c->ev_join2);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->body_stream) cudaStreamDestroy(c->body_stream);
 }
@@ -410,6 +411,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->body_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { free_all(c); free(c); return MIX_ERR_CUDA; }
@@ -899,8 +901,9 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // Multi-class probes of a large batch have two kernels of which exactly one does the work: the 16-row
   // kernel takes batches sparse in such rows (and every batch of a context with SAE weight sets), the
   // tensor-core kernel dense ones.  Where both exist, a census makes the choice first and both -- their rows
-  // no other kernel of this call touches -- run on the context's side stream, beside the streaming kernel's
-  // pass over the batch.
+  // no other kernel of this call touches -- run beside the streaming kernel's pass over the batch, each on a stream of
+  // its own: the 16-row kernel takes 4 ... 10 us to find that it has nothing to do, which on the other's stream came
+  // behind it (65536 rows of d = 4096 in requests of 256, called eagerly: 135 us, and 127).
   const bool tc = has_tc_probe_stage(c);
   const bool tc_fork = tc && !c->stage_events_on;
   CUtensorMap tm_hidden;                         // host-side encoding only: no device work, fine under capture
@@ -912,9 +915,11 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
     if (tc_fork) {
       MIX_CUDA(c, cudaEventRecord(c->ev_fork, ps));
       MIX_CUDA(c, cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
+      MIX_CUDA(c, cudaStreamWaitEvent(c->body_stream, c->ev_fork, 0));
       MIX_CUDA(c, launch_probe_tc(c, tm_hidden, T, scores_out, c->side_stream));
-      MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, c->side_stream));
       MIX_CUDA(c, cudaEventRecord(c->ev_join, c->side_stream));
+      MIX_CUDA(c, launch_probe_multiclass(c, h, T, scores_out, c->body_stream));
+      MIX_CUDA(c, cudaEventRecord(c->ev_join2, c->body_stream));
     }
   }
   // (programmatic launch only where this kernel directly follows the caller's work in the caller's stream)
@@ -931,7 +936,10 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
     MIX_CUDA(c, launch_probe_tc(c, tm_hidden, T, scores_out, ps));
     MIX_CUDA(c, tap());
   }
-  if (tc_fork) MIX_CUDA(c, cudaStreamWaitEvent(ps, c->ev_join, 0));
+  if (tc_fork) {
+    MIX_CUDA(c, cudaStreamWaitEvent(ps, c->ev_join, 0));
+    MIX_CUDA(c, cudaStreamWaitEvent(ps, c->ev_join2, 0));
+  }
   if (fork) MIX_CUDA(c, cudaEventRecord(c->ev_join, ps));
   if (c->cfg.n_groups_max > 0) {
     // (with slot chains a steering app may precede an SAE app on the same row: the hook kernel is in front of this one)

@@ -188,8 +188,9 @@ struct Ctx {
 
   // probe/steer kernels run beside the SAE chain on this stream (created with the context)
   cudaStream_t side_stream;
-  cudaStream_t body_stream;   // used only to record the body of a conditional node (mix_apply_conditional)
-  cudaEvent_t ev_fork, ev_join;
+  cudaStream_t body_stream;   // records the body of a conditional node (mix_apply_conditional); without weight sets, which rules
+                              // that out, the 16-row kernel for multi-class probes runs on it
+  cudaEvent_t ev_fork, ev_join, ev_join2;
 
   // profiling taps
   int stage_events_on;
