@@ -35,6 +35,18 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Four sums over the warp with 6 exchanges instead of 20; lanes 8c .. 8c + 7 return that of v[c].  (The same additions as in
+// warp_sum, hence the same bits.)
+__device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
+  const bool b16 = lane & 16, b8 = lane & 8;
+  const float a0 = (b16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, b16 ? v[0] : v[2], 16);
+  const float a1 = (b16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, b16 ? v[1] : v[3], 16);
+  float z = (b8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b8 ? a0 : a1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  return z;
+}
+
 // h + alpha v for one row; nvec = d / 8 16-byte vectors.  The `stride` threads that share the
 // row start at `first` (a warp: lane, 32; a CTA team: threadIdx.x, blockDim.x).
 __device__ __forceinline__ void steer_row(uint4* __restrict__ h, const uint4* __restrict__ v, float alpha,
@@ -379,6 +391,7 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
 // >= 0, in parallel with the app-table lookup, so a cold row costs two dependent round trips
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
 constexpr int kTeamVec = 4;     // NW * 32 * kTeamVec * 8 >= d_model: 8192 columns at NW = 8
+constexpr int kHookWarps = 8, kMostVec = kTeamVec;
 
 enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
 
@@ -590,51 +603,148 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
 // registers, exactly as a store and reload would; the row goes back to memory once, at the end,
 // if any app changed it.  The j-th probe of a chain writes its scores after those of the earlier
 // ones.  Control flow is uniform across the CTA.
-constexpr int kChainWarps = 8;
+// Bound by the chain of dependent loads: link -> entry -> gate -> score -> vector, app after app.  All of it that the
+// library owns -- links, entries, gate entries, single vectors (in the arena) -- is read ahead of the programmatic wait, into
+// shared memory, while the layer or hook in front still runs; behind the wait everything the caller owns is requested together
+// (row, gate scores, biases), and the probes' partial logits meet once, behind the last app.
+constexpr int kChainStaged = 2;      // single vectors of a chain that are staged (later ones are loaded when their turn comes)
 
-__global__ void __launch_bounds__(kChainWarps * 32)
+struct ChainStep {
+  int kind;              // 0: nothing to do
+  int C, act, col;       // col: the probe's first column in the row's scores
+  float alpha;           // (of a one-class probe with its vector in the arena: the bias)
+  int staged;            // place of the vector in shared memory, or -1
+  const uint4* W;
+  const float* b;
+  RowGate gate;
+};
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+
+// NV: 16-byte vectors of the row per thread.
+template <int NV>
+__global__ void __launch_bounds__(kHookWarps * 32)
 probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
                          const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates,
                          const int* __restrict__ chain_next, int n_slots, __nv_bfloat16* __restrict__ hidden, int d,
-                         float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int pdl) {
-  __shared__ float s_part[kChainWarps][kMaxClasses];
-  constexpr int NT = kChainWarps * 32;
+                         float* __restrict__ scores, int C_max, unsigned* __restrict__ status, int in_arena, int pdl) {
+  extern __shared__ uint4 s_vec[];               // [kChainStaged][nvec]
+  __shared__ float s_part[kHookWarps][kMaxClasses];   // partial logits of all the chain's probes, by column
+  __shared__ float s_dot[kMaxChain][kHookWarps];
+  __shared__ ChainStep s_step[kMaxChain];
+  __shared__ int s_n;
+  constexpr int NW = kHookWarps, NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
-  // programmatic dependent launch, as in probe_steer_team_kernel: the slot id (library-owned) may be read while the
+  // programmatic dependent launch, as in probe_steer_team_kernel: what the library owns may be read while the
   // predecessor still runs, unless a kernel has just installed the map; everything else comes after the wait, and every
   // thread waits before it leaves
   if (pdl == kPdlMapAhead) pdl_wait();
   pdl_launch_dependents();
-  int slot = __ldg(token_slot + t);
-  pdl_wait();
-  if (t >= T || slot == -1) return;
+  const int slot0 = __ldg(token_slot + t);
+  if (t >= T || slot0 == -1) {
+    pdl_wait();
+    return;
+  }
   const int nvec = d >> 3;
-  uint4* hrow = reinterpret_cast<uint4*>(hidden + (size_t)t * d);
-  uint4 hq[kTeamVec];
+  if (warp == 0) {                               // the row's apps, in order (every lane reads the same)
+    int slot = slot0, n = 0, col = 0, staged = 0;
+    while (n < kMaxChain) {
+      const int next = slot >= 0 && slot < n_slots ? __ldg(chain_next + slot) : -1;     // (requested with the entry)
+      const RowApp a = lookup(slot, t, apps, gates, n_slots, status, lane == 0, /*eval_gate=*/false);
+      ChainStep st;
+      st.kind = a.kind;
+      st.C = a.C;
+      st.act = a.act;
+      st.col = col;
+      st.alpha = a.alpha;
+      st.W = a.W;
+      st.b = a.b;
+      st.staged = -1;
+      if (staged < kChainStaged && (a.kind == MIX_STEER || a.kind == MIX_PROJECT || (a.kind == MIX_PROBE && a.C == 1))) st.staged = staged++;
+      st.gate.score = nullptr;
+      if (a.kind != 0 && a.gated) st.gate = load_gate(gates, slot, t);
+      if (lane == 0) s_step[n] = st;
+      ++n;
+      if (!a.chained) break;
+      if (a.raw_kind == MIX_PROBE) col += a.C;
+      slot = next;                               // (slot was in range: lookup() found a valid entry)
+      if (slot < 0) break;
+    }
+    if (lane == 0) s_n = n;
+  }
+  __syncthreads();
+  const int n = s_n;
+  // a thread stages the vectors that it will use itself, so nobody else has to know when they have arrived
+  auto stage = [&]() {
+    for (int i = 0; i < n; ++i) {
+      const int at = s_step[i].staged;
+      if (at < 0) continue;
 #pragma unroll
-  for (int u = 0; u < kTeamVec; ++u) {
+      for (int u = 0; u < NV; ++u) {
+        const int v = threadIdx.x + u * NT;
+        if (v < nvec) cp_async16(s_vec + at * nvec + v, s_step[i].W + v);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (in_arena) stage();
+  pdl_wait();
+  uint4* hrow = reinterpret_cast<uint4*>(hidden + (size_t)t * d);
+  uint4 hq[NV];
+#pragma unroll
+  for (int u = 0; u < NV; ++u) {
     const int v = threadIdx.x + u * NT;
     hq[u] = make_uint4(0u, 0u, 0u, 0u);
-    if (v < nvec && slot >= 0 && slot < n_slots) hq[u] = __ldcs(hrow + v);
+    if (v < nvec) hq[u] = __ldcs(hrow + v);
   }
-  bool dirty = false;
-  int col = 0;
-  for (int depth = 0; depth < kMaxChain; ++depth) {
-    const RowApp a = lookup(slot, t, apps, gates, n_slots, status, threadIdx.x == 0);
-    if ((a.kind == MIX_STEER || a.kind == MIX_PROJECT) && a.alpha != 0.f) {   // alpha = 0: identity, bit-exact
-      uint4 vq[kTeamVec];
+  if (!in_arena) stage();
+  float score[kMaxChain];                        // (all requested before one is looked at)
 #pragma unroll
-      for (int u = 0; u < kTeamVec; ++u) {
+  for (int i = 0; i < kMaxChain; ++i) {
+    score[i] = 0.f;
+    if (i < n && s_step[i].gate.score != nullptr) score[i] = __ldg(s_step[i].gate.score);
+  }
+  float bias_lo = 0.f, bias_hi = 0.f;            // of the probe that this warp will finish
+  if (warp < n && s_step[warp].kind == MIX_PROBE) {
+    const ChainStep& st = s_step[warp];
+    if (in_arena && st.C == 1) {
+      bias_lo = st.alpha;
+    } else if (st.b != nullptr) {
+      if (lane < st.C) bias_lo = __ldg(st.b + lane);
+      if (lane + 32 < st.C) bias_hi = __ldg(st.b + lane + 32);
+    }
+  }
+  unsigned open = 0u;                            // (a closed gate skips its app, not the chain behind it)
+#pragma unroll
+  for (int i = 0; i < kMaxChain; ++i)
+    if (i < n && s_step[i].kind != 0 && (s_step[i].gate.score == nullptr || gate_passes(s_step[i].gate, score[i]))) open |= 1u << i;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  bool dirty = false;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    if (!((open >> i) & 1u)) continue;
+    const ChainStep& st = s_step[i];
+    const int kind = st.kind;
+    const bool single = kind == MIX_STEER || kind == MIX_PROJECT || (kind == MIX_PROBE && st.C == 1);
+    if ((kind == MIX_STEER || kind == MIX_PROJECT) && st.alpha == 0.f) continue;     // identity, bit-exact
+    if (kind == MIX_PROBE && scores == nullptr) continue;
+    if (single) {
+      uint4 vq[NV];
+      const uint4* src = st.staged >= 0 ? s_vec + st.staged * nvec : st.W;
+#pragma unroll
+      for (int u = 0; u < NV; ++u) {
         const int v = threadIdx.x + u * NT;
         vq[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (v < nvec) vq[u] = __ldg(a.W + v);
+        if (v < nvec) vq[u] = src[v];
       }
-      float coef = a.alpha;
-      if (a.kind == MIX_PROJECT) {               // h - beta (h . r) r
+      float coef = st.alpha;
+      if (kind != MIX_STEER) {
         float dot = 0.f;
 #pragma unroll
-        for (int u = 0; u < kTeamVec; ++u) {
+        for (int u = 0; u < NV; ++u) {
           float x[8], y[8];
           unpack8(hq[u], x);
           unpack8(vq[u], y);
@@ -642,15 +752,19 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
           for (int e = 0; e < 8; ++e) dot = fmaf(x[e], y[e], dot);
         }
         dot = warp_sum(dot);
-        if (lane == 0) s_part[warp][0] = dot;
+        if (kind == MIX_PROBE) {
+          if (lane == 0) s_part[warp][st.col] = dot;
+          continue;
+        }
+        if (lane == 0) s_dot[i][warp] = dot;     // h - beta (h . r) r
         __syncthreads();
         float total = 0.f;
 #pragma unroll
-        for (int w = 0; w < kChainWarps; ++w) total += s_part[w][0];
-        coef = -a.alpha * total;
+        for (int w = 0; w < NW; ++w) total += s_dot[i][w];
+        coef = -st.alpha * total;
       }
 #pragma unroll
-      for (int u = 0; u < kTeamVec; ++u) {
+      for (int u = 0; u < NV; ++u) {
         float x[8], y[8];
         unpack8(hq[u], x);
         unpack8(vq[u], y);
@@ -659,12 +773,23 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
         hq[u] = pack8(x);
       }
       dirty = true;
-    } else if (a.kind == MIX_PROBE && scores != nullptr) {
-      for (int c0 = 0; c0 < a.C; c0 += 4) {
-        const int nc = min(4, a.C - c0);
+    } else if (kind == MIX_PROBE) {
+      const int C = st.C, col = st.col;
+      const uint4* W = st.W;
+#pragma unroll 1
+      for (int c0 = 0; c0 < C; c0 += 4) {
+        const int nc = min(4, C - c0);
+        uint4 wq[4][NV];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int u = 0; u < NV; ++u) {
+            const int v = threadIdx.x + u * NT;
+            if (c < nc && v < nvec) wq[c][u] = __ldg(W + (size_t)(c0 + c) * nvec + v);
+          }
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int u = 0; u < kTeamVec; ++u) {
+        for (int u = 0; u < NV; ++u) {
           const int v = threadIdx.x + u * NT;
           if (v < nvec) {
             float x[8];
@@ -673,42 +798,35 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
             for (int c = 0; c < 4; ++c)
               if (c < nc) {
                 float y[8];
-                unpack8(__ldg(a.W + (size_t)(c0 + c) * nvec + v), y);
+                unpack8(wq[c][u], y);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) acc[c] = fmaf(x[e], y[e], acc[c]);
               }
           }
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float z = warp_sum(acc[c]);
-          if (lane == 0 && c < nc) s_part[warp][c0 + c] = z;
-        }
-      }
-      __syncthreads();
-      if (warp == 0) {
-        for (int c = lane; c < a.C; c += 32) {
-          float z = a.b ? __ldg(a.b + c) : 0.f;
-#pragma unroll
-          for (int w = 0; w < kChainWarps; ++w) z += s_part[w][c];
-          s_part[0][c] = z;            // only this lane reads or writes column c from here on
-        }
-        __syncwarp();
-        finish_probe(s_part[0], a.C, a.act, scores + (size_t)t * C_max + col, lane);
+        const float z = warp_sum4(acc, lane);
+        if ((lane & 7) == 0 && (lane >> 3) < nc) s_part[warp][col + c0 + (lane >> 3)] = z;
       }
     }
-    if (!a.chained) break;
-    if (a.raw_kind == MIX_PROBE) col += a.C;
-    slot = __ldg(chain_next + slot);             // slot was in range: lookup() found a valid entry
-    if (slot < 0) break;
-    __syncthreads();                             // s_part is reused by the next app
   }
   if (dirty) {
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) __stcs(hrow + v, hq[u]);
     }
+  }
+  __syncthreads();
+  if (scores != nullptr && warp < n && ((open >> warp) & 1u) && s_step[warp].kind == MIX_PROBE) {       // a warp per probe
+    const ChainStep& st = s_step[warp];
+    for (int c = lane; c < st.C; c += 32) {
+      float z = c < 32 ? bias_lo : bias_hi;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) z += s_part[w][st.col + c];
+      s_part[0][st.col + c] = z;     // only this lane reads or writes the column from here on
+    }
+    __syncwarp();
+    finish_probe(&s_part[0][st.col], st.C, st.act, scores + (size_t)t * C_max + st.col, lane);
   }
 }
 
@@ -872,10 +990,19 @@ bool has_tc_probe_stage(const Ctx* c) { return has_multiclass_stage(c) && c->cfg
 
 cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float* scores, cudaStream_t s, bool allow_pdl, bool map_ahead) {
   const int pdl = (allow_pdl && (pdl_mask() & kPdlHook)) ? (map_ahead ? kPdlMapAhead : 1) : 0;
+  const int nvec = c->cfg.d_model / 8, n_vec = (nvec + kHookWarps * 32 - 1) / (kHookWarps * 32);     // n_vec: per thread
   if (c->cfg.flags & MIX_FLAG_SLOT_CHAINS) {
-    return launch_pdl(allow_pdl ? kPdlHook : 0, probe_steer_chain_kernel, dim3(c->cfg.T_max), dim3(kChainWarps * 32), 0, s,
-                      c->d_token_slot, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
-                      c->cfg.d_model, scores, c->cfg.C_max, c->d_status, pdl);
+    auto run = [&](auto kernel) {
+      return launch_pdl(allow_pdl ? kPdlHook : 0, kernel, dim3(c->cfg.T_max), dim3(kHookWarps * 32), (size_t)kChainStaged * nvec * sizeof(uint4), s,
+                        c->d_token_slot, T, c->d_apps, c->d_gates, c->d_chain_next, c->cfg.n_slots_max, hidden,
+                        c->cfg.d_model, scores, c->cfg.C_max, c->d_status, c->d_vec_arena != nullptr ? 1 : 0, pdl);
+    };
+    switch (n_vec) {
+      case 1: return run(probe_steer_chain_kernel<1>);
+      case 2: return run(probe_steer_chain_kernel<2>);
+      case 3: return run(probe_steer_chain_kernel<3>);
+      default: return run(probe_steer_chain_kernel<kMostVec>);
+    }
   } else if (c->cfg.T_max <= kTeamMaxRows) {
     auto kernel = c->cfg.n_groups_max > 0 ? probe_steer_team_kernel<8, kTeamLate>
                                           : (pdl == kPdlMapAhead ? probe_steer_team_kernel<8, kTeamMapAhead> : probe_steer_team_kernel<8, kTeamPlain>);

@@ -16,14 +16,26 @@ struct RowApp {
   const float* b;
 };
 
-// Does row t pass the gate of its slot?  (NaN fails both comparisons.)
-__device__ __forceinline__ bool gate_open(const GateEntry* __restrict__ gates, int s, int t) {
+// A row's gate: the entry, which the library owns, and -- a second step -- the score, which the caller owns.
+struct RowGate {
+  const float* score;
+  int cmp;
+  float thr;
+};
+__device__ __forceinline__ RowGate load_gate(const GateEntry* __restrict__ gates, int s, int t) {
   const int4 g0 = __ldg(reinterpret_cast<const int4*>(gates + s));        // scores ptr, stride, col
   const int4 g1 = __ldg(reinterpret_cast<const int4*>(gates + s) + 1);    // cmp, thr
-  const float* sc = reinterpret_cast<const float*>(((unsigned long long)(unsigned)g0.y << 32) | (unsigned)g0.x);
-  const float v = __ldg(sc + (size_t)t * g0.z + g0.w);
-  const float thr = __int_as_float(g1.y);
-  return g1.x == MIX_GATE_GE ? v >= thr : v < thr;
+  RowGate r;
+  r.score = reinterpret_cast<const float*>(((unsigned long long)(unsigned)g0.y << 32) | (unsigned)g0.x) + (size_t)t * g0.z + g0.w;
+  r.cmp = g1.x;
+  r.thr = __int_as_float(g1.y);
+  return r;
+}
+// Does a row with this score pass?  (NaN fails both comparisons.)
+__device__ __forceinline__ bool gate_passes(const RowGate& g, float score) { return g.cmp == MIX_GATE_GE ? score >= g.thr : score < g.thr; }
+__device__ __forceinline__ bool gate_open(const GateEntry* __restrict__ gates, int s, int t) {
+  const RowGate g = load_gate(gates, s, t);
+  return gate_passes(g, __ldg(g.score));
 }
 
 // Slot -> app for row t; flags bad slot ids; applies the slot's gate.  `leader` is the one

@@ -205,3 +205,75 @@ def test_random_chains(seed):
     out = run_gpu(w, flags=mixlib.MIX_FLAG_SLOT_CHAINS, graph=bool(seed % 2), conditional=bool(seed % 4 == 1))
     check_chain_parity(W.host(w), out, scale_with_output=True, expect_status=None)
     assert out["status"] & ~mixlib.MIX_STATUS_TOPK_GENERAL == 0
+
+
+@pytest.mark.parametrize("d", [64, 2048, 2112, 4096, 4160, 6144, 6208, 8192])
+@pytest.mark.parametrize("T", [9, 2049])
+def test_every_width_chained_and_one_by_one(d, T):
+    """The hook kernels of every row width, at the edges of the widths: a probe, a steering vector, a projection and a five-class
+    probe on one row, the third and the last gated -- in a chain, and one context each (small contexts; above 2048 rows the
+    chain's vectors stay in the caller's memory).  Scores against float64: a sum of n = d products in fp32 is within n 2^-24 of
+    the sum of their magnitudes, whatever its order."""
+    mixlib = _mixlib()
+    g = torch.Generator(device=DEV); g.manual_seed(d + T)
+    h = torch.randn((T, d), generator=g, device=DEV).to(torch.bfloat16)
+    w1 = (torch.randn((1, d), generator=g, device=DEV) * d ** -0.5).to(torch.bfloat16)
+    w5 = (torch.randn((5, d), generator=g, device=DEV) * d ** -0.5).to(torch.bfloat16)
+    v, r = [(torch.randn((d,), generator=g, device=DEV) * d ** -0.5).to(torch.bfloat16) for _ in range(2)]
+    bias = torch.randn(5, generator=g, device=DEV)
+    gate = torch.randn((T, 1), generator=g, device=DEV)
+    slots = torch.where(torch.arange(T, device=DEV) % 4 == 3, -1, 0).to(torch.int32)
+
+    def register(m, first, kinds):
+        for i, kind in enumerate(kinds):
+            s = first + i
+            if kind == "probe":
+                m.register_probe(s, w1, bias[:1], mixlib.MIX_ACT_NONE)
+            elif kind == "steer":
+                m.register_steer(s, v, 1.5)
+            elif kind == "project":
+                m.register_project(s, r, 0.75)
+            else:
+                m.register_probe(s, w5, bias, mixlib.MIX_ACT_NONE)
+            if kind in ("project", "wide"):
+                m.set_gate(s, gate, column=0, threshold=0.0)
+
+    kinds = ["probe", "steer", "project", "wide"]
+    m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=4, C_max=6, flags=mixlib.MIX_FLAG_SLOT_CHAINS)
+    register(m, 0, kinds)
+    for s in range(3):
+        m.set_chain(s, s + 1)
+    m.set_slot_map(slots, T)
+    chained, scores = h.clone(), torch.full((T, 6), 7.0, device=DEV)
+    m.apply(chained, scores)
+    torch.cuda.synchronize()
+    assert m.get_status() == 0
+    m.destroy()
+    hooked = slots == 0
+    opened = hooked & (gate[:, 0] >= 0)
+    one, one_scores, before = h.clone(), torch.full((T, 6), 7.0, device=DEV), {}
+    for kind in kinds:
+        before[kind] = one.clone()
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=1, C_max=5)
+        register(m, 0, [kind])
+        m.set_slot_map(slots, T)
+        sc = torch.full((T, 5), 7.0, device=DEV)
+        m.apply(one, sc)
+        torch.cuda.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+        if kind == "probe":
+            one_scores[:, 0] = sc[:, 0]
+        elif kind == "wide":
+            one_scores[:, 1:] = sc
+    if T <= 2048:
+        assert torch.equal(chained, one) and torch.equal(scores, one_scores)
+    assert torch.equal(chained[~hooked], h[~hooked]) and bool((scores[~hooked] == 7.0).all()) and bool((scores[~opened][:, 1:] == 7.0).all())
+    for sc, row in ((scores, chained), (one_scores, before["wide"])):
+        for col, Wm, x, rows in ((0, w1, h, hooked), (1, w5, row, opened)):
+            x64, W64 = x[rows].double(), Wm.double()
+            want = x64 @ W64.T + bias[:Wm.shape[0]].double()
+            bound = (d + 1) * 2.0 ** -24 * (x64.abs() @ W64.abs().T + bias[:Wm.shape[0]].abs().double())
+            assert bool(((sc[rows, col:col + Wm.shape[0]].double() - want).abs() <= bound).all())
+    steered = (h.double() + 1.5 * v.double()).float().to(torch.bfloat16)
+    assert bool(((before["project"] - steered)[hooked].abs() <= steered[hooked].abs() * 2.0 ** -7 + 1e-30).all())
