@@ -4,6 +4,8 @@
 // loads, fp32 FMA, shuffle reductions.  A row whose slot is -1 costs one 4-byte load.
 #include <string.h>
 
+#include <type_traits>
+
 #include "mix_internal.h"
 #include "row_lookup.cuh"
 
@@ -386,23 +388,26 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
   }
 }
 
-// Small batches (decode): one CTA of NW warps per row, the row held in registers (up to kTeamVec
-// 16-byte vectors per thread).  The row's loads are issued as soon as the slot id is known to be
+// Small batches (decode): one CTA per row, the row held in registers (NV 16-byte vectors per thread, a kernel for each width:
+// 64 registers up to d = 4096 where one for all widths had 126, i.e. four CTAs on an SM instead of two, so that the kernels of a
+// step's next layers are there, their look-ups done, when the present one ends).  The row's loads are issued as soon as the slot id is known to be
 // >= 0, in parallel with the app-table lookup, so a cold row costs two dependent round trips
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
-constexpr int kTeamVec = 4;     // NW * 32 * kTeamVec * 8 >= d_model: 8192 columns at NW = 8
-constexpr int kHookWarps = 8, kMostVec = kTeamVec;
+// Eight warps: with sixteen, which leaves each thread half as much, the sums over the warps cost more than that saves (187 rows
+// of a three-app chain, d = 5120: 38 us for four layers against 33).
+constexpr int kHookWarps = 8;
+constexpr int kMostVec = 4;     // kHookWarps * 32 * kMostVec * 8 >= d_model: 8192 columns
 
 enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
 
-template <int NW, TeamForm kForm>
-__global__ void __launch_bounds__(NW * 32)
+template <int NV, TeamForm kForm>
+__global__ void __launch_bounds__(kHookWarps * 32, NV <= 2 ? 4 : 2)
 probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
                         unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl) {
-  __shared__ float s_part[NW][kMaxClasses];
-  constexpr int NT = NW * 32;
+  __shared__ float s_part[kHookWarps][kMaxClasses];
+  constexpr int NW = kHookWarps, NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
   // Programmatic dependent launch (`pdl`: the launch asked for it): everything up to pdl_wait() reads only
@@ -432,30 +437,35 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   // Single-vector weights (steering, projection, one-class probe) were copied at registration
   // into row `slot` of the context's vector arena, so their address follows from the slot id
   // alone: the row AND its vector are requested together, before the app entry is known.
-  uint4 hq[kTeamVec], vq[kTeamVec];
+  uint4 hq[NV], vq[NV];
   // (kLate, contexts with SAE weight sets: most rows may be another kernel's; nothing is requested before the entry says
   // that the row is this one's.  1000 SAE rows of d = 2304: 6.2 -> 4.5 us.)
   const bool slot_ok = slot >= 0 && slot < n_slots;
   if (!kLate && slot_ok) {
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
     }
   }
   if (!kLate && !pdl && slot_ok) {
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) hq[u] = __ldcs(hrow + v);
     }
   }
+  // (A hint, so it may come before the wait: what the predecessor still writes of the row, it writes to this L2.  For a step
+  // whose hidden states no longer lie there: 32 layers of 256 rows, d = 4096: 2.25 -> 1.9 us a layer.)
+  if (!kLate && pdl && slot_ok && threadIdx.x * 8 < nvec) asm volatile("prefetch.global.L2 [%0];" ::"l"(hrow + threadIdx.x * 8));
   RowApp a = lookup(slot, t, apps, gates, n_slots, status, threadIdx.x == 0, /*eval_gate=*/false);
+  RowGate gate;
+  if (a.gated) gate = load_gate(gates, slot, t);
   if (pdl) pdl_wait();
   if (kLate) {
     if (a.kind == 0 || a.kind == MIX_SAE || a.kind == MIX_ROUTER) return;
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
@@ -465,12 +475,14 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   } else if (pdl) {
     if (slot_ok) {
 #pragma unroll
-      for (int u = 0; u < kTeamVec; ++u) {
+      for (int u = 0; u < NV; ++u) {
         const int v = threadIdx.x + u * NT;
         if (v < nvec) hq[u] = __ldcs(hrow + v);
       }
     }
   }
+  float score = 0.f;
+  if (a.gated) score = __ldg(gate.score);        // (requested with the row)
   // A one-class probe's bias came with the entry (registration put it into the `alpha` word); the biases of a
   // wider probe are requested as soon as the entry is here, not after the dot products they are added to.
   float bias_lo = 0.f, bias_hi = 0.f;
@@ -482,11 +494,11 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
       if (lane + 32 < a.C) bias_hi = __ldg(a.b + lane + 32);
     }
   }
-  if (a.gated && a.kind != 0 && !gate_open(gates, slot, t)) return;       // gate closed: the row passes through
+  if (a.gated && !gate_passes(gate, score)) return;       // gate closed: the row passes through
   if (a.kind == MIX_STEER) {
     if (a.alpha == 0.f) return;                  // identity; the row stays bit-exact
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         float x[8], y[8];
@@ -503,7 +515,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
     if (a.alpha == 0.f) return;
     float dot = 0.f;
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         float x[8], y[8];
@@ -521,7 +533,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
     for (int w = 0; w < NW; ++w) total += s_part[w][0];
     const float coef = -a.alpha * total;
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         float x[8], y[8];
@@ -538,7 +550,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   if (a.C == 1) {                              // the probe vector is already here
     float acc = 0.f;
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         float x[8], y[8];
@@ -553,17 +565,17 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   }
   for (int c0 = 0; c0 < (a.C == 1 ? 0 : a.C); c0 += 4) {
     const int nc = min(4, a.C - c0);
-    uint4 wq[4][kTeamVec];
+    uint4 wq[4][NV];
 #pragma unroll
     for (int c = 0; c < 4; ++c)
 #pragma unroll
-      for (int u = 0; u < kTeamVec; ++u) {
+      for (int u = 0; u < NV; ++u) {
         const int v = threadIdx.x + u * NT;
         if (c < nc && v < nvec) wq[c][u] = __ldg(a.W + (size_t)(c0 + c) * nvec + v);
       }
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int u = 0; u < kTeamVec; ++u) {
+    for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) {
         float x[8];
@@ -578,11 +590,8 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
           }
       }
     }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float z = warp_sum(acc[c]);
-      if (lane == 0 && c < nc) s_part[warp][c0 + c] = z;
-    }
+    const float z = warp_sum4(acc, lane);
+    if ((lane & 7) == 0 && (lane >> 3) < nc) s_part[warp][c0 + (lane >> 3)] = z;
   }
   __syncthreads();
   if (warp == 0) {
@@ -1004,12 +1013,22 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
       default: return run(probe_steer_chain_kernel<kMostVec>);
     }
   } else if (c->cfg.T_max <= kTeamMaxRows) {
-    auto kernel = c->cfg.n_groups_max > 0 ? probe_steer_team_kernel<8, kTeamLate>
-                                          : (pdl == kPdlMapAhead ? probe_steer_team_kernel<8, kTeamMapAhead> : probe_steer_team_kernel<8, kTeamPlain>);
-    return launch_pdl(allow_pdl ? kPdlHook : 0, kernel,
-                      dim3(c->cfg.T_max), dim3(8 * 32), 0, s, c->d_token_slot, T, c->d_apps, c->d_gates,
-                      c->cfg.n_slots_max, hidden, c->cfg.d_model, scores, c->cfg.C_max, c->d_status,
-                      reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
+    auto run = [&](auto kernel) {
+      return launch_pdl(allow_pdl ? kPdlHook : 0, kernel, dim3(c->cfg.T_max), dim3(kHookWarps * 32), 0, s, c->d_token_slot, T, c->d_apps, c->d_gates,
+                        c->cfg.n_slots_max, hidden, c->cfg.d_model, scores, c->cfg.C_max, c->d_status,
+                        reinterpret_cast<const uint4*>(c->d_vec_arena), pdl);
+    };
+    auto of_width = [&](auto nv) {
+      constexpr int NV = decltype(nv)::value;
+      if (c->cfg.n_groups_max > 0) return run(probe_steer_team_kernel<NV, kTeamLate>);
+      return pdl == kPdlMapAhead ? run(probe_steer_team_kernel<NV, kTeamMapAhead>) : run(probe_steer_team_kernel<NV, kTeamPlain>);
+    };
+    switch (n_vec) {
+      case 1: return of_width(std::integral_constant<int, 1>());
+      case 2: return of_width(std::integral_constant<int, 2>());
+      case 3: return of_width(std::integral_constant<int, 3>());
+      default: return of_width(std::integral_constant<int, kMostVec>());
+    }
   } else {
     auto run = [&](auto kernel, int warps) {
       kernel<<<(c->cfg.T_max + warps - 1) / warps, warps * 32, 0, s>>>(c->d_token_slot, T, c->d_apps, c->d_gates,
