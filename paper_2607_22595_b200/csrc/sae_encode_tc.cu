@@ -39,7 +39,10 @@ namespace {
 constexpr int kMaxStages = 8;
 constexpr int kABytes = kTileM * kTileK * 2;   // 16 KiB: 128 rows of 128 bytes
 constexpr int kBBytes = kTileN * kTileK * 2;   // 32 KiB: 256 rows of 128 bytes
-constexpr int kXchgEntries = kCandPerTile + 2;  // a top-9 list and the bound it was collected under
+constexpr int kVecs = 4;                        // tiles whose bias and scale are in shared memory
+// An epilogue warp's list of a TopK tile: up to 8 values a row and a place for what is one too many, [entry][lane], then their
+// columns.  The lists that are handed over are followed by three words a row: 9th value, number of entries, bound.
+constexpr int kListRows = kCandPerTile + 1, kListBytes = kListRows * 32 * 5, kXchgListBytes = kListBytes + 3 * 32 * 4;
 // kEnc: 0 = bf16 encoder and input; 1 = 8-bit encoder, bf16 input as two E4M3 operands; 2 = 8-bit encoder and 8-bit input
 // kPair: two CTAs (a cluster) share one 256-row x 256-feature tile: each loads its own 128 panel rows and HALF of the
 //        W_enc tile, and one tcgen05.mma.cta_group::2 instruction feeds both SMs' tensor cores -- a third less
@@ -56,14 +59,14 @@ template <int kEnc, int kEpi, bool kPair> struct TcCfg {
   // each; the two top-9 lists of a row meet in shared memory).  One warp per scheduler runs the epilogue's
   // dependent compare/select chains at a fraction of the issue rate; two interleave.
   static constexpr int kEpiWarps = kEpi;
-  static constexpr int kXchgBytes = kEpiWarps == 8 ? 2 * 4 * kXchgEntries * 32 * 8 : 0;   // [acc][quarter][entry][lane] x (value, column)
+  static constexpr int kXchgBytes = kEpiWarps == 8 ? 2 * 4 * kXchgListBytes : 0;   // [acc][quarter]: the upper-half warps' lists
   static constexpr int kThreads = 64 + kEpiWarps * 32;
-  // each epilogue warp keeps the bias (and, for codes, the feature scale) of its columns of the current tile in
-  // shared memory, fetched while the tile's main loop still runs
-  static constexpr int kEpiVecBytes = 2 * 4 * kTileN * 4;   // [bias, scale][warp][its columns] floats: 8 KiB with 4 or 8 warps
-  // survivors of the top-8 search, 8 values and columns per row, of the four lower-half warps (the upper-half warps use
-  // their hand-over place)
-  static constexpr int kPickBytes = kEpiWarps == 8 ? 4 * 32 * kCandPerTile * 5 : 0;
+  // The bias (and, for codes, the feature scale) of a tile's columns comes with the tile: the producer copies it into one of
+  // kVecs places.  bf16 kernels keep the thresholds of each epilogue warp's columns behind them.
+  static constexpr int kVecBytes = (kEnc != 0 ? 2 : 1) * kTileN * 4;
+  static constexpr int kEpiVecBytes = 2 * 4 * kTileN * 4;
+  static_assert(kVecs * kVecBytes + (kEnc == 0 ? 4 * kTileN * 4 : 0) <= kEpiVecBytes, "the tiles' vectors");
+  static constexpr int kPickBytes = kEpiWarps == 8 ? 4 * kListBytes : 0;                 // the lower-half warps' lists
   static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + 1024 /* TcShared */ + kXchgBytes + kEpiVecBytes + kPickBytes;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
@@ -76,6 +79,8 @@ struct __align__(8) TcShared {
   unsigned long long empty[kMaxStages];
   unsigned long long tmem_full[2];
   unsigned long long tmem_empty[2];
+  unsigned long long vec_full[kVecs], vec_empty[kVecs];   // a tile's bias and scale
+  unsigned long long top_full[2][4];      // [half][quarter]: that warp's 8 largest values are where the other one looks for them
   unsigned long long xchg_full[2][4];     // 8 epilogue warps: the upper-half warp's list of (accumulator, quarter) is in shared memory
   unsigned tmem_base;
   volatile int abort_flag;
@@ -259,10 +264,9 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   // 1024-byte alignment: required by the 128-byte swizzle atoms
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   TcShared* sh = reinterpret_cast<TcShared*>(tiles + Cfg::kRingBytes);
-  float* xchg_val = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sh) + 1024);
-  int* xchg_idx = reinterpret_cast<int*>(xchg_val + 2 * 4 * kXchgEntries * 32);
-  float* epi_vec = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sh) + 1024 + Cfg::kXchgBytes);
-  float* pick = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(epi_vec) + Cfg::kEpiVecBytes);
+  unsigned char* xchg = reinterpret_cast<unsigned char*>(sh) + 1024;
+  float* epi_vec = reinterpret_cast<float*>(xchg + Cfg::kXchgBytes);
+  unsigned char* pick = reinterpret_cast<unsigned char*>(epi_vec) + Cfg::kEpiVecBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // CTA pairs: rank 0 leads (it issues the pair's tensor-core instructions and owns the barriers both CTAs' copies
   // complete on); `worker` numbers the units that walk the tile list -- pairs, or single CTAs
@@ -280,7 +284,14 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&sh->tmem_full[a]), 1);
       mbar_init(smem_u32(&sh->tmem_empty[a]), kPair ? 2 * kEpiWarps : kEpiWarps);   // a pair's leader hears from both CTAs' epilogues
-      for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&sh->xchg_full[a][q]), 1);
+      for (int q = 0; q < 4; ++q) {
+        mbar_init(smem_u32(&sh->xchg_full[a][q]), 1);
+        mbar_init(smem_u32(&sh->top_full[a][q]), 1);
+      }
+    }
+    for (int v = 0; v < kVecs; ++v) {
+      mbar_init(smem_u32(&sh->vec_full[v]), 1);
+      mbar_init(smem_u32(&sh->vec_empty[v]), kEpiWarps);
     }
     sh->abort_flag = 0;
     sh->wait_cycles = test_stall ? kWaitCyclesTest : kWaitCycles;
@@ -346,8 +357,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
 
   if (warp == 0) {
     if (lane == 0) {
-      int stage = 0;
-      unsigned phase = 0;
+      int stage = 0, vec = 0;
+      unsigned phase = 0, vec_phase = 0;
       bool ok = true;
       const unsigned long long stream = l2_evict_first();
       for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
@@ -362,7 +373,20 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         // with a chain of DRAM round trips (91 rows, d = 4096, 16384 features: front 12.3 -> 8.5 us, tail 19.4 -> 15.6).
         // Tiles that several row tiles share must stay (the mixed batch's encode 441 -> 480 us with the hint).
         const bool once = sh->unit0[t.group + 1] - sh->unit0[t.group] == 1;
+        const float* b_eff = groups[t.group].b_eff;           // (requested here, used a few k-blocks later)
+        const float* w_scale = groups[t.group].w_scale;
         for (int kb = 0; kb < num_kb; ++kb) {
+          if (kb == min(3, num_kb - 1)) {       // (behind the first copies: nothing waits for these before the tile's end)
+            if (!mbar_wait(smem_u32(&sh->vec_empty[vec]), vec_phase ^ 1u, sh, status)) { ok = false; break; }
+            if (!test_stall) {
+              const unsigned bar = smem_u32(&sh->vec_full[vec]), bytes = tile_n * 4;
+              const unsigned dst = smem_u32(epi_vec) + vec * Cfg::kVecBytes;
+              mbar_expect_tx(bar, (kE4 ? 2 : 1) * bytes);
+              bulk_load(dst, b_eff + (size_t)t.n_tile * tile_n, bytes, bar);
+              if (kE4) bulk_load(dst + kTileN * 4, w_scale + (size_t)t.n_tile * tile_n, bytes, bar);
+              if (++vec == kVecs) { vec = 0; vec_phase ^= 1u; }
+            }
+          }
           if (!mbar_wait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
           // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumer's
           // bounded wait runs out and the whole CTA leaves through the time-out path.
@@ -448,7 +472,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
     const int q = warp & 3;                  // tensor-memory lane quarter this warp may read
     const int half = (warp - 2) >> 2;        // 8 epilogue warps: which 128 columns of the tile
     const int c_lo = half * epi_cols;
-    unsigned acc = 0, acc_phase = 0;
+    unsigned acc = 0, acc_phase = 0, vec = 0, vec_phase = 0;
+    unsigned top_phase = 0;
     unsigned xchg_phase = 0;                 // bit a: phase of the next hand-over through xchg_full[a][q] (TopK tiles only)
     for (int tile = worker; tile < total_tiles; tile += n_workers) {
       const Tile t = tile_of(tile);
@@ -468,30 +493,14 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
       const bool publish_tau = use_tau && tile + n_workers < total_tiles;
       unsigned tau_key = 0u;                   // 0: no bound yet
       if (use_tau) tau_key = __ldcg(tau_min + p);     // the smallest slot, as of the last time a publisher looked
-      // this warp's columns of the bias (and feature scale) go to shared memory now, while the accumulator is
-      // still being computed: read from global memory inside the loop below, 32 columns at a time between
-      // tensor-memory loads, they were four exposed round trips per tile
-      // (Not where both operands are 8-bit and the epilogue selects TopK candidates: there the epilogue, not the
-      // main loop, sets the pace -- the accumulator is ready when the warp asks for it -- so a load to wait for in
-      // front of every tile costs more than the loads spread over the loop: config 2 with 8-bit operands 240 us
-      // against 210 us.  Asking one tile ahead, the vectors held in registers meanwhile, was slower still: 256 us.)
       constexpr bool kScaled = kEnc != 0;      // the accumulator is in units of the codes
-      constexpr bool kStageVec = !(kEnc == 2 && kEpi == 8);
-      float* wb = epi_vec + (warp - 2) * kEpiColsMax;
-      float* ws = wb + kEpiWarps * kEpiColsMax;
-      const float* bias_t = groups[t.group].b_eff + (size_t)t.n_tile * tile_n + c_lo;
-      const float* wsc_t = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * tile_n + c_lo : nullptr;
-      if (kStageVec) {
-        const float* bias_g = groups[t.group].b_eff + (size_t)t.n_tile * tile_n + c_lo;
-        const float* wsc_g = kScaled ? groups[t.group].w_scale + (size_t)t.n_tile * tile_n + c_lo : nullptr;
-        for (int j = lane * 4; j < epi_cols; j += 128) {
-          *reinterpret_cast<float4*>(wb + j) = __ldg(reinterpret_cast<const float4*>(bias_g + j));
-          if (kScaled) *reinterpret_cast<float4*>(ws + j) = __ldg(reinterpret_cast<const float4*>(wsc_g + j));
-        }
-        __syncwarp();
-      }
+      // This warp's columns of the bias and the feature scale, which the producer has copied.  (Read from global memory between
+      // the tensor-memory loads they were four exposed round trips a tile; copied by each warp for itself ahead of its wait for
+      // the accumulator, a trip that 8-bit tiles, which the epilogue sets the pace of, had no time for.)
+      const float* wb = epi_vec + vec * (Cfg::kVecBytes / 4) + c_lo;
+      const float* ws = wb + kTileN;
       const float* theta_t = nullptr;
-      float* wt = kScaled || !kStageVec ? nullptr : ws;         // (the scale's place is free where there is no scale)
+      float* wt = kScaled ? nullptr : epi_vec + kVecs * kTileN + (warp - 2) * kEpiColsMax;
       bool want_bits = false, any_bits = false, jump = false, only_edits = false, any_full = false;
       unsigned edited = 0u;
       if (!topk_tile) {
@@ -538,130 +547,212 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
         }
       }
       // warp-uniform decision: tcgen05.ld below needs the whole warp
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->tmem_full[acc]), acc_phase, sh, status))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->vec_full[vec]), vec_phase, sh, status) &&
+                                       mbar_wait(smem_u32(&sh->tmem_full[acc]), acc_phase, sh, status))) break;
       tc_fence_after();
       const float ars = kE4 ? (valid ? __ldg(act_scale + p) : 0.f) : 1.f;     // power of two: the products below are exact
       const unsigned taddr = tmem_base + ((unsigned)(q * 32) << 16) + acc * kTileN;
       if (topk_tile) {
-        // the list starts out filled with a value just below the bound: whatever is not collected is at most that
+        // `below`: what is not collected is at most that; the places of a list that nothing was collected for hold it
         const float tau = tau_key > 1u ? key2f(tau_key) : -INFINITY;
-        const float below_tau = tau_key > 1u ? key2f(tau_key - 1u) : -INFINITY;
-        float tv[kCandPerTile + 1];
-        int ti[kCandPerTile + 1];
+        float below = tau_key > 1u ? key2f(tau_key - 1u) : -INFINITY;
+        auto to_z = [&](float v, float b, float s) { return kScaled ? fmaf(v, s * ars, b) : v + b; };
+        // f(first column, 8 pre-activations) over this warp's columns, 32 of them a load: what a trip of eight costs beside the
+        // work is the load's latency, also with the next load under way (eight a load 2.5 us for the networks of 64 columns and
+        // 2.5 for what is collected, 32 a load 2.3 and 1.9).  A loop still: this code runs once or a few times per call, and what
+        // is unrolled has to be fetched before it has an effect.
+        auto columns = [&](auto&& f) {
+#pragma unroll 1
+          for (int c = c_lo; c < c_lo + epi_cols; c += 32) {
+            float v[32];
+            tmem_ld32(taddr + c, v);
 #pragma unroll
-        for (int s = 0; s <= kCandPerTile; ++s) {
-          tv[s] = below_tau;
-          ti[s] = 0;
-        }
-        // Eight columns of the accumulator as pre-activations.  (Eight, in loops that stay loops: this code runs once or a few
-        // times per call, and 32 unrolled columns of it are 30 KiB of instructions to fetch before the first has an effect --
-        // more than the selection itself takes.)
-        auto load_z = [&](int c, float (&v)[8]) {
-          tmem_ld8(taddr + c, v);
+            for (int g = 0; g < 32; g += 8) {
+              float z[8];
 #pragma unroll
-          for (int i = 0; i < 8; i += 4) {
-            const float4 b4 = kStageVec ? *reinterpret_cast<const float4*>(wb + (c - c_lo) + i)
-                                        : __ldg(reinterpret_cast<const float4*>(bias_t + (c - c_lo) + i));
-            float4 s4 = make_float4(1.f, 1.f, 1.f, 1.f);
-            if (kScaled) s4 = kStageVec ? *reinterpret_cast<const float4*>(ws + (c - c_lo) + i)
-                                        : __ldg(reinterpret_cast<const float4*>(wsc_t + (c - c_lo) + i));
-            if (kE4) { s4.x *= ars; s4.y *= ars; s4.z *= ars; s4.w *= ars; }
-            v[i] = kScaled ? fmaf(v[i], s4.x, b4.x) : v[i] + b4.x;
-            v[i + 1] = kScaled ? fmaf(v[i + 1], s4.y, b4.y) : v[i + 1] + b4.y;
-            v[i + 2] = kScaled ? fmaf(v[i + 2], s4.z, b4.z) : v[i + 2] + b4.z;
-            v[i + 3] = kScaled ? fmaf(v[i + 3], s4.w, b4.w) : v[i + 3] + b4.w;
+              for (int i = 0; i < 8; i += 4) {
+                const float4 b4 = *reinterpret_cast<const float4*>(wb + (c - c_lo) + g + i);
+                float4 s4 = make_float4(1.f, 1.f, 1.f, 1.f);
+                if (kScaled) s4 = *reinterpret_cast<const float4*>(ws + (c - c_lo) + g + i);
+                z[i] = to_z(v[g + i], b4.x, s4.x);
+                z[i + 1] = to_z(v[g + i + 1], b4.y, s4.y);
+                z[i + 2] = to_z(v[g + i + 2], b4.z, s4.z);
+                z[i + 3] = to_z(v[g + i + 3], b4.w, s4.w);
+              }
+              f(c + g, z);
+            }
           }
         };
-        // Two ways to the list.  With a bound in force nearly every column fails one comparison, and the few that do not are
-        // inserted.  Without one (a call's first wave of tiles; every tile of a call that has one wave) some lane of the
-        // warp would insert at nearly every column, 60 instructions each for one lane's sake: there the 8 largest VALUES and
-        // the 9th are found first, by min / max networks in which all lanes take part (11 instructions a column), and a
-        // second look at the accumulator picks up the columns of those 8, which the lanes then sort together.
-        bool listed = false;
-        if (kEpiWarps == 8 && __any_sync(0xffffffffu, valid && tau_key <= 1u)) {
-          float top[8], ninth = -INFINITY;
+        // This warp's list: columns ascending, or sorted.  (Either way equal values stand in the order of their columns, which is
+        // all that the selection asks of it.)
+        auto handed = [&](unsigned a) { return xchg + (a * 4 + q) * kXchgListBytes; };
+        unsigned char* list = half == 1 ? handed(acc) : pick + q * kListBytes;
+        float* list_v = reinterpret_cast<float*>(list) + lane;
+        unsigned char* list_c = list + kListRows * 32 * 4 + lane;
+        float tv[kCandPerTile + 1];
+        int ti[kCandPerTile + 1];
+        int n = 0;                              // entries of the list
+        bool listed = false, sorted = false;    // sorted: the list is in tv / ti, in descending order
+        if (kEpiWarps == 8) {
+          float least = tau;                    // what is collected: this and above
+          tv[kCandPerTile] = below;
+          // With a bound in force few columns pass it.  Without one -- the row's feature tiles that finished a wave ago cannot
+          // have filled its k slots -- the 8 largest VALUES of the tile and the 9th are found first, by min / max networks in
+          // which all lanes take part (11 instructions a column); the two warps of a quarter show each other theirs, and the 8th
+          // of both is the bound, so that together they collect 8 and nobody sorts.  (Each warp collecting its own 8, sorting
+          // them and merging: 6.5 us for a tile of 128 features and 4.2 for one of 64, where this takes 5.0 and 3.4.  Both warps
+          // must come to the same answer here, so it does not hang on what either has read of the bound.)
+          const int first_wave = n_workers / (uniform_nt > 0 ? sh->unit0[n_groups] : sh->unit0[t.group + 1] - sh->unit0[t.group]) + 1;
+          const bool network = __any_sync(0xffffffffu, valid) &&
+                               (tau_slots == nullptr || k_row > kTauSlots || (t.n_tile - first_wave) * kCandPerTile < k_row);
+          if (network) {
+            float top[8], ninth = -INFINITY;
 #pragma unroll
-          for (int s = 0; s < 8; ++s) top[s] = -INFINITY;
-#pragma unroll 1
-          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
-            float b[8];
-            load_z(c, b);
+            for (int s = 0; s < 8; ++s) top[s] = -INFINITY;
+            columns([&](int, float (&b)[8]) {
 #pragma unroll
-            for (int s = 0; s < 8; ++s) b[s] = fmaxf(b[s], -INFINITY);          // (a NaN is never selected)
-            sort8_desc(b);
+              for (int s = 0; s < 8; ++s) b[s] = fmaxf(b[s], -INFINITY);          // (a NaN is never selected)
+              sort8_desc(b);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) {                                       // the 8 largest of both, and the largest of the rest
-              const float lo = fminf(top[s], b[7 - s]);
-              top[s] = fmaxf(top[s], b[7 - s]);
-              ninth = fmaxf(ninth, lo);
+              for (int s = 0; s < 8; ++s) {                                       // the 8 largest of both, and the largest of the rest
+                const float lo = fminf(top[s], b[7 - s]);
+                top[s] = fmaxf(top[s], b[7 - s]);
+                ninth = fmaxf(ninth, lo);
+              }
+              merge8_desc(top);
+            });
+            // The lower-half warp leaves its values in the other accumulator's hand-over place, which it was the last to read;
+            // the upper-half warp answers in the lower one's list, which that does not touch before it has read the answer.
+            float* to = reinterpret_cast<float*>(half == 0 ? handed(acc ^ 1u) : pick + q * kListBytes) + lane;
+            const float* from = reinterpret_cast<const float*>(half == 0 ? pick + q * kListBytes : handed(acc ^ 1u)) + lane;
+            if (half == 1 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->top_full[0][q]), top_phase, sh, status))) break;
+            float other[8], ninth2 = 0.f;
+            if (half == 1) {
+#pragma unroll
+              for (int s = 0; s < 8; ++s) other[s] = from[s * 32];
+              ninth2 = from[8 * 32];
             }
-            merge8_desc(top);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) to[s * 32] = top[s];
+            to[8 * 32] = ninth;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh->top_full[half][q]));
+            if (half == 0) {
+              if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->top_full[1][q]), top_phase, sh, status))) break;
+#pragma unroll
+              for (int s = 0; s < 8; ++s) other[s] = from[s * 32];
+              ninth2 = from[8 * 32];
+              __syncwarp();                     // (every lane has read before one writes its list there)
+            }
+            top_phase ^= 1u;
+            least = INFINITY;
+            ninth = fmaxf(ninth, ninth2);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+              least = fminf(least, fmaxf(top[s], other[7 - s]));
+              ninth = fmaxf(ninth, fminf(top[s], other[7 - s]));
+            }
+            below = -INFINITY;
+            tv[kCandPerTile] = ninth;
           }
-          float* pick_v = half == 1 ? xchg_val + (size_t)((acc * 4 + q) * kXchgEntries) * 32 : pick + q * (32 * kCandPerTile);
-          unsigned char* pick_c = half == 1 ? reinterpret_cast<unsigned char*>(xchg_idx + (size_t)((acc * 4 + q) * kXchgEntries) * 32)
-                                            : reinterpret_cast<unsigned char*>(pick + 4 * 32 * kCandPerTile) + q * (32 * kCandPerTile);
-          const float eighth = valid ? top[7] : INFINITY;
-          int n = 0;
-#pragma unroll 1
-          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
-            float v[8];
-            load_z(c, v);
+          if (!valid) least = NAN;
+          columns([&](int c, float (&z)[8]) {
+            float m = z[0];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) m = fmaxf(m, z[i]);
+            if (!__any_sync(0xffffffffu, m >= least)) return;
+            // (stored whether they pass or not, the next one over what did not: a branch around each of them, taken for some
+            // lane nearly every time, cost 86 cycles a column)
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-              const int at = min(n, kCandPerTile - 1) * 32 + lane;      // (a ninth survivor: see below)
-              if (v[i] >= eighth) {
-                pick_v[at] = v[i];
-                pick_c[at] = (unsigned char)(c - c_lo + i);
-                ++n;
-              }
+              const int at = min(n, kListRows - 1) * 32;
+              list_v[at] = z[i];
+              list_c[at] = (unsigned char)(c - c_lo + i);
+              n += z[i] >= least;
             }
-          }
-          if (__all_sync(0xffffffffu, n <= kCandPerTile)) {      // (more only where values are exactly equal: the insertion below)
-            listed = true;
+          });
+          listed = __all_sync(0xffffffffu, n <= kCandPerTile);
+          if (listed && half == 0) {
 #pragma unroll
             for (int s = 0; s < kCandPerTile; ++s) {
-              const bool in = s < n;
-              tv[s] = in ? pick_v[s * 32 + lane] : -INFINITY;
-              ti[s] = c_lo + (in ? (int)pick_c[s * 32 + lane] : 0);
+              tv[s] = s < n ? list_v[s * 32] : below;
+              ti[s] = c_lo + (s < n ? (int)list_c[s * 32] : 0);
             }
-            sort8_pairs(tv, ti);
-            tv[kCandPerTile] = ninth;
-            __syncwarp();
           }
         }
-        if (!listed && __any_sync(0xffffffffu, valid)) {
-#pragma unroll 1
-          for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
-            float v[8];
-            load_z(c, v);
-            // (the list's 9th value is at least below_tau, so the test inside top9_insert covers the bound too)
+        if (!listed) {
+          // More than 8 above the bound, or equal values at the 8th: a sorted list of 9, by insertion (kEpiWarps == 4, contexts
+          // that had no TopK set when this was launched: always).
+          below = tau_key > 1u ? key2f(tau_key - 1u) : -INFINITY;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) top9_insert(tv, ti, v[i], c + i);
+          for (int s = 0; s <= kCandPerTile; ++s) {
+            tv[s] = below;
+            ti[s] = c_lo;
           }
+          if (__any_sync(0xffffffffu, valid)) {
+#pragma unroll 1
+            for (int c = c_lo; c < c_lo + epi_cols; c += 8) {
+              float v[8];
+              tmem_ld8(taddr + c, v);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) top9_insert(tv, ti, to_z(v[i], wb[c - c_lo + i], kScaled ? ws[c - c_lo + i] : 1.f), c + i);
+            }
+          }
+          n = kCandPerTile;
+          sorted = true;
         }
         bool writer = true;
         unsigned tau_pub = tau_key;
         if (kEpiWarps == 8) {
-          // the upper-half warp hands its list over; the lower-half warp merges it into its own (its columns
-          // come first, so equal values keep the lower column in front) and writes the tile's candidates
-          float* xv = xchg_val + (size_t)((acc * 4 + q) * kXchgEntries) * 32 + lane;
-          int* xi = xchg_idx + (size_t)((acc * 4 + q) * kXchgEntries) * 32 + lane;
+          // the upper-half warp's list is where the lower-half warp finds it; that one writes the tile's candidates: both lists
+          // one behind the other where they fit (its columns come first), else the 8 largest of both
+          unsigned char* up = handed(acc);
+          float* xv = reinterpret_cast<float*>(up) + lane;
+          unsigned char* xc = up + kListRows * 32 * 4 + lane;
+          int* xw = reinterpret_cast<int*>(up + kListBytes) + lane;
           if (half == 1) {
+            if (sorted) {
 #pragma unroll
-            for (int s = 0; s <= kCandPerTile; ++s) {
-              xv[s * 32] = tv[s];
-              xi[s * 32] = ti[s];
+              for (int s = 0; s < kCandPerTile; ++s) {
+                xv[s * 32] = tv[s];
+                xc[s * 32] = (unsigned char)(ti[s] - c_lo);
+              }
             }
-            xi[(kCandPerTile + 1) * 32] = (int)tau_key;
+            xw[0] = __float_as_int(tv[kCandPerTile]);
+            xw[32] = n | (sorted ? 0x100 : 0);
+            xw[64] = (int)tau_key;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh->xchg_full[acc][q]));
             writer = false;
           } else {
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh->xchg_full[acc][q]), (xchg_phase >> acc) & 1u, sh, status))) break;
-            merge_lists(tv, ti, xv[kCandPerTile * 32], [&](int s, float& x, int& cx) { x = xv[s * 32]; cx = xi[s * 32]; });
+            const int n2 = xw[32] & 0xff;
+            const bool sorted2 = (xw[32] & 0x100) != 0;
+            const float ninth2 = __int_as_float(xw[0]);
+            if (__all_sync(0xffffffffu, n + n2 <= kCandPerTile)) {
+#pragma unroll
+              for (int s = 0; s < kCandPerTile; ++s) {
+                if (s >= n && s < n + n2) {
+                  tv[s] = xv[(s - n) * 32];
+                  ti[s] = epi_cols + (int)xc[(s - n) * 32];
+                }
+              }
+              tv[kCandPerTile] = fmaxf(tv[kCandPerTile], ninth2);
+            } else {
+              float v2[kCandPerTile + 1];
+              int c2[kCandPerTile + 1];
+#pragma unroll
+              for (int s = 0; s < kCandPerTile; ++s) {
+                v2[s] = s < n2 ? xv[s * 32] : -INFINITY;
+                c2[s] = epi_cols + (s < n2 ? (int)xc[s * 32] : 0);
+              }
+              if (!sorted) sort8_pairs(tv, ti);
+              if (!sorted2) sort8_pairs(v2, c2);
+              merge_lists(tv, ti, ninth2, [&](int s, float& x, int& cx) { x = v2[s]; cx = c2[s]; });
+            }
             // the two warps may have read the bound at different times: what is at or above the larger one is a
             // real element of the row (each warp's fillers lie below its own bound)
-            tau_pub = max(tau_key, (unsigned)xi[(kCandPerTile + 1) * 32]);
+            tau_pub = max(tau_key, (unsigned)xw[64]);
           }
         }
         xchg_phase ^= 1u << acc;
@@ -676,8 +767,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
           ci[1] = make_int4(j0 + ti[4], j0 + ti[5], j0 + ti[6], j0 + ti[7]);
           cand_ninth[slot] = tv[kCandPerTile];
           if (publish_tau) {
-            // this tile's r-th largest goes to slot (n_tile + r k/8) mod k: no two (tile, rank) pairs are the same
-            // element, eight consecutive feature tiles fill every slot, and every slot sees all ranks over time
+            // this tile's r-th candidate goes to slot (n_tile + r k/8) mod k: no two (tile, rank) pairs are the same
+            // element, eight consecutive feature tiles fill every slot, and every slot sees all places over time
             unsigned* sp = tau_slots + p * kTauSlots;
             bool raised_min = false;
             const int rank_step = max(k_row / kCandPerTile, 1);
@@ -718,11 +809,9 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
           if (valid) {
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
-              const float4 b4 = kStageVec ? *reinterpret_cast<const float4*>(wb + (c - c_lo) + i)
-                                          : __ldg(reinterpret_cast<const float4*>(bias_t + (c - c_lo) + i));
+              const float4 b4 = *reinterpret_cast<const float4*>(wb + (c - c_lo) + i);
               float4 s4 = make_float4(1.f, 1.f, 1.f, 1.f);
-              if (kScaled) s4 = kStageVec ? *reinterpret_cast<const float4*>(ws + (c - c_lo) + i)
-                                          : __ldg(reinterpret_cast<const float4*>(wsc_t + (c - c_lo) + i));
+              if (kScaled) s4 = *reinterpret_cast<const float4*>(ws + (c - c_lo) + i);
               if (kE4) { s4.x *= ars; s4.y *= ars; s4.z *= ars; s4.w *= ars; }
               float4 o;
               o.x = kScaled ? fmaf(v[i], s4.x, b4.x) : v[i] + b4.x;
@@ -762,7 +851,9 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
       if (lane == 0) {     // the accumulator is free: tell the CTA that issues the instructions
         if (kPair && !leader) mbar_arrive_cluster(mapa_cluster(smem_u32(&sh->tmem_empty[acc]), 0));
         else mbar_arrive(smem_u32(&sh->tmem_empty[acc]));
+        mbar_arrive(smem_u32(&sh->vec_empty[vec]));
       }
+      if (++vec == kVecs) { vec = 0; vec_phase ^= 1u; }
       acc ^= 1u;
       if (acc == 0) acc_phase ^= 1u;
     }

@@ -149,6 +149,13 @@ __device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Contiguous bytes into shared memory (both addresses on 16 bytes, a multiple of 16), counted on an mbarrier.
+__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
 // ---- CTA pairs (a cluster of two CTAs working on one 256-row tile with tcgen05 cta_group::2) ----
 // Rank of this CTA in its cluster; the shared::cluster address of the same variable in CTA `rank` of the cluster;
 // a cluster-wide barrier; an arrival on an mbarrier that may live in the peer CTA.
