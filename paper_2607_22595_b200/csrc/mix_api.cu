@@ -384,10 +384,11 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
     if (e == cudaSuccess && !(cfg->flags & MIX_FLAG_ENCODE_SIMT)) {
       if (load_encode_fn() != MIX_OK)
         e = cudaErrorUnknown;
-      else if ((cfg->flags & MIX_FLAG_FP8_W_ENC)    // codes: P rows (8-bit input) or 2 P rows (hi, lo) in the same buffer
-                   ? make_tmap_e4m3(&c->tmap_panel, c->d_panel, 2ull * c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK
-                   : make_tmap(&c->tmap_panel, c->d_panel, c->panel_rows_cap, cfg->d_model, kTileM) != MIX_OK)
-        e = cudaErrorUnknown;
+      for (int i = 0; i < kPanelBoxes && e == cudaSuccess; ++i)
+        if ((cfg->flags & MIX_FLAG_FP8_W_ENC)       // codes: P rows (8-bit input) or 2 P rows (hi, lo) in the same buffer
+                ? make_tmap_e4m3(&c->tmap_panel.box[i], c->d_panel, 2ull * c->panel_rows_cap, cfg->d_model, panel_box_rows(i)) != MIX_OK
+                : make_tmap(&c->tmap_panel.box[i], c->d_panel, c->panel_rows_cap, cfg->d_model, panel_box_rows(i)) != MIX_OK)
+          e = cudaErrorUnknown;
       if (e == cudaSuccess && c->d_act_scale) e = cudaMemset(c->d_act_scale, 0, c->panel_rows_cap * sizeof(float));
       if (e == cudaSuccess) e = encode_tc_prepare();
     }

@@ -119,6 +119,15 @@ struct MapInstall {
 };
 constexpr int kMapPending = 8;
 
+// Panel maps by the rows of their boxes.  What bounds the encode of a call with one narrow tile per SM is what an SM takes in,
+// some 45 bytes a clock, and a tile of few rows has no use for 128 rows of panel.
+constexpr int kPanelBoxes = 5;
+__host__ __device__ constexpr int panel_box_rows(int i) { return i == 0 ? 16 : 32 * i; }
+static_assert(panel_box_rows(kPanelBoxes - 1) == kTileM, "the last box takes a whole tile");
+struct PanelMaps {
+  CUtensorMap box[kPanelBoxes];
+};
+
 struct Ctx {
   mix_config cfg;
   int device;
@@ -184,7 +193,7 @@ struct Ctx {
   float* d_part_logits;     // [part_items(T_max)][128 rows][32] tensor-core probe kernel: partial logits of tiles whose columns are cut into parts
   int* d_part_done;         // [kPPartItems][4] finished parts of each quarter of a tile (zeroed by the census)
   CUtensorMap tmap_w_one;   // where d_tmap_w is null (the allocation-free call): the one weight set's map, at this call's tile width
-  CUtensorMap tmap_panel;   // panel map (box kTileK x kTileM, 128B swizzle)
+  PanelMaps tmap_panel;     // panel maps (boxes of kTileK columns, 128B swizzle)
 
   // probe/steer kernels run beside the SAE chain on this stream (created with the context)
   cudaStream_t side_stream;

@@ -3,14 +3,15 @@
 //   Z[p, j] = sum_i panel[p, i] * W_enc[j, i] + b_eff[j]        bf16 x bf16 -> fp32
 //
 // One persistent CTA per SM walks a device-built tile schedule (group, feature tile, row tile).
-// Warp roles:  warp 0 = TMA producer (panel tile 128x64 and W_enc tile 256x64 -- or 128x64, 64x64 where a call has few
-// tiles -- per k-block into a ring of 128-byte-swizzled shared memory: TcCfg::kStages of full-width tiles, up to kMaxStages
-// of narrower ones), warp 1 = MMA issuer (tcgen05.mma 128x256x16, fp32 accumulators in tensor memory, double
-// buffered so the epilogue of one tile overlaps the main loop of the next), warps 2..9 = epilogue, two per
-// tensor-memory lane quarter with 128 columns of the tile each (tcgen05.ld, + bias -- the warp's columns of it
-// copied to shared memory before the accumulator is waited for -- then either the fp32 pre-activations to the Z
+// Warp roles:  warp 0 and the last two = TMA producers, each with every third k-block (panel tile 128x64 and W_enc tile 256x64
+// -- or 128x64, 64x64 where a call has few tiles -- into a ring of 128-byte-swizzled shared memory: TcCfg::kStages of
+// full-width tiles, up to kMaxStages of narrower ones), warp 1 = MMA issuer (tcgen05.mma 128x256x16, fp32 accumulators in tensor
+// memory, double buffered so the epilogue of one tile overlaps the main loop of the next), warps 2..9 = epilogue, two per
+// tensor-memory lane quarter with 128 columns of the tile each (tcgen05.ld, + bias, which came with the tile
+// -- then either the fp32 pre-activations to the Z
 // scratch, or -- for TopK weight sets -- only the tile's 8 largest values per row plus its 9th, which the tail
-// kernel turns into the exact TopK; the two warps of a quarter merge their lists through shared memory).
+// kernel turns into the exact TopK; the two warps of a quarter put their lists together through shared memory).
+// Producers and issuer run their loops as whole warps and elect a lane for the instructions (elect_one says why).
 // A second form (kPair) runs on clusters of two CTAs that share a 256-row tile through
 // tcgen05.mma.cta_group::2; which form works on a call is decided on the device (see TcCfg).
 // No TMA multicast in either form.  Every wait is bounded: on expiry the CTA raises
@@ -36,9 +37,11 @@ namespace mix {
 
 namespace {
 
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 16;
 constexpr int kABytes = kTileM * kTileK * 2;   // 16 KiB: 128 rows of 128 bytes
 constexpr int kBBytes = kTileN * kTileK * 2;   // 32 KiB: 256 rows of 128 bytes
+constexpr int kCopyWarps = 3;                   // producers, each with every third k-block
+constexpr int kSharedBytes = 1280;               // room for TcShared
 constexpr int kVecs = 4;                        // tiles whose bias and scale are in shared memory
 // An epilogue warp's list of a TopK tile: up to 8 values a row and a place for what is one too many, [entry][lane], then their
 // columns.  The lists that are handed over are followed by three words a row: 9th value, number of entries, bound.
@@ -55,19 +58,20 @@ template <int kEnc, int kEpi, bool kPair> struct TcCfg {
   static constexpr int kStageBytes = kARingBytes + kBBytesCta;        // (of a full-width tile; narrower tiles leave room for more stages)
   static constexpr int kStages = kPair ? (kSplit ? 4 : 6) : (kSplit ? 3 : 4);
   static constexpr int kRingBytes = kStages * kStageBytes;
+  static_assert(kStages >= kCopyWarps, "the producers' turns");
   // epilogue warps: 4 (one per tensor-memory lane quarter, all 256 columns) or 8 (two per quarter, 128 columns
   // each; the two top-9 lists of a row meet in shared memory).  One warp per scheduler runs the epilogue's
   // dependent compare/select chains at a fraction of the issue rate; two interleave.
   static constexpr int kEpiWarps = kEpi;
   static constexpr int kXchgBytes = kEpiWarps == 8 ? 2 * 4 * kXchgListBytes : 0;   // [acc][quarter]: the upper-half warps' lists
-  static constexpr int kThreads = 64 + kEpiWarps * 32;
+  static constexpr int kThreads = (kCopyWarps + 1 + kEpiWarps) * 32;      // (and the issuer)
   // The bias (and, for codes, the feature scale) of a tile's columns comes with the tile: the producer copies it into one of
   // kVecs places.  bf16 kernels keep the thresholds of each epilogue warp's columns behind them.
   static constexpr int kVecBytes = (kEnc != 0 ? 2 : 1) * kTileN * 4;
   static constexpr int kEpiVecBytes = 2 * 4 * kTileN * 4;
   static_assert(kVecs * kVecBytes + (kEnc == 0 ? 4 * kTileN * 4 : 0) <= kEpiVecBytes, "the tiles' vectors");
   static constexpr int kPickBytes = kEpiWarps == 8 ? 4 * kListBytes : 0;                 // the lower-half warps' lists
-  static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + 1024 /* TcShared */ + kXchgBytes + kEpiVecBytes + kPickBytes;
+  static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + kSharedBytes + kXchgBytes + kEpiVecBytes + kPickBytes;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
 constexpr int kTmemCols = 512;                 // two 128 x 256 fp32 accumulators
@@ -92,13 +96,17 @@ struct __align__(8) TcShared {
   short unit0[kMaxGroups + 1];
   int utile0[kMaxGroups + 1];
 };
-static_assert(sizeof(TcShared) <= 1024, "TcShared must fit the space reserved for it");
+static_assert(sizeof(TcShared) <= kSharedBytes, "TcShared must fit the space reserved for it");
 
 using namespace tc;
 
 // Bounded wait on this kernel's shared state.
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, TcShared* sh, unsigned* status) {
   return mbar_wait_bounded(bar, parity, &sh->abort_flag, &sh->wait_cycles, status);
+}
+
+__device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, TcShared* sh, unsigned* status) {
+  return mbar_wait_bounded_warp(bar, parity, &sh->abort_flag, &sh->wait_cycles, status);
 }
 
 constexpr unsigned kIdescPair = idesc_f16(2 * kTileM, kTileN);     // the pair's instruction: M = 256
@@ -246,7 +254,7 @@ __device__ __forceinline__ void merge_lists(float (&v)[kCandPerTile + 1], int (&
 
 template <int kEnc, int kEpi, bool kPair>
 __global__ void __launch_bounds__(TcCfg<kEnc, kEpi, kPair>::kThreads, 1)
-encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_constant__ CUtensorMap tmap_w_one, const CUtensorMap* __restrict__ tmap_w, const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
+encode_tc_kernel(const __grid_constant__ PanelMaps tmap_panel, const __grid_constant__ CUtensorMap tmap_w_one, const CUtensorMap* __restrict__ tmap_w, const RouteState* __restrict__ rs_g, const GroupEntry* __restrict__ groups, int n_groups,
                  float* __restrict__ Z, long long ldz, int d, unsigned* __restrict__ status, int mode,
                  const int* __restrict__ mtile_flag, const int* __restrict__ n_flagged, float* __restrict__ cand_val,
                  int* __restrict__ cand_idx, float* __restrict__ cand_ninth, int cand_tiles, int w_tiled, int test_stall,
@@ -264,10 +272,10 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   // 1024-byte alignment: required by the 128-byte swizzle atoms
   unsigned char* tiles = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   TcShared* sh = reinterpret_cast<TcShared*>(tiles + Cfg::kRingBytes);
-  unsigned char* xchg = reinterpret_cast<unsigned char*>(sh) + 1024;
+  unsigned char* xchg = reinterpret_cast<unsigned char*>(sh) + kSharedBytes;
   float* epi_vec = reinterpret_cast<float*>(xchg + Cfg::kXchgBytes);
   unsigned char* pick = reinterpret_cast<unsigned char*>(epi_vec) + Cfg::kEpiVecBytes;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   // CTA pairs: rank 0 leads (it issues the pair's tensor-core instructions and owns the barriers both CTAs' copies
   // complete on); `worker` numbers the units that walk the tile list -- pairs, or single CTAs
   const int rank = kPair ? (int)cluster_ctarank() : 0;
@@ -308,10 +316,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   __syncthreads();
   // Feature width of this call's tiles: 256, or 128 / 64 where full-width tiles would leave half of the SMs or more without
   // one (decided by the front kernel).  A narrower tile makes a shorter stage, so the ring holds more of them.
-  const int tile_n = kPair ? kTileN : sh->rs.tile_n;
+  const int tile_n = kPair ? kTileN : uniform(sh->rs.tile_n);
   const int n_sub = kTileN / tile_n;                   // tiles per 256 features
-  const int stage_bytes = Cfg::kARingBytes + (kPair ? Cfg::kBBytesCta : tile_n * (kTileK * 2));
-  const int n_stages = min(kMaxStages, Cfg::kRingBytes / stage_bytes);
   const int epi_cols = tile_n / (kEpiWarps / 4);       // columns of a tile per epilogue warp
   if (warp < 2) {
     // this kernel's weight sets (lane g: set g): units (row tiles, or pairs of them) and tiles, numbered through.  The full
@@ -344,126 +350,161 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmap_panel, const __grid_co
   }
   tc_fence_before();
   __syncthreads();
-  const int total_tiles = sh->utile0[n_groups];
+  const int total_tiles = uniform(sh->utile0[n_groups]);
   if (total_tiles == 0) return;            // (both CTAs of a pair see the same)
   if (kPair) cluster_sync_all();           // the peer's barriers are initialised before anything is sent to them
   tc_fence_after();
-  const unsigned tmem_base = sh->tmem_base;
+  const unsigned tmem_base = (unsigned)uniform((int)sh->tmem_base);
   phase_stamp(clk, 27, stamp);
   // (the interleaved order serves the TopK epilogue's running bound; without TopK rows the plain order is a little faster)
   const int uniform_nt = sh->rs.n_topk_rows > 0 ? uniform_feature_tiles(*sh, n_groups) : 0;
   const int num_kb = d / kBlockK;
   auto tile_of = [&](int tile) { return decode_tile<kPair>(*sh, n_groups, tile, uniform_nt, rank); };
+  // The ring.  Where tiles are narrow a CTA has one at most, and its stages hold the panel rows which that one has: smaller
+  // stages, hence more of them, and of the stream of W_enc, which bounds such a call, more is under way (what a tile's
+  // instructions read behind those rows is the stage's own W_enc or the next stage, and the accumulator's rows that come of it
+  // nobody reads; all of it lies inside the CTA's shared memory).
+  int box = kPanelBoxes - 1;                           // panel box: panel_box_rows(box) rows
+  if (!kPair && n_sub > 1 && worker < total_tiles) {
+    const int rows = uniform(tile_of(worker).rows_valid);
+    while (box > 0 && panel_box_rows(box - 1) >= rows) --box;
+  }
+  const int a_bytes = panel_box_rows(box) * (kTileK * 2), a_ring = (kSplit ? 2 : 1) * a_bytes;
+  const int stage_bytes = a_ring + (kPair ? Cfg::kBBytesCta : tile_n * (kTileK * 2));
+  const int n_stages = min(kMaxStages, Cfg::kRingBytes / stage_bytes);
 
-  if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0, vec = 0;
-      unsigned phase = 0, vec_phase = 0;
-      bool ok = true;
-      const unsigned long long stream = l2_evict_first();
-      for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
-        const Tile t = tile_of(tile);
-        if (!tile_wanted(t, groups, mode, mtile_flag)) continue;
-        // (boxes of as many W_enc rows as this kernel's tile has: a map array per width)
-        // (no array: a single weight set whose map came with the launch, at the width the front kernel arrives at too)
-        const CUtensorMap* tw = tmap_w == nullptr ? &tmap_w_one : tmap_w + (kPair || n_sub == 2 ? n_groups : (n_sub == 4 ? 2 * n_groups : 0)) + t.group;
-        const int n256 = t.n_tile / n_sub, row_in_256 = kPair ? rank * (kTileN / 2) : (t.n_tile - n256 * n_sub) * tile_n;
-        // A W_enc tile that one worker alone reads goes through L2 as the first to be evicted: otherwise the stream leaves
-        // nothing of what the short kernels around it live on -- their code, the tables, the rows -- and each of them starts
-        // with a chain of DRAM round trips (91 rows, d = 4096, 16384 features: front 12.3 -> 8.5 us, tail 19.4 -> 15.6).
-        // Tiles that several row tiles share must stay (the mixed batch's encode 441 -> 480 us with the hint).
-        const bool once = sh->unit0[t.group + 1] - sh->unit0[t.group] == 1;
-        const float* b_eff = groups[t.group].b_eff;           // (requested here, used a few k-blocks later)
-        const float* w_scale = groups[t.group].w_scale;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (kb == min(3, num_kb - 1)) {       // (behind the first copies: nothing waits for these before the tile's end)
-            if (!mbar_wait(smem_u32(&sh->vec_empty[vec]), vec_phase ^ 1u, sh, status)) { ok = false; break; }
-            if (!test_stall) {
-              const unsigned bar = smem_u32(&sh->vec_full[vec]), bytes = tile_n * 4;
-              const unsigned dst = smem_u32(epi_vec) + vec * Cfg::kVecBytes;
-              mbar_expect_tx(bar, (kE4 ? 2 : 1) * bytes);
-              bulk_load(dst, b_eff + (size_t)t.n_tile * tile_n, bytes, bar);
-              if (kE4) bulk_load(dst + kTileN * 4, w_scale + (size_t)t.n_tile * tile_n, bytes, bar);
-              if (++vec == kVecs) { vec = 0; vec_phase ^= 1u; }
-            }
-          }
-          if (!mbar_wait(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
-          // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producer never fills a stage, so the consumer's
-          // bounded wait runs out and the whole CTA leaves through the time-out path.
-          if (test_stall) { ok = false; break; }
-          const unsigned bar = smem_u32(&sh->full[stage]);
-          const unsigned sa = smem_u32(tiles + stage * stage_bytes);
-          const unsigned sw = sa + Cfg::kARingBytes;
-          // W_enc tile: rows n_tile * tile_n .. of the row-major matrix, or -- when the weights were re-laid out at
-          // registration (always, for codes) -- rows of block (n256, kb) of the tile-contiguous copy
-          // [S/256][d/kBlockK][256][kBlockK]
-          const int wx = (kE4 || w_tiled) ? 0 : kb * kTileK;
-          const int wy = ((kE4 || w_tiled) ? n256 * num_kb + kb : n256) * kTileN + row_in_256;
-          if (kPair) {
-            // both CTAs' copies complete on the LEADER's barrier, which expects the bytes of both; this CTA
-            // fetches its own 128 panel rows and its half (128 features) of the W_enc tile
-            if (leader) mbar_expect_tx(bar, 2 * stage_bytes);
-            const unsigned bar_c = mapa_cluster(bar, 0);
-            tma_load_2d_pair(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar_c);
-            if (kSplit) tma_load_2d_pair(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar_c);
-            if (once) tma_load_2d_pair_hint(sw, tw, wx, wy, bar_c, stream);
-            else tma_load_2d_pair(sw, tw, wx, wy, bar_c);
-          } else {
-            mbar_expect_tx(bar, stage_bytes);
-            tma_load_2d(sa, &tmap_panel, kb * kBlockK, t.m_tile_global * kTileM, bar);
-            if (kSplit) tma_load_2d(sa + kABytes, &tmap_panel, kb * kBlockK, lo_row0 + t.m_tile_global * kTileM, bar);   // the lo codes
-            if (once) tma_load_2d_hint(sw, tw, wx, wy, bar, stream);
-            else tma_load_2d(sw, tw, wx, wy, bar);
-          }
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+  if (warp == 0 || warp >= 2 + kEpiWarps) {
+    // The producers, warp 0 and the last ones, take the k-blocks in turn.  What a k-block costs one warp is the latency of the
+    // forty instructions around its two copies, 400 cycles, whatever the copies bring; one warp for all of them bounded the
+    // calls with a narrow tile per SM (91 rows, d = 4096, 8192 features: 64 k-blocks in 15.8 us, 12.7 so; 9 rows 15.8 and 11.5).
+    // Turns go on through the tiles: a warp's next k-block is always kCopyWarps further, so that when it looks at a stage of the
+    // ring, which is at least as long, the k-block two rounds before is known to have been consumed -- the parity that it waits
+    // for means one thing only.
+    int first = warp == 0 ? 0 : warp - (1 + kEpiWarps);        // this warp's first k-block of the tile
+    int stage0 = 0, vec = 0;                                   // stage and phase of the tile's first k-block
+    unsigned phase0 = 0, vec_phase = 0;
+    bool ok = true;
+    const unsigned long long stream = l2_evict_first();
+    for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
+      const Tile t = tile_of(tile);
+      if (!tile_wanted(t, groups, mode, mtile_flag)) continue;
+      const int group = uniform(t.group), n_tile = uniform(t.n_tile), row0 = uniform(t.m_tile_global) * kTileM;
+      const CUtensorMap* tp = &tmap_panel.box[box];
+      // (boxes of as many W_enc rows as this kernel's tile has: a map array per width)
+      // (no array: a single weight set whose map came with the launch, at the width the front kernel arrives at too)
+      const CUtensorMap* tw = tmap_w == nullptr ? &tmap_w_one : tmap_w + (kPair || n_sub == 2 ? n_groups : (n_sub == 4 ? 2 * n_groups : 0)) + group;
+      const int n256 = n_tile / n_sub, row_in_256 = kPair ? rank * (kTileN / 2) : (n_tile - n256 * n_sub) * tile_n;
+      // A W_enc tile that one worker alone reads goes through L2 as the first to be evicted: otherwise the stream leaves
+      // nothing of what the short kernels around it live on -- their code, the tables, the rows -- and each of them starts
+      // with a chain of DRAM round trips (91 rows, d = 4096, 16384 features: front 12.3 -> 8.5 us, tail 19.4 -> 15.6).
+      // Tiles that several row tiles share must stay (the mixed batch's encode 441 -> 480 us with the hint).
+      const bool once = uniform(sh->unit0[group + 1] - sh->unit0[group]) == 1;
+      // W_enc tile: rows n_tile * tile_n .. of the row-major matrix, or -- when the weights were re-laid out at
+      // registration (always, for codes) -- rows of block (n256, kb) of the tile-contiguous copy
+      // [S/256][d/kBlockK][256][kBlockK]
+      const bool w_blocks = kE4 || w_tiled;
+      const int wy0 = (w_blocks ? n256 * num_kb : n256) * kTileN + row_in_256;
+      int stage = stage0 + first;
+      unsigned phase = phase0;
+      while (stage >= n_stages) { stage -= n_stages; phase ^= 1u; }
+      unsigned ready = 0u;                                     // the present stage is free, as of one k-block ago
+      for (int kb = first; kb < num_kb; kb += kCopyWarps) {
+        if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(smem_u32(&sh->empty[stage]), phase ^ 1u, sh, status)) { ok = false; break; }
+        // Test hook (MIX_FLAG_TEST_STALL_ENCODE): the producers never fill a stage, so the consumer's
+        // bounded wait runs out and the whole CTA leaves through the time-out path.
+        if (test_stall) { ok = false; break; }
+        int next = stage + kCopyWarps;
+        unsigned next_phase = phase;
+        if (next >= n_stages) { next -= n_stages; next_phase ^= 1u; }      // (n_stages >= kCopyWarps)
+        ready = mbar_test(smem_u32(&sh->empty[next]), next_phase ^ 1u);
+        const unsigned bar = smem_u32(&sh->full[stage]), sa = smem_u32(tiles + stage * stage_bytes), sw = sa + a_ring, on = elect_one();
+        const int wx = w_blocks ? 0 : kb * kTileK, wy = w_blocks ? wy0 + kb * kTileN : wy0;
+        if (kPair) {
+          // both CTAs' copies complete on the LEADER's barrier, which expects the bytes of both; this CTA
+          // fetches its own 128 panel rows and its half (128 features) of the W_enc tile
+          if (leader) mbar_expect_tx(bar, 2 * stage_bytes, on);
+          const unsigned bar_c = mapa_cluster(bar, 0);
+          tma_load_2d_pair(sa, tp, kb * kBlockK, row0, bar_c, on);
+          if (kSplit) tma_load_2d_pair(sa + a_bytes, tp, kb * kBlockK, lo_row0 + row0, bar_c, on);
+          if (once) tma_load_2d_pair_hint(sw, tw, wx, wy, bar_c, stream, on);
+          else tma_load_2d_pair(sw, tw, wx, wy, bar_c, on);
+        } else {
+          mbar_expect_tx(bar, stage_bytes, on);
+          tma_load_2d(sa, tp, kb * kBlockK, row0, bar, on);
+          if (kSplit) tma_load_2d(sa + a_bytes, tp, kb * kBlockK, lo_row0 + row0, bar, on);   // the lo codes
+          if (once) tma_load_2d_hint(sw, tw, wx, wy, bar, stream, on);
+          else tma_load_2d(sw, tw, wx, wy, bar, on);
         }
+        stage = next;
+        phase = next_phase;
       }
-      phase_stamp(clk, 28, stamp);          // the last copy of this CTA has been issued
+      if (warp == 0 && ok) {               // the tile's bias and scale, which nothing waits for before its end
+        if (!mbar_wait_warp(smem_u32(&sh->vec_empty[vec]), vec_phase ^ 1u, sh, status)) break;
+        const unsigned bar = smem_u32(&sh->vec_full[vec]), dst = smem_u32(epi_vec) + vec * Cfg::kVecBytes;
+        const float* b_eff = groups[group].b_eff + (size_t)n_tile * tile_n;
+        const float* w_scale = groups[group].w_scale + (size_t)n_tile * tile_n;
+        if (elect_one()) {
+          mbar_expect_tx(bar, (kE4 ? 2 : 1) * tile_n * 4);
+          bulk_load(dst, b_eff, tile_n * 4, bar);
+          if (kE4) bulk_load(dst + kTileN * 4, w_scale, tile_n * 4, bar);
+        }
+        if (++vec == kVecs) { vec = 0; vec_phase ^= 1u; }
+      }
+      first = (first + kCopyWarps - num_kb % kCopyWarps) % kCopyWarps;
+      const int laps = (stage0 + num_kb) / n_stages;
+      stage0 += num_kb - laps * n_stages;
+      phase0 ^= (unsigned)(laps & 1);
     }
+    if (warp == 0) phase_stamp(clk, 28, stamp);          // the last copy of this CTA has been issued (if it is this warp's)
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    if (leader) {
       const unsigned idesc = kE4 ? idesc_e4m3(kTileM, tile_n) : idesc_f16(kTileM, tile_n);   // D fp32, operands K-major
       int stage = 0;
-      unsigned phase = 0, acc = 0, acc_phase = 0;
+      unsigned phase = 0, acc = 0, acc_phase = 0, ready = 0u;
       bool ok = true;
       for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
         if (mode != 0 && !tile_wanted(tile_of(tile), groups, mode, mtile_flag)) continue;
-        if (!mbar_wait(smem_u32(&sh->tmem_empty[acc]), acc_phase ^ 1u, sh, status)) break;
+        if (!mbar_wait_warp(smem_u32(&sh->tmem_empty[acc]), acc_phase ^ 1u, sh, status)) break;
         tc_fence_after();
         const unsigned d_tmem = tmem_base + acc * kTileN;
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(smem_u32(&sh->full[stage]), phase, sh, status)) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(smem_u32(&sh->full[stage]), phase, sh, status)) { ok = false; break; }
           tc_fence_after();
           const unsigned sa = smem_u32(tiles + stage * stage_bytes);
-          const unsigned sb = sa + Cfg::kARingBytes;
+          const unsigned sb = sa + a_ring;
           const unsigned long long da = umma_desc(sa), db = umma_desc(sb);
+          const unsigned on = elect_one();
+          const int next = stage + 1 == n_stages ? 0 : stage + 1;
+          const unsigned next_phase = next == 0 ? phase ^ 1u : phase;
+          ready = mbar_test(smem_u32(&sh->full[next]), next_phase);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {   // 16 bf16 or 32 codes = 32 bytes = 2 descriptor units per step
             const unsigned accum = (unsigned)((kb | k) != 0);
             if (kPair) {
-              if (kE4) umma_e4m3_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescE4Pair, accum);
-              else umma_f16_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescPair, accum);
+              if (kE4) umma_e4m3_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescE4Pair, accum, on);
+              else umma_f16_pair(d_tmem, da + 2ull * k, db + 2ull * k, kIdescPair, accum, on);
             } else {
-              if (kE4) umma_e4m3(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum);
-              else umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum);
+              if (kE4) umma_e4m3(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum, on);
+              else umma_f16(d_tmem, da + 2ull * k, db + 2ull * k, idesc, accum, on);
             }
           }
           if (kSplit) {                   // + lo W into the same accumulator
-            const unsigned long long dl = umma_desc(sa + kABytes);
+            const unsigned long long dl = umma_desc(sa + a_bytes);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              if (kPair) umma_e4m3_pair(d_tmem, dl + 2ull * k, db + 2ull * k, kIdescE4Pair, 1u);
-              else umma_e4m3(d_tmem, dl + 2ull * k, db + 2ull * k, idesc, 1u);
+              if (kPair) umma_e4m3_pair(d_tmem, dl + 2ull * k, db + 2ull * k, kIdescE4Pair, 1u, on);
+              else umma_e4m3(d_tmem, dl + 2ull * k, db + 2ull * k, idesc, 1u, on);
             }
           }
           // the stage is free again -- in both CTAs of a pair
-          if (kPair) umma_commit_pair(smem_u32(&sh->empty[stage]));
-          else umma_commit(smem_u32(&sh->empty[stage]));
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+          if (kPair) umma_commit_pair(smem_u32(&sh->empty[stage]), on);
+          else umma_commit(smem_u32(&sh->empty[stage]), on);
+          stage = next;
+          phase = next_phase;
         }
         if (!ok) break;
-        if (kPair) umma_commit_pair(smem_u32(&sh->tmem_full[acc]));
-        else umma_commit(smem_u32(&sh->tmem_full[acc]));
+        if (kPair) umma_commit_pair(smem_u32(&sh->tmem_full[acc]), elect_one());
+        else umma_commit(smem_u32(&sh->tmem_full[acc]), elect_one());
         acc ^= 1u;
         if (acc == 0) acc_phase ^= 1u;
       }

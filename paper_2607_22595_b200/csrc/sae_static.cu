@@ -222,8 +222,9 @@ extern "C" int mix_sae_apply_static(void* hidden, int n_rows, int d_model, const
   c.h_groups = &ge;
   // The tensor maps travel with the launches (they name addresses of this call only).
   const int n_tiles = (int)(w->d_sae / kTileN);
-  if (make_tmap(&c.tmap_panel, c.d_panel, kStaticRows, d_model, kTileM) != MIX_OK ||
-      make_tmap(&c.tmap_w_one, w->W_enc, (unsigned long long)w->d_sae, d_model, tile_width(n_tiles, n_tiles, c.n_sms, c.cand_tiles)) != MIX_OK)
+  bool mapped = true;
+  for (int i = 0; i < kPanelBoxes; ++i) mapped = mapped && make_tmap(&c.tmap_panel.box[i], c.d_panel, kStaticRows, d_model, panel_box_rows(i)) == MIX_OK;
+  if (!mapped || make_tmap(&c.tmap_w_one, w->W_enc, (unsigned long long)w->d_sae, d_model, tile_width(n_tiles, n_tiles, c.n_sms, c.cand_tiles)) != MIX_OK)
     return fail(errbuf, errbuf_len, MIX_ERR_CUDA, "cuTensorMapEncodeTiled failed");
 
   // The array keeps whatever the previous call left: one small kernel rewrites every table this call reads,

@@ -17,8 +17,10 @@ __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)_
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+// `on` in this and the other instructions below that one thread issues: only where it is not 0 (see elect_one).
+__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes, unsigned on = 1u) {
+  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %2, 0;\n\t@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}"
+               ::"r"(bar), "r"(bytes), "r"(on) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -33,6 +35,19 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity) {
       : "r"(bar), "r"(parity)
       : "memory");
   return ok != 0;
+}
+
+// The same without waiting at all: has the phase completed?
+__device__ __forceinline__ unsigned mbar_test(unsigned bar, unsigned parity) {
+  unsigned ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
 }
 
 // Bounded wait.  Returns false if the wait ran longer than *cap_p clock cycles (the caller's CTA
@@ -57,10 +72,42 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity,
   return true;
 }
 
-__device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar) {
+// The same by a whole warp, which gets one answer.
+__device__ __forceinline__ bool mbar_wait_bounded_warp(unsigned bar, unsigned parity, volatile int* abort_flag,
+                                                       const long long* cap_p, unsigned* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const long long cap = *cap_p;
+  const long long t0 = clock64();
+  unsigned spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++spins & 255u) == 0u) {
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+      if (__any_sync(0xffffffffu, clock64() - t0 > cap)) {
+        *abort_flag = 1;
+        if ((threadIdx.x & 31) == 0) atomicOr(status, MIX_STATUS_WAIT_TIMEOUT);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// One lane of a converged warp, the same one every time.  A loop that issues copies or tensor-core instructions is run by the
+// whole warp with this around the instructions themselves: their operands then live in uniform registers.  Inside a branch that
+// one lane has taken each operand is moved there first, instruction by instruction -- 328 cycles to issue the four tcgen05.mma
+// and the commit of a k-block.
+__device__ __forceinline__ unsigned elect_one() {
+  unsigned one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one;
+}
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+__device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar, unsigned on = 1u) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "r"(on)
       : "memory");
 }
 
@@ -71,10 +118,12 @@ __device__ __forceinline__ unsigned long long l2_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ void tma_load_2d_hint(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar, unsigned long long policy) {
+__device__ __forceinline__ void tma_load_2d_hint(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar, unsigned long long policy,
+                                                 unsigned on = 1u) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %6, 0;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n\t}"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy), "r"(on)
       : "memory");
 }
 
@@ -95,12 +144,12 @@ __host__ __device__ constexpr unsigned idesc_f16(int m, int n) {
 }
 
 __device__ __forceinline__ void umma_f16(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned idesc,
-                                         unsigned accumulate) {
+                                         unsigned accumulate, unsigned on = 1u) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on)
       : "memory");
 }
 // kind::f8f6f4 with both operands E4M3 (format code 0), D fp32, both K-major: one instruction takes
@@ -109,16 +158,17 @@ __host__ __device__ constexpr unsigned idesc_e4m3(int m, int n) {
   return (1u << 4) | ((unsigned)(n >> 3) << 17) | ((unsigned)(m >> 4) << 24);
 }
 __device__ __forceinline__ void umma_e4m3(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned idesc,
-                                          unsigned accumulate) {
+                                          unsigned accumulate, unsigned on = 1u) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on)
       : "memory");
 }
-__device__ __forceinline__ void umma_commit(unsigned bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void umma_commit(unsigned bar, unsigned on = 1u) {
+  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+               ::"r"(bar), "r"(on) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -178,44 +228,48 @@ __device__ __forceinline__ void mbar_arrive_cluster(unsigned cluster_addr) {
 // Tile load of one CTA of a pair: the data lands in THIS CTA's shared memory, the completion bytes are counted on
 // a barrier given by its shared::cluster address, which may be the peer's (the pair's leader waits on one barrier
 // for both halves of a stage).  No multicast: each CTA fetches its own half.
-__device__ __forceinline__ void tma_load_2d_pair(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar_cluster) {
+__device__ __forceinline__ void tma_load_2d_pair(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar_cluster, unsigned on = 1u) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster), "r"(on)
       : "memory");
 }
 __device__ __forceinline__ void tma_load_2d_pair_hint(unsigned dst, const CUtensorMap* map, int x, int y, unsigned bar_cluster,
-                                                      unsigned long long policy) {
+                                                      unsigned long long policy, unsigned on = 1u) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster), "l"(policy)
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %6, 0;\n\t"
+      "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n\t}"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster), "l"(policy), "r"(on)
       : "memory");
 }
 // One instruction of the pair: M = 256 (rows 0..127 from the A tile in the leader's shared memory, 128..255 from
 // the peer's, accumulators in each CTA's own tensor memory), N = 256 with each CTA's shared memory holding 128 of
 // the B rows.  Issued by one thread of the leader CTA.
 __device__ __forceinline__ void umma_f16_pair(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned idesc,
-                                              unsigned accumulate) {
+                                              unsigned accumulate, unsigned on = 1u) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on)
       : "memory");
 }
 __device__ __forceinline__ void umma_e4m3_pair(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned idesc,
-                                               unsigned accumulate) {
+                                               unsigned accumulate, unsigned on = 1u) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on)
       : "memory");
 }
 // Arrives, once the instructions issued so far have completed, on the barrier at this offset in BOTH CTAs of the pair.
-__device__ __forceinline__ void umma_commit_pair(unsigned bar) {
+__device__ __forceinline__ void umma_commit_pair(unsigned bar, unsigned on = 1u) {
   const unsigned short mask = 3;
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(mask)
+  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %2, 0;\n\t"
+               "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+               ::"r"(bar), "h"(mask), "r"(on)
                : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(unsigned smem_slot, unsigned cols) {
