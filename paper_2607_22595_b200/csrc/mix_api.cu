@@ -735,7 +735,10 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   const unsigned long long capture = capture_of(s);
   const bool capturing = capture != 0;
   const int n_fill = map_fill(c, T_live, capturing);
-  const bool by_kernel = c->cfg.n_groups_max == 0;
+  // (Contexts with weight sets: short maps by the copy, whose long kernels leave the translation of the host page cold; from
+  // kMapSaeRows on the kernel, in whose place a copy and what it waits for on either side take 15 us.  8192 rows, d = 5120: the call
+  // 642 -> 618 us; 512 ... 2048 rows: no difference that could be told.)
+  const bool by_kernel = c->cfg.n_groups_max == 0 || T_live > kMapSaeRows;
   // where a kernel can read the map (a copy takes words that do not lie on 4 bytes too)
   const int* src = token_slot;
   if (T_live > 0 && !src_is_device) src = by_kernel ? device_view(token_slot, T_live) : nullptr;

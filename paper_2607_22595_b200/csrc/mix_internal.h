@@ -324,6 +324,7 @@ cudaError_t edit_only_prepare();   // opt in to the dynamic shared memory of the
 // The step's slot map, from memory the device can address or from the host; rows [T_live, n_fill) are set to -1.
 constexpr int kMapCopyRows = 256;          // a pinned map of up to this many rows, where the device has up to kMapCopyHooks
 constexpr int kMapCopyHooks = 3;           // contexts without weight sets, is installed by a copy
+constexpr int kMapSaeRows = 2048;          // contexts with weight sets: longer pinned maps are read by a kernel
 constexpr int kMapParamRows = 896;         // rows of a map that can travel as kernel parameters (3.5 of 4 KiB)
 cudaError_t launch_install_map(const Ctx* c, const int* src, int T_live, int n_fill, cudaStream_t s);
 cudaError_t launch_install_map_params(const Ctx* c, const int* host_src, int T_live, int n_fill, cudaStream_t s);   // 1 <= T_live <= kMapParamRows

@@ -1,5 +1,7 @@
 """The slot map from every place it can come from, shrinking and growing from call to call: rows behind the live ones
 pass through whatever the maps before had there."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -253,4 +255,42 @@ def test_a_map_in_memory_that_is_registered_in_part():
         torch.cuda.synchronize()
     finally:
         cudart.cudaHostUnregister(memory.ctypes.data + page)
+    m.destroy()
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_long_pinned_maps_of_a_context_with_weight_sets(captured, shift):
+    """Above 2048 live rows a kernel reads the map where it lies; at 2048 and below, and where it does not lie on four bytes, a
+    copy takes it.  Lengths up and down across the line, each install followed by a call."""
+    d, T = 64, 2200
+    m = Mix(d_model=d, T_max=T, n_slots_max=2, n_groups_max=1, d_sae_max=256)
+    for slot in range(2):
+        m.register_steer(slot, torch.ones(d, device="cuda", dtype=torch.bfloat16), slot + 1.0)
+    h = torch.zeros((T, d), device="cuda", dtype=torch.bfloat16)
+    rng = np.random.default_rng(shift)
+    for n in (2049, 2048, T, 1, 2100, 0, T):
+        slots = rng.integers(-1, 2, size=n).astype(np.int32)
+        pinned = torch.zeros(4 * n + 8, dtype=torch.uint8).pin_memory()
+        address = pinned.data_ptr() + shift
+        ctypes.memmove(address, slots.ctypes.data, 4 * n)
+        install = lambda: m._check(m.lib.mix_set_slot_map(m.ctx, address, n, 0, torch.cuda.current_stream().cuda_stream))
+        h.zero_()
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                install()
+                m.apply(h)
+            graph.replay()
+        else:
+            install()
+            m.apply(h)
+        torch.cuda.synchronize()
+        want = np.zeros(T, dtype=np.float32)
+        want[:n] = slots + 1.0
+        assert np.array_equal(h.float().cpu().numpy(), np.repeat(want[:, None], d, 1)), n
+        if captured:
+            del graph
+    assert m.get_status() == 0
     m.destroy()
