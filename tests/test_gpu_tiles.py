@@ -258,3 +258,53 @@ def test_padding_rows_of_a_tile_are_zero():
     assert np.array_equal(z[5:, :S], np.broadcast_to(b, (123, S)))
     assert not np.array_equal(z[:5, :S], np.broadcast_to(b, (5, S)))
     m.destroy()
+# k-blocks of a tile with every remainder of the producers' turns, several tiles a CTA (S / 256 = 300 tiles and more), on the rings
+# of three to six stages that full tiles have: bf16 on single CTAs (100 rows) and pairs (200), and both 8-bit forms
+@pytest.mark.parametrize("k_blocks", [1, 2, 3, 4, 5, 7, 8])
+@pytest.mark.parametrize("T", [100, 200])
+@pytest.mark.parametrize("fp8", [None, "weights", "input"])
+def test_turns_of_the_producers(k_blocks, T, fp8):
+    w = _workload(k_blocks * (64 if fp8 is None else 128), 300 * 256, T, W.SAE_TOPK, False, fp8=fp8)
+    sample = np.random.default_rng(k_blocks).choice(T, 6, replace=False)
+    out = run_gpu(w, flags={None: 0, "weights": 32, "input": 96}[fp8], graph=True, replays=2)
+    check_parity(W.host(w), out, rows=np.sort(sample))
+
+
+# rows for the panel boxes of 16 ... 128 rows, beside a set whose tiles have other rows
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 48, 65, 95, 98, 112])
+@pytest.mark.parametrize("act", [W.SAE_TOPK, W.SAE_JUMPRELU])
+def test_panel_boxes(T, act):
+    w = _workload(320, 2048, T + 5, act, True, n_sets=2)
+    w.token_slot[:] = np.minimum(np.arange(T + 5) // T, 1)
+    check_parity(W.host(w), run_gpu(w, graph=True, replays=2))
+
+
+@pytest.mark.parametrize("S", [1024, 128 * 256, 400 * 256])     # narrow tiles, one wave of full ones, waves with a bound in force
+@pytest.mark.parametrize("kind", ["zeros", "steps", "clustered"])
+def test_topk_of_values_that_tie_or_crowd(S, kind):
+    """Pre-activations that equal one another at and around a tile's 8th value, many zeros among them, and winners that crowd
+    in a few tiles (more than 8 of a tile, in one half of it or in both): ids and values must be the exact TopK, of equal values
+    the lower id."""
+    d, T, k = 64, 40, 24
+    w = _workload(d, S, T, W.SAE_TOPK, False, k=k)
+    g = torch.Generator(device="cuda"); g.manual_seed(S)
+    sw = w.groups[0]
+    sw.W_enc[:] = 0                                             # z[t, j] = 8 hidden[t, j % 8] * step[j] + bias[j], all exact
+    cols = torch.arange(S, device="cuda")
+    if kind == "zeros":
+        level = torch.where(torch.rand(S, generator=g, device="cuda") < 0.004, 1.0, 0.0)
+        sw.b_enc[:] = 0
+    elif kind == "steps":
+        level = torch.randint(-2, 3, (S,), generator=g, device="cuda").float()
+        sw.b_enc[:] = 0.5
+    else:
+        level = torch.where((cols % 256 >= 120) & (cols % 256 < 136) & (cols // 256 % 3 == 0), 1.0, -1.0)
+        sw.b_enc[:] = (cols % 5).float() * 0.25
+    sw.W_enc[cols, cols % 8] = level.to(torch.bfloat16)
+    w.hidden[:] = torch.randint(1, 4, (T, d), generator=g, device="cuda").to(torch.bfloat16)
+    out = run_gpu(w, graph=True, replays=2)
+    z = (w.hidden.float() @ sw.W_enc.float().T + sw.b_enc).cpu().numpy()
+    for t in range(T):
+        want = np.lexsort((np.arange(S), -z[t]))[:k]
+        assert np.array_equal(out["topk_idx"][t, :k], want), (t, out["topk_idx"][t, :k], want)
+        assert np.array_equal(out["topk_val"][t, :k], z[t][want])
