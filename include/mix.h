@@ -385,7 +385,8 @@ int mix_get_status(mix_ctx* ctx, unsigned* bits, void* stream);
    1 without SAE weight sets, else 7 (4 with MIX_FLAG_ENCODE_SIMT); one more when T_max > 2048
    and C_max > 1 (multi-class probes of large batches run in a kernel of their own), and two more
    with MIX_FLAG_SAE_EDIT_ONLY.  An uncaptured call leaves two of the 7 out until a TopK set is
-   registered: they serve its fallback. */
+   registered: they serve its fallback.  With T_max <= 2048 and without MIX_FLAG_SLOT_CHAINS the
+   first two are one launch, unless the timing taps below are on. */
 int mix_launches_per_apply(const mix_ctx* ctx);
 
 /* Per-kernel timing taps (profiling only; do not use while capturing a graph).  events: HOST

@@ -929,7 +929,12 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // (programmatic launch only where this kernel directly follows the caller's work in the caller's stream)
   const bool hook_pdl = !fork && !tc && !c->stage_events_on;
   const unsigned long long capture = c->n_map_pending || c->map_captured ? capture_of(s) : 0;
-  MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, map_is_pending(c, s, capture)));
+  // (In a small context with weight sets these rows go with the front kernel's launch, unless chains put its rows behind them or
+  // hooks are not to be launched programmatically, for A/B timing.)
+  const bool merged = c->cfg.n_groups_max > 0 && hook_pdl && (pdl_mask() & kPdlHook) && c->cfg.T_max <= kTeamMaxRows &&
+                      !(c->cfg.flags & MIX_FLAG_SLOT_CHAINS);
+  const HookRows rows = {scores_out, map_is_pending(c, s, capture) ? kPdlMapAhead : 1};
+  if (!merged) MIX_CUDA(c, launch_probe_steer(c, h, T, scores_out, ps, hook_pdl, map_is_pending(c, s, capture)));
   map_arrived(c, s, capture);
   MIX_CUDA(c, tap());
   if (has_multiclass_stage(c) && !tc_fork) {
@@ -947,7 +952,7 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   if (fork) MIX_CUDA(c, cudaEventRecord(c->ev_join, ps));
   if (c->cfg.n_groups_max > 0) {
     // (with slot chains a steering app may precede an SAE app on the same row: the hook kernel is in front of this one)
-    MIX_CUDA(c, launch_front(c, h, T, s, small && !c->stage_events_on, handle, conditional ? 1 : 0));   // routing + row pack
+    MIX_CUDA(c, launch_front(c, h, T, s, small && !c->stage_events_on, handle, conditional ? 1 : 0, merged ? &rows : nullptr));   // routing + row pack
     MIX_CUDA(c, tap());
     const int rc = conditional ? sae_chain_conditional(c, h, s, graph, handle) : sae_chain(c, h, s, tap);
     if (rc != MIX_OK) return rc;

@@ -293,8 +293,13 @@ cudaError_t launch_router(const Ctx* c, float* logits, int n_experts, int T, cud
 // Routing + row pack in one launch.  cond/use_cond: graph-conditional handle the kernel sets to (SAE rows
 // routed > 0); plain calls pass 0, 0
 // pdl: the kernel in front of it in the stream is the hook kernel
-cudaError_t launch_front(const Ctx* c, const __nv_bfloat16* hidden, int T, cudaStream_t s, bool pdl = false, unsigned long long cond = 0,
-                         int use_cond = 0);
+// rows: the rows of the other apps are part of the launch (see front_kernel), which then follows the caller's own work.
+struct HookRows {
+  float* scores;
+  int pdl;                           // 1 or kPdlMapAhead: as launch_probe_steer tells its kernels
+};
+cudaError_t launch_front(const Ctx* c, __nv_bfloat16* hidden, int T, cudaStream_t s, bool pdl = false, unsigned long long cond = 0,
+                         int use_cond = 0, const HookRows* rows = nullptr);
 int front_chunks(int T_max);       // chunks of token rows the front kernel classifies: sizes d_front_counts / d_front_sync
 // bf16 [rows, d] row-major, boxes of 64 columns x box_rows rows, 128-byte swizzle; host work only
 int make_tmap(CUtensorMap* out, const void* base, unsigned long long rows, int d, int box_rows);

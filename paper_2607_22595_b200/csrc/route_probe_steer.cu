@@ -7,47 +7,12 @@
 #include <type_traits>
 
 #include "mix_internal.h"
+#include "hook_row.cuh"
 #include "row_lookup.cuh"
 
 namespace mix {
 
 namespace {
-
-__device__ __forceinline__ void unpack8(const uint4& q, float* f) {
-  const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&q);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float2 t = __bfloat1622float2(p[i]);
-    f[2 * i] = t.x;
-    f[2 * i + 1] = t.y;
-  }
-}
-
-__device__ __forceinline__ uint4 pack8(const float* f) {
-  uint4 q;
-  __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(&q);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-  return q;
-}
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Four sums over the warp with 6 exchanges instead of 20; lanes 8c .. 8c + 7 return that of v[c].  (The same additions as in
-// warp_sum, hence the same bits.)
-__device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
-  const bool b16 = lane & 16, b8 = lane & 8;
-  const float a0 = (b16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, b16 ? v[0] : v[2], 16);
-  const float a1 = (b16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, b16 ? v[1] : v[3], 16);
-  float z = (b8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b8 ? a0 : a1, 8);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-  return z;
-}
 
 // h + alpha v for one row; nvec = d / 8 16-byte vectors.  The `stride` threads that share the
 // row start at `first` (a warp: lane, 32; a CTA team: threadIdx.x, blockDim.x).
@@ -136,39 +101,6 @@ __device__ __forceinline__ void probe_dots(const uint4* const* __restrict__ h, c
   for (int r = 0; r < RB; ++r)
 #pragma unroll
     for (int c = 0; c < NC; ++c) out[r][c] = warp_sum(acc[r][c]);
-}
-
-// 1 / (1 + e^-z) with the hardware exponential and reciprocal: a few instructions instead of the two library
-// routines' hundred on the one-warp tail of a decode step (0.28 us of a 3 us step); the relative error stays
-// below 1e-5 for |z| < 80, two orders under the 1e-3 the scores are held to.
-__device__ __forceinline__ float fast_sigmoid(float z) { return __frcp_rn(1.f + __expf(-z)); }
-
-// Logits (bias included) of one row in `logit` -> scores.  One warp; C <= 64.
-__device__ __forceinline__ void finish_probe(const float* logit, int C, int act, float* __restrict__ out, int lane) {
-  if (C == 1) {                                  // the decode step's case: one lane, no cross-lane work
-    if (lane == 0) {
-      const float z = logit[0];
-      out[0] = act == MIX_ACT_NONE ? z : (act == MIX_ACT_SOFTMAX ? 1.f : fast_sigmoid(z));
-    }
-    return;
-  }
-  float z0 = lane < C ? logit[lane] : -INFINITY;
-  float z1 = lane + 32 < C ? logit[lane + 32] : -INFINITY;
-  if (act == MIX_ACT_SOFTMAX) {
-    float m = fmaxf(z0, z1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const float e0 = lane < C ? expf(z0 - m) : 0.f;
-    const float e1 = lane + 32 < C ? expf(z1 - m) : 0.f;
-    const float sum = warp_sum(e0 + e1);
-    z0 = e0 / sum;
-    z1 = e1 / sum;
-  } else if (act == MIX_ACT_SIGMOID) {
-    z0 = fast_sigmoid(z0);
-    z1 = fast_sigmoid(z1);
-  }
-  if (lane < C) out[lane] = z0;
-  if (lane + 32 < C) out[lane + 32] = z1;
 }
 
 constexpr int kCoopMaxClasses = 32;    // widest probe the cooperative tensor-core pass takes
@@ -393,11 +325,6 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
 // step's next layers are there, their look-ups done, when the present one ends).  The row's loads are issued as soon as the slot id is known to be
 // >= 0, in parallel with the app-table lookup, so a cold row costs two dependent round trips
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
-// Eight warps: with sixteen, which leaves each thread half as much, the sums over the warps cost more than that saves (187 rows
-// of a three-app chain, d = 5120: 38 us for four layers against 33).
-constexpr int kHookWarps = 8;
-constexpr int kMostVec = 4;     // kHookWarps * 32 * kMostVec * 8 >= d_model: 8192 columns
-
 enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
 
 template <int NV, TeamForm kForm>
