@@ -891,9 +891,9 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // joined back into the caller's stream with events, which stream capture turns into graph
   // edges), the SAE chain on the caller's stream.  With the timing taps on, everything runs in
   // order on the caller's stream so that the per-stage times mean something.
-  // In contexts of up to 2048 rows the hook kernel is a few microseconds, less than fork and join cost on the host and on
-  // the stream: there both run in the caller's stream, the front kernel launched programmatically, so that its look-ups
-  // overlap the hook kernel (tiny configuration, eagerly: 41 -> 38 us; 555 rows with 8-bit input: 213 -> 203).
+  // In contexts of up to 2048 rows the hook rows are a few microseconds, less than fork and join cost on the host and on
+  // the stream (tiny configuration, eagerly: 41 -> 38 us; 555 rows with 8-bit input: 213 -> 203): there they are part of the
+  // front kernel's launch, or, with chains, a kernel in front of it, the front kernel launched programmatically.
   const bool small = c->cfg.T_max <= kTeamMaxRows || (c->cfg.flags & MIX_FLAG_SLOT_CHAINS);
   const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on && !small;
   cudaStream_t ps = fork ? c->side_stream : s;

@@ -315,7 +315,7 @@ __device__ __forceinline__ void write_route(const FrontArgs& a, int total, int n
 //      the small count table and scans it.  The publishing CTAs never wait before they publish, and CTAs are dispatched in
 //      index order, so whoever waits, waits for work that is already running.  The rows of a CTA are found through the
 //      scan and the published records.
-// Launched programmatically behind the hook kernel of a small context: what is read before the wait is the slot map and the
+// Launched programmatically behind the caller's work, or the hook kernel, of a small context: what is read before the wait is the slot map and the
 // tables, as in that kernel; gates, `hidden` and everything that is written come after it.
 // Then CTA b packs panel rows [8 b, 8 b + 8), one per warp.  The last CTA -- whose panel rows a call seldom needs -- writes
 // what exists once (routing result, tile -> weight-set map, conditional handle), beside the others' packing.  The last CTA
