@@ -321,14 +321,16 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
 }
 
 // Small batches (decode): one CTA per row, the row held in registers (NV 16-byte vectors per thread, a kernel for each width:
-// 64 registers up to d = 4096 where one for all widths had 126, i.e. four CTAs on an SM instead of two, so that the kernels of a
-// step's next layers are there, their look-ups done, when the present one ends).  The row's loads are issued as soon as the slot id is known to be
+// 52 ... 72 registers up to d = 4096 where one for all widths had 126, i.e. three or four CTAs on an SM instead of two, so that the
+// kernels of a step's next layers are there, their look-ups done, when the present one ends; held to 64, i.e. four CTAs, the form of
+// two vectors was no faster there, 148 us for 32 layers, and slower where probes are wide: 22 rows, 16 classes, three layers 28.0 us
+// against 26.0).  The row's loads are issued as soon as the slot id is known to be
 // >= 0, in parallel with the app-table lookup, so a cold row costs two dependent round trips
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
 enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
 
 template <int NV, TeamForm kForm>
-__global__ void __launch_bounds__(kHookWarps * 32, NV <= 2 ? 4 : 2)
+__global__ void __launch_bounds__(kHookWarps * 32, NV == 1 ? 4 : (NV == 2 ? 3 : 2))
 probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
                         const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
