@@ -544,7 +544,9 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
 // Bound by the chain of dependent loads: link -> entry -> gate -> score -> vector, app after app.  All of it that the
 // library owns -- links, entries, gate entries, single vectors (in the arena) -- is read ahead of the programmatic wait, into
 // shared memory, while the layer or hook in front still runs; behind the wait everything the caller owns is requested together
-// (row, gate scores, biases), and the probes' partial logits meet once, behind the last app.
+// (row, gate scores, biases), and the probes' partial logits meet once, behind the last app -- unless a gate further down the
+// chain looks at a score that an earlier probe of the chain writes: separate calls decide it on the new score, so the probes in
+// front of it are finished before its turn.
 constexpr int kChainStaged = 2;      // single vectors of a chain that are staged (later ones are loaded when their turn comes)
 
 struct ChainStep {
@@ -561,9 +563,12 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
 }
 
-// NV: 16-byte vectors of the row per thread.
+// NV: 16-byte vectors of the row per thread.  (The bounds hold the CTAs an SM takes to what the registers came to by themselves
+// before a chain could stop half-way.  That costs the chains that do not stop 0.5 us over four layers of 187 rows, d = 5120: 31.7 ->
+// 32.2 us, with the comparison of addresses in the walk and the turn back marked as the rare one; with the scores finished by a
+// second copy of the code below it was 33.5, with the comparison behind the wait 33.2.)
 template <int NV>
-__global__ void __launch_bounds__(kHookWarps * 32)
+__global__ void __launch_bounds__(kHookWarps * 32, NV == 1 ? 4 : (NV == 2 ? 3 : 2))
 probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
                          const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates,
                          const int* __restrict__ chain_next, int n_slots, __nv_bfloat16* __restrict__ hidden, int d,
@@ -573,6 +578,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
   __shared__ float s_dot[kMaxChain][kHookWarps];
   __shared__ ChainStep s_step[kMaxChain];
   __shared__ int s_n;
+  __shared__ unsigned s_own;                     // steps whose gate looks at a column of an earlier probe of this chain
   constexpr int NW = kHookWarps, NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
@@ -587,8 +593,10 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
     return;
   }
   const int nvec = d >> 3;
+  float* const row_scores = scores + (size_t)t * C_max;
   if (warp == 0) {                               // the row's apps, in order (every lane reads the same)
     int slot = slot0, n = 0, col = 0, staged = 0;
+    unsigned own_bits = 0u;
     while (n < kMaxChain) {
       const int next = slot >= 0 && slot < n_slots ? __ldg(chain_next + slot) : -1;     // (requested with the entry)
       const RowApp a = lookup(slot, t, apps, gates, n_slots, status, lane == 0, /*eval_gate=*/false);
@@ -604,6 +612,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       if (staged < kChainStaged && (a.kind == MIX_STEER || a.kind == MIX_PROJECT || (a.kind == MIX_PROBE && a.C == 1))) st.staged = staged++;
       st.gate.score = nullptr;
       if (a.kind != 0 && a.gated) st.gate = load_gate(gates, slot, t);
+      if (st.gate.score != nullptr && scores != nullptr && st.gate.score >= row_scores && st.gate.score < row_scores + col) own_bits |= 1u << n;
       if (lane == 0) s_step[n] = st;
       ++n;
       if (!a.chained) break;
@@ -611,7 +620,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       slot = next;                               // (slot was in range: lookup() found a valid entry)
       if (slot < 0) break;
     }
-    if (lane == 0) s_n = n;
+    if (lane == 0) s_n = n, s_own = own_bits;
   }
   __syncthreads();
   const int n = s_n;
@@ -643,7 +652,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
 #pragma unroll
   for (int i = 0; i < kMaxChain; ++i) {
     score[i] = 0.f;
-    if (i < n && s_step[i].gate.score != nullptr) score[i] = __ldg(s_step[i].gate.score);
+    if (i < n && s_step[i].gate.score != nullptr) score[i] = ld_score(s_step[i].gate.score);
   }
   float bias_lo = 0.f, bias_hi = 0.f;            // of the probe that this warp will finish
   if (warp < n && s_step[warp].kind == MIX_PROBE) {
@@ -660,9 +669,13 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
   for (int i = 0; i < kMaxChain; ++i)
     if (i < n && s_step[i].kind != 0 && (s_step[i].gate.score == nullptr || gate_passes(s_step[i].gate, score[i]))) open |= 1u << i;
   asm volatile("cp.async.wait_all;" ::: "memory");
+  unsigned own = s_own, finished = 0u;
   bool dirty = false;
+  int i = 0;
+again:                                           // up to the next step that is gated on a score of this chain
+  const int end = __builtin_expect(own != 0u, 0) ? __ffs(own) - 1 : n;
 #pragma unroll 1
-  for (int i = 0; i < n; ++i) {
+  for (; i < end; ++i) {
     if (!((open >> i) & 1u)) continue;
     const ChainStep& st = s_step[i];
     const int kind = st.kind;
@@ -747,7 +760,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       }
     }
   }
-  if (dirty) {
+  if (own == 0u && dirty) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
@@ -755,7 +768,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
     }
   }
   __syncthreads();
-  if (scores != nullptr && warp < n && ((open >> warp) & 1u) && s_step[warp].kind == MIX_PROBE) {       // a warp per probe
+  if (scores != nullptr && warp < end && (((open & ~finished) >> warp) & 1u) && s_step[warp].kind == MIX_PROBE) {       // a warp per probe
     const ChainStep& st = s_step[warp];
     for (int c = lane; c < st.C; c += 32) {
       float z = c < 32 ? bias_lo : bias_hi;
@@ -764,7 +777,17 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       s_part[0][st.col + c] = z;     // only this lane reads or writes the column from here on
     }
     __syncwarp();
-    finish_probe(&s_part[0][st.col], st.C, st.act, scores + (size_t)t * C_max + st.col, lane);
+    finish_probe(&s_part[0][st.col], st.C, st.act, row_scores + st.col, lane);
+  }
+  if (__builtin_expect(own != 0u, 0)) {
+    // The score that step `end` is gated on now stands where separate calls would leave it; if that probe's gate was closed, it is
+    // what was there before.
+    finished = (1u << end) - 1u;
+    __syncthreads();
+    open &= ~(1u << end);
+    if (gate_passes(s_step[end].gate, ld_score(s_step[end].gate.score))) open |= 1u << end;
+    own &= own - 1u;
+    goto again;
   }
 }
 

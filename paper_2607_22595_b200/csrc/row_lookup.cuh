@@ -31,6 +31,13 @@ __device__ __forceinline__ RowGate load_gate(const GateEntry* __restrict__ gates
   r.thr = __int_as_float(g1.y);
   return r;
 }
+// The score, by a load that neither the compiler nor a cache answers with what was there earlier: the kernel in front, whose end a
+// programmatic launch waits for half-way, or an earlier probe of the same chain may just have written it.
+__device__ __forceinline__ float ld_score(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
 // Does a row with this score pass?  (NaN fails both comparisons.)
 __device__ __forceinline__ bool gate_passes(const RowGate& g, float score) { return g.cmp == MIX_GATE_GE ? score >= g.thr : score < g.thr; }
 __device__ __forceinline__ bool gate_open(const GateEntry* __restrict__ gates, int s, int t) {

@@ -277,3 +277,112 @@ def test_every_width_chained_and_one_by_one(d, T):
             assert bool(((sc[rows, col:col + Wm.shape[0]].double() - want).abs() <= bound).all())
     steered = (h.double() + 1.5 * v.double()).float().to(torch.bfloat16)
     assert bool(((before["project"] - steered)[hooked].abs() <= steered[hooked].abs() * 2.0 ** -7 + 1e-30).all())
+
+
+# ------------------------------------------------------------------ gates on scores of the same chain
+# app: (kind, gate), gate: (column of the chain's scores, comparison, threshold) or None; "p1" and "p2" have one class, "wide" has five
+OWN_GATES = {
+    "write on a raw logit": [("p1", None), ("steer", (0, W.GATE_GE, 0.0))],
+    "write on a softmax class": [("steer", None), ("wide", None), ("project", (3, W.GATE_LT, 0.2))],
+    "read on a read on a read": [("p1", None), ("wide", (0, W.GATE_GE, 0.0)), ("p2", (2, W.GATE_GE, 0.2)), ("steer", (6, W.GATE_LT, 0.0))],
+    "two on one, the second on its opposite": [("project", None), ("p2", None), ("steer", (0, W.GATE_GE, 0.0)), ("p1", (0, W.GATE_LT, 0.0))],
+    "own column and a later probe's": [("p1", (0, W.GATE_GE, 0.0)), ("steer", (2, W.GATE_GE, 0.2)), ("wide", None)],
+}
+CLASSES = {"p1": 1, "p2": 1, "wide": 5}
+
+
+@pytest.mark.parametrize("d,T", [(64, 9), (2112, 64), (8192, 21), (320, 2049)])
+@pytest.mark.parametrize("form", sorted(OWN_GATES))
+def test_a_gate_on_a_score_of_its_own_chain_is_decided_as_separate_calls_decide_it(form, d, T):
+    """Separate calls that write the same score buffer decide a gate on what an earlier probe of the chain has just written there,
+    or, where that probe's gate was closed or the probe comes later, on what was there before.  The buffer holds the opposite
+    decisions to begin with.  Above 2048 rows the kernels add in another order: there a row counts if its gated scores lie
+    further from their thresholds than two such sums may differ (n = d products of fp32: 2 n 2^-24 times the sum of their
+    magnitudes, which is at most the product of the norms, here below twice the row's), and a written row is equal to one rounding
+    to bf16 per write."""
+    mixlib = _mixlib()
+    apps = OWN_GATES[form]
+    C = 7
+    g = torch.Generator(device=DEV); g.manual_seed(d + T)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device=DEV)
+    h = rnd(T, d).to(torch.bfloat16)
+    Wt = {k: (rnd(n, d) * d ** -0.5).to(torch.bfloat16) for k, n in CLASSES.items()}
+    bias = {k: rnd(n) for k, n in CLASSES.items()}
+    v, r = [(rnd(d) * d ** -0.5).to(torch.bfloat16) for _ in range(2)]
+    slots = torch.where(torch.arange(T, device=DEV) % 4 == 3, -1, 0).to(torch.int32)
+
+    def register(m, s, kind, gate, buf):
+        if kind in CLASSES:
+            m.register_probe(s, Wt[kind], bias[kind], mixlib.MIX_ACT_SOFTMAX if kind == "wide" else mixlib.MIX_ACT_NONE)
+        elif kind == "steer":
+            m.register_steer(s, v, 1.5)
+        else:
+            m.register_project(s, r, 0.75)
+        if gate is not None:
+            m.set_gate(s, buf, column=gate[0], cmp=gate[1], threshold=gate[2])
+
+    def buffer(old):              # the scores, and room behind them for a call whose first column is not the buffer's
+        flat = torch.zeros((T + 1) * C, device=DEV)
+        flat[:T * C] = old.flatten()
+        return flat
+
+    def separate(old):
+        flat, x, col = buffer(old), h.clone(), 0
+        for kind, gate in apps:
+            m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=1, C_max=C)
+            register(m, 0, kind, gate, flat[:T * C].view(T, C))
+            m.set_slot_map(slots, T)
+            m.apply(x, flat[col:col + T * C].view(T, C))
+            torch.cuda.synchronize()
+            assert m.get_status() == 0
+            m.destroy()
+            col += CLASSES.get(kind, 0)
+        return x, flat[:T * C].view(T, C)
+
+    def chained(old, graph):
+        flat, x = buffer(old), h.clone()
+        scores = flat[:T * C].view(T, C)
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=len(apps), C_max=C, flags=mixlib.MIX_FLAG_SLOT_CHAINS)
+        for s, (kind, gate) in enumerate(apps):
+            register(m, s, kind, gate, scores)
+        for s in range(len(apps) - 1):
+            m.set_chain(s, s + 1)
+        m.set_slot_map(slots, T)
+        s = torch.cuda.Stream(); s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            if graph:
+                gr = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(gr, stream=s):
+                    m.apply(x, scores, stream=s)
+                gr.replay()
+            else:
+                m.apply(x, scores, stream=s)
+        torch.cuda.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+        return x, scores
+
+    cuts = {c: t for _, gate in apps if gate is not None for c, _, t in [gate]}
+    fresh = separate(torch.full((T, C), 9.0, device=DEV))[1]
+    old = 9.0 - fresh
+    for c, thr in cuts.items():
+        old[:, c] = 2 * thr - fresh[:, c]
+    want_x, want_s = separate(old)
+    hooked = slots == 0
+    if T > 2048:
+        near = torch.zeros(T, dtype=torch.bool, device=DEV)
+        for c, thr in cuts.items():
+            near |= (want_s[:, c] - thr).abs() <= 2 * d * 2.0 ** -24 * 2 * h.float().norm(dim=1)
+        assert int(near.sum()) < T // 8
+        rows = ~near
+    else:
+        rows = torch.ones(T, dtype=torch.bool, device=DEV)
+    for graph in (False, True):
+        x, sc = chained(old, graph)
+        if T > 2048:
+            diff = (x.float() - want_x.float()).abs()[rows]
+            assert bool((diff <= (want_x.float().abs()[rows] + 1.5 * v.float().abs()) * 2.0 ** -7 + 1e-6).all())
+            assert bool(((sc - want_s).abs()[rows] <= SCORE_TOL).all())
+        else:
+            assert torch.equal(x, want_x) and torch.equal(sc, want_s)
+        assert torch.equal(x[~hooked], h[~hooked]) and torch.equal(sc[~hooked], old[~hooked])
