@@ -114,7 +114,7 @@ __device__ __forceinline__ void team_row(int first_cta, const int* __restrict__ 
     }
   }
   float score = 0.f;
-  if (a.gated) score = __ldg(gate.score);        // (requested with the row)
+  if (a.gated) score = ld_score(gate.score);     // (requested with the row)
   // A one-class probe's bias came with the entry (registration put it into the `alpha` word); the biases of a
   // wider probe are requested as soon as the entry is here, not after the dot products they are added to.
   float bias_lo = 0.f, bias_hi = 0.f;

@@ -411,7 +411,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
     }
   }
   float score = 0.f;
-  if (a.gated) score = __ldg(gate.score);        // (requested with the row)
+  if (a.gated) score = ld_score(gate.score);     // (requested with the row)
   // A one-class probe's bias came with the entry (registration put it into the `alpha` word); the biases of a
   // wider probe are requested as soon as the entry is here, not after the dot products they are added to.
   float bias_lo = 0.f, bias_hi = 0.f;

@@ -31,8 +31,9 @@ __device__ __forceinline__ RowGate load_gate(const GateEntry* __restrict__ gates
   r.thr = __int_as_float(g1.y);
   return r;
 }
-// The score, by a load that neither the compiler nor a cache answers with what was there earlier: the kernel in front, whose end a
-// programmatic launch waits for half-way, or an earlier probe of the same chain may just have written it.
+// The score, by an ordinary load of the GPU's memory: the read-only path (__ldg) is for what nobody writes while the kernel runs, and the
+// kernel in front, which a programmatic launch overlaps, or an earlier probe of the same chain writes scores.  A kernel that starts
+// before the chain kernel in front of it has ended may find rows next to its own in an L1 that this one filled ahead of their probes.
 __device__ __forceinline__ float ld_score(const float* p) {
   float v;
   asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
@@ -42,7 +43,7 @@ __device__ __forceinline__ float ld_score(const float* p) {
 __device__ __forceinline__ bool gate_passes(const RowGate& g, float score) { return g.cmp == MIX_GATE_GE ? score >= g.thr : score < g.thr; }
 __device__ __forceinline__ bool gate_open(const GateEntry* __restrict__ gates, int s, int t) {
   const RowGate g = load_gate(gates, s, t);
-  return gate_passes(g, __ldg(g.score));
+  return gate_passes(g, ld_score(g.score));
 }
 
 // Slot -> app for row t; flags bad slot ids; applies the slot's gate.  `leader` is the one

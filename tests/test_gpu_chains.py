@@ -386,3 +386,57 @@ def test_a_gate_on_a_score_of_its_own_chain_is_decided_as_separate_calls_decide_
         else:
             assert torch.equal(x, want_x) and torch.equal(sc, want_s)
         assert torch.equal(x[~hooked], h[~hooked]) and torch.equal(sc[~hooked], old[~hooked])
+
+
+@pytest.mark.parametrize("T,classes", [(96, 1), (700, 3), (2200, 2)])
+def test_an_sae_app_gated_on_a_score_of_its_own_chain(T, classes):
+    """The routing kernel, which starts while the chain kernel in front of it still runs, decides the gate on the score that the chain
+    has written, as separate calls do.  The buffer holds the opposite decisions; a row's scores share 32 bytes with its neighbours'."""
+    mixlib = _mixlib()
+    d, S = 256, 512
+    g = torch.Generator(device=DEV); g.manual_seed(T)
+    h = torch.randn((T, d), generator=g, device=DEV).to(torch.bfloat16)
+    sign = torch.where(torch.arange(T, device=DEV) % 2 == 0, 1.0, -1.0)
+    Wp = torch.zeros((classes, d), dtype=torch.bfloat16, device=DEV)
+    Wp[:, 0] = 1.0
+    h[:, 0] = (2.0 * sign).to(torch.bfloat16)                    # the logit: +-2, exactly, in every kernel
+    sae = W.make_sae_weights(g, DEV, d, S, W.SAE_RELU)
+    slots = torch.where(torch.arange(T, device=DEV) % 5 == 4, -1, 0).to(torch.int32)
+
+    def context(n_slots, groups, flags):
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=n_slots, n_groups_max=groups, C_max=classes, k_max=1, r_max=2, d_sae_max=S, flags=flags)
+        if groups:
+            m.register_sae_weights(0, S, sae.act, 0, sae.W_enc, sae.b_enc, sae.W_dec)
+        return m
+
+    def sae_app(m, slot, scores):
+        m.register_sae_app(slot, 0, [3, 300], [2.0, -1.5], [0, 0], True)
+        m.set_gate(slot, scores, column=classes - 1, threshold=0.0)
+
+    def run(m, x, scores):
+        m.set_slot_map(slots, T)
+        s = torch.cuda.Stream(); s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            m.apply(x, scores, stream=s)
+        torch.cuda.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+
+    old = (-2.0 * sign)[:, None].repeat(1, classes)
+    want, want_scores = h.clone(), old.clone()
+    m = context(1, 0, 0)
+    m.register_probe(0, Wp, None, mixlib.MIX_ACT_NONE)
+    run(m, want, want_scores)
+    m = context(1, 1, 0)
+    sae_app(m, 0, want_scores)
+    run(m, want, None)
+    for _ in range(4):
+        x, scores = h.clone(), old.clone()
+        m = context(2, 1, mixlib.MIX_FLAG_SLOT_CHAINS)
+        m.register_probe(0, Wp, None, mixlib.MIX_ACT_NONE)
+        sae_app(m, 1, scores)
+        m.set_chain(0, 1)
+        run(m, x, scores)
+        assert torch.equal(scores, want_scores) and torch.equal(x, want)
+    changed = (want != h).any(dim=1)
+    assert torch.equal(changed, (slots == 0) & (sign > 0))
