@@ -288,7 +288,7 @@ int mix_set_gate(mix_ctx* ctx, int slot, const float* scores, int row_stride, in
    (Above 2048 rows the two add up a probe's logit in different orders: there they agree to fp32 rounding.)
    Every app keeps its own gate: a closed gate skips that app only.  A gate on a score that an earlier probe of the
    same chain writes for the same row in this call is decided on the new score, as in separate calls; one on a score
-   that the call writes for another row may see the old one or the new.  The probes of a chain write
+   that the call writes for another row may see the old one or the new, the row as a whole.  The probes of a chain write
    their scores side by side: a probe's first column in scores_out[t, :] is the total n_classes of
    the chain's earlier probes (whether their gates were open or not), so the sum over a chain
    must not exceed C_max.  An SAE app can only be the last app of a chain; router apps cannot be

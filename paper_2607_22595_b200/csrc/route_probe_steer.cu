@@ -564,9 +564,9 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 }
 
 // NV: 16-byte vectors of the row per thread.  (The bounds hold the CTAs an SM takes to what the registers came to by themselves
-// before a chain could stop half-way.  That costs the chains that do not stop 0.5 us over four layers of 187 rows, d = 5120: 31.7 ->
-// 32.2 us, with the comparison of addresses in the walk and the turn back marked as the rare one; with the scores finished by a
-// second copy of the code below it was 33.5, with the comparison behind the wait 33.2.)
+// before a chain could stop half-way.  That, and the gates decided by one warp for all, costs the chains that do not stop 0.7 us over
+// four layers of 187 rows, d = 5120: 30.9 -> 31.6 us, with the comparison of addresses in the walk and the turn back marked as the
+// rare one; with the scores finished by a second copy of the code below it was 1.3 us more, with the comparison behind the wait 1.0.)
 template <int NV>
 __global__ void __launch_bounds__(kHookWarps * 32, NV == 1 ? 4 : (NV == 2 ? 3 : 2))
 probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
@@ -578,7 +578,8 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
   __shared__ float s_dot[kMaxChain][kHookWarps];
   __shared__ ChainStep s_step[kMaxChain];
   __shared__ int s_n;
-  __shared__ unsigned s_own;                     // steps whose gate looks at a column of an earlier probe of this chain
+  __shared__ unsigned s_free, s_gated, s_own;    // steps without a gate; with one; with one on a column of an earlier probe of this chain
+  __shared__ unsigned s_passed;
   constexpr int NW = kHookWarps, NT = NW * 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
@@ -596,7 +597,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
   float* const row_scores = scores + (size_t)t * C_max;
   if (warp == 0) {                               // the row's apps, in order (every lane reads the same)
     int slot = slot0, n = 0, col = 0, staged = 0;
-    unsigned own_bits = 0u;
+    unsigned free_bits = 0u, gated_bits = 0u, own_bits = 0u;
     while (n < kMaxChain) {
       const int next = slot >= 0 && slot < n_slots ? __ldg(chain_next + slot) : -1;     // (requested with the entry)
       const RowApp a = lookup(slot, t, apps, gates, n_slots, status, lane == 0, /*eval_gate=*/false);
@@ -610,9 +611,16 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       st.b = a.b;
       st.staged = -1;
       if (staged < kChainStaged && (a.kind == MIX_STEER || a.kind == MIX_PROJECT || (a.kind == MIX_PROBE && a.C == 1))) st.staged = staged++;
-      st.gate.score = nullptr;
-      if (a.kind != 0 && a.gated) st.gate = load_gate(gates, slot, t);
-      if (st.gate.score != nullptr && scores != nullptr && st.gate.score >= row_scores && st.gate.score < row_scores + col) own_bits |= 1u << n;
+      // (Registration keeps a chain's columns within C_max.  A walk that a registration on another stream overtakes may meet the old
+      // link and the new, wider probe: it must not leave the row's scores, or shared memory.)
+      if (a.kind == MIX_SAE || (a.kind == MIX_PROBE && col + a.C > C_max)) st.kind = 0;     // (an SAE app: the front kernel's, gate and all)
+      if (st.kind != 0 && a.gated) {
+        st.gate = load_gate(gates, slot, t);
+        if (scores != nullptr && st.gate.score >= row_scores && st.gate.score < row_scores + col) own_bits |= 1u << n;
+        else gated_bits |= 1u << n;
+      } else if (st.kind != 0) {
+        free_bits |= 1u << n;
+      }
       if (lane == 0) s_step[n] = st;
       ++n;
       if (!a.chained) break;
@@ -620,7 +628,7 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       slot = next;                               // (slot was in range: lookup() found a valid entry)
       if (slot < 0) break;
     }
-    if (lane == 0) s_n = n, s_own = own_bits;
+    if (lane == 0) s_n = n, s_free = free_bits, s_gated = gated_bits, s_own = own_bits;
   }
   __syncthreads();
   const int n = s_n;
@@ -648,12 +656,11 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
     if (v < nvec) hq[u] = __ldcs(hrow + v);
   }
   if (!in_arena) stage();
-  float score[kMaxChain];                        // (all requested before one is looked at)
-#pragma unroll
-  for (int i = 0; i < kMaxChain; ++i) {
-    score[i] = 0.f;
-    if (i < n && s_step[i].gate.score != nullptr) score[i] = ld_score(s_step[i].gate.score);
-  }
+  // Gates are decided once for the row, by the first warp, a lane each: a score may be one that another row of this call is just
+  // writing, and threads that read it for themselves could part ways in front of the barriers below.
+  const unsigned gated = s_gated;
+  float score = 0.f;
+  if (warp == 0 && ((gated >> lane) & 1u)) score = ld_score(s_step[lane].gate.score);
   float bias_lo = 0.f, bias_hi = 0.f;            // of the probe that this warp will finish
   if (warp < n && s_step[warp].kind == MIX_PROBE) {
     const ChainStep& st = s_step[warp];
@@ -664,10 +671,15 @@ probe_steer_chain_kernel(const int* __restrict__ token_slot, int T,
       if (lane + 32 < st.C) bias_hi = __ldg(st.b + lane + 32);
     }
   }
-  unsigned open = 0u;                            // (a closed gate skips its app, not the chain behind it)
-#pragma unroll
-  for (int i = 0; i < kMaxChain; ++i)
-    if (i < n && s_step[i].kind != 0 && (s_step[i].gate.score == nullptr || gate_passes(s_step[i].gate, score[i]))) open |= 1u << i;
+  unsigned open = s_free;                        // (a closed gate skips its app, not the chain behind it)
+  if (gated != 0u) {
+    if (warp == 0) {
+      const unsigned passed = __ballot_sync(0xffffffffu, ((gated >> lane) & 1u) && gate_passes(s_step[lane].gate, score));
+      if (lane == 0) s_passed = passed;
+    }
+    __syncthreads();
+    open |= s_passed;
+  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   unsigned own = s_own, finished = 0u;
   bool dirty = false;

@@ -440,3 +440,42 @@ def test_an_sae_app_gated_on_a_score_of_its_own_chain(T, classes):
         assert torch.equal(scores, want_scores) and torch.equal(x, want)
     changed = (want != h).any(dim=1)
     assert torch.equal(changed, (slots == 0) & (sign > 0))
+
+
+@pytest.mark.parametrize("d,T", [(512, 2048), (8192, 700)])
+def test_a_gate_on_another_rows_score_of_the_same_call_decides_the_whole_row(d, T):
+    """Such a gate may see the score that was there or the one that the call writes, in another block at that moment; either way the
+    row is written as a whole, and so are the scores behind the write."""
+    mixlib = _mixlib()
+    g = torch.Generator(device=DEV); g.manual_seed(d)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device=DEV)
+    h = rnd(T, d).to(torch.bfloat16)
+    w1, w5 = [(rnd(n, d) * d ** -0.5).to(torch.bfloat16) for n in (1, 5)]
+    r = (rnd(d) * d ** -0.5).to(torch.bfloat16)
+    slots = torch.zeros(T, dtype=torch.int32, device=DEV)
+    flat = torch.zeros((T + 1) * 6, device=DEV)             # the call's scores, and the row behind them: row t is gated on row t + 1
+    scores, ahead = flat[:T * 6].view(T, 6), flat[6:].view(T, 6)
+
+    def run(old, threshold):
+        flat.fill_(old)
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=3, C_max=6, flags=mixlib.MIX_FLAG_SLOT_CHAINS)
+        m.register_probe(0, w1, None, mixlib.MIX_ACT_NONE)
+        m.register_project(1, r, 0.75)
+        m.set_gate(1, ahead, column=0, threshold=threshold)
+        m.register_probe(2, w5, None, mixlib.MIX_ACT_NONE)
+        m.set_chain(0, 1)
+        m.set_chain(1, 2)
+        m.set_slot_map(slots, T)
+        x = h.clone()
+        m.apply(x, scores)
+        torch.cuda.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+        return x, scores.clone()
+
+    opened, closed = run(9.0, -1e30), run(9.0, 1e30)
+    for old in (-1e9, 1e9, -1e9, 1e9):
+        x, sc = run(old, 0.0)
+        is_open = (x == opened[0]).all(dim=1) & (sc == opened[1]).all(dim=1)
+        is_closed = (x == closed[0]).all(dim=1) & (sc == closed[1]).all(dim=1)
+        assert bool((is_open | is_closed).all()) and not bool((is_open & is_closed).any())
