@@ -274,7 +274,9 @@ int mix_update_sae_edits(mix_ctx* ctx, int slot, int n_edit, const int* idx, con
    the raw logit); it is read when the later mix_apply() runs, so both calls can sit in one
    captured graph.  scores == NULL removes the gate.  Registering the slot again also removes
    it.  Stream-ordered, not captured.  Works for every app kind (a gated probe writes no score
-   for rows whose gate is closed).  Errors: OUT_OF_RANGE (slot), INVALID_ARG (slot not
+   for rows whose gate is closed).  An SAE app may be gated on a score that the same mix_apply() writes for another row, if
+   the gate is set when the call is enqueued or captured: it is decided on the new score.  Any other app on such a score (chains:
+   see below), or on a score that anything else writes while the call runs, is not: the row's threads may see different values.  Errors: OUT_OF_RANGE (slot), INVALID_ARG (slot not
    registered, bad cmp, row_stride < 1, column outside [0, row_stride)). */
 int mix_set_gate(mix_ctx* ctx, int slot, const float* scores, int row_stride, int column, int cmp, float threshold,
                  void* stream);

@@ -87,12 +87,35 @@ void free_all(mix_ctx* c) {
   if (c->owned_w_tiled)
     for (int g = 0; g < c->cfg.n_groups_max; ++g) cudaFree(c->owned_w_tiled[g]);
   free(c->owned_w_tiled);
+  free(c->sae_gates);
   free(c->owned_b_eff); free(c->h_apps); free(c->h_groups); free(c->h_chain_next); free(c->h_edit_idx);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_join2) cudaEventDestroy(c->ev_join2);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->body_stream) cudaStreamDestroy(c->body_stream);
+}
+
+void forget_sae_gate(mix_ctx* c, int slot) {
+  for (int i = 0; i < c->n_sae_gates; ++i)
+    if (c->sae_gates[i].slot == slot) {
+      c->sae_gates[i] = c->sae_gates[--c->n_sae_gates];
+      return;
+    }
+}
+
+// Does an SAE app's gate look at scores that a call on T rows writes for other rows than the one it decides?  (A gate on the same
+// buffer that looks at its own row's columns -- scores of an earlier call, since the row's app is an SAE app -- does not.)
+bool sae_gates_look_across(const mix_ctx* c, const float* scores_out, int T) {
+  if (c->n_sae_gates == 0 || scores_out == nullptr || T == 0) return false;
+  const long long C = c->cfg.C_max, n = T;
+  for (int i = 0; i < c->n_sae_gates; ++i) {
+    const SaeGate& g = c->sae_gates[i];
+    const long long at = ((intptr_t)g.scores - (intptr_t)scores_out) / (long long)sizeof(float);    // of the first score, from the call's first
+    if (at >= n * C || at + (n - 1) * g.stride < 0) continue;
+    if (g.stride != C || at < 0 || at >= C) return true;
+  }
+  return false;
 }
 
 int check_slot(mix_ctx* c, int slot) {
@@ -317,10 +340,11 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   c->h_groups = static_cast<GroupEntry*>(calloc(G > 0 ? G : 1, sizeof(GroupEntry)));
   c->h_chain_next = static_cast<int*>(malloc(NS * sizeof(int)));
   c->h_edit_idx = static_cast<int*>(calloc((size_t)NS * c->cfg.r_max, sizeof(int)));
+  c->sae_gates = static_cast<SaeGate*>(calloc(NS, sizeof(SaeGate)));
   if (c->h_chain_next) memset(c->h_chain_next, 0xff, NS * sizeof(int));
   c->owned_b_eff = static_cast<float**>(calloc(G > 0 ? G : 1, sizeof(float*)));
   c->owned_w_tiled = static_cast<__nv_bfloat16**>(calloc(G > 0 ? G : 1, sizeof(__nv_bfloat16*)));
-  if (!c->h_apps || !c->h_groups || !c->h_chain_next || !c->h_edit_idx || !c->owned_b_eff || !c->owned_w_tiled) { free_all(c); free(c); return MIX_ERR_NO_MEMORY; }
+  if (!c->h_apps || !c->h_groups || !c->h_chain_next || !c->h_edit_idx || !c->sae_gates || !c->owned_b_eff || !c->owned_w_tiled) { free_all(c); free(c); return MIX_ERR_NO_MEMORY; }
   bool ok = true;
   ok = ok && dev_alloc(&c->d_token_slot, T) == cudaSuccess;
   ok = ok && dev_alloc(&c->d_apps, NS) == cudaSuccess;
@@ -378,6 +402,7 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   if (e == cudaSuccess && G > 0) {
     e = cudaMemset(c->d_panel, 0, (size_t)c->panel_rows_cap * cfg->d_model * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMemset(c->d_route, 0, sizeof(RouteState));
+    if (e == cudaSuccess) e = cudaMemset(c->d_row_rec, 0, c->panel_rows_cap * sizeof(RowRec));
     if (e == cudaSuccess) e = cudaMemset(c->d_front_sync, 0, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_panel_row, 0xff, c->panel_rows_cap * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_mtile_group, 0xff, c->panel_rows_cap / kTileM * sizeof(int));
@@ -616,6 +641,7 @@ int mix_register_app(mix_ctx* c, int slot, int kind, const void* desc, void* str
     }
     if (old_next >= 0) MIX_CUDA(c, cudaMemcpyAsync(c->d_chain_next + slot, c->h_chain_next + slot, sizeof(int), cudaMemcpyHostToDevice, s));
   }
+  forget_sae_gate(c, slot);
   // The bias of a one-class probe travels in the entry itself (its `alpha` word is otherwise unused): the
   // one-CTA-per-row kernel then has it with the entry instead of one dependent load later.
   const float* bias_src = (c->d_vec_arena && kind == MIX_PROBE && e.n_classes == 1) ? e.b : nullptr;
@@ -627,6 +653,7 @@ int mix_unregister_app(mix_ctx* c, int slot, void* stream) {
   int rc = check_slot(c, slot);
   if (rc != MIX_OK) return rc;
   memset(&c->h_apps[slot], 0, sizeof(AppEntry));
+  forget_sae_gate(c, slot);
   const int zero = 0;
   MIX_CUDA(c, cudaMemcpyAsync(&c->d_apps[slot].valid, &zero, sizeof(int), cudaMemcpyHostToDevice,
                               static_cast<cudaStream_t>(stream)));
@@ -670,6 +697,7 @@ int mix_set_gate(mix_ctx* c, int slot, const float* scores, int row_stride, int 
   int kind = c->h_apps[slot].kind & ~kKindGated;
   if (!scores) {                      // remove: drop the flag first, the entry may then go stale
     c->h_apps[slot].kind = kind;
+    forget_sae_gate(c, slot);
     MIX_CUDA(c, cudaMemcpyAsync(&c->d_apps[slot].kind, &kind, sizeof(int), cudaMemcpyHostToDevice, s));
     return MIX_OK;
   }
@@ -688,6 +716,8 @@ int mix_set_gate(mix_ctx* c, int slot, const float* scores, int row_stride, int 
     MIX_CUDA(c, cudaMemcpyAsync(&c->d_apps[slot].kind, &kind, sizeof(int), cudaMemcpyHostToDevice, s));
   MIX_CUDA(c, cudaMemcpyAsync(c->d_gates + slot, &g, sizeof(g), cudaMemcpyHostToDevice, s));
   kind |= kKindGated;
+  forget_sae_gate(c, slot);
+  if ((kind & kKindMask) == MIX_SAE) c->sae_gates[c->n_sae_gates++] = {scores + column, slot, row_stride};
   c->h_apps[slot].kind = kind;
   MIX_CUDA(c, cudaMemcpyAsync(&c->d_apps[slot].kind, &kind, sizeof(int), cudaMemcpyHostToDevice, s));
   return MIX_OK;
@@ -894,8 +924,12 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // In contexts of up to 2048 rows the hook rows are a few microseconds, less than fork and join cost on the host and on
   // the stream (tiny configuration, eagerly: 41 -> 38 us; 555 rows with 8-bit input: 213 -> 203): there they are part of the
   // front kernel's launch, or, with chains, a kernel in front of it, the front kernel launched programmatically.
+  // Neither where an SAE app is gated on a score that this call writes for another row: there the hook kernels run in front of the
+  // front kernel, which decides such a gate on the new score.  Beside them it would find some scores written and some not, and its
+  // CTAs, each of which works out the routing of a call of up to 1024 rows for itself, could come to different routings.
+  const bool in_order = sae_gates_look_across(c, scores_out, T);
   const bool small = c->cfg.T_max <= kTeamMaxRows || (c->cfg.flags & MIX_FLAG_SLOT_CHAINS);
-  const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on && !small;
+  const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on && !small && !in_order;
   cudaStream_t ps = fork ? c->side_stream : s;
   if (fork) {
     MIX_CUDA(c, cudaEventRecord(c->ev_fork, s));
@@ -927,7 +961,7 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
     }
   }
   // (programmatic launch only where this kernel directly follows the caller's work in the caller's stream)
-  const bool hook_pdl = !fork && !tc && !c->stage_events_on;
+  const bool hook_pdl = !fork && !tc && !c->stage_events_on && !in_order;
   const unsigned long long capture = c->n_map_pending || c->map_captured ? capture_of(s) : 0;
   // (In a small context with weight sets these rows go with the front kernel's launch, unless chains put its rows behind them or
   // hooks are not to be launched programmatically, for A/B timing.)

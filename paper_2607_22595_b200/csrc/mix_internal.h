@@ -128,6 +128,12 @@ struct PanelMaps {
   CUtensorMap box[kPanelBoxes];
 };
 
+// A gate of an SAE app, as the host knows it: where its scores lie.
+struct SaeGate {
+  const float* scores;      // of column `col` of row 0
+  int slot, stride;
+};
+
 struct Ctx {
   mix_config cfg;
   int device;
@@ -158,6 +164,8 @@ struct Ctx {
   // host mirrors (validation only)
   AppEntry* h_apps;
   GroupEntry* h_groups;
+  SaeGate* sae_gates;       // [n_slots_max], the first n_sae_gates in use
+  int n_sae_gates;
   int topk_seen;            // a TopK set has been registered
   float** owned_b_eff;      // per group: library-owned folded bias or null
   __nv_bfloat16** owned_w_tiled;   // per group: library-owned tile-contiguous copy of W_enc or null

@@ -247,3 +247,58 @@ def test_router_logit_steering_matches_oracle_and_leaves_hidden_alone():
         if ref.kind[t] == 0:
             assert np.array_equal(out["hidden"][t], wh.hidden[t])
     assert out["status"] == mixlib.MIX_STATUS_BAD_SLOT              # slot 7 was never registered
+
+
+@pytest.mark.parametrize("T_max,T", [(64, 64), (1000, 1000), (1500, 1500), (2600, 600), (2600, 2600)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_an_sae_app_gated_on_a_score_that_the_same_call_writes_for_the_row_in_front(T_max, T, graph):
+    """It is decided on the new score, as behind a call for the probes alone; the buffer holds the opposite decisions."""
+    import paper_2607_22595_b200 as mixlib
+    d, S, C = 256, 512, 2
+    g = torch.Generator(device=DEV); g.manual_seed(T_max + T)
+    h = torch.randn((T_max, d), generator=g, device=DEV).to(torch.bfloat16)
+    sign = torch.where(torch.arange(T_max, device=DEV) // 2 % 3 == 0, 1.0, -1.0)
+    Wp = torch.zeros((C, d), dtype=torch.bfloat16, device=DEV)
+    Wp[:, 0] = 1.0
+    h[:, 0] = (2.0 * sign).to(torch.bfloat16)                       # the logits: +-2, exactly, in every kernel
+    sae = W.make_sae_weights(g, DEV, d, S, W.SAE_RELU)
+    slots = (torch.arange(T_max, device=DEV) % 2).to(torch.int32)   # probe, SAE app, probe, ...
+    flat = torch.zeros((T_max + 1) * C, device=DEV)
+    behind, scores = flat[:T_max * C].view(T_max, C), flat[C:].view(T_max, C)      # row t of `behind` is row t - 1 of `scores`
+
+    def run(slot_maps, gate_first):
+        flat.zero_()
+        scores[:T] = (-2.0 * sign)[:T, None]
+        m = mixlib.Mix(d_model=d, T_max=T_max, n_slots_max=2, n_groups_max=1, C_max=C, k_max=1, r_max=2, d_sae_max=S)
+        m.register_sae_weights(0, S, sae.act, 0, sae.W_enc, sae.b_enc, sae.W_dec)
+        m.register_probe(0, Wp, None, mixlib.MIX_ACT_NONE)
+        m.register_sae_app(1, 0, [3, 300], [2.0, -1.5], [0, 0], True)
+        if gate_first:                                              # one that is replaced, taken away and set again
+            m.set_gate(1, torch.zeros((T_max, C), device=DEV), column=0, threshold=1.0)
+            m.set_gate(1, None)
+        m.set_gate(1, behind, column=1, threshold=0.0)
+        x = h.clone()
+        s = torch.cuda.Stream(); s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            for slot_map in slot_maps:
+                m.set_slot_map(slot_map, T)
+                if graph:
+                    gr = torch.cuda.CUDAGraph()
+                    with torch.cuda.graph(gr, stream=s):
+                        m.apply(x, scores, T=T, stream=s)
+                    gr.replay()
+                else:
+                    m.apply(x, scores, T=T, stream=s)
+                s.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+        return x, scores.clone()
+
+    one = [torch.where(slots == k, slots, -1).to(torch.int32) for k in (0, 1)]
+    want = run(one, False)
+    for i in range(4):
+        got = run([slots], i % 2 == 1)
+        assert torch.equal(got[1], want[1]) and torch.equal(got[0], want[0])
+    changed = (want[0] != h).any(dim=1)
+    rows = torch.arange(T_max, device=DEV)
+    assert torch.equal(changed, (slots == 1) & (rows < T) & (sign.roll(1) > 0))
