@@ -327,7 +327,7 @@ probe_multiclass_kernel(const int* __restrict__ token_slot, int T,
 // against 26.0).  The row's loads are issued as soon as the slot id is known to be
 // >= 0, in parallel with the app-table lookup, so a cold row costs two dependent round trips
 // (slot, then entry + data) instead of three.  Control flow is uniform across the CTA.
-enum TeamForm { kTeamPlain, kTeamMapAhead, kTeamLate };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
+enum TeamForm { kTeamPlain, kTeamMapAhead };   // (forms of their own: as flags they cost the plain step 2.81 -> 2.86 us)
 
 template <int NV, TeamForm kForm>
 __global__ void __launch_bounds__(kHookWarps * 32, NV == 1 ? 4 : (NV == 2 ? 3 : 2))
@@ -336,8 +336,7 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
                         __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
                         unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int pdl) {
   __shared__ float s_part[kHookWarps][kMaxClasses];
-  constexpr int NW = kHookWarps, NT = NW * 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NT = kHookWarps * 32;
   const int t = blockIdx.x;                      // < T_max: the slot map has an entry for every row
   // Programmatic dependent launch (`pdl`: the launch asked for it): everything up to pdl_wait() reads only
   // tables the LIBRARY owns -- slot map, app entry, vector arena; copies write them, which are complete before a kernel
@@ -349,12 +348,11 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   // row is then requested together with the vector and the app entry, one round trip earlier.  Behind a map that a
   // kernel installed (kPdlMapAhead) the wait comes first, and only then the trigger: a successor that reads the map
   // early must not start before the map is there.
-  if (kForm == kTeamMapAhead || (kForm == kTeamLate && pdl == kPdlMapAhead)) {
+  if (kForm == kTeamMapAhead) {
     pdl_wait();
     pdl_launch_dependents();
     pdl = 0;
   }
-  constexpr bool kLate = kForm == kTeamLate;
   if (pdl) pdl_launch_dependents();
   const int slot = __ldg(token_slot + t);
   if (t >= T || slot == -1) {
@@ -367,17 +365,15 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   // into row `slot` of the context's vector arena, so their address follows from the slot id
   // alone: the row AND its vector are requested together, before the app entry is known.
   uint4 hq[NV], vq[NV];
-  // (kLate, contexts with SAE weight sets: most rows may be another kernel's; nothing is requested before the entry says
-  // that the row is this one's.  1000 SAE rows of d = 2304: 6.2 -> 4.5 us.)
   const bool slot_ok = slot >= 0 && slot < n_slots;
-  if (!kLate && slot_ok) {
+  if (slot_ok) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
       if (v < nvec) vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
     }
   }
-  if (!kLate && !pdl && slot_ok) {
+  if (!pdl && slot_ok) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
@@ -386,153 +382,30 @@ probe_steer_team_kernel(const int* __restrict__ token_slot, int T,
   }
   // (A hint, so it may come before the wait: what the predecessor still writes of the row, it writes to this L2.  For a step
   // whose hidden states no longer lie there: 32 layers of 256 rows, d = 4096: 2.25 -> 1.9 us a layer.)
-  if (!kLate && pdl && slot_ok && threadIdx.x * 8 < nvec) asm volatile("prefetch.global.L2 [%0];" ::"l"(hrow + threadIdx.x * 8));
+  if (pdl && slot_ok && threadIdx.x * 8 < nvec) asm volatile("prefetch.global.L2 [%0];" ::"l"(hrow + threadIdx.x * 8));
   RowApp a = lookup(slot, t, apps, gates, n_slots, status, threadIdx.x == 0, /*eval_gate=*/false);
   RowGate gate;
   if (a.gated) gate = load_gate(gates, slot, t);
   if (pdl) pdl_wait();
-  if (kLate) {
-    if (a.kind == 0 || a.kind == MIX_SAE || a.kind == MIX_ROUTER) return;
+  if (pdl && slot_ok) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        vq[u] = __ldg(vec_arena + (size_t)slot * nvec + v);
-        hq[u] = __ldcs(hrow + v);
-      }
-    }
-  } else if (pdl) {
-    if (slot_ok) {
-#pragma unroll
-      for (int u = 0; u < NV; ++u) {
-        const int v = threadIdx.x + u * NT;
-        if (v < nvec) hq[u] = __ldcs(hrow + v);
-      }
+      if (v < nvec) hq[u] = __ldcs(hrow + v);
     }
   }
-  float score = 0.f;
-  if (a.gated) score = ld_score(gate.score);     // (requested with the row)
-  // A one-class probe's bias came with the entry (registration put it into the `alpha` word); the biases of a
-  // wider probe are requested as soon as the entry is here, not after the dot products they are added to.
-  float bias_lo = 0.f, bias_hi = 0.f;
-  if (a.kind == MIX_PROBE && warp == 0) {
-    if (a.C == 1) {
-      bias_lo = a.alpha;
-    } else if (a.b != nullptr) {
-      if (lane < a.C) bias_lo = __ldg(a.b + lane);
-      if (lane + 32 < a.C) bias_hi = __ldg(a.b + lane + 32);
-    }
-  }
-  if (a.gated && !gate_passes(gate, score)) return;       // gate closed: the row passes through
-  if (a.kind == MIX_STEER) {
-    if (a.alpha == 0.f) return;                  // identity; the row stays bit-exact
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        float x[8], y[8];
-        unpack8(hq[u], x);
-        unpack8(vq[u], y);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = fmaf(a.alpha, y[e], x[e]);
-        __stcs(hrow + v, pack8(x));
-      }
-    }
-    return;
-  }
-  if (a.kind == MIX_PROJECT) {                 // h - beta (h . r) r
-    if (a.alpha == 0.f) return;
-    float dot = 0.f;
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        float x[8], y[8];
-        unpack8(hq[u], x);
-        unpack8(vq[u], y);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dot = fmaf(x[e], y[e], dot);
-      }
-    }
-    dot = warp_sum(dot);
-    if (lane == 0) s_part[warp][0] = dot;
-    __syncthreads();
-    float total = 0.f;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) total += s_part[w][0];
-    const float coef = -a.alpha * total;
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        float x[8], y[8];
-        unpack8(hq[u], x);
-        unpack8(vq[u], y);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = fmaf(coef, y[e], x[e]);
-        __stcs(hrow + v, pack8(x));
-      }
-    }
-    return;
-  }
-  if (a.kind != MIX_PROBE || scores == nullptr) return;
-  if (a.C == 1) {                              // the probe vector is already here
-    float acc = 0.f;
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        float x[8], y[8];
-        unpack8(hq[u], x);
-        unpack8(vq[u], y);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc = fmaf(x[e], y[e], acc);
-      }
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) s_part[warp][0] = acc;
-  }
-  for (int c0 = 0; c0 < (a.C == 1 ? 0 : a.C); c0 += 4) {
-    const int nc = min(4, a.C - c0);
-    uint4 wq[4][NV];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int u = 0; u < NV; ++u) {
-        const int v = threadIdx.x + u * NT;
-        if (c < nc && v < nvec) wq[c][u] = __ldg(a.W + (size_t)(c0 + c) * nvec + v);
-      }
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * NT;
-      if (v < nvec) {
-        float x[8];
-        unpack8(hq[u], x);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (c < nc) {
-            float y[8];
-            unpack8(wq[c][u], y);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[c] = fmaf(x[e], y[e], acc[c]);
-          }
-      }
-    }
-    const float z = warp_sum4(acc, lane);
-    if ((lane & 7) == 0 && (lane >> 3) < nc) s_part[warp][c0 + (lane >> 3)] = z;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    for (int c = lane; c < a.C; c += 32) {
-      float z = c < 32 ? bias_lo : bias_hi;
-#pragma unroll
-      for (int w = 0; w < NW; ++w) z += s_part[w][c];
-      s_part[0][c] = z;            // only this lane reads or writes column c from here on
-    }
-    __syncwarp();
-    finish_probe(s_part[0], a.C, a.act, scores + (size_t)t * C_max, lane);
-  }
+  row_app<NV>(a, gate, hq, vq, hrow, nvec, scores == nullptr ? nullptr : scores + (size_t)t * C_max, s_part);
+}
+
+// Contexts with weight sets, where these rows are not part of the front kernel's launch (see apply_impl); never launched programmatically.
+template <int NV>
+__global__ void __launch_bounds__(kHookWarps * 32, NV == 1 ? 4 : (NV == 2 ? 3 : 2))
+probe_steer_late_kernel(const int* __restrict__ token_slot, int T,
+                        const AppEntry* __restrict__ apps, const GateEntry* __restrict__ gates, int n_slots,
+                        __nv_bfloat16* __restrict__ hidden, int d, float* __restrict__ scores, int C_max,
+                        unsigned* __restrict__ status, const uint4* __restrict__ vec_arena, int) {
+  __shared__ float s_part[kHookWarps][kMaxClasses];
+  late_row<NV>(0, token_slot, T, apps, gates, n_slots, hidden, d, scores, C_max, status, vec_arena, s_part);
 }
 
 // Contexts with slot chains: one CTA per row, the row held in registers while the apps of its chain
@@ -984,7 +857,7 @@ cudaError_t launch_probe_steer(const Ctx* c, __nv_bfloat16* hidden, int T, float
     };
     auto of_width = [&](auto nv) {
       constexpr int NV = decltype(nv)::value;
-      if (c->cfg.n_groups_max > 0) return run(probe_steer_team_kernel<NV, kTeamLate>);
+      if (c->cfg.n_groups_max > 0) return run(probe_steer_late_kernel<NV>);
       return pdl == kPdlMapAhead ? run(probe_steer_team_kernel<NV, kTeamMapAhead>) : run(probe_steer_team_kernel<NV, kTeamPlain>);
     };
     switch (n_vec) {

@@ -343,7 +343,7 @@ front_kernel(const FrontArgs a) {
     static_assert(kHookWarps * 32 == kFrontThreads, "a CTA per row");
     if (cta >= a.n_front) {
       __shared__ float s_part[kHookWarps][kMaxClasses];
-      team_row<NV>(a.n_front, a.token_slot, a.T, a.apps, a.gates, a.n_slots, a.rows, a.d, a.scores, a.C_max, a.status, a.vec_arena, s_part);
+      late_row<NV>(a.n_front, a.token_slot, a.T, a.apps, a.gates, a.n_slots, a.rows, a.d, a.scores, a.C_max, a.status, a.vec_arena, s_part);
       return;
     }
   }

@@ -792,3 +792,57 @@ def test_weight_sets_dealt_between_single_ctas_and_cta_pairs(rows_per_set):
                    topk_val=tk_val.cpu().numpy(), n_active=n_act.cpu().numpy(), status=m.get_status())
         check_parity(W.host(w), out)
     m.destroy()
+
+
+@pytest.mark.parametrize("d,form", [(d, form) for d in (64, 2048, 2112, 4096, 4160, 6144, 6208, 8192) for form in ("bf16", "fp8", "fp8_act")
+                                    if form == "bf16" or d % 128 == 0])
+def test_every_width_of_the_other_apps_rows_beside_sae_rows(d, form):
+    """Small contexts with weight sets: the rows of probes, steering vectors and projections are part of the routing kernel's launch,
+    whose form follows the row width and the encoder's; with the timing taps on they are a kernel in front of it.  Either way
+    they have the bits that a context without weight sets gives them, and the SAE rows those of a call on them alone."""
+    mixlib = _mixlib()
+    T, S, C = 45, 256, 37
+    flags = {"bf16": 0, "fp8": mixlib.MIX_FLAG_FP8_W_ENC, "fp8_act": mixlib.MIX_FLAG_FP8_W_ENC | mixlib.MIX_FLAG_FP8_ACT}[form]
+    g = torch.Generator(device=DEV); g.manual_seed(d)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device=DEV)
+    h = rnd(T, d).to(torch.bfloat16)
+    probes = [(rnd(n, d) * d ** -0.5).to(torch.bfloat16) for n in (1, 5, C)]
+    v, r = [(rnd(d) * d ** -0.5).to(torch.bfloat16) for _ in range(2)]
+    bias, gate = rnd(C), rnd(T, 1)
+    sae = W.make_sae_weights(g, DEV, d, S, W.SAE_RELU, fp8=form != "bf16")
+    slots = (torch.arange(T, device=DEV) * 7 % 10 - 1).to(torch.int32)             # -1: no app; 7, 8: SAE apps
+
+    def run(with_set, slot_map, taps=False):
+        m = mixlib.Mix(d_model=d, T_max=T, n_slots_max=9, C_max=C, flags=flags if with_set else 0,
+                       **(dict(n_groups_max=1, k_max=1, r_max=2, d_sae_max=S) if with_set else {}))
+        m.register_probe(0, probes[0], bias[:1], mixlib.MIX_ACT_SIGMOID)
+        m.register_steer(1, v, 1.5)
+        m.register_project(2, r, 0.75)
+        m.register_probe(3, probes[1], None, mixlib.MIX_ACT_SOFTMAX)
+        m.register_probe(4, probes[2], bias, mixlib.MIX_ACT_NONE)
+        m.register_project(5, r, -1.25)
+        m.register_probe(6, probes[0], None, mixlib.MIX_ACT_NONE)
+        if with_set:
+            m.register_sae_weights(0, S, sae.act, 0, sae.W_enc, sae.b_enc, sae.W_dec, w_scale=sae.w_scale)
+            m.register_sae_app(7, 0, [3, 200], [2.0, -1.5], [0, 0], True)
+            m.register_sae_app(8, 0, [5], [0.0], [1], False)
+        for s in (4, 5, 6) + ((8,) if with_set else ()):
+            m.set_gate(s, gate, column=0, threshold=0.0)
+        m.set_slot_map(slot_map, T)
+        if taps:
+            m.set_stage_events([torch.cuda.Event(enable_timing=True) for _ in range(m.launches_per_apply() + 1)])
+        x, scores = h.clone(), torch.full((T, C), 7.0, device=DEV)
+        m.apply(x, scores)
+        torch.cuda.synchronize()
+        assert m.get_status() == 0
+        m.destroy()
+        return x, scores
+
+    is_sae = slots >= 7
+    others = run(False, torch.where(is_sae, -1, slots))
+    alone = run(True, torch.where(is_sae, slots, -1))
+    for taps in (False, True):
+        x, scores = run(True, slots, taps)
+        assert torch.equal(scores, others[1])
+        assert torch.equal(x[~is_sae], others[0][~is_sae]) and torch.equal(x[is_sae], alone[0][is_sae])
+    assert bool((alone[0] != h).any(dim=1)[slots == 7].all()) and bool((others[0] != h).any(dim=1)[(slots == 1) | (slots == 2)].all())
