@@ -277,6 +277,15 @@ def test_every_width_chained_and_one_by_one(d, T):
             assert bool(((sc[rows, col:col + Wm.shape[0]].double() - want).abs() <= bound).all())
     steered = (h.double() + 1.5 * v.double()).float().to(torch.bfloat16)
     assert bool(((before["project"] - steered)[hooked].abs() <= steered[hooked].abs() * 2.0 ** -7 + 1e-30).all())
+    # Rows: the write is one fp32 operation per element whatever the kernel, so where the projection's gate is closed a chained row has the
+    # same bits.  Where it is open, the two dot products may differ by twice the bound above, and a bf16 rounding may fall to either side.
+    assert torch.equal(chained[hooked & ~opened], one[hooked & ~opened])
+    s64, r64 = before["project"][opened].double(), r.double()
+    err = 0.75 * (d + 1) * 2.0 ** -24 * (s64.abs() @ r64.abs())[:, None] * r64.abs()
+    projected = s64 - 0.75 * (s64 @ r64)[:, None] * r64
+    for got in (chained, one):
+        diff = (got[opened].double() - projected).abs()
+        assert bool((diff <= err + projected.abs() * (2.0 ** -8 + 2.0 ** -22) + 1e-30).all())
 
 
 # ------------------------------------------------------------------ gates on scores of the same chain
