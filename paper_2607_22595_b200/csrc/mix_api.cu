@@ -402,7 +402,6 @@ int mix_create(mix_ctx** out, const mix_config* cfg) {
   if (e == cudaSuccess && G > 0) {
     e = cudaMemset(c->d_panel, 0, (size_t)c->panel_rows_cap * cfg->d_model * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMemset(c->d_route, 0, sizeof(RouteState));
-    if (e == cudaSuccess) e = cudaMemset(c->d_row_rec, 0, c->panel_rows_cap * sizeof(RowRec));
     if (e == cudaSuccess) e = cudaMemset(c->d_front_sync, 0, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_panel_row, 0xff, c->panel_rows_cap * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_mtile_group, 0xff, c->panel_rows_cap / kTileM * sizeof(int));
