@@ -307,9 +307,10 @@ int mix_set_chain(mix_ctx* ctx, int slot, int next_slot, void* stream);
    Install the token->slot map for the next mix_apply calls: token_slot int32[T_live]
    (host if src_is_device == 0, else device), -1 = no app.  Rows >= T_live are pass-through.
    One operation on the stream into a fixed device buffer: from device memory a kernel; from host memory an async
-   copy or, in contexts without weight sets, mostly a kernel, which reads memory that the device can address where it
-   lies and takes up to 896 rows of any other among its parameters; two operations where a map that is copied is
-   shorter than the one before (the rows in between are set to -1).
+   copy or, in contexts without weight sets mostly and in the others where T_live > 2048, a kernel, which reads memory
+   that the device can address (pinned, registered, managed) where it lies when the stream gets there.  Of any other host
+   memory a context without weight sets takes up to 896 rows among a kernel's parameters, and everything else is copied.  Two
+   operations where a map that is copied is shorter than the one before (the rows in between are set to -1).
    Meant to be called between replays.  A captured call reads its source, which must then stay valid as long as the
    graph, at every replay; from the capture on every install of the context sets all rows up to T_max, since a
    replay may have put a longer map in front of it.
@@ -343,18 +344,19 @@ int mix_set_feature_out(mix_ctx* ctx, int* topk_idx, float* topk_val, int* n_act
    device fp32 [T_max, C_max] or NULL; only the first n_classes entries of probe rows are
    written.  Enqueues kernels on `stream` (when the context has SAE weight sets, more than 2048 rows
    and no slot chains, the probe / steering kernels run on a context-owned side stream forked from and joined back into `stream`
-   by events, so they overlap the SAE chain; in a context for more than 2048 rows with multi-class
-   probes and no SAE weight sets, the two kernels for those run on two such streams beside the
-   streaming kernel) and returns; safe to capture.  In a context without SAE weight sets and
-   T_max <= 2048 the kernel is launched with programmatic stream serialization (see
-   mix_set_pdl_mask): if the kernel in front of it in `stream` lets its successor start early, the
+   by events, so they overlap the SAE chain, unless an SAE app is gated on a score that this call writes for another
+   row; in a context for more than 2048 rows with multi-class probes and no SAE weight sets, the two kernels for
+   those run on two such streams beside the streaming kernel) and returns; safe to capture.  In a context with
+   T_max <= 2048 or slot chains the first kernel is launched with programmatic stream serialization (see
+   mix_set_pdl_mask; not beside such a gate): if the kernel in front of it in `stream` lets its successor start early, the
    part that looks up the slot map, app entry and single-vector weights -- tables the library owns --
    overlaps that kernel (unless that kernel is the one that installed the map); `hidden`, gate scores and
    multi-class probe weights are read only after the predecessor has completed and flushed, and the
    grid does not end before it.  Behind any other kernel nothing changes.  One launch shape follows
    from what is registered when the call is enqueued or captured -- the encode's epilogue warps
    (TopK weight set present or not); this is performance only: either shape handles every
-   registration, so tables rewritten after a capture are still applied correctly.  Device-side
+   registration, so tables rewritten after a capture are still applied correctly (but for the gates just named: see
+   mix_set_gate).  Device-side
    problems (bad slot ids, ...) are reported through the status word, never by faulting.
    Errors: INVALID_ARG (NULL hidden, misaligned), OUT_OF_RANGE (T), CUDA (launch failure). */
 int mix_apply(mix_ctx* ctx, void* hidden, int T, float* scores_out, void* stream);
@@ -386,12 +388,14 @@ int mix_apply_router(mix_ctx* ctx, float* logits, int n_experts, int T, void* st
    reads when it chooses to, never raised as a fault.) */
 int mix_get_status(mix_ctx* ctx, unsigned* bits, void* stream);
 
-/* Number of kernels one mix_apply() call launches on this context (fixed at mix_create):
-   1 without SAE weight sets, else 7 (4 with MIX_FLAG_ENCODE_SIMT); one more when T_max > 2048
-   and C_max > 1 (multi-class probes of large batches run in a kernel of their own), and two more
-   with MIX_FLAG_SAE_EDIT_ONLY.  An uncaptured call leaves two of the 7 out until a TopK set is
-   registered: they serve its fallback.  With T_max <= 2048 and without MIX_FLAG_SLOT_CHAINS the
-   first two are one launch, unless the timing taps below are on. */
+/* Number of stages of one mix_apply() call on this context (fixed at mix_create), which the timing taps below time one
+   by one and which no call exceeds in launches: 1 without SAE weight sets, else 7 (4 with MIX_FLAG_ENCODE_SIMT); with
+   T_max > 2048, C_max > 1 and no MIX_FLAG_SLOT_CHAINS one more (multi-class probes of large batches have a kernel of their own), or three more
+   without weight sets (two kernels, and the census that chooses between them); two more with
+   MIX_FLAG_SAE_EDIT_ONLY.  Without the taps a call may launch fewer kernels: the first two of the 7 (or 4) are one launch where
+   T_max <= 2048 (unless MIX_FLAG_SLOT_CHAINS, a gate that looks at other rows' scores of the call, or
+   mix_set_pdl_mask without the hook kernel's bit keeps them apart), the encode on CTA pairs is left out where no call of the
+   context can use it, and until a TopK set is registered an uncaptured call leaves out the two that serve its fallback. */
 int mix_launches_per_apply(const mix_ctx* ctx);
 
 /* Per-kernel timing taps (profiling only; do not use while capturing a graph).  events: HOST

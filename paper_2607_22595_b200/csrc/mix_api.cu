@@ -765,8 +765,9 @@ int mix_set_slot_map(mix_ctx* c, const int* token_slot, int T_live, int src_is_d
   const bool capturing = capture != 0;
   const int n_fill = map_fill(c, T_live, capturing);
   // (Contexts with weight sets: short maps by the copy, whose long kernels leave the translation of the host page cold; from
-  // kMapSaeRows on the kernel, in whose place a copy and what it waits for on either side take 15 us.  8192 rows, d = 5120: the call
-  // 642 -> 618 us; 512 ... 2048 rows: no difference that could be told.)
+  // kMapSaeRows on the kernel.  8192 rows, d = 5120: 19.0 us from the last kernel of one replay to the first of the next with a copy, 8.3 with
+  // the kernel; maps and replays in a row 609 and 592 us in the median, runs of either differing by more than that; one by one 605 either
+  // way.  512 ... 2048 rows: no difference that could be told.)
   const bool by_kernel = c->cfg.n_groups_max == 0 || T_live > kMapSaeRows;
   // where a kernel can read the map (a copy takes words that do not lie on 4 bytes too)
   const int* src = token_slot;

@@ -695,8 +695,8 @@ router_kernel(const int* __restrict__ token_slot, int T,
 // and more each on the stream and on the host.
 // Contexts without SAE weight sets, of which a step has one per layer, take a map in host memory by kernel too: read over
 // PCIe where it lies if the device can address it (2.9 us of stream time against 4.0 for a copy), among the kernel's
-// parameters if it is pageable and short (1.1 us).  Contexts with weight sets keep the copy: their long kernels leave the
-// translation of the host page cold, and the same read takes 5.3 us.
+// parameters if it is pageable and short (1.1 us).  Contexts with weight sets keep the copy up to 2048 rows: their long kernels
+// leave the translation of the host page cold, and the same read takes 5.3 us.
 // 32 maps of 256 rows and the replay of 32 layers behind them: 260 us with two copies a map, 204 with one, 160 with this.
 // Launched programmatically: a kernel is scheduled while its predecessor ends, and waits for it before it touches
 // anything (the predecessor may still read the old map, or write the source).

@@ -323,8 +323,8 @@ __device__ __forceinline__ void write_route(const FrontArgs& a, int total, int n
 // kPack: 0 the bf16 row, 1 E4M3 hi + lo (exact split), 2 E4M3 quantised.
 // NV > 0 (contexts of up to 2048 rows, without chains): the rows of probes, steering vectors and projections, which no other
 // part of the call touches, go with this launch, a CTA each behind the others, NV vectors of the row a thread.  As a kernel in front
-// of this one they were a launch for the host and 1.1 ... 4 us on the stream: 64 rows called eagerly, d = 512, 35.7 -> 33.9 us; 1000 SAE
-// rows of d = 2304, 206.5 -> 204.2; 91 of d = 4096 in a graph, 61.6 -> 60.9.
+// of this one they were a launch for the host and 1 ... 4 us on the stream: 64 rows called eagerly, d = 512, 34.4 -> 33.5 us; 1000 SAE
+// rows of d = 2304, 206 -> 203.8; 91 of d = 4096 in a graph, 60.5 -> 60.1.
 template <int kPack, int NV>
 __global__ void __launch_bounds__(kFrontThreads, NV == 0 ? 1 : (NV <= 2 ? 3 : 2))
 front_kernel(const FrontArgs a) {

@@ -109,8 +109,9 @@ struct ZRow {            // all pre-activations of the row; position = feature i
 };
 struct CandRow {         // per-tile candidates of the fused encode epilogue, their keys staged in shared memory.
   // The id of a candidate is its POSITION in the row's candidate array: positions run tile by tile, and inside a
-  // tile by decreasing value with the lower column first among equal values, so among equal keys position order
-  // is feature-id order -- the tie rule -- and the feature ids are fetched for the k winners only.
+  // tile by column, or, where the epilogue had to sort, by decreasing value.  Either way equal values stand with the
+  // lower column first, so among equal keys position order is feature-id order -- the tie rule -- and the feature ids are
+  // fetched for the k winners only.
   const unsigned* key_s;
   int n;
   __device__ __forceinline__ unsigned key(int i) const { return key_s[i]; }
