@@ -258,6 +258,8 @@ def test_padding_rows_of_a_tile_are_zero():
     assert np.array_equal(z[5:, :S], np.broadcast_to(b, (123, S)))
     assert not np.array_equal(z[:5, :S], np.broadcast_to(b, (5, S)))
     m.destroy()
+
+
 # k-blocks of a tile with every remainder of the producers' turns, several tiles a CTA (S / 256 = 300 tiles and more), on the rings
 # of three to six stages that full tiles have: bf16 on single CTAs (100 rows) and pairs (200), and both 8-bit forms
 @pytest.mark.parametrize("k_blocks", [1, 2, 3, 4, 5, 7, 8])
@@ -289,7 +291,7 @@ def test_topk_of_values_that_tie_or_crowd(S, kind):
     w = _workload(d, S, T, W.SAE_TOPK, False, k=k)
     g = torch.Generator(device="cuda"); g.manual_seed(S)
     sw = w.groups[0]
-    sw.W_enc[:] = 0                                             # z[t, j] = 8 hidden[t, j % 8] * step[j] + bias[j], all exact
+    sw.W_enc[:] = 0                                             # z[t, j] = hidden[t, j % 8] * level[j] + bias[j], all exact
     cols = torch.arange(S, device="cuda")
     if kind == "zeros":
         level = torch.where(torch.rand(S, generator=g, device="cuda") < 0.004, 1.0, 0.0)
