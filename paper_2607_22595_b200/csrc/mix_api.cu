@@ -927,7 +927,8 @@ int apply_impl(mix_ctx* c, void* hidden, int T, float* scores_out, void* stream,
   // Neither where an SAE app is gated on a score that this call writes for another row: there the hook kernels run in front of the
   // front kernel, which decides such a gate on the new score.  Beside them it would find some scores written and some not, and its
   // CTAs, each of which works out the routing of a call of up to 1024 rows for itself, could come to different routings.
-  const bool in_order = sae_gates_look_across(c, scores_out, T);
+  // (With chains that is the order of every call.)
+  const bool in_order = !(c->cfg.flags & MIX_FLAG_SLOT_CHAINS) && sae_gates_look_across(c, scores_out, T);
   const bool small = c->cfg.T_max <= kTeamMaxRows || (c->cfg.flags & MIX_FLAG_SLOT_CHAINS);
   const bool fork = c->cfg.n_groups_max > 0 && !c->stage_events_on && !small && !in_order;
   cudaStream_t ps = fork ? c->side_stream : s;

@@ -250,7 +250,7 @@ def test_router_logit_steering_matches_oracle_and_leaves_hidden_alone():
 
 
 @pytest.mark.parametrize("T_max,T", [(64, 64), (1000, 1000), (1500, 1500), (2600, 600), (2600, 2600)])
-@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("graph", [False, True, "conditional"])
 def test_an_sae_app_gated_on_a_score_that_the_same_call_writes_for_the_row_in_front(T_max, T, graph):
     """It is decided on the new score, as behind a call for the probes alone; the buffer holds the opposite decisions."""
     import paper_2607_22595_b200 as mixlib
@@ -285,7 +285,7 @@ def test_an_sae_app_gated_on_a_score_that_the_same_call_writes_for_the_row_in_fr
                 if graph:
                     gr = torch.cuda.CUDAGraph()
                     with torch.cuda.graph(gr, stream=s):
-                        m.apply(x, scores, T=T, stream=s)
+                        (m.apply_conditional if graph == "conditional" else m.apply)(x, scores, T=T, stream=s)
                     gr.replay()
                 else:
                     m.apply(x, scores, T=T, stream=s)
